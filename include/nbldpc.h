@@ -218,7 +218,10 @@ int nbldpc_decode_batch(const nbldpc_job *jobs, int n_jobs, void *workspace_dev,
  * for GF(128) and GF(256) codes.  nbldpc_code_create picks a default variant
  * per field order and a frames-per-block value from the code size;
  * nbldpc_code_autotune measures every valid pair on the caller's frames and
- * keeps the fastest.
+ * keeps the fastest.  A batch of too few frames to fill the GPU this way (how
+ * few depends on the code, the message width and early_stop; minimal schedule)
+ * decodes each frame on a cluster of 2..16 blocks, with the same outputs and no
+ * message slots, unless nbldpc_code_set_tuning has pinned the launch shape.
  */
 typedef struct nbldpc_tune_result {
   int variant;
@@ -228,8 +231,8 @@ typedef struct nbldpc_tune_result {
 
 int nbldpc_code_get_tuning(const nbldpc_code *code, int *variant, int *frames_per_block);
 
-/* Set the tuning by hand (variant 0..7, frames_per_block 1, 2, 4 or 8); NBLDPC_ERR_UNSUPPORTED if
- * that pair does not fit the device or the code.  Not concurrent with any other call on the same
+/* Set the tuning by hand (variant 0..7, frames_per_block 1, 2, 4 or 8), for batches of every size;
+ * NBLDPC_ERR_UNSUPPORTED if that pair does not fit the device or the code.  Not concurrent with any other call on the same
  * handle (a decode reads the tuning).  Switching a code to 16-bit messages or to the Table 1
  * schedule keeps bit 0 of its variant only. */
 int nbldpc_code_set_tuning(nbldpc_code *code, int variant, int frames_per_block);

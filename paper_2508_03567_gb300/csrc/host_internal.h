@@ -61,6 +61,9 @@ struct nbldpc_code {
   unsigned long long* work_counter = nullptr;   // device counter of visited convolution pairs (optional)
   int mb = 1;                          // message bytes per symbol (1: 8-bit messages, 2: 16-bit)
   int cnp_schedule = NBLDPC_CNP_MINIMAL;   // check-node convolutions: 3(d-2) or Table 1's 3d-4
+  int split_max = 0;                   // largest cluster of the split-frame kernel (0: not for this code's mode)
+  int smem_optin = 0;                  // shared memory a block may take
+  bool pinned = false;                 // the launch shape was set by nbldpc_code_set_tuning: every batch takes it
   nbldpc_host::Plan plan{};            // single-code launch shape (fpb chosen by default or by the autotuner)
   int fft_status = NBLDPC_ERR_UNSUPPORTED;   // FFT-SPA launch shape below valid when NBLDPC_OK
   int fft_dc = 0, fft_dv = 0;          // FFT-SPA check-node form (dc 0: lane per edge) and column-degree bucket

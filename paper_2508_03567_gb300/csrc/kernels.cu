@@ -63,4 +63,14 @@ const void* NBLDPC_CAT(kernel_q, NBLDPC_KQ)(int v, int mb, int t1, int dreg) {
 #endif
 }
 
+#if NBLDPC_KQ > 0
+// Address of the kernel that decodes a frame on a cluster of blocks, for mb-byte
+// messages (minimal schedule): the layout and the convolutions of the default variant.
+const void* NBLDPC_CAT(split_kernel_q, NBLDPC_KQ)(int mb) {
+  constexpr int Q = NBLDPC_KQ, V = (Q >= 16 && Q <= 64) ? 1 : 0;
+  return mb == 2 ? reinterpret_cast<const void*>(&mma_split_kernel<Q, V, 2, false>)
+                 : reinterpret_cast<const void*>(&mma_split_kernel<Q, V, 1, (Q >= 128)>);
+}
+#endif
+
 }  // namespace nbldpc

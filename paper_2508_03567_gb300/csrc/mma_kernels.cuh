@@ -760,6 +760,34 @@ __device__ __forceinline__ bool decode_frame_warp4(const JobDesc& job, int frame
   return true;
 }
 
+// ---------------------------------------------------------------- one frame on several SMs
+// A thread-block cluster decodes one frame: rank k of the cluster owns the
+// checks [k * cpc, (k + 1) * cpc) with the message rows of their edges, and the
+// columns [k * npc, (k + 1) * npc) with their reliabilities and decisions, all
+// in its shared memory.  The check-node pass is local to a rank; the variable-
+// node pass and the syndrome reach the other ranks' rows and decisions through
+// distributed shared memory, with one cluster barrier after each pass.
+struct SplitCtx {
+  int rank, size;
+  int r0, r1, n0, n1;         // the rank's checks and columns
+  int e0;                     // first edge of the rank's checks
+  int npc;                    // columns per rank
+  const uint8_t* gam;         // the rank's reliability rows (shared memory)
+  uint8_t* const* vrow;       // message row of each edge of the rank's columns, in column order
+  int* flags;                 // [2][kMaxSplit] syndrome flags of the ranks
+};
+constexpr int kMaxSplit = 16;
+
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+// address of this rank's shared-memory object p in rank r's shared memory
+template <class T> __device__ __forceinline__ T* at_rank(T* p, int r) {
+  uint64_t d;
+  asm("mapa.u64 %0, %1, %2;" : "=l"(d) : "l"(p), "r"(r));
+  return reinterpret_cast<T*>(d);
+}
+
 // ---------------------------------------------------------------- one frame
 // Decodes frame `frame` of `job` with the nthr threads of one frame slot
 // (slot thread index stid, named barrier bar_id).  sblob holds the job's code
@@ -771,10 +799,13 @@ __device__ __forceinline__ bool decode_frame_warp4(const JobDesc& job, int frame
 // schedule).  W4: a GF(4) frame slot of one warp may take the one-warp form
 // (decode_frame_warp4; resident-message kernels, which have the registers for it).
 // D > 0: every check of the code has degree D (a compile-time loop bound and
-// vector layout; 0: the degrees are read per check).
-template <class g, int MB, bool T1, bool REG4 = true, bool PR = false, bool W4 = false, int D = 0>
-__device__ __forceinline__ void decode_frame(const JobDesc& job, int frame, uint8_t* X, const unsigned char* sblob,
-                                             uint8_t* chat, unsigned char* scratch, int stid, int nthr, int bar_id) {
+// vector layout; 0: the degrees are read per check).  SP: the threads are those of
+// one rank of a cluster that decodes the frame together (sc; X then holds the
+// message rows of the rank's own edges).
+template <class g, int MB, bool T1, bool REG4 = true, bool PR = false, bool W4 = false, int D = 0, bool SP = false>
+__device__ __forceinline__ void decode_frame(const JobDesc& job, int frame, uint8_t* Xown, const unsigned char* sblob,
+                                             uint8_t* chat, unsigned char* scratch, int stid, int nthr, int bar_id,
+                                             const SplitCtx* sc = nullptr) {
   constexpr int Q = g::Q;
   constexpr int PW = g::PW;
   constexpr int RS = Q * MB;                 // bytes of one message row
@@ -783,7 +814,7 @@ __device__ __forceinline__ void decode_frame(const JobDesc& job, int frame, uint
   static_assert(!PR || (g::G == 32 && MB == 1 && !T1), "pruned convolutions: 32-lane groups, 8-bit, minimal");
   if constexpr (Q == 4 && MB == 1 && !T1 && REG4 && W4) {
     // one warp per frame: a slot of 32 threads
-    if (nthr == 32 && decode_frame_warp4<D == 4 ? 4 : 0>(job, frame, X, sblob, stid)) return;
+    if (nthr == 32 && decode_frame_warp4<D == 4 ? 4 : 0>(job, frame, Xown, sblob, stid)) return;
   }
   // pairs (x, y) the convolutions visit in this frame (counted when job.work is set)
   const bool counting = job.work != nullptr;
@@ -839,6 +870,27 @@ __device__ __forceinline__ void decode_frame(const JobDesc& job, int frame, uint
   // B ping-pong = vec(2 dmax - 2), vec(2 dmax - 1), R = vec(2 dmax)
   const int vF = dm - 1, vB = 2 * dm - 2, vR = 2 * dm;
   const uint8_t* gam = job.gamma + (size_t)frame * job.n * Q;
+  // rows are addressed by edge number: a rank's area starts with the row of its first edge
+  uint8_t* X = SP ? Xown - (ptrdiff_t)sc->e0 * RS : Xown;
+  const int r_first = SP ? sc->r0 : 0, r_last = SP ? sc->r1 : job.m;
+  const int n_first = SP ? sc->n0 : 0, n_last = SP ? sc->n1 : job.n;
+  // reliabilities of the columns of the variable-node pass, message row of entry k of
+  // the column-ordered edge list, decision of column c
+  const uint8_t* vgam = SP ? sc->gam - (ptrdiff_t)n_first * Q : gam;
+  const int k_first = SP ? vn_ptr[n_first] : 0;
+  auto vn_row = [&](int k) -> uint8_t* {
+    if constexpr (SP) return sc->vrow[k - k_first];
+    else return X + (size_t)vn_edge[k] * RS;
+  };
+  auto decision = [&](int c) -> int {
+    if constexpr (SP) return *at_rank(chat + c, c / sc->npc);
+    else return chat[c];
+  };
+  // end of a pass: its messages and decisions are visible to every thread of the frame
+  auto pass_sync = [&]() {
+    if constexpr (SP) cluster_barrier();
+    else slot_sync(bar_id, nthr);
+  };
 
     // ---- variable-node pass (Alg. 2, VNP and hard decision):
     //   S(a) = gamma(a) + sum over edges of beta(a);  c = argmin S (lowest a)
@@ -849,15 +901,15 @@ __device__ __forceinline__ void decode_frame(const JobDesc& job, int frame, uint
     // 16-bit messages: the same pass on 32-bit sums, one symbol per register
     auto vnp_wide = [&](bool first, bool want_alpha) {
       constexpr int NB = VBPL;
-      for (int vn = vgrp; vn < job.n; vn += nvgroups) {
+      for (int vn = n_first + vgrp; vn < n_last; vn += nvgroups) {
         int S[NB];
-        const uint8_t* gr = gam + (size_t)vn * Q + vgl * NB;
+        const uint8_t* gr = vgam + (ptrdiff_t)vn * Q + vgl * NB;
 #pragma unroll
         for (int i = 0; i < NB; ++i) S[i] = gr[i];
         const int k0 = vn_ptr[vn], k1 = vn_ptr[vn + 1];
         if (!first) {
           for (int k = k0; k < k1; ++k) {
-            const uint16_t* br = reinterpret_cast<const uint16_t*>(X + (size_t)vn_edge[k] * RS) + vgl * NB;
+            const uint16_t* br = reinterpret_cast<const uint16_t*>(vn_row(k)) + vgl * NB;
 #pragma unroll
             for (int i = 0; i < NB; ++i) S[i] += br[i];
           }
@@ -869,7 +921,7 @@ __device__ __forceinline__ void decode_frame(const JobDesc& job, int frame, uint
         if (vgl == 0) chat[vn] = (uint8_t)(key & 0xFF);
         if (!first && want_alpha) {
           for (int k = k0; k < k1; ++k) {
-            uint16_t* row = reinterpret_cast<uint16_t*>(X + (size_t)vn_edge[k] * RS) + vgl * NB;
+            uint16_t* row = reinterpret_cast<uint16_t*>(vn_row(k)) + vgl * NB;
             int t[NB];
             int mn = 0x7FFFFFFF;
 #pragma unroll
@@ -884,8 +936,7 @@ __device__ __forceinline__ void decode_frame(const JobDesc& job, int frame, uint
 
     // 16-bit messages start from alpha^(0) = gamma widened into every edge row
     auto init_wide = [&]() {
-      const int nnz = row_ptr[job.m];
-      for (int i = stid; i < nnz * Q; i += nthr) {
+      for (int i = row_ptr[r_first] * Q + stid; i < row_ptr[r_last] * Q; i += nthr) {
         const int e = i / Q, a = i % Q;
         reinterpret_cast<uint16_t*>(X)[i] = gam[(size_t)edge_col[e] * Q + a];
       }
@@ -894,17 +945,17 @@ __device__ __forceinline__ void decode_frame(const JobDesc& job, int frame, uint
     // q <= 16 with every variable node in one pass of the slot's lanes: each lane
     // keeps its node's gamma words in registers from the first pass on (the later
     // passes then start without a global-memory load)
-    const bool gamma_regs = kGammaRegs && job.n <= nvgroups;
+    const bool gamma_regs = kGammaRegs && n_last - n_first <= nvgroups;
     auto vnp = [&](bool first, bool want_alpha) {
       // symbol values of this lane's packed words: (a, a + 1), a = vgl * VBPL + 2 i
       const uint32_t vsym0 = (uint32_t)(vgl * VBPL) * 0x10001u + 0x10000u;
-      for (int vn = vgrp; vn < job.n; vn += nvgroups) {
+      for (int vn = n_first + vgrp; vn < n_last; vn += nvgroups) {
         uint32_t S[VW];
         if (gamma_regs && !first) {
 #pragma unroll
           for (int i = 0; i < VW; ++i) S[i] = gcache[i];
         } else {
-          load_pairs<VBPL>(gam + (size_t)vn * Q + vgl * VBPL, S);
+          load_pairs<VBPL>(vgam + (ptrdiff_t)vn * Q + vgl * VBPL, S);
           if (gamma_regs) {
 #pragma unroll
             for (int i = 0; i < VW; ++i) gcache[i] = S[i];
@@ -914,7 +965,7 @@ __device__ __forceinline__ void decode_frame(const JobDesc& job, int frame, uint
         if (!first) {
           for (int k = k0; k < k1; ++k) {
             uint32_t b[VW];
-            load_pairs<VBPL>(X + (size_t)vn_edge[k] * Q + vgl * VBPL, b);
+            load_pairs<VBPL>(vn_row(k) + vgl * VBPL, b);
 #pragma unroll
             for (int i = 0; i < VW; ++i) S[i] += b[i];
           }
@@ -940,7 +991,7 @@ __device__ __forceinline__ void decode_frame(const JobDesc& job, int frame, uint
         }
         if (!first && want_alpha) {
           for (int k = k0; k < k1; ++k) {
-            uint8_t* row = X + (size_t)vn_edge[k] * Q + vgl * VBPL;
+            uint8_t* row = vn_row(k) + vgl * VBPL;
             uint32_t t[VW];
             load_pairs<VBPL>(row, t);
 #pragma unroll
@@ -959,18 +1010,26 @@ __device__ __forceinline__ void decode_frame(const JobDesc& job, int frame, uint
       }
     };
 
-    // ---- syndrome of chat over all checks (slot-wide)
+    // ---- syndrome of chat over all checks (slot-wide, cluster-wide for SP)
+    int flag_set = 0;
     auto syndrome_ok = [&]() -> bool {
       int bad = 0;
-      for (int r = stid; r < job.m; r += nthr) {
+      for (int r = r_first + stid; r < r_last; r += nthr) {
         int sy = 0;
         for (int e = row_ptr[r]; e < row_ptr[r + 1]; ++e) {
-          const int c = chat[edge_col[e]];
+          const int c = decision(edge_col[e]);
           if (c) sy ^= exp2[glog[c] + edge_lh[e]];
         }
         bad |= sy;
       }
-      return slot_sync_or(bar_id, nthr, bad) == 0;
+      bad = slot_sync_or(bar_id, nthr, bad);
+      if constexpr (SP) {      // every rank's flag to every rank; two sets, so that a late reader's stays
+        if (stid < sc->size) at_rank(sc->flags + flag_set * kMaxSplit + sc->rank, stid)[0] = bad;
+        cluster_barrier();
+        for (int k = 0; k < sc->size; ++k) bad |= sc->flags[flag_set * kMaxSplit + k];
+        flag_set ^= 1;
+      }
+      return bad == 0;
     };
 
     // ---- check-node pass (Alg. 2, F & B matrices and beta), one group per check
@@ -1014,7 +1073,7 @@ __device__ __forceinline__ void decode_frame(const JobDesc& job, int frame, uint
       }
     };
     auto cnp = [&](bool first) {
-      for (int r = grp; r < job.m; r += ngroups) {
+      for (int r = r_first + grp; r < r_last; r += ngroups) {
         const int e0 = row_ptr[r], d = D > 0 ? D : row_ptr[r + 1] - e0;
         if constexpr (kScatter) {
           for (int c = gl; c < d * CH; c += g::G) scatter_piece(first, e0, c);
@@ -1138,7 +1197,7 @@ __device__ __forceinline__ void decode_frame(const JobDesc& job, int frame, uint
                              (uint32_t)((((i3 >> 1) << 2) | ((i3 & 1) << 1)) << 12);
         *reinterpret_cast<uint32_t*>(X + (size_t)e * 4) = __byte_perm(R.x, R.y, sel);
       };
-      for (int r = stid; r < job.m; r += nthr) {
+      for (int r = r_first + stid; r < r_last; r += nthr) {
         const int e0 = row_ptr[r], d = row_ptr[r + 1] - e0;
         if (counting && d > 2) work += 16ull * 3 * (d - 2);
         // The last P and F are tracked as the loops run (Plast = P_{d-1}, Flast =
@@ -1188,13 +1247,13 @@ __device__ __forceinline__ void decode_frame(const JobDesc& job, int frame, uint
     // tested, so the stop test runs once, after the last iteration.
     const bool es = job.early_stop != 0;
     if constexpr (MB == 2) vnp_wide(true, false); else vnp(true, false);   // c^(0) = argmin gamma
-    slot_sync(bar_id, nthr);
+    pass_sync();
     bool ok = (es || job.max_iters == 0) ? syndrome_ok() : false;
     int iters = 0;
     if (!(es && ok)) {
       if constexpr (MB == 2) {
         init_wide();
-        slot_sync(bar_id, nthr);
+        pass_sync();
       }
       for (int k = 1; k <= job.max_iters; ++k) {
         if constexpr (Q == 4 && MB == 1 && !T1 && REG4) {
@@ -1202,17 +1261,17 @@ __device__ __forceinline__ void decode_frame(const JobDesc& job, int frame, uint
         } else {
           cnp(MB == 1 && k == 1);
         }
-        slot_sync(bar_id, nthr);
+        pass_sync();
         if constexpr (MB == 2) vnp_wide(false, k < job.max_iters); else vnp(false, k < job.max_iters);
-        slot_sync(bar_id, nthr);
+        pass_sync();
         iters = k;
         if (es || k == job.max_iters) ok = syndrome_ok();
         if (es && ok) break;
       }
     }
-    for (int i = stid; i < job.n; i += nthr) job.out_sym[(size_t)frame * job.n + i] = chat[i];
+    for (int i = n_first + stid; i < n_last; i += nthr) job.out_sym[(size_t)frame * job.n + i] = chat[i];
     if (counting && work) atomicAdd(job.work, work);
-    if (stid == 0) {
+    if (stid == 0 && (!SP || sc->rank == 0)) {
       job.out_iters[frame] = iters;
       job.out_ok[frame] = ok ? 1 : 0;
     }
@@ -1323,6 +1382,70 @@ __global__ void __launch_bounds__(XS ? kResidentThreads : 256, XS ? 2 : PR ? NBL
     }
     slot_sync(bar_id, nthr);
   }
+}
+
+// ---------------------------------------------------------------- the kernel of split frames
+// One cluster per frame (grid: frames * cluster size).  Shared memory of a rank:
+// code blob | decisions (n_cap bytes, indexed by column) | flags | row table |
+// reliabilities of its columns | check-node scratch | message rows of its edges.
+struct SplitParams {
+  JobDesc job;
+  int size;                   // ranks per frame
+  int cpc, npc;               // checks and columns per rank
+  int chat_off, flag_off, row_off, gam_off, scratch_off, x_off;
+};
+
+template <int Q, int V, int MB, bool PR>
+__global__ void __launch_bounds__(kResidentThreads, 2) mma_split_kernel(const __grid_constant__ SplitParams p) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  constexpr int RS = Q * MB;
+  const JobDesc& job = p.job;
+  const int tid = threadIdx.x, nthr = blockDim.x;
+  const int rank = blockIdx.x % p.size, frame = blockIdx.x / p.size;
+  unsigned char* sblob = smem;
+  for (int i = tid; i < job.off.bytes / 16; i += nthr)
+    reinterpret_cast<uint4*>(sblob)[i] = reinterpret_cast<const uint4*>(job.blob)[i];
+  SplitCtx sc;
+  sc.rank = rank;
+  sc.size = p.size;
+  sc.r0 = min(rank * p.cpc, job.m);
+  sc.r1 = min(sc.r0 + p.cpc, job.m);
+  sc.n0 = min(rank * p.npc, job.n);
+  sc.n1 = min(sc.n0 + p.npc, job.n);
+  sc.npc = p.npc;
+  sc.flags = reinterpret_cast<int*>(smem + p.flag_off);
+  uint8_t** vrow = reinterpret_cast<uint8_t**>(smem + p.row_off);
+  sc.vrow = vrow;
+  uint8_t* sgam = smem + p.gam_off;
+  sc.gam = sgam;
+  // reliabilities of the rank's columns (rows of q bytes; 4-byte words when q >= 4: gamma is 16-byte aligned)
+  {
+    const uint8_t* src = job.gamma + ((size_t)frame * job.n + sc.n0) * Q;
+    const int bytes = (sc.n1 - sc.n0) * Q;
+    if constexpr (Q >= 16) {
+      for (int i = tid; i < bytes / 16; i += nthr)
+        reinterpret_cast<uint4*>(sgam)[i] = reinterpret_cast<const uint4*>(src)[i];
+    } else if constexpr (Q >= 4) {
+      for (int i = tid; i < bytes / 4; i += nthr)
+        reinterpret_cast<uint32_t*>(sgam)[i] = reinterpret_cast<const uint32_t*>(src)[i];
+    } else {
+      for (int i = tid; i < bytes; i += nthr) sgam[i] = src[i];
+    }
+  }
+  __syncthreads();
+  const uint16_t* row_ptr = reinterpret_cast<const uint16_t*>(sblob + job.off.row_ptr);
+  const uint16_t* vn_ptr = reinterpret_cast<const uint16_t*>(sblob + job.off.vn_ptr);
+  const uint16_t* vn_edge = reinterpret_cast<const uint16_t*>(sblob + job.off.vn_edge);
+  const uint16_t* edge_row = reinterpret_cast<const uint16_t*>(job.blob + job.off.edge_row);
+  sc.e0 = row_ptr[sc.r0];
+  uint8_t* X = smem + p.x_off;
+  for (int k = vn_ptr[sc.n0] + tid; k < vn_ptr[sc.n1]; k += nthr) {
+    const int e = vn_edge[k], owner = edge_row[e] / p.cpc;
+    vrow[k - vn_ptr[sc.n0]] = at_rank(X, owner) + (size_t)(e - row_ptr[owner * p.cpc]) * RS;
+  }
+  cluster_barrier();           // the row table is complete, and every rank of the cluster runs
+  decode_frame<Geo<Q, V>, MB, false, true, PR, false, 0, true>(job, frame, X, sblob, smem + p.chat_off,
+                                                               smem + p.scratch_off, tid, nthr, 1, &sc);
 }
 
 }  // namespace nbldpc

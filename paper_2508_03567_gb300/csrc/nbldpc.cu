@@ -5,6 +5,7 @@
 // of the min-max kernels.  FFT-SPA decodes are in fftspa_host.cu.
 #include "nbldpc.h"
 
+#include <algorithm>
 #include <cstdio>
 #include <cstring>
 #include <new>
@@ -60,6 +61,14 @@ const void* kernel_q32(int v, int mb, int t1, int dreg);
 const void* kernel_q64(int v, int mb, int t1, int dreg);
 const void* kernel_q128(int v, int mb, int t1, int dreg);
 const void* kernel_q256(int v, int mb, int t1, int dreg);
+const void* split_kernel_q2(int mb);
+const void* split_kernel_q4(int mb);
+const void* split_kernel_q8(int mb);
+const void* split_kernel_q16(int mb);
+const void* split_kernel_q32(int mb);
+const void* split_kernel_q64(int mb);
+const void* split_kernel_q128(int mb);
+const void* split_kernel_q256(int mb);
 }  // namespace nbldpc
 
 namespace {
@@ -91,6 +100,21 @@ const void* kernel_for(int q, int v, int km, int dreg = 0) {
 // the regular check degree that selects a specialised kernel (see kernel_for), else 0
 int kernel_dreg(int q, int v, int km, int dreg) {
   return ((q == 64 || q == 4) && km == 1 && v >= 2 && v <= 3 && dreg == 4) ? 4 : 0;
+}
+
+// kernel that decodes a frame on a cluster of blocks (minimal schedule)
+const void* split_kernel_for(int q, int mb) {
+  switch (q) {
+    case 2: return nbldpc::split_kernel_q2(mb);
+    case 4: return nbldpc::split_kernel_q4(mb);
+    case 8: return nbldpc::split_kernel_q8(mb);
+    case 16: return nbldpc::split_kernel_q16(mb);
+    case 32: return nbldpc::split_kernel_q32(mb);
+    case 64: return nbldpc::split_kernel_q64(mb);
+    case 128: return nbldpc::split_kernel_q128(mb);
+    case 256: return nbldpc::split_kernel_q256(mb);
+  }
+  return nullptr;
 }
 
 template <int Q> int lanes(int v) { return v ? nbldpc::Geo<Q, 1>::G : nbldpc::Geo<Q, 0>::G; }
@@ -148,6 +172,40 @@ int prepare_kernel(int q, int v, int km, int dreg, int dev, int smem_optin) {
     done = true;
   }
   return NBLDPC_OK;
+}
+
+// Largest cluster of split-frame blocks (16, else the portable 8) that the device
+// runs for a field order and message width; 0 when the kernel cannot be prepared.
+// The kernel attributes are set and the device asked once.
+int g_split_max[64][8][2] = {};
+
+int split_max(int q, int mb, int dev, int smem_optin) {
+  std::lock_guard<std::mutex> lk(g_attr_mu);
+  if (dev < 0 || dev >= 64) return 0;
+  int& mx = g_split_max[dev][nbldpc::ilog2(q) - 1][mb - 1];
+  if (mx == 0) {
+    const void* k = split_kernel_for(q, mb);
+    mx = -1;
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_optin) == cudaSuccess) {
+      mx = 8;
+      cudaLaunchConfig_t cfg{};
+      cudaLaunchAttribute at{};
+      at.id = cudaLaunchAttributeClusterDimension;
+      at.val.clusterDim.x = nbldpc::kMaxSplit;
+      at.val.clusterDim.y = at.val.clusterDim.z = 1;
+      cfg.gridDim = dim3(nbldpc::kMaxSplit);
+      cfg.blockDim = dim3(nbldpc::kResidentThreads);
+      cfg.dynamicSmemBytes = (size_t)smem_optin;
+      cfg.attrs = &at;
+      cfg.numAttrs = 1;
+      int n = 0;
+      if (cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+          cudaOccupancyMaxActiveClusters(&n, k, &cfg) == cudaSuccess && n >= 1)
+        mx = nbldpc::kMaxSplit;
+      cudaGetLastError();      // a refused query is not a later call's error
+    }
+  }
+  return mx < 0 ? 0 : mx;
 }
 
 struct CodeNeeds {       // what one code asks of a frame slot
@@ -243,6 +301,11 @@ int configure(nbldpc_code* c, int variant, int fpb) {
   if (st != NBLDPC_OK) return st;
   c->variant = variant;
   c->plan = pl;
+  int optin = 0;
+  c->split_max = 0;
+  if (kmode(c) != 3 && cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device) == cudaSuccess)
+    c->split_max = split_max(c->q, c->mb, c->device, optin);
+  c->smem_optin = optin;
   return NBLDPC_OK;
 }
 
@@ -300,9 +363,117 @@ int launch_plan(const void* kernel, const Plan& pl, nbldpc::LaunchParams& lp, in
   return NBLDPC_OK;
 }
 
+// ---- frames split over the blocks of a cluster ------------------------------
+// Shape of a split launch: ranks per frame, threads per rank, shared memory of a rank.
+struct SplitShape {
+  int size = 0, threads = 0, smem = 0;
+  nbldpc::SplitParams p{};
+};
+
+int split_layout_variant(int q) { return (q >= 16 && q <= 64) ? 1 : 0; }   // kernels.cu: split_kernel_q*
+
+// Lay out a rank's shared memory; size 0 when it does not fit the device.
+SplitShape split_layout(const nbldpc_code* c, int size, int threads) {
+  SplitShape s;
+  const int G = group_lanes(c->q, split_layout_variant(c->q));
+  s.p.size = size;
+  s.p.cpc = (c->m + size - 1) / size;
+  s.p.npc = (c->n + size - 1) / size;
+  const long long edges_r = std::min<long long>(c->nnz, (long long)s.p.cpc * c->dmax);
+  const long long edges_n = std::min<long long>(c->nnz, (long long)s.p.npc * c->vmax);
+  size_t o = c->off.bytes;
+  auto take = [&](size_t bytes) { const size_t at = o; o = round_up(o + bytes, 16); return (int)at; };
+  s.p.chat_off = take((size_t)c->n);
+  s.p.flag_off = take(2 * nbldpc::kMaxSplit * sizeof(int));
+  s.p.row_off = take((size_t)edges_n * sizeof(void*));
+  s.p.gam_off = take((size_t)s.p.npc * c->q);
+  s.p.scratch_off = take((size_t)(threads / G) * group_bytes(c->q, c->dmax, c->mb));
+  s.p.x_off = take((size_t)edges_r * c->q * c->mb);
+  if (o > (size_t)c->smem_optin) return SplitShape{};
+  s.size = size;
+  s.threads = threads;
+  s.smem = (int)o;
+  return s;
+}
+
+// Threads of the split-frame blocks of one shape that an SM holds (80 registers a thread).
+int split_resident(const nbldpc_code* c, const SplitShape& s) {
+  const int by_smem = (c->smem_optin + 1024) / (s.smem + 1024), by_regs = 65536 / (80 * s.threads);
+  return std::min(by_smem, by_regs) * s.threads;
+}
+
+// The split shape of a batch, or size 0 for the one-block-per-frame kernels.
+//
+// One block per frame leaves SMs idle below their number, and with early stop
+// it leaves them idle at the end of a batch, when the last frames run all their
+// iterations (a GF(64) N=576 frame: 58 us an iteration on one SM, 9.5 us on
+// 16).  Measured on GB300, us per decode of up to 20 or 30 iterations, one
+// block per frame against this rule: GF(64) N=576, 1 / 96 / 200 / 1000 frames
+// 1103 / 1158 / 1937 / 3721 against 180 / 481 / 846 / 3299; GF(256) (2,6) N=384,
+// 1 / 96 / 200 frames 7328 / 7818 / 9626 against 689 / 3498 / 8051; GF(256) (2,8)
+// N=128, 17 frames 3939 against 1217; GF(16) N=1024, 1 / 200 / 1000 frames
+// 837 / 882 / 1613 against 161 / 432 / 1436; GF(8) N=512, 1 / 200 frames 225 / 256
+// against 113 / 183.
+//  - More ranks and threads for fewer frames, so that the SMs are filled and the
+//    frame's chain of passes is as short as they allow.
+//  - No more 128-thread ranks than the frame has check-node lanes for.
+//  - q <= 4 stays (the check-node pass there is shorter than a cluster barrier).
+//  - Up to twice the frames that the one-block kernels hold at once when frames
+//    stop early (beyond it the tail is short and the ranks' barriers cost 2-5 %);
+//    half of them where the ranks fill an SM less than three quarters as full
+//    (GF(256): 400 frames of N=384 12.9 ms against 15.6) or q = 8; a third when
+//    every frame runs the same iterations (no tail: 1000 frames 7.1 ms against 7.7).
+//  - 16-bit messages: half of them from q = 64 (200 frames 2.9 against 2.3 ms; 1000
+//    frames 5.1 against 10.0), else a quarter (GF(16): 48 frames 1.72 against 0.89 ms,
+//    200 frames 1.93 against 2.11).
+SplitShape split_shape(const nbldpc_code* c, int frames, int early_stop) {
+  if (c->split_max == 0 || c->pinned || c->q <= 4) return SplitShape{};
+  const long long slots = (long long)c->plan.grid_max * c->plan.fpb;
+  if (frames > 2 * slots) return SplitShape{};
+  const int sms = c->plan.grid_max / c->plan.per_sm;
+  const int G = group_lanes(c->q, split_layout_variant(c->q));
+  int size = frames <= sms / 8 ? 16 : 8;
+  int threads = frames <= 3 * sms / 8 ? 384 : frames <= 3 * sms / 4 ? 256 : 128;
+  size = std::min(size, c->split_max);
+  while (size > 2 && (long long)size * 128 > (long long)c->m * G * 5 / 4) size /= 2;
+  const int cpc = (c->m + size - 1) / size;
+  threads = std::min(threads, std::max(128, (int)round_up((size_t)cpc * G, 32)));
+  SplitShape s = split_layout(c, size, threads);
+  while (s.size == 0 && threads > 64) s = split_layout(c, size, threads = (threads - 1) / 64 * 64);
+  if (s.size == 0) return s;
+  long long most = early_stop ? 2 * slots : slots / 3;
+  if (c->mb == 2) most = std::min(most, c->q >= 64 ? slots / 2 : slots / 4);
+  else if (c->q == 8 || 4 * split_resident(c, s) < 3 * c->plan.per_sm * c->plan.threads) most = std::min(most, slots / 2);
+  return frames <= most ? s : SplitShape{};
+}
+
+int launch_split(const nbldpc_code* c, SplitShape& s, const nbldpc::JobDesc& job, cudaStream_t st) {
+  s.p.job = job;
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = (unsigned)s.size;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.gridDim = dim3((unsigned)job.frames * (unsigned)s.size);
+  cfg.blockDim = dim3((unsigned)s.threads);
+  cfg.dynamicSmemBytes = (size_t)s.smem;
+  cfg.stream = st;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  void* args[] = {&s.p};
+  if (cudaLaunchKernelExC(&cfg, split_kernel_for(c->q, c->mb), args) != cudaSuccess) return NBLDPC_ERR_CUDA;
+  g_launches.fetch_add(1, std::memory_order_relaxed);
+  return NBLDPC_OK;
+}
+
+// split: small batches may go to the split-frame kernel (not while the autotuner times a tuning)
 int launch(const nbldpc_code* c, const uint8_t* gamma, int frames, int max_iters, int early_stop, uint8_t* sym,
-           int32_t* iters, uint8_t* ok, void* ws, cudaStream_t st, bool count = true) {
+           int32_t* iters, uint8_t* ok, void* ws, cudaStream_t st, bool count = true, bool split = true) {
   if (frames == 0) return NBLDPC_OK;
+  if (split) {
+    SplitShape s = split_shape(c, frames, early_stop);
+    if (s.size) return launch_split(c, s, job_desc(c, gamma, frames, max_iters, early_stop, sym, iters, ok, 0, count), st);
+  }
   nbldpc::LaunchParams lp{};
   lp.jobs[0] = job_desc(c, gamma, frames, max_iters, early_stop, sym, iters, ok, 0, count);
   lp.njobs = 1;
@@ -352,6 +523,11 @@ int nbldpc_decode_noalloc(const nbldpc_code* c, const uint8_t* gamma_dev, int fr
   }
   st = cuda_status(cudaGetLastError());
   if (st != NBLDPC_OK) return st;
+  SplitShape sp = split_shape(c, frames, early_stop);
+  if (sp.size)
+    return launch_split(c, sp,
+                        job_desc(c, gamma_dev, frames, max_iters, early_stop, out_sym_dev, out_iters_dev, out_ok_dev, 0),
+                        reinterpret_cast<cudaStream_t>(cuda_stream));
   void* scratch = nullptr;
   st = noalloc_scratch(&scratch);
   if (st != NBLDPC_OK) return st;
@@ -550,7 +726,9 @@ int nbldpc_code_set_tuning(nbldpc_code* c, int variant, int frames_per_block) {
     return NBLDPC_ERR_ARG;
   const int st = check_device(c);
   if (st != NBLDPC_OK) return st;
-  return configure(c, variant, frames_per_block);
+  const int st2 = configure(c, variant, frames_per_block);
+  if (st2 == NBLDPC_OK) c->pinned = true;
+  return st2;
 }
 
 int nbldpc_code_set_message_bits(nbldpc_code* c, int bits) {
@@ -725,13 +903,13 @@ int nbldpc_code_autotune(nbldpc_code* c, const uint8_t* gamma_dev, int frames, i
       if (configure(c, v, fpb) != NBLDPC_OK) continue;
       // one untimed decode, then the fastest of kTuneReps timed decodes with fixed iterations
       // (pairs within 1-2 % of each other would otherwise swap places from run to run)
-      st = launch(c, gamma_dev, frames, max_iters, 0, sym, its, okb, dws, s, false);
+      st = launch(c, gamma_dev, frames, max_iters, 0, sym, its, okb, dws, s, false, false);
       if (st != NBLDPC_OK) break;
       float ms = 3.4e38f;
       for (int rep = 0; rep < kTuneReps && st == NBLDPC_OK; ++rep) {
         float t = 0.f;
         if (cudaEventRecord(e0, s) != cudaSuccess) { st = NBLDPC_ERR_CUDA; break; }
-        st = launch(c, gamma_dev, frames, max_iters, 0, sym, its, okb, dws, s, false);
+        st = launch(c, gamma_dev, frames, max_iters, 0, sym, its, okb, dws, s, false, false);
         if (st != NBLDPC_OK) break;
         if (cudaEventRecord(e1, s) != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess ||
             cudaEventElapsedTime(&t, e0, e1) != cudaSuccess) {

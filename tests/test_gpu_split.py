@@ -1,0 +1,85 @@
+"""GPU parity of the split-frame kernels: a small batch decodes each frame on a
+cluster of blocks (the rule is in split_shape, csrc/nbldpc.cu).  Bar: bit-exact
+against the oracle, and the same outputs as the one-block-per-frame kernels,
+which a handle with a pinned tuning (nbldpc_code_set_tuning) keeps."""
+import os
+
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2508_03567_gb300 import binding, inputs as I
+
+pytestmark = pytest.mark.gpu
+THREADS = os.cpu_count() or 4
+
+
+def irregular(q, n, m, seed, dmax):
+    """Rows of degree 2..dmax, every column used, random coefficients."""
+    rng = np.random.default_rng(seed)
+    h = np.zeros((m, n), np.int64)
+    for r in range(m):
+        h[r, rng.choice(n, int(rng.integers(2, dmax + 1)), replace=False)] = 1
+    for c in np.nonzero(~h.any(0))[0]:
+        h[int(rng.integers(m)), c] = 1
+    h *= rng.integers(1, q, h.shape)
+    return I.code_from_dense(h, q, I.PRIMITIVE_POLY[q])
+
+
+# fewer checks than ranks, rows and columns that do not divide by the ranks, ragged degrees
+CODES = [("tiny", 16, 8, 5), ("ragged", 8, 70, 33), ("ragged", 32, 61, 31), ("ragged", 64, 45, 19), ("ragged", 128, 30, 13),
+         ("ragged", 256, 26, 9), ("regular", 8, 64, 4), ("regular", 16, 100, 4), ("regular", 64, 576, 4),
+         ("regular", 256, 128, 8)]
+
+
+def make(kind, q, n, x):
+    if kind == "regular":
+        return I.make_regular_code(q, n, 2, x, seed=q + n)
+    return irregular(q, n, x, q + n, 4 if kind == "tiny" else 6)
+
+
+@pytest.mark.parametrize("bits", [8, 16])
+@pytest.mark.parametrize("kind,q,n,x", CODES)
+def test_small_batches_match_the_oracle_and_the_one_block_kernels(kind, q, n, x, bits):
+    code = make(kind, q, n, x)
+    rng = np.random.default_rng(3 * q + n)
+    dec, one = binding.Decoder.from_code(code), binding.Decoder.from_code(code)
+    if bits == 16:
+        dec.set_message_bits(16)
+        one.set_message_bits(16)
+    one.set_tuning(*one.tuning())
+    for frames in (1, 3, 25, 70, 130):          # every cluster size and block size of the rule
+        g = rng.integers(0, 48, (frames, code.n, q)).astype(np.uint8)
+        g[np.arange(frames)[:, None], np.arange(code.n)[None, :], rng.integers(0, q, (frames, code.n))] = 0
+        g[0] = rng.choice(np.array([0, 255], np.uint8), g[0].shape)
+        gd = torch.as_tensor(g).cuda()
+        for iters, early in ((6, 1), (3, 0), (0, 1), (0, 0)):
+            got = [t.cpu().numpy() for t in dec.decode(gd, iters, early)]
+            ref = [t.cpu().numpy() for t in one.decode(gd, iters, early)]
+            k = min(frames, 8)
+            want = oracle.decode(code, g[:k], iters, early, threads=THREADS, cap=65535 if bits == 16 else 255)
+            for name, a, b, w in zip(("symbols", "iterations", "ok"), got, ref, want):
+                assert np.array_equal(a, b), f"{name}: {frames} frames, {iters} iterations, early {early}"
+                assert np.array_equal(a[:k], w), f"{name} against the oracle: {frames} frames, {iters} iterations"
+
+
+def test_split_decode_replays_from_a_cuda_graph():
+    code = I.workload_code("gf64_n576_dv2_dc4")
+    dec = binding.Decoder.from_code(code)
+    g = I.make_batch(code, 2.0, 5, 9).gamma.cuda()
+    sym = torch.empty((9, code.n), dtype=torch.uint8, device="cuda")
+    its, ok = torch.empty(9, dtype=torch.int32, device="cuda"), torch.empty(9, dtype=torch.uint8, device="cuda")
+    ws = dec.workspace(9, "cuda")
+    s = torch.cuda.Stream()
+    s.wait_stream(torch.cuda.current_stream())
+    binding.nbldpc_decode(dec.handle, g, 9, 20, 1, sym, its, ok, ws, stream=s)
+    s.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=s):
+        binding.nbldpc_decode(dec.handle, g, 9, 20, 1, sym, its, ok, ws, stream=s)
+    g.copy_(I.make_batch(code, 1.5, 6, 9).gamma.cuda())
+    graph.replay()
+    torch.cuda.synchronize()
+    for a, w in zip((sym, its, ok), oracle.decode(code, g.cpu().numpy(), 20, 1, threads=THREADS)):
+        assert np.array_equal(a.cpu().numpy(), w)
