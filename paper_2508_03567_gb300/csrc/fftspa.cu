@@ -15,24 +15,26 @@ namespace nbldpc {
 // <= dv (2, 4 or 8) and check degrees <= dc (4 or 8: distributed check-node
 // pass), or dc = 0 (lane-per-edge check-node pass, q <= 64, check degree
 // <= 32), and its block size; null when there is none.
-template <int DC, int DV> const void* fft_entry(int* threads) {
+// split: the kernel that decodes a frame on a cluster of blocks.
+template <int DC, int DV> const void* fft_entry(int split, int* threads) {
   if (threads) *threads = FftThreads<NBLDPC_FQ, DC, DV>::v;
-  return reinterpret_cast<const void*>(&fftspa_decode_kernel<NBLDPC_FQ, DC, DV>);
+  return split ? reinterpret_cast<const void*>(&fftspa_split_kernel<NBLDPC_FQ, DC, DV>)
+               : reinterpret_cast<const void*>(&fftspa_decode_kernel<NBLDPC_FQ, DC, DV>);
 }
 
-template <int DC> const void* fft_entry_dv(int dv, int* threads) {
-  if (dv == 2) return fft_entry<DC, 2>(threads);
-  if (dv == 4) return fft_entry<DC, 4>(threads);
-  if (dv == 8) return fft_entry<DC, 8>(threads);
+template <int DC> const void* fft_entry_dv(int dv, int split, int* threads) {
+  if (dv == 2) return fft_entry<DC, 2>(split, threads);
+  if (dv == 4) return fft_entry<DC, 4>(split, threads);
+  if (dv == 8) return fft_entry<DC, 8>(split, threads);
   return nullptr;
 }
 
-const void* NBLDPC_CAT(fft_kernel_q, NBLDPC_FQ)(int dc, int dv, int* threads) {
+const void* NBLDPC_CAT(fft_kernel_q, NBLDPC_FQ)(int dc, int dv, int split, int* threads) {
 #if NBLDPC_FQ <= 64
-  if (dc == 0) return fft_entry_dv<0>(dv, threads);
+  if (dc == 0) return fft_entry_dv<0>(dv, split, threads);
 #endif
-  if (dc == 4) return fft_entry_dv<4>(dv, threads);
-  if (dc == 8) return fft_entry_dv<8>(dv, threads);
+  if (dc == 4) return fft_entry_dv<4>(dv, split, threads);
+  if (dc == 8) return fft_entry_dv<8>(dv, split, threads);
   return nullptr;
 }
 

@@ -4,6 +4,8 @@
 // launches of the FFT-SPA kernels, device- and host-buffer entry points.
 #include "nbldpc.h"
 
+#include <algorithm>
+
 #include "fftspa_kernels.cuh"
 #include "host_internal.h"
 
@@ -12,28 +14,28 @@ static_assert(sizeof(nbldpc::FftParams) < 4000, "kernel parameter space");
 using namespace nbldpc_host;
 
 namespace nbldpc {   // defined in fftspa.cu, one translation unit per field order
-const void* fft_kernel_q2(int dc, int dv, int* threads);
-const void* fft_kernel_q4(int dc, int dv, int* threads);
-const void* fft_kernel_q8(int dc, int dv, int* threads);
-const void* fft_kernel_q16(int dc, int dv, int* threads);
-const void* fft_kernel_q32(int dc, int dv, int* threads);
-const void* fft_kernel_q64(int dc, int dv, int* threads);
-const void* fft_kernel_q128(int dc, int dv, int* threads);
-const void* fft_kernel_q256(int dc, int dv, int* threads);
+const void* fft_kernel_q2(int dc, int dv, int split, int* threads);
+const void* fft_kernel_q4(int dc, int dv, int split, int* threads);
+const void* fft_kernel_q8(int dc, int dv, int split, int* threads);
+const void* fft_kernel_q16(int dc, int dv, int split, int* threads);
+const void* fft_kernel_q32(int dc, int dv, int split, int* threads);
+const void* fft_kernel_q64(int dc, int dv, int split, int* threads);
+const void* fft_kernel_q128(int dc, int dv, int split, int* threads);
+const void* fft_kernel_q256(int dc, int dv, int split, int* threads);
 }  // namespace nbldpc
 
 namespace {
 
-const void* fft_kernel_for(int q, int dc, int dv, int* threads = nullptr) {
+const void* fft_kernel_for(int q, int dc, int dv, int split, int* threads = nullptr) {
   switch (q) {
-    case 2: return nbldpc::fft_kernel_q2(dc, dv, threads);
-    case 4: return nbldpc::fft_kernel_q4(dc, dv, threads);
-    case 8: return nbldpc::fft_kernel_q8(dc, dv, threads);
-    case 16: return nbldpc::fft_kernel_q16(dc, dv, threads);
-    case 32: return nbldpc::fft_kernel_q32(dc, dv, threads);
-    case 64: return nbldpc::fft_kernel_q64(dc, dv, threads);
-    case 128: return nbldpc::fft_kernel_q128(dc, dv, threads);
-    case 256: return nbldpc::fft_kernel_q256(dc, dv, threads);
+    case 2: return nbldpc::fft_kernel_q2(dc, dv, split, threads);
+    case 4: return nbldpc::fft_kernel_q4(dc, dv, split, threads);
+    case 8: return nbldpc::fft_kernel_q8(dc, dv, split, threads);
+    case 16: return nbldpc::fft_kernel_q16(dc, dv, split, threads);
+    case 32: return nbldpc::fft_kernel_q32(dc, dv, split, threads);
+    case 64: return nbldpc::fft_kernel_q64(dc, dv, split, threads);
+    case 128: return nbldpc::fft_kernel_q128(dc, dv, split, threads);
+    case 256: return nbldpc::fft_kernel_q256(dc, dv, split, threads);
   }
   return nullptr;
 }
@@ -47,7 +49,10 @@ const void* fft_kernel_for(int q, int dc, int dv, int* threads = nullptr) {
 #define NBLDPC_FFT_LANE_MAXQ 4
 #endif
 
-bool g_fft_attr_done[64][8][3][3] = {};   // device, log2(q) - 1, check-node form, column-degree bucket
+// device, log2(q) - 1, check-node form, column-degree bucket: the kernels' attributes are
+// set; the largest cluster of the split-frame kernel (-1: none)
+bool g_fft_attr_done[64][8][3][3] = {};
+int g_fft_split_max[64][8][3][3] = {};
 
 }  // namespace
 
@@ -64,7 +69,7 @@ int nbldpc_host::fft_configure(nbldpc_code* c) {
   const int dv = c->vmax <= 2 ? 2 : (c->vmax <= 4 ? 4 : (c->vmax <= 8 ? 8 : 0));
   if (dc < 0 || !dv) return NBLDPC_ERR_UNSUPPORTED;
   int threads = 0;
-  const void* k = fft_kernel_for(c->q, dc, dv, &threads);
+  const void* k = fft_kernel_for(c->q, dc, dv, 0, &threads);
   if (!k) return NBLDPC_ERR_UNSUPPORTED;
   int dev = 0, sms = 0, optin = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
@@ -82,12 +87,19 @@ int nbldpc_host::fft_configure(nbldpc_code* c) {
   if (pl.smem > optin) return NBLDPC_ERR_UNSUPPORTED;
   {
     std::lock_guard<std::mutex> lk(g_attr_mu);
-    bool& done = g_fft_attr_done[dev][nbldpc::ilog2(c->q) - 1][dc == 0 ? 0 : (dc == 4 ? 1 : 2)][dv == 2 ? 0 : (dv == 4 ? 1 : 2)];
+    const int iq = nbldpc::ilog2(c->q) - 1, ic = dc == 0 ? 0 : (dc == 4 ? 1 : 2), iv = dv == 2 ? 0 : (dv == 4 ? 1 : 2);
+    bool& done = g_fft_attr_done[dev][iq][ic][iv];
+    int& split = g_fft_split_max[dev][iq][ic][iv];
+    int split_threads = 0;
+    const void* ks = fft_kernel_for(c->q, dc, dv, 1, &split_threads);
     if (!done) {
       if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, optin) != cudaSuccess)
         return NBLDPC_ERR_CUDA;
+      split = split_kernel_prepare(ks, split_threads, optin);
       done = true;
     }
+    c->fft_split_max = split;
+    c->fft_split_threads = split_threads;
   }
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pl.per_sm, k, pl.threads, pl.smem) != cudaSuccess)
     return NBLDPC_ERR_CUDA;
@@ -102,10 +114,82 @@ int nbldpc_host::fft_configure(nbldpc_code* c) {
 
 namespace {
 
+// Shape of a split launch (see nbldpc.cu): ranks per frame, threads per rank, shared memory of a rank.
+struct FftSplitShape {
+  int size = 0, threads = 0, smem = 0;
+  nbldpc::FftSplitParams p{};
+};
+
+// Lay out a rank's shared memory; size 0 when it does not fit the device.
+FftSplitShape fft_split_layout(const nbldpc_code* c, int size, int threads) {
+  FftSplitShape s;
+  const bool lane_form = c->fft_dc == 0;
+  s.p.size = size;
+  s.p.cpc = ((lane_form ? c->ntasks : c->m) + size - 1) / size;
+  s.p.npc = (c->n + size - 1) / size;
+  // a warp task holds at most 32 edges
+  const long long edges_r = std::min<long long>(c->nnz, (long long)s.p.cpc * (lane_form ? 32 : c->dmax));
+  const long long edges_n = std::min<long long>(c->nnz, (long long)s.p.npc * c->vmax);
+  size_t o = round_up((size_t)c->off.fft_bytes, 16);
+  auto take = [&](size_t bytes) { const size_t at = o; o = round_up(o + bytes, 256); return (int)at; };
+  s.p.chat_off = take((size_t)c->n);
+  s.p.flag_off = take(2 * nbldpc::kMaxSplit * sizeof(int));
+  s.p.row_off = take((size_t)edges_n * sizeof(void*));
+  s.p.w_off = take(lane_form ? (size_t)threads * c->q * sizeof(float) : 0);
+  s.p.x_off = take((size_t)edges_r * c->q * sizeof(float));
+  if (o > (size_t)c->smem_optin) return FftSplitShape{};
+  s.size = size;
+  s.threads = threads;
+  s.smem = (int)o;
+  return s;
+}
+
+// The split shape of a batch, or size 0 for the one-block-per-frame kernel.
+//
+// The one-block kernel gives a frame one SM.  A cluster shortens a frame's
+// passes, but the variable-node pass then reads the other ranks' rows: at
+// throughput it is slower (GF(64) N=576, 4096 frames: 5.6 ms against 8.2 ms at
+// best), so it serves batches that leave SMs idle.  Measured on GB300, us per
+// decode of up to 20 iterations with early stop, one block against this rule:
+// GF(64) N=576, 1 / 48 / 200 / 400 frames 311 / 362 / 646 / 843 against 88 / 249 /
+// 572 / 945 (not taken); GF(16) N=1024, 1 / 96 / 200 frames 337 / 339 / 449 against
+// 116 / 236 / 346; GF(256) N=384, 1 / 96 / 200 frames 1971 / 1952 / 2551 against
+// 273 / 1068 / 2115; GF(8) N=512, 48 frames 162 against 121.
+//  - 128-thread ranks and few frames only where a frame has fewer than 1024
+//    check-node lanes, none below 400 (GF(16) N=100: 72 against 80 at one frame).
+//  - The lane-per-edge form (q <= 4) up to 3/8 frame per SM (GF(4) N=1024,
+//    48 / 96 frames: 153 / 153 against 117 / 161).
+//  - Equal iterations for every frame have no tail to shorten: up to 3/8 frame
+//    per SM (96 frames of GF(64) N=576: 168 against 214), and for q <= 32 between
+//    one frame per SM and one and a half, which the one-block kernel takes in two
+//    waves (200 frames of GF(16) N=1024, 5 iterations: 183 against 162).
+FftSplitShape fft_split_shape(const nbldpc_code* c, int frames, int early_stop) {
+  if (c->fft_split_max == 0) return FftSplitShape{};
+  const bool lane_form = c->fft_dc == 0;
+  const int sms = c->fft_plan.grid_max / c->fft_plan.per_sm;
+  const int lanes = lane_form ? c->nnz : c->m * (c->q == 256 ? 32 : c->q / 4);
+  if (lanes < 400) return FftSplitShape{};
+  const int few = 3 * sms / 8, two_waves = 3 * sms / 2;
+  const bool most = frames <= few || (frames <= two_waves && lanes >= 1024 && !lane_form &&
+                                      (early_stop || (c->q <= 32 && frames > sms)));
+  if (!most) return FftSplitShape{};
+  int size = frames <= sms / 8 ? 16 : frames <= 3 * sms / 4 ? 8 : 4;
+  int threads = c->q == 64 || c->q == 128 ? c->fft_split_threads / 2 : 256;
+  if (lanes < 1024) {
+    size = 8;
+    threads = 128;
+  }
+  size = std::min(size, c->fft_split_max);
+  FftSplitShape s = fft_split_layout(c, size, threads);
+  while (s.size == 0 && threads > 64) s = fft_split_layout(c, size, threads = (threads - 1) / 64 * 64);
+  return s;
+}
+
 int fft_launch(const nbldpc_code* c, const float* prob, int frames, int max_iters, int early_stop, uint8_t* sym,
                int32_t* iters, uint8_t* ok, float* app, void* ws, cudaStream_t st) {
   const Plan& pl = c->fft_plan;
   nbldpc::FftParams fp{};
+  fp.job.ntasks = c->ntasks;
   fp.job.blob = c->blob_dev;
   fp.job.off = c->off;
   fp.job.prob = prob;
@@ -119,17 +203,21 @@ int fft_launch(const nbldpc_code* c, const float* prob, int frames, int max_iter
   fp.job.frames = frames;
   fp.job.max_iters = max_iters;
   fp.job.early_stop = early_stop ? 1 : 0;
+  FftSplitShape sp = fft_split_shape(c, frames, early_stop);
+  if (sp.size) {
+    sp.p.job = fp.job;
+    return split_launch(fft_kernel_for(c->q, c->fft_dc, c->fft_dv, 1), frames, sp.size, sp.threads, sp.smem, &sp.p, st);
+  }
   fp.counter = reinterpret_cast<unsigned int*>(ws);
   fp.msg = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(ws) + 256);
   fp.slot_floats = pl.slot_bytes / sizeof(float);
   fp.blob_cap = pl.blob_cap;
   fp.n_cap = pl.n_cap;
   fp.w_off = (int)round_up((size_t)(pl.blob_cap + pl.n_cap + 16), 256);
-  fp.job.ntasks = c->ntasks;
   cudaError_t e = cudaMemsetAsync(ws, 0, sizeof(unsigned int), st);
   if (e != cudaSuccess) return NBLDPC_ERR_CUDA;
   void* args[] = {&fp};
-  e = cudaLaunchKernel(fft_kernel_for(c->q, c->fft_dc, c->fft_dv), dim3(grid_for(pl, frames)), dim3(pl.threads),
+  e = cudaLaunchKernel(fft_kernel_for(c->q, c->fft_dc, c->fft_dv, 0), dim3(grid_for(pl, frames)), dim3(pl.threads),
                        args, (size_t)pl.smem, st);
   if (e != cudaSuccess) return NBLDPC_ERR_CUDA;
   g_launches.fetch_add(1, std::memory_order_relaxed);

@@ -487,10 +487,12 @@ __device__ __forceinline__ void gray_gather(float (&acc)[Q], const int (&a4)[ilo
 // ---------------------------------------------------------------- one frame
 // DC >= every check degree (register arrays of the distributed check-node
 // pass), or DC = 0: the lane-per-edge check-node pass (q <= 64, check degree
-// <= 32); DV >= every column degree.
-template <class g, int DC, int DV>
-__device__ __forceinline__ void fft_decode_frame(const FftJob& job, int frame, float* X, const unsigned char* sblob,
-                                                 uint8_t* chat, float* wsm) {
+// <= 32); DV >= every column degree.  SP: the block is one rank of a cluster
+// that decodes the frame together (SplitCtx of mma_kernels.cuh; X then holds the
+// message rows of the rank's own edges, in its shared memory).
+template <class g, int DC, int DV, bool SP = false>
+__device__ __forceinline__ void fft_decode_frame(const FftJob& job, int frame, float* Xown, const unsigned char* sblob,
+                                                 uint8_t* chat, float* wsm, const SplitCtx* sc = nullptr) {
   using vg = VnpGeo<g::Q, DV>;
   constexpr int Q = g::Q, R = g::R, RV = vg::RV;
   const uint8_t* exp2 = sblob + job.off.exp2;        // x^(i mod (q-1)), i < 2(q-1)
@@ -515,12 +517,31 @@ __device__ __forceinline__ void fft_decode_frame(const FftJob& job, int frame, f
   const unsigned vmask = group_mask<vg::VG>(lane);
   const float* pf = job.prob + (size_t)frame * job.n * Q;
   float* app = job.out_app ? job.out_app + (size_t)frame * job.n * Q : nullptr;
+  // rows are addressed by edge number: a rank's area starts with the row of its first edge
+  float* X = SP ? Xown - (ptrdiff_t)sc->e0 * Q : Xown;
+  const int r_first = SP ? sc->r0 : 0, r_last = SP ? sc->r1 : job.m;
+  const int n_first = SP ? sc->n0 : 0, n_last = SP ? sc->n1 : job.n;
+  const int k_first = SP ? vn_ptr[n_first] : 0;
+  // message row of entry k of the column-ordered edge list, decision of column c
+  auto vn_row = [&](int k) -> float* {
+    if constexpr (SP) return reinterpret_cast<float*>(sc->vrow[k - k_first]);
+    else return X + (size_t)vn_edge[k] * Q;
+  };
+  auto decision = [&](int c) -> int {
+    if constexpr (SP) return *at_rank(chat + c, c / sc->npc);
+    else return chat[c];
+  };
+  // end of a pass: its messages and decisions are visible to every thread of the frame
+  auto pass_sync = [&]() {
+    if constexpr (SP) cluster_barrier();
+    else __syncthreads();
+  };
 
   // ---- variable-node pass (Alg. 1, VNP and decision):
   //   z_e(x) = p(x) prod over the other edges of v'(x), u_e = z_e / sum z_e
   //   c = argmax_x p(x) prod over all edges of v'(x)   (lowest symbol on ties)
   auto vnp = [&](bool first, bool want_u) {
-    for (int vn = vgrp; vn < job.n; vn += nvgroups) {
+    for (int vn = n_first + vgrp; vn < n_last; vn += nvgroups) {
       float pv[RV], T[RV];
       load_vec<RV>(pf + (size_t)vn * Q + vgl * RV, pv);
 #pragma unroll
@@ -530,7 +551,7 @@ __device__ __forceinline__ void fft_decode_frame(const FftJob& job, int frame, f
 #pragma unroll
       for (int a = 0; a < DV; ++a) {
         if (!first && a < dv) {
-          load_vec<RV>(X + (size_t)vn_edge[k0 + a] * Q + vgl * RV, V[a]);
+          load_vec<RV>(vn_row(k0 + a) + vgl * RV, V[a]);
 #pragma unroll
           for (int r = 0; r < RV; ++r) T[r] *= V[a][r];
         } else {
@@ -568,25 +589,33 @@ __device__ __forceinline__ void fft_decode_frame(const FftJob& job, int frame, f
               z[r] = t;
             }
             normalize_vec<vg>(z, vmask);
-            store_vec<RV>(X + (size_t)vn_edge[k0 + a] * Q + vgl * RV, z);
+            store_vec<RV>(vn_row(k0 + a) + vgl * RV, z);
           }
         }
       }
     }
   };
 
-  // ---- syndrome of chat over all checks (block-wide)
+  // ---- syndrome of chat over all checks (block-wide, cluster-wide for SP)
+  int flag_set = 0;
   auto syndrome_ok = [&]() -> bool {
     int bad = 0;
-    for (int r = tid; r < job.m; r += nthr) {
+    for (int r = r_first + tid; r < r_last; r += nthr) {
       int sy = 0;
       for (int e = row_ptr[r]; e < row_ptr[r + 1]; ++e) {
-        const int c = chat[edge_col[e]];
+        const int c = decision(edge_col[e]);
         if (c) sy ^= exp2[glog[c] + edge_lh[e]];
       }
       bad |= sy;
     }
-    return __syncthreads_or(bad) == 0;
+    bad = __syncthreads_or(bad);
+    if constexpr (SP) {        // every rank's flag to every rank; two sets, so that a late reader's stays
+      if (tid < sc->size) at_rank(sc->flags + flag_set * kMaxSplit + sc->rank, tid)[0] = bad;
+      cluster_barrier();
+      for (int k = 0; k < sc->size; ++k) bad |= sc->flags[flag_set * kMaxSplit + k];
+      flag_set ^= 1;
+    }
+    return bad == 0;
   };
 
 
@@ -599,7 +628,7 @@ __device__ __forceinline__ void fft_decode_frame(const FftJob& job, int frame, f
     const int w_row0 = (int)(reinterpret_cast<unsigned char*>(wsm) - fft_smem);   // byte offset, 256-aligned
     float* wrow = wsm + ((size_t)warp * 32 + lane) * Q;        // this lane's transformed vector
     const int swz = row_swz<Q>(lane);
-    for (int t = warp; t < job.ntasks; t += nwarps) {
+    for (int t = (SP ? sc->t0 : 0) + warp; t < (SP ? sc->t1 : job.ntasks); t += nwarps) {
       const int eb = row_ptr[task_c0[t]], ee = row_ptr[task_c0[t + 1]];
       const int e = eb + lane;
       const bool valid = e < ee;
@@ -665,7 +694,7 @@ __device__ __forceinline__ void fft_decode_frame(const FftJob& job, int frame, f
     const int y0s = SF ? (y0 ^ (gl & ((1 << RL) - 1))) : y0;
     const bool y0snz = y0s != 0;
     const int ly0s = y0snz ? glog[y0s] : 0;
-    for (int r = grp; r < job.m; r += ngroups) {
+    for (int r = r_first + grp; r < r_last; r += ngroups) {
       const int e0 = row_ptr[r], d = row_ptr[r + 1] - e0;
       float W[DC][R];
       // absent edges (d < DC) enter the product as the transform of the unit
@@ -730,22 +759,22 @@ __device__ __forceinline__ void fft_decode_frame(const FftJob& job, int frame, f
 
   // ---- decode one frame
   vnp(true, false);                                  // c^(0) = argmax p
-  __syncthreads();
+  pass_sync();
   bool ok = syndrome_ok();
   int iters = 0;
   if (!(job.early_stop && ok)) {
     for (int k = 1; k <= job.max_iters; ++k) {
       if constexpr (DC == 0) cnp_lane(k == 1); else cnp(k == 1);
-      __syncthreads();
+      pass_sync();
       vnp(false, k < job.max_iters);
-      __syncthreads();
+      pass_sync();
       iters = k;
       ok = syndrome_ok();
       if (job.early_stop && ok) break;
     }
   }
-  for (int i = tid; i < job.n; i += nthr) job.out_sym[(size_t)frame * job.n + i] = chat[i];
-  if (tid == 0) {
+  for (int i = n_first + tid; i < n_last; i += nthr) job.out_sym[(size_t)frame * job.n + i] = chat[i];
+  if (tid == 0 && (!SP || sc->rank == 0)) {
     job.out_iters[frame] = iters;
     job.out_ok[frame] = ok ? 1 : 0;
   }
@@ -783,6 +812,72 @@ __global__ void __launch_bounds__(FftThreads<Q, DC, DV>::v, 1) fftspa_decode_ker
     fft_decode_frame<FftGeo<Q>, DC, DV>(job, frame, X, sblob, chat, wsm);
     __syncthreads();
   }
+}
+
+// ---------------------------------------------------------------- the kernel of split frames
+// One cluster per frame (grid: frames * cluster size).  Shared memory of a rank:
+// code blob | decisions (indexed by column) | flags | row table | transformed vectors
+// (lane-per-edge form) | message rows of its edges.  In the lane-per-edge form a
+// rank owns whole warp tasks, else cpc checks.
+struct FftSplitParams {
+  FftJob job;
+  int size;                   // ranks per frame
+  int cpc, npc;               // warp tasks (lane-per-edge form) or checks per rank, columns per rank
+  int chat_off, flag_off, row_off, w_off, x_off;
+};
+
+// (The one-block kernel's launch bounds, so its registers per thread; a rank is
+// launched with fewer threads and an SM holds several.)
+template <int Q, int DC, int DV>
+__global__ void __launch_bounds__(FftThreads<Q, DC, DV>::v, 1)
+    fftspa_split_kernel(const __grid_constant__ FftSplitParams p) {
+  unsigned char* smem = fft_smem;
+  const FftJob& job = p.job;
+  const int tid = threadIdx.x, nthr = blockDim.x;
+  const int rank = blockIdx.x % p.size, frame = blockIdx.x / p.size;
+  unsigned char* sblob = smem;
+  for (int i = tid; i < job.off.fft_bytes / 16; i += nthr)
+    reinterpret_cast<uint4*>(sblob)[i] = reinterpret_cast<const uint4*>(job.blob)[i];
+  __syncthreads();
+  const uint16_t* row_ptr = reinterpret_cast<const uint16_t*>(sblob + job.off.row_ptr);
+  const uint16_t* vn_ptr = reinterpret_cast<const uint16_t*>(sblob + job.off.vn_ptr);
+  const uint16_t* vn_edge = reinterpret_cast<const uint16_t*>(sblob + job.off.vn_edge);
+  const uint16_t* edge_row = reinterpret_cast<const uint16_t*>(sblob + job.off.edge_row);
+  const uint16_t* task_c0 = reinterpret_cast<const uint16_t*>(sblob + job.off.task_c0);
+  // first check of rank k's share
+  auto first_check = [&](int k) -> int {
+    if constexpr (DC == 0) return task_c0[min(k * p.cpc, job.ntasks)];
+    else return min(k * p.cpc, job.m);
+  };
+  SplitCtx sc;
+  sc.rank = rank;
+  sc.size = p.size;
+  sc.t0 = min(rank * p.cpc, job.ntasks);
+  sc.t1 = min(sc.t0 + p.cpc, job.ntasks);
+  sc.r0 = first_check(rank);
+  sc.r1 = first_check(rank + 1);
+  sc.n0 = min(rank * p.npc, job.n);
+  sc.n1 = min(sc.n0 + p.npc, job.n);
+  sc.npc = p.npc;
+  sc.e0 = row_ptr[sc.r0];
+  sc.gam = nullptr;
+  sc.flags = reinterpret_cast<int*>(smem + p.flag_off);
+  uint8_t** vrow = reinterpret_cast<uint8_t**>(smem + p.row_off);
+  sc.vrow = vrow;
+  float* X = reinterpret_cast<float*>(smem + p.x_off);
+  for (int k = vn_ptr[sc.n0] + tid; k < vn_ptr[sc.n1]; k += nthr) {
+    const int e = vn_edge[k], r = edge_row[e];
+    int owner = 0;
+    if constexpr (DC == 0) {
+      while (owner + 1 < p.size && first_check(owner + 1) <= r) ++owner;
+    } else {
+      owner = r / p.cpc;
+    }
+    vrow[k - vn_ptr[sc.n0]] = reinterpret_cast<uint8_t*>(at_rank(X, owner) + (size_t)(e - row_ptr[first_check(owner)]) * Q);
+  }
+  cluster_barrier();           // the row table is complete, and every rank of the cluster runs
+  fft_decode_frame<FftGeo<Q>, DC, DV, true>(job, frame, X, sblob, smem + p.chat_off,
+                                            reinterpret_cast<float*>(smem + p.w_off), &sc);
 }
 
 }  // namespace nbldpc

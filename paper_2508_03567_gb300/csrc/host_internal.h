@@ -67,6 +67,7 @@ struct nbldpc_code {
   nbldpc_host::Plan plan{};            // single-code launch shape (fpb chosen by default or by the autotuner)
   int fft_status = NBLDPC_ERR_UNSUPPORTED;   // FFT-SPA launch shape below valid when NBLDPC_OK
   int fft_dc = 0, fft_dv = 0;          // FFT-SPA check-node form (dc 0: lane per edge) and column-degree bucket
+  int fft_split_max = 0, fft_split_threads = 0;   // largest cluster and block of the FFT-SPA split-frame kernel
   int ntasks = 0;                      // FFT-SPA warp tasks (blob section)
   nbldpc_host::Plan fft_plan{};
   std::mutex mu;                       // guards the lazily created copy stream
@@ -88,6 +89,51 @@ inline int check_device(const nbldpc_code* c) {
 // FFT-SPA launch shape of a code (fftspa_host.cu): NBLDPC_OK, NBLDPC_ERR_UNSUPPORTED
 // when no FFT-SPA kernel covers the code, or NBLDPC_ERR_CUDA.
 int fft_configure(nbldpc_code* c);
+
+// ---- frames split over the blocks of a cluster ------------------------------
+// Set a split-frame kernel's attributes; the largest cluster that the device runs
+// for it (16, else the portable 8), or 0 when it cannot be prepared.
+inline int split_kernel_prepare(const void* kernel, int threads, int smem_optin) {
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_optin) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = nbldpc::kMaxSplit;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.gridDim = dim3(nbldpc::kMaxSplit);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = (size_t)smem_optin;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  int n = 0;
+  const bool wide = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+                    cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) == cudaSuccess && n >= 1;
+  cudaGetLastError();          // a refused query is not a later call's error
+  return wide ? nbldpc::kMaxSplit : 8;
+}
+
+// Queue one cluster of `size` blocks per frame.
+inline int split_launch(const void* kernel, int frames, int size, int threads, int smem, void* params,
+                        cudaStream_t st) {
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = (unsigned)size;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.gridDim = dim3((unsigned)frames * (unsigned)size);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = (size_t)smem;
+  cfg.stream = st;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  void* args[] = {params};
+  if (cudaLaunchKernelExC(&cfg, kernel, args) != cudaSuccess) return NBLDPC_ERR_CUDA;
+  g_launches.fetch_add(1, std::memory_order_relaxed);
+  return NBLDPC_OK;
+}
 
 // ---- host-buffer decodes (nbldpc_decode_host, nbldpc_fftspa_decode_host) ------
 // One chunk's device buffers: input rows, symbols, iterations, ok flags, decoder workspace.

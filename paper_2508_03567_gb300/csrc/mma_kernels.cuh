@@ -771,6 +771,7 @@ struct SplitCtx {
   int rank, size;
   int r0, r1, n0, n1;         // the rank's checks and columns
   int e0;                     // first edge of the rank's checks
+  int t0, t1;                 // the rank's warp tasks (FFT-SPA, lane-per-edge form)
   int npc;                    // columns per rank
   const uint8_t* gam;         // the rank's reliability rows (shared memory)
   uint8_t* const* vrow;       // message row of each edge of the rank's columns, in column order
@@ -936,7 +937,8 @@ __device__ __forceinline__ void decode_frame(const JobDesc& job, int frame, uint
 
     // 16-bit messages start from alpha^(0) = gamma widened into every edge row
     auto init_wide = [&]() {
-      for (int i = row_ptr[r_first] * Q + stid; i < row_ptr[r_last] * Q; i += nthr) {
+      const int first = SP ? row_ptr[r_first] * Q : 0, last = row_ptr[r_last] * Q;
+      for (int i = first + stid; i < last; i += nthr) {
         const int e = i / Q, a = i % Q;
         reinterpret_cast<uint16_t*>(X)[i] = gam[(size_t)edge_col[e] * Q + a];
       }

@@ -184,26 +184,8 @@ int split_max(int q, int mb, int dev, int smem_optin) {
   if (dev < 0 || dev >= 64) return 0;
   int& mx = g_split_max[dev][nbldpc::ilog2(q) - 1][mb - 1];
   if (mx == 0) {
-    const void* k = split_kernel_for(q, mb);
-    mx = -1;
-    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_optin) == cudaSuccess) {
-      mx = 8;
-      cudaLaunchConfig_t cfg{};
-      cudaLaunchAttribute at{};
-      at.id = cudaLaunchAttributeClusterDimension;
-      at.val.clusterDim.x = nbldpc::kMaxSplit;
-      at.val.clusterDim.y = at.val.clusterDim.z = 1;
-      cfg.gridDim = dim3(nbldpc::kMaxSplit);
-      cfg.blockDim = dim3(nbldpc::kResidentThreads);
-      cfg.dynamicSmemBytes = (size_t)smem_optin;
-      cfg.attrs = &at;
-      cfg.numAttrs = 1;
-      int n = 0;
-      if (cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
-          cudaOccupancyMaxActiveClusters(&n, k, &cfg) == cudaSuccess && n >= 1)
-        mx = nbldpc::kMaxSplit;
-      cudaGetLastError();      // a refused query is not a later call's error
-    }
+    mx = split_kernel_prepare(split_kernel_for(q, mb), nbldpc::kResidentThreads, smem_optin);
+    if (mx == 0) mx = -1;
   }
   return mx < 0 ? 0 : mx;
 }
@@ -449,21 +431,7 @@ SplitShape split_shape(const nbldpc_code* c, int frames, int early_stop) {
 
 int launch_split(const nbldpc_code* c, SplitShape& s, const nbldpc::JobDesc& job, cudaStream_t st) {
   s.p.job = job;
-  cudaLaunchConfig_t cfg{};
-  cudaLaunchAttribute at{};
-  at.id = cudaLaunchAttributeClusterDimension;
-  at.val.clusterDim.x = (unsigned)s.size;
-  at.val.clusterDim.y = at.val.clusterDim.z = 1;
-  cfg.gridDim = dim3((unsigned)job.frames * (unsigned)s.size);
-  cfg.blockDim = dim3((unsigned)s.threads);
-  cfg.dynamicSmemBytes = (size_t)s.smem;
-  cfg.stream = st;
-  cfg.attrs = &at;
-  cfg.numAttrs = 1;
-  void* args[] = {&s.p};
-  if (cudaLaunchKernelExC(&cfg, split_kernel_for(c->q, c->mb), args) != cudaSuccess) return NBLDPC_ERR_CUDA;
-  g_launches.fetch_add(1, std::memory_order_relaxed);
-  return NBLDPC_OK;
+  return split_launch(split_kernel_for(c->q, c->mb), job.frames, s.size, s.threads, s.smem, &s.p, st);
 }
 
 // split: small batches may go to the split-frame kernel (not while the autotuner times a tuning)

@@ -64,6 +64,29 @@ def test_small_batches_match_the_oracle_and_the_one_block_kernels(kind, q, n, x,
                 assert np.array_equal(a[:k], w), f"{name} against the oracle: {frames} frames, {iters} iterations"
 
 
+@pytest.mark.parametrize("q,n,m,dmax", [(2, 400, 180, 6), (4, 300, 140, 12), (8, 300, 210, 6), (16, 161, 101, 4),
+                                        (32, 97, 53, 8), (64, 61, 31, 4), (128, 40, 17, 6), (256, 33, 14, 8)])
+def test_small_fftspa_batches_match_the_one_block_kernel(q, n, m, dmax):
+    """Same arithmetic in the same order: the frames of a small batch (cluster of blocks) equal, bit
+    for bit and with their a-posteriori vectors, the same frames inside a batch of 600 (one block
+    per frame)."""
+    code = irregular(q, n, m, q + n, dmax)
+    if np.bincount(code.col_idx, minlength=n).max() > 8:
+        pytest.skip("column degree outside the FFT-SPA kernels")
+    rng = np.random.default_rng(q)
+    p = rng.dirichlet(np.full(q, 0.05), (600, n)).astype(np.float32) + np.float32(1e-6)
+    p[0, 0] = 0.0                                # a vector without positive entries
+    p[1] = rng.choice(np.array([0.0, 1.0], np.float32), p[1].shape)
+    pd = torch.as_tensor(p).cuda()
+    dec = binding.Decoder.from_code(code)
+    for iters, early in ((5, 1), (2, 0), (0, 1)):
+        ref = [t.cpu().numpy() for t in dec.fftspa_decode(pd, iters, early, want_app=True)]
+        for frames in (1, 2, 30, 100, 220):
+            got = [t.cpu().numpy() for t in dec.fftspa_decode(pd[:frames].contiguous(), iters, early, want_app=True)]
+            for name, a, b in zip(("symbols", "iterations", "ok", "app"), got, ref):
+                assert np.array_equal(a, b[:frames]), f"{name}: {frames} frames, {iters} iterations, early {early}"
+
+
 def test_split_decode_replays_from_a_cuda_graph():
     code = I.workload_code("gf64_n576_dv2_dc4")
     dec = binding.Decoder.from_code(code)
