@@ -47,6 +47,10 @@ const void* NBLDPC_CAT(kernel_q, NBLDPC_KQ)(int v, int mb, int t1, int dreg) {
       return (v & 1) ? reinterpret_cast<const void*>(&mma_decode_kernel<NBLDPC_KQ, 1, 1, false, true, false, 4>)
                      : reinterpret_cast<const void*>(&mma_decode_kernel<NBLDPC_KQ, 0, 1, false, true, false, 4>);
 #endif
+#if NBLDPC_KQ == 8 || NBLDPC_KQ == 16 || NBLDPC_KQ == 32
+    // (one lane per check: the layouts of the group form do not differ here)
+    return reinterpret_cast<const void*>(&mma_decode_kernel<NBLDPC_KQ, 0, 1, false, true>);
+#endif
     return (v & 1) ? reinterpret_cast<const void*>(&mma_decode_kernel<NBLDPC_KQ, 1, 1, false, true>)
                    : reinterpret_cast<const void*>(&mma_decode_kernel<NBLDPC_KQ, 0, 1, false, true>);
   }
@@ -63,13 +67,18 @@ const void* NBLDPC_CAT(kernel_q, NBLDPC_KQ)(int v, int mb, int t1, int dreg) {
 #endif
 }
 
-#if NBLDPC_KQ > 0
+#if NBLDPC_KQ >= 8
 // Address of the kernel that decodes a frame on a cluster of blocks, for mb-byte
-// messages (minimal schedule): the layout and the convolutions of the default variant.
+// messages (minimal schedule): the layout and the convolutions of the default variant
+// (GF(8): 16-bit messages only).
 const void* NBLDPC_CAT(split_kernel_q, NBLDPC_KQ)(int mb) {
   constexpr int Q = NBLDPC_KQ, V = (Q >= 16 && Q <= 64) ? 1 : 0;
-  return mb == 2 ? reinterpret_cast<const void*>(&mma_split_kernel<Q, V, 2, false>)
-                 : reinterpret_cast<const void*>(&mma_split_kernel<Q, V, 1, (Q >= 128)>);
+  if (mb == 2) return reinterpret_cast<const void*>(&mma_split_kernel<Q, V, 2, false>);
+#if NBLDPC_KQ == 8
+  return nullptr;
+#else
+  return reinterpret_cast<const void*>(&mma_split_kernel<Q, V, 1, (Q >= 128)>);
+#endif
 }
 #endif
 

@@ -60,7 +60,7 @@ __device__ __forceinline__ uint32_t vmax2_fma(uint32_t a, uint32_t b) {
 #endif
 template <int Q> struct VnpBytes {
   static constexpr int v = Q == 2 ? 2 : Q == 4 ? 4 : Q == 8 ? 8 : Q == 64 ? NBLDPC_VBPL_64
-                         : Q == 256 ? NBLDPC_VBPL_256 : 8;
+                         : Q == 256 ? NBLDPC_VBPL_256 : Q >= 16 && Q <= 32 ? 16 : 8;
 };
 
 // LB: lane bits of x (the shuffle offset d runs over them); SB: lane bits that
@@ -419,7 +419,9 @@ __device__ __forceinline__ int pr_conv(const uint32_t* __restrict__ A, const uin
 
 // ---------------------------------------------------------------- parameters
 struct CodeBlob {           // offsets (bytes) into the code blob
-  int exp2, log, row_ptr, edge_col, edge_lh, edge_lhi, vn_ptr, vn_edge, bytes;
+  int exp2, log, row_ptr, edge_col, edge_lh, edge_lhi, vn_ptr, vn_edge;
+  int perm;                   // q = 8, 16, 32: byte selectors of every multiplication (PermRow)
+  int bytes;
   // FFT-SPA section, after `bytes` (the min-max kernels stage only [0, bytes)):
   // check of each edge, first check of each warp task, transposed-multiplication basis
   int edge_row, task_c0, at_log, fft_bytes;
@@ -580,6 +582,134 @@ __device__ __forceinline__ uint2 conv4(uint2 a, uint2 b) {
                     vmin2(vmin2(vmax2(a0, b.y), vmax2(a1, s1)), vmin2(vmax2(a2, b.x), vmax2(a3, s0))));
 }
 
+
+// ---------------------------------------------------------------- q = 8, 16, 32 in registers
+// One lane per check: a message vector is W = q / 2 words of 16-bit pairs (or q / 4
+// words of bytes) in the lane's registers.  y's register part picks the words and
+// its lowest bit swaps their halves, so every index is static: a convolution is
+// W * q maxima and minima with no shuffle and no shared memory, and the pass is bound
+// by the ALU pipe (80 % busy at GF(16) N=1024; the 8- and 16-lane groups spent as
+// much on shuffles, vector loads and stores, and group barriers).  Resident-message
+// kernels only.  Measured on GB300, group form against this: GF(16) (2,4) N=1024,
+// 4096 frames 4.60 against 2.21 ms; GF(8) (2,4) N=512, 8192 frames 2.10 against 0.89 ms;
+// GF(32) (3,6) N=600, 2999 frames 9.24 against 7.79 ms.
+template <int Q> __host__ __device__ constexpr bool reg_form() { return Q == 8 || Q == 16 || Q == 32; }
+
+// C(x) = min_y max(A(y), B(x ^ y)) (B's halves are swapped for the odd y and back).
+// Two y at a time, so that their two minima are one three-operand instruction (one
+// at a time the compiler kept two: GF(32) N=600 10 % slower).  Half of the maxima on
+// the FMA pipe (GF(16) N=1024, 0 to 4 eighths: 2.49, 2.42, 2.34, 2.31, 2.25 ms).
+// q = 32 keeps the loop over the lowest bit of y rolled (500 instructions a turn).
+template <int W>
+__device__ __forceinline__ void conv_reg(const uint32_t (&A)[W], uint32_t (&B)[W], uint32_t (&C)[W]) {
+  constexpr int F = W / 2;             // words whose maxima run on the FMA pipe (see FmaEighths)
+#pragma unroll
+  for (int w = 0; w < W; ++w) C[w] = 0xFFFFFFFFu;
+#pragma unroll(W >= 16 ? 1 : 2)
+  for (int half = 0; half < 2; ++half) {
+    const uint32_t sel = half ? 0x3232u : 0x1010u;
+#pragma unroll
+    for (int i = 0; i < W; i += 2) {
+      const uint32_t a0 = __byte_perm(A[i], 0, sel), a1 = __byte_perm(A[i + 1], 0, sel);
+#pragma unroll
+      for (int w = 0; w < W; ++w) {
+        const uint32_t m0 = w < F ? vmax2_fma(a0, B[w ^ i]) : vmax2(a0, B[w ^ i]);
+        const uint32_t m1 = w < F ? vmax2_fma(a1, B[w ^ i ^ 1]) : vmax2(a1, B[w ^ i ^ 1]);
+        C[w] = __vimin3_u16x2(C[w], m0, m1);
+      }
+    }
+#pragma unroll
+    for (int w = 0; w < W; ++w) B[w] = __byte_perm(B[w], 0, 0x1032);
+  }
+}
+
+// Byte selectors of "element y of the result is element h y of the argument" for
+// the q / 4 words of a row: a selector among the eight bytes of a word pair for
+// each word, and masks that choose between the pairs (bit 3 of h y, then bit 4).
+template <int Q> struct PermRow {
+  static constexpr int NB = Q / 4;
+  static constexpr int sel_bytes = Q == 8 ? 4 : Q == 16 ? 16 : 16;   // NB 16-bit selectors (q = 16: padded)
+  static constexpr int masks = Q == 8 ? 0 : Q == 16 ? 1 : 2;
+  static constexpr int bytes = sel_bytes + masks * Q;
+};
+
+template <int Q>
+__device__ __forceinline__ void gather_row(const uint32_t (&r)[Q / 4], uint32_t (&o)[Q / 4], const uint8_t* t) {
+  constexpr int NB = Q / 4;
+  uint32_t s[NB / 2];
+  if constexpr (Q == 8) {
+    s[0] = *reinterpret_cast<const uint32_t*>(t);
+  } else if constexpr (Q == 16) {
+    const uint2 v = *reinterpret_cast<const uint2*>(t);
+    s[0] = v.x; s[1] = v.y;
+  } else {
+    const uint4 v = *reinterpret_cast<const uint4*>(t);
+    s[0] = v.x; s[1] = v.y; s[2] = v.z; s[3] = v.w;
+  }
+  const uint32_t* m = reinterpret_cast<const uint32_t*>(t + PermRow<Q>::sel_bytes);
+  uint32_t mk[PermRow<Q>::masks ? PermRow<Q>::masks * NB : 1];
+  if constexpr (Q >= 16) {
+#pragma unroll
+    for (int i = 0; i < PermRow<Q>::masks * NB; i += 4) {
+      const uint4 v = *reinterpret_cast<const uint4*>(m + i);
+      mk[i] = v.x; mk[i + 1] = v.y; mk[i + 2] = v.z; mk[i + 3] = v.w;
+    }
+  }
+#pragma unroll
+  for (int w = 0; w < NB; ++w) {
+    const uint32_t sl = (w & 1) ? s[w / 2] >> 16 : s[w / 2];      // (the permute reads 16 bits of it)
+    uint32_t v = __byte_perm(r[0], r[1], sl);
+    if constexpr (Q >= 16) {
+      const uint32_t v1 = __byte_perm(r[2], r[3], sl);
+      v = (v & ~mk[w]) | (v1 & mk[w]);
+    }
+    if constexpr (Q >= 32) {
+      const uint32_t v2 = __byte_perm(r[4], r[5], sl), v3 = __byte_perm(r[6], r[7], sl);
+      const uint32_t u = (v2 & ~mk[w]) | (v3 & mk[w]);
+      v = (v & ~mk[NB + w]) | (u & mk[NB + w]);
+    }
+    o[w] = v;
+  }
+}
+
+// a row of Q bytes to and from Q / 4 words
+template <int Q> __device__ __forceinline__ void load_row(const uint8_t* p, uint32_t (&r)[Q / 4]) {
+  if constexpr (Q == 8) {
+    const uint2 v = *reinterpret_cast<const uint2*>(p);
+    r[0] = v.x; r[1] = v.y;
+  } else {
+#pragma unroll
+    for (int i = 0; i < Q / 16; ++i) {
+      const uint4 v = reinterpret_cast<const uint4*>(p)[i];
+      r[4 * i] = v.x; r[4 * i + 1] = v.y; r[4 * i + 2] = v.z; r[4 * i + 3] = v.w;
+    }
+  }
+}
+template <int Q> __device__ __forceinline__ void store_row(uint8_t* p, const uint32_t (&r)[Q / 4]) {
+  if constexpr (Q == 8) {
+    *reinterpret_cast<uint2*>(p) = make_uint2(r[0], r[1]);
+  } else {
+#pragma unroll
+    for (int i = 0; i < Q / 16; ++i)
+      reinterpret_cast<uint4*>(p)[i] = make_uint4(r[4 * i], r[4 * i + 1], r[4 * i + 2], r[4 * i + 3]);
+  }
+}
+template <int NB> __device__ __forceinline__ void unpack_row(const uint32_t (&r)[NB], uint32_t (&v)[2 * NB]) {
+#pragma unroll
+  for (int i = 0; i < NB; ++i) {
+    v[2 * i] = __byte_perm(r[i], 0, 0x4140);
+    v[2 * i + 1] = __byte_perm(r[i], 0, 0x4342);
+  }
+}
+template <int NB> __device__ __forceinline__ void pack_row(const uint32_t (&v)[2 * NB], uint32_t (&r)[NB]) {
+#pragma unroll
+  for (int i = 0; i < NB; ++i) r[i] = __byte_perm(v[2 * i], v[2 * i + 1], 0x6420);
+}
+
+// shared scratch of a frame slot of nthr lanes: F_1..F_{d-3} of each lane's check, as bytes
+template <int Q> __host__ __device__ constexpr int reg_scratch_bytes(int nthr, int dmax) {
+  return dmax > 3 ? nthr * (dmax - 3) * Q : 0;
+}
 
 // ---------------------------------------------------------------- q = 4, one warp per frame
 // A frame of a small GF(4) code (at most 32 checks of degree <= kW4Deg, columns
@@ -1245,6 +1375,81 @@ __device__ __forceinline__ void decode_frame(const JobDesc& job, int frame, uint
       }
     };
 
+    // ---- check-node pass for q = 8, 16, 32 in registers: one lane per check of any
+    // degree.  The lane reads an edge's row when it needs P_j (beta_j overwrites it only
+    // after that) and parks F_1..F_{d-3} as bytes in the slot's shared scratch.  At q = 32
+    // beta_j and B_j share one convolution's code: with three in line, frames in different
+    // passes evicted each other's instructions (N=96: no_instruction 2.3 stalls per issue,
+    // 3.33 ms against 2.91; with a single one for F_j too, N=600 was 5 % slower).
+    auto cnp_reg = [&](bool first) {
+      if constexpr (reg_form<Q>()) {
+        constexpr int W = Q / 2, NB = Q / 4;
+        const uint8_t* perm = sblob + job.off.perm;
+        auto load_p = [&](int e, uint32_t (&P)[W]) {       // P_j(y) = alpha_j(h^-1 y)
+          uint32_t r[NB], o[NB];
+          load_row<Q>(first ? gam + (size_t)edge_col[e] * Q : X + (size_t)e * Q, r);
+          gather_row<Q>(r, o, perm + edge_lhi[e] * PermRow<Q>::bytes);
+          unpack_row<NB>(o, P);
+        };
+        auto store_packed = [&](int e, const uint32_t (&r)[NB]) {   // beta_j(a) = R(h a)
+          uint32_t o[NB];
+          gather_row<Q>(r, o, perm + edge_lh[e] * PermRow<Q>::bytes);
+          store_row<Q>(X + (size_t)e * Q, o);
+        };
+        auto store_beta = [&](int e, const uint32_t (&R)[W]) {
+          uint32_t r[NB];
+          pack_row<NB>(R, r);
+          store_packed(e, r);
+        };
+        uint8_t* fs = scratch + (size_t)stid * Q;                // F_j of this lane: fs + (j - 1) * nthr * Q
+        for (int r = r_first + stid; r < r_last; r += nthr) {
+          const int e0 = row_ptr[r], d = D > 0 ? D : row_ptr[r + 1] - e0;
+          if (counting && d > 2) work += (unsigned long long)Q * Q * 3 * (d - 2);
+          uint32_t a[W], b[W], c[W];
+          // forward: F_0 = P_0, F_j = F_{j-1} (*) P_j
+          load_p(e0, a);
+#pragma unroll 1
+          for (int j = 1; j <= d - 2; ++j) {
+            load_p(e0 + j, b);
+            conv_reg<W>(a, b, c);
+            if (j <= d - 3) {
+              uint32_t f[NB];
+              pack_row<NB>(c, f);
+              store_row<Q>(fs + (size_t)(j - 1) * nthr * Q, f);
+            }
+#pragma unroll
+            for (int w = 0; w < W; ++w) a[w] = c[w];
+          }
+          load_p(e0 + d - 1, b);                                 // B_{d-1} = P_{d-1}
+          store_beta(e0 + d - 1, a);                             // beta_{d-1} = F_{d-2}
+          // backward: beta_j = F_{j-1} (*) B_{j+1}, B_j = B_{j+1} (*) P_j
+#pragma unroll 1
+          for (int j = d - 2; j >= 1; --j) {
+            if (j == 1) {
+              load_p(e0, a);
+            } else {
+              uint32_t f[NB];
+              load_row<Q>(fs + (size_t)(j - 2) * nthr * Q, f);
+              unpack_row<NB>(f, a);
+            }
+            uint32_t be[NB];
+#pragma unroll(W >= 16 ? 1 : 2)
+            for (int s = 0; s < 2; ++s) {
+              if (s) {
+                load_p(e0 + j, a);
+                store_packed(e0 + j, be);
+              }
+              conv_reg<W>(b, a, c);
+              if (!s) pack_row<NB>(c, be);
+            }
+#pragma unroll
+            for (int w = 0; w < W; ++w) b[w] = c[w];
+          }
+          store_beta(e0, b);                                     // beta_0 = B_1
+        }
+      }
+    };
+
     // ---- decode one frame.  Without early stop only the final decision is
     // tested, so the stop test runs once, after the last iteration.
     const bool es = job.early_stop != 0;
@@ -1260,6 +1465,8 @@ __device__ __forceinline__ void decode_frame(const JobDesc& job, int frame, uint
       for (int k = 1; k <= job.max_iters; ++k) {
         if constexpr (Q == 4 && MB == 1 && !T1 && REG4) {
           if (job.dmax <= kRegDeg) cnp_regs4(k == 1); else cnp(k == 1);
+        } else if constexpr (reg_form<Q>() && MB == 1 && !T1 && W4) {
+          cnp_reg(k == 1);
         } else {
           cnp(MB == 1 && k == 1);
         }
@@ -1420,18 +1627,17 @@ __global__ void __launch_bounds__(kResidentThreads, 2) mma_split_kernel(const __
   sc.vrow = vrow;
   uint8_t* sgam = smem + p.gam_off;
   sc.gam = sgam;
-  // reliabilities of the rank's columns (rows of q bytes; 4-byte words when q >= 4: gamma is 16-byte aligned)
+  // reliabilities of the rank's columns (gamma is 16-byte aligned)
   {
     const uint8_t* src = job.gamma + ((size_t)frame * job.n + sc.n0) * Q;
     const int bytes = (sc.n1 - sc.n0) * Q;
+    static_assert(Q >= 8, "rows of 8-byte words");
     if constexpr (Q >= 16) {
       for (int i = tid; i < bytes / 16; i += nthr)
         reinterpret_cast<uint4*>(sgam)[i] = reinterpret_cast<const uint4*>(src)[i];
-    } else if constexpr (Q >= 4) {
-      for (int i = tid; i < bytes / 4; i += nthr)
-        reinterpret_cast<uint32_t*>(sgam)[i] = reinterpret_cast<const uint32_t*>(src)[i];
     } else {
-      for (int i = tid; i < bytes; i += nthr) sgam[i] = src[i];
+      for (int i = tid; i < bytes / 8; i += nthr)
+        reinterpret_cast<uint2*>(sgam)[i] = reinterpret_cast<const uint2*>(src)[i];
     }
   }
   __syncthreads();

@@ -61,8 +61,6 @@ const void* kernel_q32(int v, int mb, int t1, int dreg);
 const void* kernel_q64(int v, int mb, int t1, int dreg);
 const void* kernel_q128(int v, int mb, int t1, int dreg);
 const void* kernel_q256(int v, int mb, int t1, int dreg);
-const void* split_kernel_q2(int mb);
-const void* split_kernel_q4(int mb);
 const void* split_kernel_q8(int mb);
 const void* split_kernel_q16(int mb);
 const void* split_kernel_q32(int mb);
@@ -102,11 +100,10 @@ int kernel_dreg(int q, int v, int km, int dreg) {
   return ((q == 64 || q == 4) && km == 1 && v >= 2 && v <= 3 && dreg == 4) ? 4 : 0;
 }
 
-// kernel that decodes a frame on a cluster of blocks (minimal schedule)
+// kernel that decodes a frame on a cluster of blocks (minimal schedule), null where
+// split_shape never takes it
 const void* split_kernel_for(int q, int mb) {
   switch (q) {
-    case 2: return nbldpc::split_kernel_q2(mb);
-    case 4: return nbldpc::split_kernel_q4(mb);
     case 8: return nbldpc::split_kernel_q8(mb);
     case 16: return nbldpc::split_kernel_q16(mb);
     case 32: return nbldpc::split_kernel_q32(mb);
@@ -184,7 +181,8 @@ int split_max(int q, int mb, int dev, int smem_optin) {
   if (dev < 0 || dev >= 64) return 0;
   int& mx = g_split_max[dev][nbldpc::ilog2(q) - 1][mb - 1];
   if (mx == 0) {
-    mx = split_kernel_prepare(split_kernel_for(q, mb), nbldpc::kResidentThreads, smem_optin);
+    const void* k = split_kernel_for(q, mb);
+    mx = k ? split_kernel_prepare(k, nbldpc::kResidentThreads, smem_optin) : 0;
     if (mx == 0) mx = -1;
   }
   return mx < 0 ? 0 : mx;
@@ -194,17 +192,35 @@ struct CodeNeeds {       // what one code asks of a frame slot
   int q, variant, mb, dmax, blob, n;
   size_t msg;
   int dreg;              // regular check degree (0: the rows differ)
+  int m;
 };
 
 CodeNeeds needs_of(const nbldpc_code* c, int variant, int mb) {
   return CodeNeeds{c->q, variant, mb, c->dmax, c->off.bytes, c->n, round_up((size_t)c->nnz * c->q * mb, 256),
-                   c->dreg};
+                   c->dreg, c->m};
+}
+
+// Field orders whose resident-message kernels take the register form of the check-node
+// pass (one lane per check).
+bool reg_form(int q) { return q == 8 || q == 16 || q == 32; }
+
+// Threads of a frame slot of those kernels: the checks in as few rounds as 384 threads
+// allow, and no more threads than these rounds need.
+int reg_threads(int m) {
+  const int rounds = (m + nbldpc::kResidentThreads - 1) / nbldpc::kResidentThreads;
+  return (int)round_up((size_t)(m + rounds - 1) / rounds, 32);
+}
+
+int reg_scratch(int q, int nthr, int dmax) {
+  return q == 8 ? nbldpc::reg_scratch_bytes<8>(nthr, dmax)
+                : q == 16 ? nbldpc::reg_scratch_bytes<16>(nthr, dmax) : nbldpc::reg_scratch_bytes<32>(nthr, dmax);
 }
 
 // Plan a launch of kernel (kq, kv, kernel mode km) with fpb frame slots per block for a set of codes.
 // Variants 2 and 3 keep each frame's messages in shared memory: blocks of
 // nbldpc::kResidentThreads threads (1, 2 or 4 frame slots) or of 256 threads with
-// 8 one-warp slots, no message slots in the workspace.
+// 8 one-warp slots (q = 8, 16, 32: at most nbldpc::kResidentThreads threads, as many
+// a slot as its checks need), no message slots in the workspace.
 int make_plan(int kq, int kv, int km, int fpb, const CodeNeeds* cs, int nc, Plan* out) {
   int dev = 0, sms = 0, optin = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
@@ -212,8 +228,11 @@ int make_plan(int kq, int kv, int km, int fpb, const CodeNeeds* cs, int nc, Plan
       cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess)
     return NBLDPC_ERR_CUDA;
   const bool resident = kv >= 0 && (kv & 2);
-  const int threads = resident ? (fpb == 8 ? kThreads : nbldpc::kResidentThreads) : kThreads;
+  const bool reg = resident && reg_form(kq);
+  const int threads = reg ? fpb * reg_threads(cs[0].m)
+                          : resident ? (fpb == 8 ? kThreads : nbldpc::kResidentThreads) : kThreads;
   if (fpb < 1 || threads % fpb) return NBLDPC_ERR_ARG;
+  if (reg && threads > nbldpc::kResidentThreads) return NBLDPC_ERR_UNSUPPORTED;
   if (resident && km != 1) return NBLDPC_ERR_UNSUPPORTED;
   const int nthr = threads / fpb;
   if (nthr < 32 || nthr % 32) return NBLDPC_ERR_UNSUPPORTED;
@@ -224,7 +243,8 @@ int make_plan(int kq, int kv, int km, int fpb, const CodeNeeds* cs, int nc, Plan
   for (int i = 0; i < nc; ++i) {
     const int G = group_lanes(cs[i].q, cs[i].variant & 1);
     if (G > nthr) return NBLDPC_ERR_UNSUPPORTED;
-    const int s = (nthr / G) * group_bytes(cs[i].q, cs[i].dmax, cs[i].mb);
+    const int s = reg ? reg_scratch(cs[i].q, nthr, cs[i].dmax)
+                      : (nthr / G) * group_bytes(cs[i].q, cs[i].dmax, cs[i].mb);
     if (s > scratch) scratch = s;
     if (cs[i].blob > pl.blob_cap) pl.blob_cap = cs[i].blob;
     if (cs[i].n > pl.n_cap) pl.n_cap = cs[i].n;
@@ -253,12 +273,12 @@ int make_plan(int kq, int kv, int km, int fpb, const CodeNeeds* cs, int nc, Plan
 }
 
 // Variant when nothing better is known: the one measured fastest for the
-// benchmark codes on GB300 (GF(16), GF(32): layout 1; GF(64): layout 1 with
-// the messages in shared memory; GF(4): layout 0 with the messages in shared
+// benchmark codes on GB300 (GF(8) to GF(64): layout 1 from GF(16) on, with the
+// messages in shared memory; GF(4): layout 0 with the messages in shared
 // memory; GF(128), GF(256): pruned convolutions, layout 0 (GF(256) (2,6) N=384:
 // 2.8x the dense kernel; GF(128) (2,4) N=256: 35.6 against 41.1 ms); otherwise
 // layout 0).
-int default_variant(int q) { return q >= 128 ? 4 : q == 64 ? 3 : q == 4 ? 2 : (q >= 16 && q <= 32) ? 1 : 0; }
+int default_variant(int q) { return q >= 128 ? 4 : (q >= 16 && q <= 64) ? 3 : q >= 4 ? 2 : 0; }
 
 // GF(4) codes a single warp decodes alone (one-warp frame slots: at most 32
 // checks of degree <= 4, columns of degree <= 2): GF(4) N=48 (2,4) 17-18 us per
@@ -289,6 +309,28 @@ int configure(nbldpc_code* c, int variant, int fpb) {
     c->split_max = split_max(c->q, c->mb, c->device, optin);
   c->smem_optin = optin;
   return NBLDPC_OK;
+}
+
+// The register form (q = 8, 16, 32) with the frames per block that keep most threads of an
+// SM resident, the larger of equals (GF(16) N=100: 4 frames 845 us, 2 frames 887; GF(32)
+// (2,8) N=508, where two frames leave 8 warps: 1 frame 7.87 ms, 2 frames 8.99).  q = 32 with
+// a fifth of the lanes without a check stays in the group form (N=96, 48 checks on 64 lanes:
+// 2.93 ms against 2.74; N=128, 64 checks: 2.44 against 2.85).
+int configure_reg(nbldpc_code* c, int variant) {
+  const int nthr = reg_threads(c->m), rounds = (c->m + nthr - 1) / nthr;
+  if (c->q == 32 && 5 * c->m <= 4 * nthr * rounds) return NBLDPC_ERR_UNSUPPORTED;
+  const CodeNeeds need = needs_of(c, variant, c->mb);
+  int best = 0, most = 0;
+  for (int fpb = 1; fpb <= 8 && fpb * nthr <= nbldpc::kResidentThreads; fpb *= 2) {
+    Plan pl{};
+    const int st = make_plan(c->q, variant, kmode(c), fpb, &need, 1, &pl);
+    if (st == NBLDPC_ERR_CUDA) return st;
+    if (st == NBLDPC_OK && pl.per_sm * pl.threads >= most) {
+      most = pl.per_sm * pl.threads;
+      best = fpb;
+    }
+  }
+  return best ? configure(c, variant, best) : NBLDPC_ERR_UNSUPPORTED;
 }
 
 size_t decode_ws_bytes(const nbldpc_code* c, int frames) { return ws_bytes(c->plan, frames); }
@@ -393,23 +435,28 @@ int split_resident(const nbldpc_code* c, const SplitShape& s) {
 // block per frame against this rule: GF(64) N=576, 1 / 96 / 200 / 1000 frames
 // 1103 / 1158 / 1937 / 3721 against 180 / 481 / 846 / 3299; GF(256) (2,6) N=384,
 // 1 / 96 / 200 frames 7328 / 7818 / 9626 against 689 / 3498 / 8051; GF(256) (2,8)
-// N=128, 17 frames 3939 against 1217; GF(16) N=1024, 1 / 200 / 1000 frames
-// 837 / 882 / 1613 against 161 / 432 / 1436; GF(8) N=512, 1 / 200 frames 225 / 256
-// against 113 / 183.
+// N=128, 17 frames 3939 against 1217; GF(32) N=600, 1 / 96 / 450 frames (register
+// form) 836 / 841 / 1576 against 171 / 439 / 1353; GF(16) N=1024, 1 / 48 frames
+// 235 / 236 against 116 / 182.
 //  - More ranks and threads for fewer frames, so that the SMs are filled and the
 //    frame's chain of passes is as short as they allow.
 //  - No more 128-thread ranks than the frame has check-node lanes for.
-//  - q <= 4 stays (the check-node pass there is shorter than a cluster barrier).
+//  - q <= 8 stays (GF(8) N=512, one frame 83 against 109: the passes are shorter
+//    than the cluster's barriers), but for the 16-bit messages of q = 8.
+//  - The register form (q = 16, 32) is fast enough alone from 5/8 frame per SM on at
+//    q = 16 (200 frames of N=1024 351 against 346, of N=444 251 against 284), from
+//    three on at q = 32 (700 frames 1960 against 1985); 3/8 and 5/8 without early stop
+//    (96 frames of GF(16) 126 against 158, 152 of GF(32) 431 against 446).
 //  - Up to twice the frames that the one-block kernels hold at once when frames
 //    stop early (beyond it the tail is short and the ranks' barriers cost 2-5 %);
 //    half of them where the ranks fill an SM less than three quarters as full
-//    (GF(256): 400 frames of N=384 12.9 ms against 15.6) or q = 8; a third when
+//    (GF(256): 400 frames of N=384 12.9 ms against 15.6); a third when
 //    every frame runs the same iterations (no tail: 1000 frames 7.1 ms against 7.7).
 //  - 16-bit messages: half of them from q = 64 (200 frames 2.9 against 2.3 ms; 1000
 //    frames 5.1 against 10.0), else a quarter (GF(16): 48 frames 1.72 against 0.89 ms,
 //    200 frames 1.93 against 2.11).
 SplitShape split_shape(const nbldpc_code* c, int frames, int early_stop) {
-  if (c->split_max == 0 || c->pinned || c->q <= 4) return SplitShape{};
+  if (c->split_max == 0 || c->pinned) return SplitShape{};
   const long long slots = (long long)c->plan.grid_max * c->plan.fpb;
   if (frames > 2 * slots) return SplitShape{};
   const int sms = c->plan.grid_max / c->plan.per_sm;
@@ -425,7 +472,9 @@ SplitShape split_shape(const nbldpc_code* c, int frames, int early_stop) {
   if (s.size == 0) return s;
   long long most = early_stop ? 2 * slots : slots / 3;
   if (c->mb == 2) most = std::min(most, c->q >= 64 ? slots / 2 : slots / 4);
-  else if (c->q == 8 || 4 * split_resident(c, s) < 3 * c->plan.per_sm * c->plan.threads) most = std::min(most, slots / 2);
+  else if (reg_form(c->q) && (c->variant & 2))
+    most = c->q == 16 ? (early_stop ? 5 : 3) * sms / 8 : early_stop ? 3 * sms : 5 * sms / 8;
+  else if (4 * split_resident(c, s) < 3 * c->plan.per_sm * c->plan.threads) most = std::min(most, slots / 2);
   return frames <= most ? s : SplitShape{};
 }
 
@@ -570,6 +619,9 @@ int nbldpc_code_create(int q, uint32_t prim_poly, int n_cols, int n_rows, const 
   off.edge_lhi = take((size_t)nnz);
   off.vn_ptr = take(2 * ((size_t)n_cols + 1));
   off.vn_edge = take(2 * (size_t)nnz);
+  const int perm_row = q == 8 ? nbldpc::PermRow<8>::bytes : q == 16 ? nbldpc::PermRow<16>::bytes
+                     : q == 32 ? nbldpc::PermRow<32>::bytes : 0;
+  off.perm = take((size_t)perm_row * (q - 1));
   off.bytes = (int)o;
   // FFT-SPA section: warp tasks pack consecutive checks with at most 32 edges in all
   std::vector<uint16_t> tasks;
@@ -600,6 +652,17 @@ int nbldpc_code_create(int q, uint32_t prim_poly, int n_cols, int n_rows, const 
         at[lc * pbits + i] = (uint8_t)a;
       }
   }
+  // selectors of "byte y is byte h y of the row" for h = x^lh (PermRow): nibbles of the low
+  // three bits of h y, then one mask word per four bytes for bit 3 and for bit 4
+  for (int lh = 0; perm_row && lh < q - 1; ++lh)
+    for (int y = 0; y < q; ++y) {
+      unsigned char* t = &blob[off.perm + (size_t)lh * perm_row];
+      const int i = y ? exp2[lg[y] + lh] : 0;
+      t[y / 2] |= (unsigned char)((i & 7) << (4 * (y & 1)));
+      const int sel = q == 8 ? nbldpc::PermRow<8>::sel_bytes : 16;
+      if (q >= 16 && (i & 8)) t[sel + y] = 0xFF;
+      if (q >= 32 && (i & 16)) t[sel + q + y] = 0xFF;
+    }
   memcpy(&blob[off.exp2], exp2.data(), 2 * (size_t)q);
   memcpy(&blob[off.log], lg.data(), (size_t)q);
   uint16_t* rp = reinterpret_cast<uint16_t*>(&blob[off.row_ptr]);
@@ -647,7 +710,8 @@ int nbldpc_code_create(int q, uint32_t prim_poly, int n_cols, int n_rows, const 
     // the resident-message form (384-thread blocks of 1, 2 or 4 frames) must fit shared
     // memory; otherwise the same layout with the messages in the workspace
     const int v = default_variant(q), fpb = default_fpb(c);
-    st = v >= 2 ? configure(c, v, (v & 2) && fpb > 4 && !warp4_code(c) ? 4 : fpb) : NBLDPC_ERR_UNSUPPORTED;
+    if (reg_form(q)) st = configure_reg(c, v);
+    else st = v >= 2 ? configure(c, v, (v & 2) && fpb > 4 && !warp4_code(c) ? 4 : fpb) : NBLDPC_ERR_UNSUPPORTED;
     if (st == NBLDPC_ERR_UNSUPPORTED) st = configure(c, v & 1, fpb);
   }
   if (st == NBLDPC_OK) {
@@ -707,7 +771,7 @@ int nbldpc_code_set_message_bits(nbldpc_code* c, int bits) {
   c->mb = bits / 8;
   // resident messages serve 8-bit codes only: a 16-bit code keeps the layout in the workspace form
   const int v = c->mb == 1 ? c->variant : c->variant & 1;
-  const int st = configure(c, v, v == c->variant ? c->plan.fpb : 1);
+  const int st = configure(c, v, v == c->variant ? c->plan.fpb : reg_form(c->q) && !c->pinned ? default_fpb(c) : 1);
   if (st != NBLDPC_OK) c->mb = old;
   return st;
 }
@@ -726,7 +790,7 @@ int nbldpc_code_set_cnp_schedule(nbldpc_code* c, int schedule) {
   c->cnp_schedule = schedule;
   // the schedule is a separate kernel; resident messages serve the minimal schedule only
   const int v = schedule == NBLDPC_CNP_MINIMAL ? c->variant : c->variant & 1;
-  const int st = configure(c, v, v == c->variant ? c->plan.fpb : 1);
+  const int st = configure(c, v, v == c->variant ? c->plan.fpb : reg_form(c->q) && !c->pinned ? default_fpb(c) : 1);
   if (st != NBLDPC_OK) c->cnp_schedule = old;
   return st;
 }
@@ -778,7 +842,9 @@ static int batch_plan(const nbldpc_job* jobs, int n_jobs, Plan* pl, int* total) 
     if (st != NBLDPC_OK) return st;
     if (kmode(c) != 1) return NBLDPC_ERR_UNSUPPORTED;   // mixed-code launches: 8-bit messages, minimal schedule
     need[i] = needs_of(c, c->variant & 1, 1);
-    if (c->plan.fpb < fpb) fpb = c->plan.fpb;
+    // the all-field kernel runs the group form: its slots are not the register form's
+    const int f = reg_form(c->q) && !c->pinned ? default_fpb(c) : c->plan.fpb;
+    if (f < fpb) fpb = f;
     t += jobs[i].frames;
   }
   if (t > 0x7FFFFFFF) return NBLDPC_ERR_ARG;
