@@ -15,26 +15,28 @@ namespace nbldpc {
 // <= dv (2, 4 or 8) and check degrees <= dc (4 or 8: distributed check-node
 // pass), or dc = 0 (lane-per-edge check-node pass, q <= 64, check degree
 // <= 32), and its block size; null when there is none.
-// split: the kernel that decodes a frame on a cluster of blocks.
-template <int DC, int DV> const void* fft_entry(int split, int* threads) {
+// form: 0 some message rows in the global slot, 1 all in shared memory, 2 the kernel that
+// decodes a frame on a cluster of blocks.
+template <int DC, int DV> const void* fft_entry(int form, int* threads) {
   if (threads) *threads = FftThreads<NBLDPC_FQ, DC, DV>::v;
-  return split ? reinterpret_cast<const void*>(&fftspa_split_kernel<NBLDPC_FQ, DC, DV>)
-               : reinterpret_cast<const void*>(&fftspa_decode_kernel<NBLDPC_FQ, DC, DV>);
+  return form == 2   ? reinterpret_cast<const void*>(&fftspa_split_kernel<NBLDPC_FQ, DC, DV>)
+         : form == 1 ? reinterpret_cast<const void*>(&fftspa_decode_kernel<NBLDPC_FQ, DC, DV, true>)
+                     : reinterpret_cast<const void*>(&fftspa_decode_kernel<NBLDPC_FQ, DC, DV, false>);
 }
 
-template <int DC> const void* fft_entry_dv(int dv, int split, int* threads) {
-  if (dv == 2) return fft_entry<DC, 2>(split, threads);
-  if (dv == 4) return fft_entry<DC, 4>(split, threads);
-  if (dv == 8) return fft_entry<DC, 8>(split, threads);
+template <int DC> const void* fft_entry_dv(int dv, int form, int* threads) {
+  if (dv == 2) return fft_entry<DC, 2>(form, threads);
+  if (dv == 4) return fft_entry<DC, 4>(form, threads);
+  if (dv == 8) return fft_entry<DC, 8>(form, threads);
   return nullptr;
 }
 
-const void* NBLDPC_CAT(fft_kernel_q, NBLDPC_FQ)(int dc, int dv, int split, int* threads) {
+const void* NBLDPC_CAT(fft_kernel_q, NBLDPC_FQ)(int dc, int dv, int form, int* threads) {
 #if NBLDPC_FQ <= 64
-  if (dc == 0) return fft_entry_dv<0>(dv, split, threads);
+  if (dc == 0) return fft_entry_dv<0>(dv, form, threads);
 #endif
-  if (dc == 4) return fft_entry_dv<4>(dv, split, threads);
-  if (dc == 8) return fft_entry_dv<8>(dv, split, threads);
+  if (dc == 4) return fft_entry_dv<4>(dv, form, threads);
+  if (dc == 8) return fft_entry_dv<8>(dv, form, threads);
   return nullptr;
 }
 

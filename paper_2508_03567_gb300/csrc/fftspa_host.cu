@@ -14,28 +14,33 @@ static_assert(sizeof(nbldpc::FftParams) < 4000, "kernel parameter space");
 using namespace nbldpc_host;
 
 namespace nbldpc {   // defined in fftspa.cu, one translation unit per field order
-const void* fft_kernel_q2(int dc, int dv, int split, int* threads);
-const void* fft_kernel_q4(int dc, int dv, int split, int* threads);
-const void* fft_kernel_q8(int dc, int dv, int split, int* threads);
-const void* fft_kernel_q16(int dc, int dv, int split, int* threads);
-const void* fft_kernel_q32(int dc, int dv, int split, int* threads);
-const void* fft_kernel_q64(int dc, int dv, int split, int* threads);
-const void* fft_kernel_q128(int dc, int dv, int split, int* threads);
-const void* fft_kernel_q256(int dc, int dv, int split, int* threads);
+const void* fft_kernel_q2(int dc, int dv, int form, int* threads);
+const void* fft_kernel_q4(int dc, int dv, int form, int* threads);
+const void* fft_kernel_q8(int dc, int dv, int form, int* threads);
+const void* fft_kernel_q16(int dc, int dv, int form, int* threads);
+const void* fft_kernel_q32(int dc, int dv, int form, int* threads);
+const void* fft_kernel_q64(int dc, int dv, int form, int* threads);
+const void* fft_kernel_q128(int dc, int dv, int form, int* threads);
+const void* fft_kernel_q256(int dc, int dv, int form, int* threads);
 }  // namespace nbldpc
 
 namespace {
 
-const void* fft_kernel_for(int q, int dc, int dv, int split, int* threads = nullptr) {
+// Shared memory left to the L1 cache when the message rows do not all fit.  Measured on
+// GB300 (8, 16, 24, 48 KB, us): GF(64) N=576, 4096 frames of 10 iterations 7247, 7288,
+// 7317, 7404; GF(256) (2,8) N=128, 1000 frames 1735, 1765, 1816, 1921.
+constexpr int kFftL1 = 8192;
+
+const void* fft_kernel_for(int q, int dc, int dv, int form, int* threads = nullptr) {
   switch (q) {
-    case 2: return nbldpc::fft_kernel_q2(dc, dv, split, threads);
-    case 4: return nbldpc::fft_kernel_q4(dc, dv, split, threads);
-    case 8: return nbldpc::fft_kernel_q8(dc, dv, split, threads);
-    case 16: return nbldpc::fft_kernel_q16(dc, dv, split, threads);
-    case 32: return nbldpc::fft_kernel_q32(dc, dv, split, threads);
-    case 64: return nbldpc::fft_kernel_q64(dc, dv, split, threads);
-    case 128: return nbldpc::fft_kernel_q128(dc, dv, split, threads);
-    case 256: return nbldpc::fft_kernel_q256(dc, dv, split, threads);
+    case 2: return nbldpc::fft_kernel_q2(dc, dv, form, threads);
+    case 4: return nbldpc::fft_kernel_q4(dc, dv, form, threads);
+    case 8: return nbldpc::fft_kernel_q8(dc, dv, form, threads);
+    case 16: return nbldpc::fft_kernel_q16(dc, dv, form, threads);
+    case 32: return nbldpc::fft_kernel_q32(dc, dv, form, threads);
+    case 64: return nbldpc::fft_kernel_q64(dc, dv, form, threads);
+    case 128: return nbldpc::fft_kernel_q128(dc, dv, form, threads);
+    case 256: return nbldpc::fft_kernel_q256(dc, dv, form, threads);
   }
   return nullptr;
 }
@@ -51,7 +56,7 @@ const void* fft_kernel_for(int q, int dc, int dv, int split, int* threads = null
 
 // device, log2(q) - 1, check-node form, column-degree bucket: the kernels' attributes are
 // set; the largest cluster of the split-frame kernel (-1: none)
-bool g_fft_attr_done[64][8][3][3] = {};
+bool g_fft_attr_done[64][8][3][3][2] = {};
 int g_fft_split_max[64][8][3][3] = {};
 
 }  // namespace
@@ -59,8 +64,8 @@ int g_fft_split_max[64][8][3][3] = {};
 // Launch shape of the FFT-SPA kernel for a code: check-node form and degree
 // buckets, block size (one frame per SM), shared memory (code blob, decisions,
 // control word, and for the lane-per-edge form one transformed vector per
-// lane), resident blocks, message slot of nnz * q floats.
-int nbldpc_host::fft_configure(nbldpc_code* c) {
+// lane, then message rows), resident blocks, message slot of nnz * q floats.
+int nbldpc_host::fft_configure(nbldpc_code* c, const int32_t* row_ptr) {
   // check-node form: lane per edge (dc 0: check degree <= 32) for small fields
   // and for q <= 64 codes with a check of degree > 8; otherwise the
   // distributed form with the check degree bucket 4 or 8
@@ -69,8 +74,7 @@ int nbldpc_host::fft_configure(nbldpc_code* c) {
   const int dv = c->vmax <= 2 ? 2 : (c->vmax <= 4 ? 4 : (c->vmax <= 8 ? 8 : 0));
   if (dc < 0 || !dv) return NBLDPC_ERR_UNSUPPORTED;
   int threads = 0;
-  const void* k = fft_kernel_for(c->q, dc, dv, 0, &threads);
-  if (!k) return NBLDPC_ERR_UNSUPPORTED;
+  if (!fft_kernel_for(c->q, dc, dv, 0, &threads)) return NBLDPC_ERR_UNSUPPORTED;
   int dev = 0, sms = 0, optin = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
@@ -85,21 +89,36 @@ int nbldpc_host::fft_configure(nbldpc_code* c) {
   const int w_area = dc == 0 ? threads * c->q * (int)sizeof(float) : 0;   // one transformed vector per lane
   pl.slot_smem = pl.smem = (int)round_up((size_t)(pl.blob_cap + pl.n_cap + 16), 256) + w_area;
   if (pl.smem > optin) return NBLDPC_ERR_UNSUPPORTED;
+  // the rest of the shared memory holds message rows: all of them, or those of the first
+  // checks, whole warps of them
+  const int row_bytes = c->q * (int)sizeof(float);
+  const long long room = optin - pl.smem;
+  int rows = c->nnz;
+  if ((long long)rows * row_bytes > room) {
+    const long long most = std::max(0LL, (room - kFftL1) / row_bytes);
+    const int step = dc == 0 ? 1 : 32 / (c->q == 256 ? 32 : c->q / 4);   // checks of a warp
+    int r = 0;
+    while (r + step <= c->m && row_ptr[r + step] <= most) r += step;
+    rows = row_ptr[r];
+  }
+  pl.xs_off = pl.smem;
+  pl.smem += (int)round_up((size_t)rows * row_bytes, 16);
+  c->fft_res_edges = rows;
+  c->fft_form = rows == c->nnz ? 1 : 0;
+  const void* k = fft_kernel_for(c->q, dc, dv, c->fft_form);
   {
     std::lock_guard<std::mutex> lk(g_attr_mu);
     const int iq = nbldpc::ilog2(c->q) - 1, ic = dc == 0 ? 0 : (dc == 4 ? 1 : 2), iv = dv == 2 ? 0 : (dv == 4 ? 1 : 2);
-    bool& done = g_fft_attr_done[dev][iq][ic][iv];
+    bool& done = g_fft_attr_done[dev][iq][ic][iv][c->fft_form];
     int& split = g_fft_split_max[dev][iq][ic][iv];
-    int split_threads = 0;
-    const void* ks = fft_kernel_for(c->q, dc, dv, 1, &split_threads);
     if (!done) {
       if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, optin) != cudaSuccess)
         return NBLDPC_ERR_CUDA;
-      split = split_kernel_prepare(ks, split_threads, optin);
+      if (split == 0) split = split_kernel_prepare(fft_kernel_for(c->q, dc, dv, 2), threads, optin);
       done = true;
     }
     c->fft_split_max = split;
-    c->fft_split_threads = split_threads;
+    c->fft_split_threads = threads;
   }
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pl.per_sm, k, pl.threads, pl.smem) != cudaSuccess)
     return NBLDPC_ERR_CUDA;
@@ -148,36 +167,36 @@ FftSplitShape fft_split_layout(const nbldpc_code* c, int size, int threads) {
 //
 // The one-block kernel gives a frame one SM.  A cluster shortens a frame's
 // passes, but the variable-node pass then reads the other ranks' rows: at
-// throughput it is slower (GF(64) N=576, 4096 frames: 5.6 ms against 8.2 ms at
+// throughput it is slower (GF(64) N=576, 4096 frames: 5.5 ms against 8.2 ms at
 // best), so it serves batches that leave SMs idle.  Measured on GB300, us per
 // decode of up to 20 iterations with early stop, one block against this rule:
-// GF(64) N=576, 1 / 48 / 200 / 400 frames 311 / 362 / 646 / 843 against 88 / 249 /
-// 572 / 945 (not taken); GF(16) N=1024, 1 / 96 / 200 frames 337 / 339 / 449 against
-// 116 / 236 / 346; GF(256) N=384, 1 / 96 / 200 frames 1971 / 1952 / 2551 against
-// 273 / 1068 / 2115; GF(8) N=512, 48 frames 162 against 121.
-//  - 128-thread ranks and few frames only where a frame has fewer than 1024
-//    check-node lanes, none below 400 (GF(16) N=100: 72 against 80 at one frame).
-//  - The lane-per-edge form (q <= 4) up to 3/8 frame per SM (GF(4) N=1024,
-//    48 / 96 frames: 153 / 153 against 117 / 161).
+// GF(64) N=576, 1 / 48 / 200 frames 299 / 356 / 628 against 88 / 245 / 586; GF(16)
+// N=1024, 1 / 96 / 200 frames 299 / 304 / 400 against 116 / 235 / 357; GF(256) N=384,
+// 1 / 96 / 200 frames 1872 / 1881 / 2421 against 276 / 1054 / 2096.
+//  - The fewer check-node lanes a frame has, the fewer frames: from 2000 on, one and
+//    a half frames per SM; from 1024 on, 3/8 (GF(256) (2,8) N=128, 48 / 96 frames:
+//    519 / 519 against 366 / 550); from 400 on, and in the lane-per-edge form, 1/8
+//    (GF(4) N=1024, 1 / 96 frames: 132 / 130 against 95 / 161), none below (GF(16)
+//    N=100, one frame: 72 against 80).
 //  - Equal iterations for every frame have no tail to shorten: up to 3/8 frame
-//    per SM (96 frames of GF(64) N=576: 168 against 214), and for q <= 32 between
-//    one frame per SM and one and a half, which the one-block kernel takes in two
-//    waves (200 frames of GF(16) N=1024, 5 iterations: 183 against 162).
+//    per SM (96 frames of GF(64) N=576: 164 against 229), and for q <= 32 between
+//    one frame per SM and four thirds, which the one-block kernel takes in two
+//    waves (200 frames of GF(32) N=600, 5 iterations: 292 against 279).
 FftSplitShape fft_split_shape(const nbldpc_code* c, int frames, int early_stop) {
   if (c->fft_split_max == 0) return FftSplitShape{};
   const bool lane_form = c->fft_dc == 0;
   const int sms = c->fft_plan.grid_max / c->fft_plan.per_sm;
-  const int lanes = lane_form ? c->nnz : c->m * (c->q == 256 ? 32 : c->q / 4);
+  const int lanes = lane_form ? 512 : c->m * (c->q == 256 ? 32 : c->q / 4);
   if (lanes < 400) return FftSplitShape{};
-  const int few = 3 * sms / 8, two_waves = 3 * sms / 2;
-  const bool most = frames <= few || (frames <= two_waves && lanes >= 1024 && !lane_form &&
-                                      (early_stop || (c->q <= 32 && frames > sms)));
-  if (!most) return FftSplitShape{};
+  const int few = lanes < 1024 ? sms / 8 : 3 * sms / 8;
+  const bool more = lanes >= 2000 && (early_stop ? frames <= 3 * sms / 2
+                                                 : c->q <= 32 && frames > sms && frames <= 4 * sms / 3);
+  if (frames > few && !more) return FftSplitShape{};
   int size = frames <= sms / 8 ? 16 : frames <= 3 * sms / 4 ? 8 : 4;
   int threads = c->q == 64 || c->q == 128 ? c->fft_split_threads / 2 : 256;
   if (lanes < 1024) {
     size = 8;
-    threads = 128;
+    threads = lane_form ? 256 : 128;
   }
   size = std::min(size, c->fft_split_max);
   FftSplitShape s = fft_split_layout(c, size, threads);
@@ -206,7 +225,7 @@ int fft_launch(const nbldpc_code* c, const float* prob, int frames, int max_iter
   FftSplitShape sp = fft_split_shape(c, frames, early_stop);
   if (sp.size) {
     sp.p.job = fp.job;
-    return split_launch(fft_kernel_for(c->q, c->fft_dc, c->fft_dv, 1), frames, sp.size, sp.threads, sp.smem, &sp.p, st);
+    return split_launch(fft_kernel_for(c->q, c->fft_dc, c->fft_dv, 2), frames, sp.size, sp.threads, sp.smem, &sp.p, st);
   }
   fp.counter = reinterpret_cast<unsigned int*>(ws);
   fp.msg = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(ws) + 256);
@@ -214,10 +233,12 @@ int fft_launch(const nbldpc_code* c, const float* prob, int frames, int max_iter
   fp.blob_cap = pl.blob_cap;
   fp.n_cap = pl.n_cap;
   fp.w_off = (int)round_up((size_t)(pl.blob_cap + pl.n_cap + 16), 256);
+  fp.x_off = pl.xs_off;
+  fp.res_edges = c->fft_res_edges;
   cudaError_t e = cudaMemsetAsync(ws, 0, sizeof(unsigned int), st);
   if (e != cudaSuccess) return NBLDPC_ERR_CUDA;
   void* args[] = {&fp};
-  e = cudaLaunchKernel(fft_kernel_for(c->q, c->fft_dc, c->fft_dv, 0), dim3(grid_for(pl, frames)), dim3(pl.threads),
+  e = cudaLaunchKernel(fft_kernel_for(c->q, c->fft_dc, c->fft_dv, c->fft_form), dim3(grid_for(pl, frames)), dim3(pl.threads),
                        args, (size_t)pl.smem, st);
   if (e != cudaSuccess) return NBLDPC_ERR_CUDA;
   g_launches.fetch_add(1, std::memory_order_relaxed);

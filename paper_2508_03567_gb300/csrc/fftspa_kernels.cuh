@@ -53,7 +53,8 @@ struct FftParams {
   float* msg;                 // message slots, one per block: [nnz][q] floats
   size_t slot_floats;
   int blob_cap, n_cap;        // shared-memory layout: blob, decisions, control word,
-  int w_off;                  // then (q <= 64, 256-byte aligned) the transformed vectors, 32 * q floats per warp
+  int w_off;                  // then (q <= 64, 256-byte aligned) the transformed vectors, 32 * q floats per warp,
+  int x_off, res_edges;       // and the message rows of the first res_edges edges
 };
 
 // Elements per lane and block size of the distributed check-node form at
@@ -488,11 +489,14 @@ __device__ __forceinline__ void gray_gather(float (&acc)[Q], const int (&a4)[ilo
 // DC >= every check degree (register arrays of the distributed check-node
 // pass), or DC = 0: the lane-per-edge check-node pass (q <= 64, check degree
 // <= 32); DV >= every column degree.  SP: the block is one rank of a cluster
-// that decodes the frame together (SplitCtx of mma_kernels.cuh; X then holds the
-// message rows of the rank's own edges, in its shared memory).
-template <class g, int DC, int DV, bool SP = false>
-__device__ __forceinline__ void fft_decode_frame(const FftJob& job, int frame, float* Xown, const unsigned char* sblob,
-                                                 uint8_t* chat, float* wsm, const SplitCtx* sc = nullptr) {
+// that decodes the frame together (SplitCtx of mma_kernels.cuh).  Message rows: of
+// edge e in shared memory, Xs + e q, for e < res_edges, else in the block's global
+// slot, Xg + e q (SP: the rank's own edges at Xs, all in its shared memory).
+// RES: res_edges covers every edge.
+template <class g, int DC, int DV, bool RES, bool SP = false>
+__device__ __forceinline__ void fft_decode_frame(const FftJob& job, int frame, float* Xs, float* Xg, int res_edges,
+                                                 const unsigned char* sblob, uint8_t* chat, float* wsm,
+                                                 const SplitCtx* sc = nullptr) {
   using vg = VnpGeo<g::Q, DV>;
   constexpr int Q = g::Q, R = g::R, RV = vg::RV;
   const uint8_t* exp2 = sblob + job.off.exp2;        // x^(i mod (q-1)), i < 2(q-1)
@@ -517,15 +521,18 @@ __device__ __forceinline__ void fft_decode_frame(const FftJob& job, int frame, f
   const unsigned vmask = group_mask<vg::VG>(lane);
   const float* pf = job.prob + (size_t)frame * job.n * Q;
   float* app = job.out_app ? job.out_app + (size_t)frame * job.n * Q : nullptr;
-  // rows are addressed by edge number: a rank's area starts with the row of its first edge
-  float* X = SP ? Xown - (ptrdiff_t)sc->e0 * Q : Xown;
+  auto row = [&](int e) -> float* {
+    if constexpr (SP) return Xs + (size_t)(e - sc->e0) * Q;
+    else if constexpr (RES) return Xs + (size_t)e * Q;
+    else return (e < res_edges ? Xs : Xg) + (size_t)e * Q;
+  };
   const int r_first = SP ? sc->r0 : 0, r_last = SP ? sc->r1 : job.m;
   const int n_first = SP ? sc->n0 : 0, n_last = SP ? sc->n1 : job.n;
   const int k_first = SP ? vn_ptr[n_first] : 0;
   // message row of entry k of the column-ordered edge list, decision of column c
   auto vn_row = [&](int k) -> float* {
     if constexpr (SP) return reinterpret_cast<float*>(sc->vrow[k - k_first]);
-    else return X + (size_t)vn_edge[k] * Q;
+    else return row(vn_edge[k]);
   };
   auto decision = [&](int c) -> int {
     if constexpr (SP) return *at_rank(chat + c, c / sc->npc);
@@ -634,7 +641,7 @@ __device__ __forceinline__ void fft_decode_frame(const FftJob& job, int frame, f
       const bool valid = e < ee;
       if (valid) {
         float v[Q];
-        load_vec<Q>(first ? pf + (size_t)edge_col[e] * Q : X + (size_t)e * Q, v);   // u^(0) = p
+        load_vec<Q>(first ? pf + (size_t)edge_col[e] * Q : row(e), v);   // u^(0) = p
         wht_full<Q>(v);                                                            // W_e = FFT(u_e)
         if constexpr (Q >= 4) {
 #pragma unroll
@@ -674,7 +681,7 @@ __device__ __forceinline__ void fft_decode_frame(const FftJob& job, int frame, f
         wht_full<Q>(acc);                                                          // inverse FFT (times q)
 #pragma unroll
         for (int i = 0; i < Q; ++i) acc[i] = fmaxf(acc[i] * (1.f / Q), 0.f);       // v'_e, rounding below 0 -> 0
-        store_vec<Q>(X + (size_t)e * Q, acc);
+        store_vec<Q>(row(e), acc);
       }
       __syncwarp();
     }
@@ -694,8 +701,8 @@ __device__ __forceinline__ void fft_decode_frame(const FftJob& job, int frame, f
     const int y0s = SF ? (y0 ^ (gl & ((1 << RL) - 1))) : y0;
     const bool y0snz = y0s != 0;
     const int ly0s = y0snz ? glog[y0s] : 0;
-    for (int r = r_first + grp; r < r_last; r += ngroups) {
-      const int e0 = row_ptr[r], d = row_ptr[r + 1] - e0;
+    // one check of edges e0 .. e0 + d - 1; `at(e)` is the row of edge e
+    auto check = [&](int e0, int d, auto at) {
       float W[DC][R];
       // absent edges (d < DC) enter the product as the transform of the unit
       // vector at 0, all ones; in the select-free form an odd number of them
@@ -717,7 +724,7 @@ __device__ __forceinline__ void fft_decode_frame(const FftJob& job, int frame, f
           int idx[R];
           perm_index<g>(idx, exp2, edge_lhi[e], ly0s, y0snz);
           // u'_j(y) = u_j(h_j^-1 y); u^(0) = p on the first pass
-          const float* src = first ? pf + (size_t)edge_col[e] * Q : X + (size_t)e * Q;
+          const float* src = first ? pf + (size_t)edge_col[e] * Q : at(e);
 #pragma unroll
           for (int i = 0; i < R; ++i) W[j][i] = src[idx[i]];
           if constexpr (SF) wht_sf<g, false>(W[j], gl, gmask);
@@ -745,13 +752,23 @@ __device__ __forceinline__ void fft_decode_frame(const FftJob& job, int frame, f
           int idx[R];
           perm_index<g>(idx, exp2, edge_lhi[e], ly0, y0nz);
           // v'_j(h_j^-1 y) = v_j(y): inverse transform / q, negative rounding -> 0
-          float* dst = X + (size_t)e * Q;
+          float* dst = at(e);
           static_for<0, R>([&](auto I) {
             constexpr int i = decltype(I)::value;
             const float t = SF ? v[i] * sf_coef<T.out[i], g::G>(gl) : v[i];
             dst[idx[i]] = fmaxf(t * (1.f / Q), 0.f);
           });
         }
+      }
+    };
+    for (int r = r_first + grp; r < r_last; r += ngroups) {
+      const int e0 = row_ptr[r], d = row_ptr[r + 1] - e0;
+      if constexpr (SP || RES) {
+        check(e0, d, row);
+      } else {
+        // (the host ends res_edges between two warps' checks, so that a check is on one side)
+        if (e0 < res_edges) check(e0, d, [&](int e) { return Xs + (size_t)e * Q; });
+        else check(e0, d, [&](int e) { return Xg + (size_t)e * Q; });
       }
     }
     }
@@ -793,7 +810,7 @@ template <int Q, int DC, int DV> struct FftThreads {
 
 // Persistent blocks, one frame at a time; DC / DV bound the check and column
 // degrees of the code (register arrays of the two passes).
-template <int Q, int DC, int DV>
+template <int Q, int DC, int DV, bool RES>
 __global__ void __launch_bounds__(FftThreads<Q, DC, DV>::v, 1) fftspa_decode_kernel(const __grid_constant__ FftParams p) {
   unsigned char* smem = fft_smem;
   unsigned char* sblob = smem;
@@ -801,6 +818,7 @@ __global__ void __launch_bounds__(FftThreads<Q, DC, DV>::v, 1) fftspa_decode_ker
   volatile int* ctl = reinterpret_cast<volatile int*>(smem + p.blob_cap + p.n_cap);
   const FftJob& job = p.job;
   float* X = p.msg + (size_t)blockIdx.x * p.slot_floats;
+  float* Xs = reinterpret_cast<float*>(smem + p.x_off);
   float* wsm = reinterpret_cast<float*>(smem + p.w_off);
   for (int i = threadIdx.x; i < job.off.fft_bytes / 16; i += blockDim.x)
     reinterpret_cast<uint4*>(sblob)[i] = reinterpret_cast<const uint4*>(job.blob)[i];
@@ -809,7 +827,7 @@ __global__ void __launch_bounds__(FftThreads<Q, DC, DV>::v, 1) fftspa_decode_ker
     __syncthreads();
     const int frame = ctl[0];
     if (frame >= job.frames) break;
-    fft_decode_frame<FftGeo<Q>, DC, DV>(job, frame, X, sblob, chat, wsm);
+    fft_decode_frame<FftGeo<Q>, DC, DV, RES>(job, frame, Xs, X, p.res_edges, sblob, chat, wsm);
     __syncthreads();
   }
 }
@@ -876,7 +894,7 @@ __global__ void __launch_bounds__(FftThreads<Q, DC, DV>::v, 1)
     vrow[k - vn_ptr[sc.n0]] = reinterpret_cast<uint8_t*>(at_rank(X, owner) + (size_t)(e - row_ptr[first_check(owner)]) * Q);
   }
   cluster_barrier();           // the row table is complete, and every rank of the cluster runs
-  fft_decode_frame<FftGeo<Q>, DC, DV, true>(job, frame, X, sblob, smem + p.chat_off,
+  fft_decode_frame<FftGeo<Q>, DC, DV, true, true>(job, frame, X, nullptr, 0, sblob, smem + p.chat_off,
                                             reinterpret_cast<float*>(smem + p.w_off), &sc);
 }
 

@@ -68,6 +68,7 @@ struct nbldpc_code {
   int fft_status = NBLDPC_ERR_UNSUPPORTED;   // FFT-SPA launch shape below valid when NBLDPC_OK
   int fft_dc = 0, fft_dv = 0;          // FFT-SPA check-node form (dc 0: lane per edge) and column-degree bucket
   int fft_split_max = 0, fft_split_threads = 0;   // largest cluster and block of the FFT-SPA split-frame kernel
+  int fft_res_edges = 0, fft_form = 0; // edges whose FFT-SPA messages stay in shared memory; 1 when that is all
   int ntasks = 0;                      // FFT-SPA warp tasks (blob section)
   nbldpc_host::Plan fft_plan{};
   std::mutex mu;                       // guards the lazily created copy stream
@@ -88,7 +89,7 @@ inline int check_device(const nbldpc_code* c) {
 
 // FFT-SPA launch shape of a code (fftspa_host.cu): NBLDPC_OK, NBLDPC_ERR_UNSUPPORTED
 // when no FFT-SPA kernel covers the code, or NBLDPC_ERR_CUDA.
-int fft_configure(nbldpc_code* c);
+int fft_configure(nbldpc_code* c, const int32_t* row_ptr);
 
 // ---- frames split over the blocks of a cluster ------------------------------
 // Set a split-frame kernel's attributes; the largest cluster that the device runs

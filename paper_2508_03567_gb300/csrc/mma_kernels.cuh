@@ -420,10 +420,12 @@ __device__ __forceinline__ int pr_conv(const uint32_t* __restrict__ A, const uin
 // ---------------------------------------------------------------- parameters
 struct CodeBlob {           // offsets (bytes) into the code blob
   int exp2, log, row_ptr, edge_col, edge_lh, edge_lhi, vn_ptr, vn_edge;
-  int perm;                   // q = 8, 16, 32: byte selectors of every multiplication (PermRow)
-  int bytes;
-  // FFT-SPA section, after `bytes` (the min-max kernels stage only [0, bytes)):
-  // check of each edge, first check of each warp task, transposed-multiplication basis
+  // q = 8, 16, 32: byte selectors of every multiplication (PermRow), staged at `perm`
+  // behind the sections above, from perm_src behind the FFT-SPA section
+  int perm, perm_src;
+  int bytes;                  // staged by the min-max kernels
+  // FFT-SPA section, from `perm` on (the min-max kernels do not stage it): check of each
+  // edge, first check of each warp task, transposed-multiplication basis
   int edge_row, task_c0, at_log, fft_bytes;
 };
 
@@ -443,6 +445,13 @@ struct JobDesc {
   int item_begin;             // index of this job's first frame in the launch's work list
   unsigned long long* work;   // optional: adds the (x, y) pairs the convolutions visit (null: no count)
 };
+
+// Copy the sections of the code description that the min-max kernels read to shared memory.
+__device__ __forceinline__ void stage_blob(unsigned char* sblob, const JobDesc& job, int tid, int nthr) {
+  const int common = job.off.perm / 16, skip = (job.off.perm_src - job.off.perm) / 16;
+  for (int i = tid; i < job.off.bytes / 16; i += nthr)
+    reinterpret_cast<uint4*>(sblob)[i] = reinterpret_cast<const uint4*>(job.blob)[i < common ? i : i + skip];
+}
 
 constexpr int kMaxJobs = 32;
 
@@ -1570,8 +1579,7 @@ __global__ void __launch_bounds__(XS ? kResidentThreads : 256, XS ? 2 : PR ? NBL
     const JobDesc& job = (QSEL == 0) ? p.jobs[j] : p.jobs[0];
     const int frame = item - job.item_begin;
     if (j != staged) {      // stage the code description (GF tables, H, variable-node view)
-      for (int i = stid; i < job.off.bytes / 16; i += nthr)
-        reinterpret_cast<uint4*>(sblob)[i] = reinterpret_cast<const uint4*>(job.blob)[i];
+      stage_blob(sblob, job, stid, nthr);
       staged = j;
       slot_sync(bar_id, nthr);
     }
@@ -1612,8 +1620,7 @@ __global__ void __launch_bounds__(kResidentThreads, 2) mma_split_kernel(const __
   const int tid = threadIdx.x, nthr = blockDim.x;
   const int rank = blockIdx.x % p.size, frame = blockIdx.x / p.size;
   unsigned char* sblob = smem;
-  for (int i = tid; i < job.off.bytes / 16; i += nthr)
-    reinterpret_cast<uint4*>(sblob)[i] = reinterpret_cast<const uint4*>(job.blob)[i];
+  stage_blob(sblob, job, tid, nthr);
   SplitCtx sc;
   sc.rank = rank;
   sc.size = p.size;

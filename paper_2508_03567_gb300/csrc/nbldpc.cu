@@ -621,8 +621,8 @@ int nbldpc_code_create(int q, uint32_t prim_poly, int n_cols, int n_rows, const 
   off.vn_edge = take(2 * (size_t)nnz);
   const int perm_row = q == 8 ? nbldpc::PermRow<8>::bytes : q == 16 ? nbldpc::PermRow<16>::bytes
                      : q == 32 ? nbldpc::PermRow<32>::bytes : 0;
-  off.perm = take((size_t)perm_row * (q - 1));
-  off.bytes = (int)o;
+  off.perm = (int)o;
+  off.bytes = (int)(o + round_up((size_t)perm_row * (q - 1), 16));
   // FFT-SPA section: warp tasks pack consecutive checks with at most 32 edges in all
   std::vector<uint16_t> tasks;
   for (int r = 0; r < n_rows;) {
@@ -637,6 +637,7 @@ int nbldpc_code_create(int q, uint32_t prim_poly, int n_cols, int n_rows, const 
   off.task_c0 = take(2 * tasks.size());
   off.at_log = take((size_t)(q - 1) * pbits);
   off.fft_bytes = (int)o;
+  off.perm_src = take((size_t)perm_row * (q - 1));
   std::vector<unsigned char> blob(o, 0);
   {
     uint16_t* er = reinterpret_cast<uint16_t*>(&blob[off.edge_row]);
@@ -656,7 +657,7 @@ int nbldpc_code_create(int q, uint32_t prim_poly, int n_cols, int n_rows, const 
   // three bits of h y, then one mask word per four bytes for bit 3 and for bit 4
   for (int lh = 0; perm_row && lh < q - 1; ++lh)
     for (int y = 0; y < q; ++y) {
-      unsigned char* t = &blob[off.perm + (size_t)lh * perm_row];
+      unsigned char* t = &blob[off.perm_src + (size_t)lh * perm_row];
       const int i = y ? exp2[lg[y] + lh] : 0;
       t[y / 2] |= (unsigned char)((i & 7) << (4 * (y & 1)));
       const int sel = q == 8 ? nbldpc::PermRow<8>::sel_bytes : 16;
@@ -715,7 +716,7 @@ int nbldpc_code_create(int q, uint32_t prim_poly, int n_cols, int n_rows, const 
     if (st == NBLDPC_ERR_UNSUPPORTED) st = configure(c, v & 1, fpb);
   }
   if (st == NBLDPC_OK) {
-    c->fft_status = fft_configure(c);
+    c->fft_status = fft_configure(c, row_ptr);
     if (c->fft_status == NBLDPC_ERR_CUDA) st = NBLDPC_ERR_CUDA;
   }
   if (st != NBLDPC_OK) {
