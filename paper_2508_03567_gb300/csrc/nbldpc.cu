@@ -452,9 +452,10 @@ int split_resident(const nbldpc_code* c, const SplitShape& s) {
 //    half of them where the ranks fill an SM less than three quarters as full
 //    (GF(256): 400 frames of N=384 12.9 ms against 15.6); a third when
 //    every frame runs the same iterations (no tail: 1000 frames 7.1 ms against 7.7).
-//  - 16-bit messages: half of them from q = 64 (200 frames 2.9 against 2.3 ms; 1000
-//    frames 5.1 against 10.0), else a quarter (GF(16): 48 frames 1.72 against 0.89 ms,
-//    200 frames 1.93 against 2.11).
+//  - 16-bit messages: as many frames as the one-block kernels hold, half at q = 8
+//    (GF(64) N=576, 1 / 96 / 450 frames 1583 / 1655 / 3662 against 187 / 574 / 1910;
+//    GF(256) N=384, 200 frames 26.3 against 11.8 ms; GF(8) N=512, 200 / 450 frames
+//    243 / 271 against 184 / 324).
 SplitShape split_shape(const nbldpc_code* c, int frames, int early_stop) {
   if (c->split_max == 0 || c->pinned) return SplitShape{};
   const long long slots = (long long)c->plan.grid_max * c->plan.fpb;
@@ -471,7 +472,7 @@ SplitShape split_shape(const nbldpc_code* c, int frames, int early_stop) {
   while (s.size == 0 && threads > 64) s = split_layout(c, size, threads = (threads - 1) / 64 * 64);
   if (s.size == 0) return s;
   long long most = early_stop ? 2 * slots : slots / 3;
-  if (c->mb == 2) most = std::min(most, c->q >= 64 ? slots / 2 : slots / 4);
+  if (c->mb == 2) most = std::min(most, c->q == 8 ? slots / 2 : slots);
   else if (reg_form(c->q) && (c->variant & 2))
     most = c->q == 16 ? (early_stop ? 5 : 3) * sms / 8 : early_stop ? 3 * sms : 5 * sms / 8;
   else if (4 * split_resident(c, s) < 3 * c->plan.per_sm * c->plan.threads) most = std::min(most, slots / 2);
