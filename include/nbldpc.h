@@ -216,8 +216,8 @@ int nbldpc_decode_batch(const nbldpc_job *jobs, int n_jobs, void *workspace_dev,
  * a few phases; the outputs are the same bit for bit.  Bit 2 needs a layout of
  * 32-lane groups (both layouts of GF(128) and GF(256), layout 0 of GF(64)),
  * 8-bit messages and the minimal schedule, and excludes bit 1 (otherwise
- * NBLDPC_ERR_UNSUPPORTED).  Mixed-code batches use the layout bit, and bit 2
- * for GF(128) and GF(256) codes.  nbldpc_code_create picks a default variant
+ * NBLDPC_ERR_UNSUPPORTED).  Mixed-code batches have one kernel form per field
+ * order whatever the variant (GF(128) and GF(256) pruned).  nbldpc_code_create picks a default variant
  * per field order and a frames-per-block value from the code size;
  * nbldpc_code_autotune measures every valid pair on the caller's frames and
  * keeps the fastest.  A batch of too few frames to fill the GPU this way (how

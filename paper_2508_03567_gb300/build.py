@@ -37,7 +37,9 @@ def _stale() -> bool:
 
 
 def _units():
-    units = [(os.path.join(CSRC, "kernels.cu"), f"kernels_q{q}.o", [f"-DNBLDPC_KQ={q}"]) for q in KERNEL_UNITS]
+    # (the mixed-code kernels call a function per field order: the launch bounds' 80 registers bind those too)
+    units = [(os.path.join(CSRC, "kernels.cu"), f"kernels_q{q}.o",
+              [f"-DNBLDPC_KQ={q}"] + (["-maxrregcount=80"] if q == 0 else [])) for q in KERNEL_UNITS]
     units += [(os.path.join(CSRC, "fftspa.cu"), f"fftspa_q{q}.o", [f"-DNBLDPC_FQ={q}"]) for q in FFT_UNITS]
     units.append((os.path.join(CSRC, "nbldpc.cu"), "nbldpc.o", []))
     units.append((os.path.join(CSRC, "fftspa_host.cu"), "fftspa_host.o", []))

@@ -67,6 +67,11 @@ const void* NBLDPC_CAT(kernel_q, NBLDPC_KQ)(int v, int mb, int t1, int dreg) {
 #endif
 }
 
+#if NBLDPC_KQ == 0
+// Address of the mixed-code kernel that decodes each frame on a cluster of blocks.
+const void* split_kernel_q0() { return reinterpret_cast<const void*>(&mma_split_batch_kernel<0>); }
+#endif
+
 #if NBLDPC_KQ >= 8
 // Address of the kernel that decodes a frame on a cluster of blocks, for mb-byte
 // messages (minimal schedule): the layout and the convolutions of the default variant

@@ -17,6 +17,8 @@
 #pragma once
 
 #include <cstdint>
+#include <type_traits>
+
 #include <cuda_runtime.h>
 
 namespace nbldpc {
@@ -278,31 +280,34 @@ __device__ __forceinline__ void mm_conv(const uint32_t* __restrict__ A, const ui
 // approximation; the work is the number of entries folded in, about
 // 17 of 256 for the GF(256) decoder's vectors instead of 256.
 //
-// One group of 32 lanes (one warp, so every branch below is warp-uniform);
-// lane L owns x = L * OPL + k (k < OPL), kept as OPL/2 packed pairs.  For
-// y = L' * OPL + i, x ^ y = (L ^ L') * OPL + (k ^ i): one aligned vector load of
-// block L ^ L' of the other side, and a permutation inside the block that
-// depends only on i, which the unrolled loop over i makes static.
+// One group of 32 lanes (one warp, so every branch below is warp-uniform).
+// Vectors are q bytes; lane L owns x = L * OPL + k (k < OPL), kept as OPL/2 packed
+// pairs.  For y = L' * OPL + i, x ^ y = (L ^ L') * OPL + (k ^ i): one aligned vector
+// load of block L ^ L' from copy i of the other side, whose blocks are permuted by
+// k -> k ^ i (OPL copies, written once per convolution).  The entries of a phase are
+// compacted into a list of records (value << 16 | byte offset of copy and block), so
+// that folding two of them in is a list load, two block loads and the maxima and
+// minima, with no search (a quarter of the maxima on the FMA pipe at q = 256).  Bound by
+// the ALU pipe (70 % busy): about 120 instructions a phase and 13 an entry.  Measured on
+// GB300 against finding an entry by ffs over a ballot and its value by shuffle, in eight
+// loops a phase: GF(256) (2,6) N=384, 4096 frames 52.1 against 46.9 ms; GF(256) (2,8)
+// N=128, 3000 frames 19.5 against 17.1 (the byte vectors also leave three blocks an SM);
+// GF(128) (2,4) N=256, 8192 frames 38.0 against 36.0.
 // tprev: prediction of max_x C(x) (the previous convolution's maximum); it
 // picks the side with fewer entries below it and the first phase's bound.
-// SW (q >= 128, else null): a scratch vector for the other side with the two
-// halves of every word exchanged, so that the odd i read their block without
-// permuting it.
+// tmp: kPrTmp<q> bytes of scratch.
 // Returns max_x C(x); with folded non-null, adds the number of entries folded in
-// (each entry is q pairs (x, y)).  Inputs and output must not alias.
+// (each entry is q pairs (x, y)).  C may be A or B: both are read before C is written.
 #ifndef NBLDPC_PRUNE_BACK
-#define NBLDPC_PRUNE_BACK 4          // first phase: hi = tprev - NBLDPC_PRUNE_BACK
-#endif
-#ifndef NBLDPC_PRUNE_UNROLL
-#define NBLDPC_PRUNE_UNROLL 2        // entries folded in per loop step
-#endif
-#ifndef NBLDPC_PRUNE_FMA
-#define NBLDPC_PRUNE_FMA 0           // eighths of the maxima on the FMA pipe
+#define NBLDPC_PRUNE_BACK 1          // first phase: hi = tprev - NBLDPC_PRUNE_BACK (4: 47.7 ms, -1: 47.7)
 #endif
 #ifndef NBLDPC_PRUNE_PHASES
 #define NBLDPC_PRUNE_PHASES 6        // after this many phases hi jumps to M
 #endif
-template <int NW> __device__ __forceinline__ void load_words(const uint32_t* p, uint32_t (&w)[NW]) {
+constexpr int kPrList = 64;          // records of the list (a longer phase is folded in parts)
+template <int Q> constexpr int kPrTmp = (Q / 32) * 2 * Q + (kPrList + 2) * 4 + 8;
+
+template <int NW> __device__ __forceinline__ void load_words(const unsigned char* p, uint32_t (&w)[NW]) {
   if constexpr (NW == 4) {
     const uint4 v = *reinterpret_cast<const uint4*>(p);
     w[0] = v.x; w[1] = v.y; w[2] = v.z; w[3] = v.w;
@@ -310,19 +315,40 @@ template <int NW> __device__ __forceinline__ void load_words(const uint32_t* p, 
     const uint2 v = *reinterpret_cast<const uint2*>(p);
     w[0] = v.x; w[1] = v.y;
   } else {
-    w[0] = p[0];
+    w[0] = *reinterpret_cast<const uint32_t*>(p);
   }
+}
+template <int NW> __device__ __forceinline__ void store_words(unsigned char* p, const uint32_t (&w)[NW]) {
+  if constexpr (NW == 4) *reinterpret_cast<uint4*>(p) = make_uint4(w[0], w[1], w[2], w[3]);
+  else if constexpr (NW == 2) *reinterpret_cast<uint2*>(p) = make_uint2(w[0], w[1]);
+  else *reinterpret_cast<uint32_t*>(p) = w[0];
 }
 
 template <class g>
-__device__ __forceinline__ int pr_conv(const uint32_t* __restrict__ A, const uint32_t* __restrict__ B,
-                                       uint16_t* __restrict__ C, uint32_t* __restrict__ SW, int lane, int tprev,
-                                       int* folded) {
+__device__ __forceinline__ int pr_conv(const uint8_t* A, const uint8_t* B, uint8_t* C, unsigned char* tmp, int lane,
+                                       int tprev, int* folded) {
   constexpr int OPL = g::Q / 32, NW = OPL / 2;
+  constexpr int BB = 2 * OPL, CB = 2 * g::Q;         // bytes of a block and of a copy
   static_assert(g::G == 32 && OPL >= 2 && NW <= 4, "one warp per convolution");
+  uint32_t* list = reinterpret_cast<uint32_t*>(tmp + OPL * CB);
+  // the lane's bytes of both sides (OPL bytes in one or two words), and as 16-bit pairs
+  uint32_t a8[2] = {0u, 0u}, b8[2] = {0u, 0u};
+  if constexpr (OPL == 8) {
+    const uint2 x = *reinterpret_cast<const uint2*>(A + lane * 8), y = *reinterpret_cast<const uint2*>(B + lane * 8);
+    a8[0] = x.x; a8[1] = x.y; b8[0] = y.x; b8[1] = y.y;
+  } else if constexpr (OPL == 4) {
+    a8[0] = *reinterpret_cast<const uint32_t*>(A + lane * 4);
+    b8[0] = *reinterpret_cast<const uint32_t*>(B + lane * 4);
+  } else {
+    a8[0] = *reinterpret_cast<const uint16_t*>(A + lane * 2);
+    b8[0] = *reinterpret_cast<const uint16_t*>(B + lane * 2);
+  }
   uint32_t a[NW], b[NW];
-  load_words<NW>(A + lane * NW, a);
-  load_words<NW>(B + lane * NW, b);
+#pragma unroll
+  for (int w = 0; w < NW; ++w) {
+    a[w] = __byte_perm(a8[w >> 1], 0, (w & 1) ? 0x4342 : 0x4140);
+    b[w] = __byte_perm(b8[w >> 1], 0, (w & 1) ? 0x4342 : 0x4140);
+  }
   // side: fewer entries <= tprev.  Per 16-bit half, 0x8000 + t - v has bit 15
   // set exactly when v <= t (values and t below 2^15: no borrow between halves)
   const uint32_t kt = 0x80008000u + (uint32_t)tprev * 0x10001u;
@@ -332,94 +358,97 @@ __device__ __forceinline__ int pr_conv(const uint32_t* __restrict__ A, const uin
     ca += __popc((kt - a[w]) & 0x80008000u);
     cb += __popc((kt - b[w]) & 0x80008000u);
   }
-  ca = (int)__reduce_add_sync(0xFFFFFFFFu, (unsigned)ca);
-  cb = (int)__reduce_add_sync(0xFFFFFFFFu, (unsigned)cb);
-  const bool swap = cb < ca;
-  const uint32_t* V = swap ? A : B;
-  uint32_t u[NW];
-  int left[OPL];                       // entry values still to fold in (0x10000 once folded)
+  const unsigned cc = __reduce_add_sync(0xFFFFFFFFu, (unsigned)(ca | (cb << 16)));
+  const bool swap = (cc >> 16) < (cc & 0xFFFFu);
+  const uint32_t e0 = swap ? b8[0] : a8[0], e1 = swap ? b8[1] : a8[1];   // the entries' values
+  uint32_t left[NW];                   // entries still to fold in (0x4000 added once listed)
 #pragma unroll
   for (int w = 0; w < NW; ++w) {
-    u[w] = swap ? b[w] : a[w];
-    left[2 * w] = (int)(u[w] & 0xFFFFu);
-    left[2 * w + 1] = (int)(u[w] >> 16);
+    left[w] = swap ? b[w] : a[w];
+    b[w] = swap ? a[w] : b[w];         // the other side
   }
-  constexpr bool kSw = g::Q >= 128;
-  if constexpr (kSw) {
+  // copies of the other side
+  const int lane_off = lane * BB;
+#pragma unroll
+  for (int i = 0; i < OPL; i += 2) {
     uint32_t t[NW];
 #pragma unroll
-    for (int w = 0; w < NW; ++w) t[w] = __byte_perm(swap ? a[w] : b[w], 0, 0x1032);
-    if constexpr (NW == 4) *reinterpret_cast<uint4*>(SW + lane * NW) = make_uint4(t[0], t[1], t[2], t[3]);
-    else *reinterpret_cast<uint2*>(SW + lane * NW) = make_uint2(t[0], t[1]);
-    __syncwarp();
+    for (int w = 0; w < NW; ++w) t[w] = b[w ^ (i >> 1)];
+    store_words<NW>(tmp + i * CB + lane_off, t);
+#pragma unroll
+    for (int w = 0; w < NW; ++w) t[w] = __byte_perm(t[w], 0, 0x1032);
+    store_words<NW>(tmp + (i + 1) * CB + lane_off, t);
   }
+  const unsigned lt = (1u << lane) - 1u;
   uint32_t acc[NW];
 #pragma unroll
   for (int w = 0; w < NW; ++w) acc[w] = 0xFFFFFFFFu;
-  int hi = max(tprev - NBLDPC_PRUNE_BACK, 0), M = 0;
+  int hi = max(tprev - NBLDPC_PRUNE_BACK, 0), M = 0, total = 0;
   for (int phase = 1;; ++phase) {
-    unsigned bal[OPL];
+    // entries <= hi not yet listed: element 2 w at bit 12 + w, element 2 w + 1 at bit 28 + w
+    const uint32_t kh = 0x80008000u + (uint32_t)min(hi, 0x3FFF) * 0x10001u;
+    uint32_t mm = 0;
 #pragma unroll
-    for (int i = 0; i < OPL; ++i) {
-      const bool p = left[i] <= hi;
-      bal[i] = __ballot_sync(0xFFFFFFFFu, p);
-      if (p) left[i] = 0x10000;
+    for (int w = 0; w < NW; ++w) {
+      const uint32_t m = (kh - left[w]) & 0x80008000u;
+      left[w] |= m >> 1;
+      mm |= m >> (3 - w);
     }
-#pragma unroll
-    for (int i = 0; i < OPL; ++i) {
-      unsigned m = bal[i];
-      while (m) {
-        // NBLDPC_PRUNE_UNROLL entries per step (a repeated entry changes no minimum)
-        int lp[NBLDPC_PRUNE_UNROLL];
-        lp[0] = __ffs(m) - 1;
-        m &= m - 1;
-#pragma unroll
-        for (int k = 1; k < NBLDPC_PRUNE_UNROLL; ++k) {
-          lp[k] = m ? __ffs(m) - 1 : lp[0];
-          m &= m - 1;
-        }
-        uint32_t uy[NBLDPC_PRUNE_UNROLL], v[NBLDPC_PRUNE_UNROLL][NW];
-#pragma unroll
-        for (int k = 0; k < NBLDPC_PRUNE_UNROLL; ++k) {
-          uy[k] = __byte_perm(__shfl_sync(0xFFFFFFFFu, u[i >> 1], lp[k]), 0, (i & 1) ? 0x3232 : 0x1010);
-          load_words<NW>(((i & 1) && kSw ? SW : V) + (lane ^ lp[k]) * NW, v[k]);
-        }
+    int n = 0;                         // records in the list
+    for (;;) {
+      const unsigned bal = __ballot_sync(0xFFFFFFFFu, mm != 0);
+      if (mm) {
+        const int bit = 31 - __clz(mm);
+        mm ^= 1u << bit;
+        const int i = ((bit & 15) - 12) * 2 + (bit >> 4);
+        const uint32_t v = __byte_perm(e0, e1, 0x8880 + i) & 0xFFu;
+        list[n + __popc(bal & lt)] = (v << 16) | (uint32_t)(i * CB + lane_off);
+      }
+      n += __popc(bal);
+      if (bal && n <= kPrList - 32) continue;
+      total += n;
+      __syncwarp();                    // (and, the first time, the copies are complete)
+      if (n & 1) {                     // an odd list ends with its last record twice
+        if (lane == 0) list[n] = list[n - 1];
+        __syncwarp();
+      }
+      for (int k = 0; k < n; k += 2) {
+        const uint2 r = *reinterpret_cast<const uint2*>(list + k);
+        uint32_t v0[NW], v1[NW];
+        load_words<NW>(tmp + ((r.x ^ (uint32_t)lane_off) & 0xFFFFu), v0);
+        load_words<NW>(tmp + ((r.y ^ (uint32_t)lane_off) & 0xFFFFu), v1);
+        const uint32_t u0 = __byte_perm(r.x, 0, 0x3232), u1 = __byte_perm(r.y, 0, 0x3232);
 #pragma unroll
         for (int w = 0; w < NW; ++w)
-#pragma unroll
-          for (int k = 0; k < NBLDPC_PRUNE_UNROLL; ++k) {
-            uint32_t t = v[k][w ^ (i >> 1)];
-            if ((i & 1) && !kSw) t = __byte_perm(t, 0, 0x1032);
-            acc[w] = vmin2(acc[w], (w * NBLDPC_PRUNE_UNROLL + k) * 8 < NBLDPC_PRUNE_FMA * NW * NBLDPC_PRUNE_UNROLL
-                                       ? vmax2_fma(t, uy[k]) : vmax2(t, uy[k]));
-          }
+          acc[w] = w < NW / 4 ? __vimin3_u16x2(acc[w], vmax2_fma(v0[w], u0), vmax2_fma(v1[w], u1))
+                           : __vimin3_u16x2(acc[w], vmax2(v0[w], u0), vmax2(v1[w], u1));
       }
+      if (!bal) break;
+      n = 0;
+      __syncwarp();
     }
     uint32_t mx = acc[0];
 #pragma unroll
     for (int w = 1; w < NW; ++w) mx = vmax2(mx, acc[w]);
     M = (int)__reduce_max_sync(0xFFFFFFFFu, max(mx & 0xFFFFu, mx >> 16));
-    if (M <= hi || hi >= 0xFFFF) break;                     // (the second: every entry folded in)
+    if (M <= hi || hi >= 255) break;                        // (the second: every entry folded in)
     if (M == 0xFFFF) hi = 2 * hi + 8;                       // nothing folded in yet
     else if (phase >= NBLDPC_PRUNE_PHASES) hi = M;
     else hi = min(M, max(hi + 2, (hi + M + 1) >> 1));
   }
-  if (folded) {               // folded entries carry 0x10000
-    int f = 0;
+  if (folded) *folded += total;
+  uint32_t c8[2] = {0u, 0u};
 #pragma unroll
-    for (int i = 0; i < OPL; ++i) f += left[i] >> 16;
-    *folded += (int)__reduce_add_sync(0xFFFFFFFFu, (unsigned)f);
-  }
-  uint32_t* c32 = reinterpret_cast<uint32_t*>(C) + lane * NW;
-  if constexpr (NW == 4) *reinterpret_cast<uint4*>(c32) = make_uint4(acc[0], acc[1], acc[2], acc[3]);
-  else if constexpr (NW == 2) *reinterpret_cast<uint2*>(c32) = make_uint2(acc[0], acc[1]);
-  else c32[0] = acc[0];
+  for (int w = 0; w < NW; w += 2) c8[w >> 1] = __byte_perm(acc[w], NW > 1 ? acc[w | 1] : 0u, 0x6420);
+  if constexpr (OPL == 8) *reinterpret_cast<uint2*>(C + lane * 8) = make_uint2(c8[0], c8[1]);
+  else if constexpr (OPL == 4) *reinterpret_cast<uint32_t*>(C + lane * 4) = c8[0];
+  else *reinterpret_cast<uint16_t*>(C + lane * 2) = (uint16_t)c8[0];
   return M;
 }
 
 // ---------------------------------------------------------------- parameters
 struct CodeBlob {           // offsets (bytes) into the code blob
-  int exp2, log, row_ptr, edge_col, edge_lh, edge_lhi, vn_ptr, vn_edge;
+  int exp2, log, row_ptr, edge_lh, edge_lhi, edge_col, vn_ptr, vn_edge;   // (in this order)
   // q = 8, 16, 32: byte selectors of every multiplication (PermRow), staged at `perm`
   // behind the sections above, from perm_src behind the FFT-SPA section
   int perm, perm_src;
@@ -429,7 +458,8 @@ struct CodeBlob {           // offsets (bytes) into the code blob
   int edge_row, task_c0, at_log, fft_bytes;
 };
 
-// One code and the frames to decode with it.
+// One code and the frames to decode with it.  (The mixed-code kernel reads edge_col and
+// the variable-node view from the blob in global memory, through L1, and stages the rest.)
 struct JobDesc {
   const unsigned char* blob;  // code description (device)
   CodeBlob off;
@@ -438,7 +468,9 @@ struct JobDesc {
   int32_t* out_iters;         // [frames]
   uint8_t* out_ok;            // [frames]
   int q, n, m, dmax, vmax;    // field order, columns, rows, largest row and column degree
-  int variant;                // bit 0: layout; bit 2: pruned convolutions (q >= 128, mixed-code kernel)
+  int perm_at;                // where the permutation selectors are staged, behind the other staged sections
+  int reg;                    // mixed-code kernel: register form of the check-node pass (q = 8, 16, 32), or
+                              // every check of degree 4 (q = 64)
   int key16;                  // (255 * (max column degree + 1) + 1) * q <= 65536: 16-bit argmin keys
   int group_bytes;            // per-group shared scratch for this code
   int frames, max_iters, early_stop;
@@ -446,10 +478,12 @@ struct JobDesc {
   unsigned long long* work;   // optional: adds the (x, y) pairs the convolutions visit (null: no count)
 };
 
-// Copy the sections of the code description that the min-max kernels read to shared memory.
-__device__ __forceinline__ void stage_blob(unsigned char* sblob, const JobDesc& job, int tid, int nthr) {
-  const int common = job.off.perm / 16, skip = (job.off.perm_src - job.off.perm) / 16;
-  for (int i = tid; i < job.off.bytes / 16; i += nthr)
+// Copy the sections of the code description that the min-max kernels read to shared memory:
+// [0, common) bytes, then the permutation selectors.
+__device__ __forceinline__ void stage_blob(unsigned char* sblob, const JobDesc& job, int common_bytes, int tid, int nthr) {
+  const int common = common_bytes / 16, skip = (job.off.perm_src - common_bytes) / 16;
+  const int n = common + (job.off.bytes - job.off.perm) / 16;
+  for (int i = tid; i < n; i += nthr)
     reinterpret_cast<uint4*>(sblob)[i] = reinterpret_cast<const uint4*>(job.blob)[i < common ? i : i + skip];
 }
 
@@ -470,6 +504,11 @@ struct LaunchParams {
   int static_items;           // 1: no more items than frame slots; slot s takes item s (no counter)
 };
 
+// Control words of a frame slot, then (mixed-code kernel) a copy of its job.
+__host__ __device__ constexpr int ctl_bytes(int qsel) {
+  return 16 + (qsel == 0 ? (int)(sizeof(JobDesc) + 15) / 16 * 16 : 0);
+}
+
 // Threads of a block whose frame keeps its messages in shared memory (two
 // blocks per SM: the same 24 warps as three 256-thread blocks).
 constexpr int kResidentThreads = 384;
@@ -481,11 +520,12 @@ template <int Q> __host__ __device__ constexpr bool scatter_perm() { return Q >=
 
 // per-group shared scratch: the d incoming rows (q symbols of mb bytes each;
 // not with the scatter permutation) and 2*dmax+1 16-bit vectors: P_0..P_{d-1},
-// F_1..F_{d-2}, two B vectors and the middle beta R; q >= 128: one more, the
-// pruned convolution's half-swapped copy of its second operand
-template <int Q> __host__ __device__ constexpr int group_scratch_bytes(int dmax, int mb = 1) {
-  return (scatter_perm<Q>() ? 0 : ((dmax * Q * mb + 15) / 16) * 16) +
-         (2 * dmax + 1 + (Q >= 128 ? 1 : 0)) * vec_bytes<Q>();
+// F_1..F_{d-2}, two B vectors and the middle beta R.  Pruned convolutions: the
+// vectors are bytes, B_j takes the place of P_j and the middle beta that of F_{j-1},
+// and the copies and the list of pr_conv follow.
+template <int Q> __host__ __device__ constexpr int group_scratch_bytes(int dmax, int mb = 1, bool pr = false) {
+  return pr ? ((2 * dmax - 2) * Q + kPrTmp<Q> + 15) / 16 * 16
+            : (scatter_perm<Q>() ? 0 : ((dmax * Q * mb + 15) / 16) * 16) + (2 * dmax + 1) * vec_bytes<Q>();
 }
 
 // named barrier over the threads of one frame slot (ids 1..fpb)
@@ -766,16 +806,16 @@ template <int Q> __host__ __device__ constexpr int reg_scratch_bytes(int nthr, i
 constexpr int kW4Deg = 4;
 template <int DW>
 __device__ __forceinline__ bool decode_frame_warp4(const JobDesc& job, int frame, uint8_t* X,
-                                                   const unsigned char* sblob, int lane) {
+                                                   const unsigned char* sblob, const unsigned char* cold, int lane) {
   if (job.m > 32 || job.dmax > kW4Deg || job.vmax > 2) return false;
   const uint8_t* exp2 = sblob + job.off.exp2;
   const uint8_t* glog = sblob + job.off.log;
   const uint16_t* row_ptr = reinterpret_cast<const uint16_t*>(sblob + job.off.row_ptr);
-  const uint16_t* edge_col = reinterpret_cast<const uint16_t*>(sblob + job.off.edge_col);
+  const uint16_t* edge_col = reinterpret_cast<const uint16_t*>(cold + job.off.edge_col);
   const uint8_t* edge_lh = sblob + job.off.edge_lh;
   const uint8_t* edge_lhi = sblob + job.off.edge_lhi;
-  const uint16_t* vn_ptr = reinterpret_cast<const uint16_t*>(sblob + job.off.vn_ptr);
-  const uint16_t* vn_edge = reinterpret_cast<const uint16_t*>(sblob + job.off.vn_edge);
+  const uint16_t* vn_ptr = reinterpret_cast<const uint16_t*>(cold + job.off.vn_ptr);
+  const uint16_t* vn_edge = reinterpret_cast<const uint16_t*>(cold + job.off.vn_edge);
   const uint8_t* gam = job.gamma + (size_t)frame * job.n * 4;
   const bool mine = lane < job.m;
   const int e0 = mine ? row_ptr[lane] : 0, d = mine ? row_ptr[lane + 1] - e0 : 0;
@@ -962,7 +1002,8 @@ template <class T> __device__ __forceinline__ T* at_rank(T* p, int r) {
 // Decodes frame `frame` of `job` with the nthr threads of one frame slot
 // (slot thread index stid, named barrier bar_id).  sblob holds the job's code
 // description, chat[n] the decisions, scratch the per-group buffers; X is the
-// slot's message area ([nnz][q] bytes).
+// slot's message area ([nnz][q] bytes); cold: where edge_col and the variable-node view
+// of the description are (sblob, or the blob in global memory).
 // REG4: q = 4 codes take the register form of the check-node pass (single-field
 // kernels; the all-field kernel keeps the group form).  PR: the check-node
 // convolutions are pruned (pr_conv; 32-lane groups, 8-bit messages, minimal
@@ -974,8 +1015,8 @@ template <class T> __device__ __forceinline__ T* at_rank(T* p, int r) {
 // message rows of the rank's own edges).
 template <class g, int MB, bool T1, bool REG4 = true, bool PR = false, bool W4 = false, int D = 0, bool SP = false>
 __device__ __forceinline__ void decode_frame(const JobDesc& job, int frame, uint8_t* Xown, const unsigned char* sblob,
-                                             uint8_t* chat, unsigned char* scratch, int stid, int nthr, int bar_id,
-                                             const SplitCtx* sc = nullptr) {
+                                             const unsigned char* cold, uint8_t* chat, unsigned char* scratch,
+                                             int stid, int nthr, int bar_id, const SplitCtx* sc = nullptr) {
   constexpr int Q = g::Q;
   constexpr int PW = g::PW;
   constexpr int RS = Q * MB;                 // bytes of one message row
@@ -984,7 +1025,7 @@ __device__ __forceinline__ void decode_frame(const JobDesc& job, int frame, uint
   static_assert(!PR || (g::G == 32 && MB == 1 && !T1), "pruned convolutions: 32-lane groups, 8-bit, minimal");
   if constexpr (Q == 4 && MB == 1 && !T1 && REG4 && W4) {
     // one warp per frame: a slot of 32 threads
-    if (nthr == 32 && decode_frame_warp4<D == 4 ? 4 : 0>(job, frame, Xown, sblob, stid)) return;
+    if (nthr == 32 && decode_frame_warp4<D == 4 ? 4 : 0>(job, frame, Xown, sblob, cold, stid)) return;
   }
   // pairs (x, y) the convolutions visit in this frame (counted when job.work is set)
   const bool counting = job.work != nullptr;
@@ -992,11 +1033,11 @@ __device__ __forceinline__ void decode_frame(const JobDesc& job, int frame, uint
   const uint8_t* exp2 = sblob + job.off.exp2;        // x^(i mod (q-1)), i < 2(q-1)
   const uint8_t* glog = sblob + job.off.log;         // log_x(v), v >= 1
   const uint16_t* row_ptr = reinterpret_cast<const uint16_t*>(sblob + job.off.row_ptr);
-  const uint16_t* edge_col = reinterpret_cast<const uint16_t*>(sblob + job.off.edge_col);
+  const uint16_t* edge_col = reinterpret_cast<const uint16_t*>(cold + job.off.edge_col);
   const uint8_t* edge_lh = sblob + job.off.edge_lh;    // log_x(h) of each edge
   const uint8_t* edge_lhi = sblob + job.off.edge_lhi;  // log_x(h^-1) of each edge
-  const uint16_t* vn_ptr = reinterpret_cast<const uint16_t*>(sblob + job.off.vn_ptr);
-  const uint16_t* vn_edge = reinterpret_cast<const uint16_t*>(sblob + job.off.vn_edge);
+  const uint16_t* vn_ptr = reinterpret_cast<const uint16_t*>(cold + job.off.vn_ptr);
+  const uint16_t* vn_edge = reinterpret_cast<const uint16_t*>(cold + job.off.vn_edge);
 
   const int lane = threadIdx.x & 31;
   // check-node groups (G lanes per check)
@@ -1030,14 +1071,16 @@ __device__ __forceinline__ void decode_frame(const JobDesc& job, int frame, uint
   // de-permutation: log of the first symbol this lane writes (-1 for symbol 0)
   const int da_log0 = gl ? (int)glog[gl * g::BPL] : -1;
 
-  unsigned char* gs = scratch + (size_t)grp * job.group_bytes;
+  unsigned char* gs = scratch + (size_t)grp * (PR ? group_scratch_bytes<Q>(job.dmax, 1, true) : job.group_bytes);
   uint8_t* stage = gs;                                                   // [dmax][q * MB] bytes (staged rows)
   const int dm = D > 0 ? D : job.dmax;
   unsigned char* vecs = gs + (kScatter ? 0 : ((dm * RS + 15) / 16) * 16);
-  auto vec = [&](int i) { return reinterpret_cast<uint32_t*>(vecs + (size_t)i * g::VB); };
-  auto vec16 = [&](int i) { return reinterpret_cast<uint16_t*>(vecs + (size_t)i * g::VB); };
+  using Sym = std::conditional_t<PR, uint8_t, uint16_t>;     // a vector's elements
+  constexpr int VB = PR ? Q : g::VB;
+  auto vec = [&](int i) { return reinterpret_cast<uint32_t*>(vecs + (size_t)i * VB); };
+  auto vec16 = [&](int i) { return reinterpret_cast<Sym*>(vecs + (size_t)i * VB); };
   // vectors: P_j = vec(j) (j < dmax), F_j = vec(dmax + j - 1) (1 <= j <= d-2),
-  // B ping-pong = vec(2 dmax - 2), vec(2 dmax - 1), R = vec(2 dmax)
+  // B ping-pong = vec(2 dmax - 2), vec(2 dmax - 1), R = vec(2 dmax) (neither if PR)
   const int vF = dm - 1, vB = 2 * dm - 2, vR = 2 * dm;
   const uint8_t* gam = job.gamma + (size_t)frame * job.n * Q;
   // rows are addressed by edge number: a rank's area starts with the row of its first edge
@@ -1217,7 +1260,7 @@ __device__ __forceinline__ void decode_frame(const JobDesc& job, int frame, uint
       const int j = c / CH, part = c - j * CH;
       const int lh = edge_lh[e0 + j];
       const int h1 = exp2[lh], h2 = exp2[lh + 1], h4 = exp2[lh + 2];
-      uint16_t* Pv = vec16(j);
+      Sym* Pv = vec16(j);
       if constexpr (MB == 2) {
         int v[8];
         if (first) load_ints<8>(gam + (size_t)edge_col[e0 + j] * Q + part * 8, v);
@@ -1243,18 +1286,18 @@ __device__ __forceinline__ void decode_frame(const JobDesc& job, int frame, uint
 #pragma unroll
         for (int k = 0; k < 16; ++k) {
           const int y = yb ^ ((k & 1) ? h1 : 0) ^ ((k & 2) ? h2 : 0) ^ ((k & 4) ? h4 : 0) ^ ((k & 8) ? h8 : 0);
-          Pv[y] = (uint16_t)__byte_perm(w[k >> 2], 0, 0x4440 | (k & 3));
+          Pv[y] = (Sym)__byte_perm(w[k >> 2], 0, 0x4440 | (k & 3));
         }
       }
     };
     // predictions of max_x C(x), one per kind of convolution (F, B, beta): each
     // kind's maxima follow their own distribution
     int tpred[3] = {24, 24, 24};
-    auto conv = [&](const uint32_t* A, const uint32_t* B, uint16_t* C, int kind) {
+    auto conv = [&](const uint32_t* A, const uint32_t* B, Sym* C, int kind) {
       if constexpr (PR) {
         int folded = 0;
-        tpred[kind] = pr_conv<g>(A, B, C, Q >= 128 ? vec(2 * dm + 1) : nullptr, gl, tpred[kind],
-                                 counting ? &folded : nullptr);
+        tpred[kind] = pr_conv<g>(reinterpret_cast<const uint8_t*>(A), reinterpret_cast<const uint8_t*>(B), C,
+                                 vecs + (size_t)(2 * dm - 2) * VB, gl, tpred[kind], counting ? &folded : nullptr);
         if (counting && gl == 0) work += (unsigned long long)folded * Q;
       } else {
         mm_conv<g, MB == 1>(A, B, C, cl, gmask);
@@ -1307,7 +1350,7 @@ __device__ __forceinline__ void decode_frame(const JobDesc& job, int frame, uint
         group_sync<g::G>(gmask);
         // beta_j(a) = R_j(h_j a), written over the edge's message row; the lane's
         // symbols are a0 + i (a0 = gl * BPL, i < BPL) and h (a0 + i) = h a0 ^ h i
-        auto depermute = [=](const uint16_t* R16, int e) {
+        auto depermute = [=](const Sym* R16, int e) {
           const int lh = edge_lh[e];
           const int base = da_log0 >= 0 ? (int)exp2[da_log0 + lh] : 0;
           int hb[3] = {0, 0, 0};
@@ -1344,10 +1387,11 @@ __device__ __forceinline__ void decode_frame(const JobDesc& job, int frame, uint
         int pp = 0;
         for (int j = d - 2; j >= 1; --j) {
           const int fj = (j == 1) ? 0 : vF + j - 1;
-          conv(vec(fj), vec(bcur), vec16(vR), 2);
+          const int ro = PR ? fj : vR;
+          conv(vec(fj), vec(bcur), vec16(ro), 2);
           group_sync<g::G>(gmask);
-          depermute(vec16(vR), e0 + j);
-          const int bn = vB + pp;
+          depermute(vec16(ro), e0 + j);
+          const int bn = PR ? j : vB + pp;
           conv(vec(bcur), vec(j), vec16(bn), 1);
           group_sync<g::G>(gmask);
           bcur = bn;
@@ -1435,7 +1479,7 @@ __device__ __forceinline__ void decode_frame(const JobDesc& job, int frame, uint
     auto cnp_reg = [&](bool first) {
       if constexpr (reg_form<Q>()) {
         constexpr int W = Q / 2, NB = Q / 4;
-        const uint8_t* perm = sblob + job.off.perm;
+        const uint8_t* perm = sblob + job.perm_at;
         auto load_p = [&](int e, uint32_t (&P)[W]) {       // P_j(y) = alpha_j(h^-1 y)
           uint32_t r[NB], o[NB];
           load_row<Q>(first ? gam + (size_t)edge_col[e] * Q : X + (size_t)e * Q, r);
@@ -1541,7 +1585,7 @@ __device__ __forceinline__ void decode_frame(const JobDesc& job, int frame, uint
 // Persistent blocks of fpb frame slots; every slot takes work items (a frame
 // of one job) from a global counter until the list is exhausted.  QSEL = q,
 // VSEL = variant compiles the path of one field order and layout (single-code
-// launches); QSEL = 0, VSEL = -1 compiles every path (mixed-code launches).
+// launches); QSEL = 0, VSEL = -1 compiles every field order (mixed-code launches).
 // Resident 256-thread blocks per SM the register allocation must allow: the
 // q >= 128 paths need more than 85 registers per thread without spilling.
 #ifndef NBLDPC_MINB_64
@@ -1556,28 +1600,57 @@ __device__ __forceinline__ void decode_frame(const JobDesc& job, int frame, uint
 #ifndef NBLDPC_MINB_PRUNE
 #define NBLDPC_MINB_PRUNE 3
 #endif
+// The mixed-code kernel (QSEL = 0) has no dense q >= 128 path and fits 80 registers too.
 template <int QSEL, int VSEL> struct MinBlocks {
-  static constexpr int v = QSEL == 0 ? 2 : QSEL >= 128 ? NBLDPC_MINB_WIDE
+  static constexpr int v = QSEL == 0 ? 3 : QSEL >= 128 ? NBLDPC_MINB_WIDE
                          : (QSEL == 64 ? (VSEL == 1 ? 3 : NBLDPC_MINB_64) : 4);
 };
 
-// VSEL = 0 or 1 compiles one layout variant; VSEL = -1 both (chosen per job,
-// and for q >= 128 with or without pruned convolutions, bit 2 of the job's variant).
-template <int Q, int VSEL, int MB, bool T1 = false, bool PR = false, bool W4 = false, int D = 0>
-__device__ __forceinline__ void decode_variant(const JobDesc& job, int frame, uint8_t* X, const unsigned char* sblob,
-                                               uint8_t* chat, unsigned char* scratch, int stid, int nthr,
-                                               int bar_id) {
-  if constexpr (VSEL >= 0) {
-    decode_frame<Geo<Q, VSEL>, MB, T1, true, PR, W4, D>(job, frame, X, sblob, chat, scratch, stid, nthr, bar_id);
-  } else if (Q >= 128 && (job.variant & 4)) {
-    if constexpr (Q >= 128) {
-      if (job.variant & 1) decode_frame<Geo<Q, 1>, MB, T1, false, true>(job, frame, X, sblob, chat, scratch, stid, nthr, bar_id);
-      else decode_frame<Geo<Q, 0>, MB, T1, false, true>(job, frame, X, sblob, chat, scratch, stid, nthr, bar_id);
+// The mixed-code kernels' form of field order Q: the default layout, with pruned
+// convolutions for q >= 128; SP: the split-frame kernel's.
+template <int Q> __host__ __device__ constexpr int mixed_layout() { return Q >= 16 && Q <= 64 ? 1 : 0; }
+
+// Where a frame slot of a mixed-code launch keeps its things in shared memory (byte
+// offsets); X: its message area there (SP), else its global slot.
+struct MixedSlot {
+  int job, blob, chat, scratch, x, sc;
+  uint8_t* X;
+};
+
+// A function of its own: in line, the persistent kernel's frame loop kept a dozen registers
+// across every path, and the paths spilled at 80.  It takes offsets, so that its accesses are
+// shared-memory ones.
+template <int Q, bool REG, bool SP, int D = 0>
+__device__ __noinline__ void decode_mixed(MixedSlot m, int frame, int stid, int nthr, int bar_id) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  const JobDesc& job = *reinterpret_cast<const JobDesc*>(smem + m.job);
+  uint8_t* X = SP ? smem + m.x : m.X;
+  decode_frame<Geo<Q, mixed_layout<Q>()>, 1, false, true, (Q >= 128), REG, D, SP>(
+      job, frame, X, smem + m.blob, SP ? smem + m.blob : job.blob, smem + m.chat, smem + m.scratch, stid, nthr, bar_id,
+      reinterpret_cast<const SplitCtx*>(smem + m.sc));
+}
+
+template <bool SP>
+__device__ __forceinline__ void decode_any(const JobDesc& job, const MixedSlot& m, int frame, int stid, int nthr,
+                                           int bar_id) {
+  if constexpr (!SP) {
+    if (job.reg) {
+      if (job.q == 64) decode_mixed<64, false, SP, 4>(m, frame, stid, nthr, bar_id);
+      else if (job.q == 8) decode_mixed<8, true, SP>(m, frame, stid, nthr, bar_id);
+      else if (job.q == 16) decode_mixed<16, true, SP>(m, frame, stid, nthr, bar_id);
+      else decode_mixed<32, true, SP>(m, frame, stid, nthr, bar_id);
+      return;
     }
-  } else if ((job.variant & 1) == 0) {
-    decode_frame<Geo<Q, 0>, MB, T1, false>(job, frame, X, sblob, chat, scratch, stid, nthr, bar_id);
-  } else {
-    decode_frame<Geo<Q, 1>, MB, T1, false>(job, frame, X, sblob, chat, scratch, stid, nthr, bar_id);
+  }
+  switch (job.q) {
+    case 2: decode_mixed<2, false, SP>(m, frame, stid, nthr, bar_id); break;
+    case 4: decode_mixed<4, !SP, SP>(m, frame, stid, nthr, bar_id); break;
+    case 8: decode_mixed<8, false, SP>(m, frame, stid, nthr, bar_id); break;
+    case 16: decode_mixed<16, false, SP>(m, frame, stid, nthr, bar_id); break;
+    case 32: decode_mixed<32, false, SP>(m, frame, stid, nthr, bar_id); break;
+    case 64: decode_mixed<64, false, SP>(m, frame, stid, nthr, bar_id); break;
+    case 128: decode_mixed<128, false, SP>(m, frame, stid, nthr, bar_id); break;
+    default: decode_mixed<256, false, SP>(m, frame, stid, nthr, bar_id); break;
   }
 }
 
@@ -1601,7 +1674,9 @@ __global__ void __launch_bounds__(XS ? kResidentThreads : 256, XS ? 2 : PR ? NBL
   unsigned char* sblob = base;
   uint8_t* chat = base + p.blob_cap;
   volatile int* ctl = reinterpret_cast<volatile int*>(base + p.blob_cap + p.n_cap);
-  unsigned char* scratch = base + p.blob_cap + p.n_cap + 16;
+  constexpr int kCtl = ctl_bytes(QSEL);
+  unsigned char* scratch = base + p.blob_cap + p.n_cap + kCtl;
+  JobDesc* sjob = reinterpret_cast<JobDesc*>(base + p.blob_cap + p.n_cap + 16);   // (QSEL = 0)
   uint8_t* X = XS ? base + p.xs_off : p.msg + ((size_t)blockIdx.x * p.fpb + slot) * p.slot_bytes;
   int staged = -1;
 
@@ -1621,51 +1696,54 @@ __global__ void __launch_bounds__(XS ? kResidentThreads : 256, XS ? 2 : PR ? NBL
     const JobDesc& job = (QSEL == 0) ? p.jobs[j] : p.jobs[0];
     const int frame = item - job.item_begin;
     if (j != staged) {      // stage the code description (GF tables, H, variable-node view)
-      stage_blob(sblob, job, stid, nthr);
+      stage_blob(sblob, job, job.perm_at, stid, nthr);
+      if constexpr (QSEL == 0) {
+        for (int i = stid; i < (int)(sizeof(JobDesc) / 4); i += nthr)
+          reinterpret_cast<uint32_t*>(sjob)[i] = reinterpret_cast<const uint32_t*>(&job)[i];
+      }
       staged = j;
       slot_sync(bar_id, nthr);
     }
-    if constexpr (QSEL != 0) {
-      decode_variant<QSEL, VSEL, MB, T1, PR, XS, D>(job, frame, X, sblob, chat, scratch, stid, nthr, bar_id);
-    } else {
-      switch (job.q) {
-        case 2: decode_variant<2, -1, 1>(job, frame, X, sblob, chat, scratch, stid, nthr, bar_id); break;
-        case 4: decode_variant<4, -1, 1>(job, frame, X, sblob, chat, scratch, stid, nthr, bar_id); break;
-        case 8: decode_variant<8, -1, 1>(job, frame, X, sblob, chat, scratch, stid, nthr, bar_id); break;
-        case 16: decode_variant<16, -1, 1>(job, frame, X, sblob, chat, scratch, stid, nthr, bar_id); break;
-        case 32: decode_variant<32, -1, 1>(job, frame, X, sblob, chat, scratch, stid, nthr, bar_id); break;
-        case 64: decode_variant<64, -1, 1>(job, frame, X, sblob, chat, scratch, stid, nthr, bar_id); break;
-        case 128: decode_variant<128, -1, 1>(job, frame, X, sblob, chat, scratch, stid, nthr, bar_id); break;
-        default: decode_variant<256, -1, 1>(job, frame, X, sblob, chat, scratch, stid, nthr, bar_id); break;
-      }
-    }
+    if constexpr (QSEL != 0)
+      decode_frame<Geo<QSEL, VSEL>, MB, T1, true, PR, XS, D>(job, frame, X, sblob, sblob, chat, scratch, stid, nthr,
+                                                                   bar_id);
+    else
+      decode_any<false>(*sjob,
+                        MixedSlot{(int)(reinterpret_cast<unsigned char*>(sjob) - smem), (int)(sblob - smem),
+                                  (int)(chat - smem), (int)(scratch - smem), 0, 0, X},
+                        frame, stid, nthr, bar_id);
     slot_sync(bar_id, nthr);
   }
 }
 
-// ---------------------------------------------------------------- the kernel of split frames
+// ---------------------------------------------------------------- the kernels of split frames
 // One cluster per frame (grid: frames * cluster size).  Shared memory of a rank:
-// code blob | decisions (n_cap bytes, indexed by column) | flags | row table |
-// reliabilities of its columns | check-node scratch | message rows of its edges.
-struct SplitParams {
-  JobDesc job;
-  int size;                   // ranks per frame
+// code blob | decisions (indexed by column) | flags | row table | reliabilities of
+// its columns | check-node scratch | message rows of its edges.
+struct SplitLayout {
   int cpc, npc;               // checks and columns per rank
   int chat_off, flag_off, row_off, gam_off, scratch_off, x_off;
 };
+struct SplitParams {          // one code
+  JobDesc job;
+  int size;                   // ranks per frame
+  SplitLayout lay;
+};
+struct SplitBatchParams {     // mixed codes; the jobs' frames form one list
+  JobDesc jobs[kMaxJobs];
+  SplitLayout lay[kMaxJobs];
+  int njobs, size;
+  int job_off, sc_off;        // the rank's copies of its job and SplitCtx in shared memory
+};
 
-template <int Q, int V, int MB, bool PR>
-__global__ void __launch_bounds__(kResidentThreads, 2) mma_split_kernel(const __grid_constant__ SplitParams p) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  constexpr int RS = Q * MB;
-  const JobDesc& job = p.job;
+// Set up this rank of a frame's cluster (code description, reliabilities, row table); rs:
+// bytes of a message row.
+__device__ __forceinline__ void split_setup(const JobDesc& job, const SplitLayout& p, int frame, int rank, int size,
+                                            int q, int rs, unsigned char* smem, SplitCtx& sc) {
   const int tid = threadIdx.x, nthr = blockDim.x;
-  const int rank = blockIdx.x % p.size, frame = blockIdx.x / p.size;
-  unsigned char* sblob = smem;
-  stage_blob(sblob, job, tid, nthr);
-  SplitCtx sc;
+  stage_blob(smem, job, job.off.perm, tid, nthr);
   sc.rank = rank;
-  sc.size = p.size;
+  sc.size = size;
   sc.r0 = min(rank * p.cpc, job.m);
   sc.r1 = min(sc.r0 + p.cpc, job.m);
   sc.n0 = min(rank * p.npc, job.n);
@@ -1676,33 +1754,59 @@ __global__ void __launch_bounds__(kResidentThreads, 2) mma_split_kernel(const __
   sc.vrow = vrow;
   uint8_t* sgam = smem + p.gam_off;
   sc.gam = sgam;
-  // reliabilities of the rank's columns (gamma is 16-byte aligned)
-  {
-    const uint8_t* src = job.gamma + ((size_t)frame * job.n + sc.n0) * Q;
-    const int bytes = (sc.n1 - sc.n0) * Q;
-    static_assert(Q >= 8, "rows of 8-byte words");
-    if constexpr (Q >= 16) {
-      for (int i = tid; i < bytes / 16; i += nthr)
-        reinterpret_cast<uint4*>(sgam)[i] = reinterpret_cast<const uint4*>(src)[i];
-    } else {
-      for (int i = tid; i < bytes / 8; i += nthr)
-        reinterpret_cast<uint2*>(sgam)[i] = reinterpret_cast<const uint2*>(src)[i];
-    }
+  const uint8_t* src = job.gamma + ((size_t)frame * job.n + sc.n0) * q;   // (gamma is 16-byte aligned)
+  const int bytes = (sc.n1 - sc.n0) * q;
+  if (q >= 16) {
+    for (int i = tid; i < bytes / 16; i += nthr)
+      reinterpret_cast<uint4*>(sgam)[i] = reinterpret_cast<const uint4*>(src)[i];
+  } else {
+    for (int i = tid; i < bytes / 2; i += nthr)
+      reinterpret_cast<uint16_t*>(sgam)[i] = reinterpret_cast<const uint16_t*>(src)[i];
   }
   __syncthreads();
-  const uint16_t* row_ptr = reinterpret_cast<const uint16_t*>(sblob + job.off.row_ptr);
-  const uint16_t* vn_ptr = reinterpret_cast<const uint16_t*>(sblob + job.off.vn_ptr);
-  const uint16_t* vn_edge = reinterpret_cast<const uint16_t*>(sblob + job.off.vn_edge);
+  const uint16_t* row_ptr = reinterpret_cast<const uint16_t*>(smem + job.off.row_ptr);
+  const uint16_t* vn_ptr = reinterpret_cast<const uint16_t*>(smem + job.off.vn_ptr);
+  const uint16_t* vn_edge = reinterpret_cast<const uint16_t*>(smem + job.off.vn_edge);
   const uint16_t* edge_row = reinterpret_cast<const uint16_t*>(job.blob + job.off.edge_row);
   sc.e0 = row_ptr[sc.r0];
   uint8_t* X = smem + p.x_off;
   for (int k = vn_ptr[sc.n0] + tid; k < vn_ptr[sc.n1]; k += nthr) {
     const int e = vn_edge[k], owner = edge_row[e] / p.cpc;
-    vrow[k - vn_ptr[sc.n0]] = at_rank(X, owner) + (size_t)(e - row_ptr[owner * p.cpc]) * RS;
+    vrow[k - vn_ptr[sc.n0]] = at_rank(X, owner) + (size_t)(e - row_ptr[owner * p.cpc]) * rs;
   }
   cluster_barrier();           // the row table is complete, and every rank of the cluster runs
-  decode_frame<Geo<Q, V>, MB, false, true, PR, false, 0, true>(job, frame, X, sblob, smem + p.chat_off,
-                                                               smem + p.scratch_off, tid, nthr, 1, &sc);
+}
+
+template <int Q, int V, int MB, bool PR>
+__global__ void __launch_bounds__(kResidentThreads, 2) mma_split_kernel(const __grid_constant__ SplitParams p) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int rank = blockIdx.x % p.size, frame = blockIdx.x / p.size;
+  SplitCtx sc;
+  split_setup(p.job, p.lay, frame, rank, p.size, Q, Q * MB, smem, sc);
+  decode_frame<Geo<Q, V>, MB, false, true, PR, false, 0, true>(p.job, frame, smem + p.lay.x_off, smem, smem,
+                                                               smem + p.lay.chat_off, smem + p.lay.scratch_off,
+                                                               threadIdx.x, blockDim.x, 1, &sc);
+}
+
+// 8-bit messages, minimal schedule.  (A template, so that only the mixed-code unit compiles it.)
+template <int QSEL>
+__global__ void __launch_bounds__(kResidentThreads, 2) mma_split_batch_kernel(const __grid_constant__ SplitBatchParams p) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int rank = blockIdx.x % p.size, item = blockIdx.x / p.size;
+  int j = 0;
+  while (j + 1 < p.njobs && item >= p.jobs[j + 1].item_begin) ++j;
+  const JobDesc& job = p.jobs[j];
+  const SplitLayout& lay = p.lay[j];
+  const int frame = item - job.item_begin;
+  JobDesc* sjob = reinterpret_cast<JobDesc*>(smem + p.job_off);
+  for (int i = threadIdx.x; i < (int)(sizeof(JobDesc) / 4); i += blockDim.x)
+    reinterpret_cast<uint32_t*>(sjob)[i] = reinterpret_cast<const uint32_t*>(&job)[i];
+  SplitCtx sc;
+  split_setup(job, lay, frame, rank, p.size, job.q, job.q, smem, sc);
+  if (threadIdx.x == 0) *reinterpret_cast<SplitCtx*>(smem + p.sc_off) = sc;
+  __syncthreads();
+  decode_any<true>(*sjob, MixedSlot{p.job_off, 0, lay.chat_off, lay.scratch_off, lay.x_off, p.sc_off, nullptr}, frame,
+                   threadIdx.x, blockDim.x, 1);
 }
 
 }  // namespace nbldpc

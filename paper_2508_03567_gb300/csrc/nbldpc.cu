@@ -15,7 +15,7 @@
 #include "mma_kernels.cuh"
 
 static_assert(nbldpc::kMaxJobs == NBLDPC_MAX_BATCH_JOBS, "job table size");
-static_assert(sizeof(nbldpc::LaunchParams) < 32000, "kernel parameter space");
+static_assert(sizeof(nbldpc::LaunchParams) < 32000 && sizeof(nbldpc::SplitBatchParams) < 32000, "kernel parameter space");
 
 std::atomic<uint64_t> nbldpc_host::g_launches{0};
 std::mutex nbldpc_host::g_attr_mu;
@@ -61,6 +61,7 @@ const void* kernel_q32(int v, int mb, int t1, int dreg);
 const void* kernel_q64(int v, int mb, int t1, int dreg);
 const void* kernel_q128(int v, int mb, int t1, int dreg);
 const void* kernel_q256(int v, int mb, int t1, int dreg);
+const void* split_kernel_q0();
 const void* split_kernel_q8(int mb);
 const void* split_kernel_q16(int mb);
 const void* split_kernel_q32(int mb);
@@ -101,9 +102,10 @@ int kernel_dreg(int q, int v, int km, int dreg) {
 }
 
 // kernel that decodes a frame on a cluster of blocks (minimal schedule), null where
-// split_shape never takes it
+// split_shape never takes it; q = 0: mixed codes, 8-bit messages
 const void* split_kernel_for(int q, int mb) {
   switch (q) {
+    case 0: return nbldpc::split_kernel_q0();
     case 8: return nbldpc::split_kernel_q8(mb);
     case 16: return nbldpc::split_kernel_q16(mb);
     case 32: return nbldpc::split_kernel_q32(mb);
@@ -113,6 +115,8 @@ const void* split_kernel_for(int q, int mb) {
   }
   return nullptr;
 }
+
+int mixed_layout(int q) { return q >= 16 && q <= 64 ? 1 : 0; }   // as in mma_kernels.cuh
 
 template <int Q> int lanes(int v) { return v ? nbldpc::Geo<Q, 1>::G : nbldpc::Geo<Q, 0>::G; }
 
@@ -130,16 +134,16 @@ int group_lanes(int q, int v) {
   return 0;
 }
 
-int group_bytes(int q, int dmax, int mb) {
+int group_bytes(int q, int dmax, int mb, bool pr) {
   switch (q) {
     case 2: return nbldpc::group_scratch_bytes<2>(dmax, mb);
     case 4: return nbldpc::group_scratch_bytes<4>(dmax, mb);
     case 8: return nbldpc::group_scratch_bytes<8>(dmax, mb);
     case 16: return nbldpc::group_scratch_bytes<16>(dmax, mb);
     case 32: return nbldpc::group_scratch_bytes<32>(dmax, mb);
-    case 64: return nbldpc::group_scratch_bytes<64>(dmax, mb);
-    case 128: return nbldpc::group_scratch_bytes<128>(dmax, mb);
-    case 256: return nbldpc::group_scratch_bytes<256>(dmax, mb);
+    case 64: return nbldpc::group_scratch_bytes<64>(dmax, mb, pr);
+    case 128: return nbldpc::group_scratch_bytes<128>(dmax, mb, pr);
+    case 256: return nbldpc::group_scratch_bytes<256>(dmax, mb, pr);
   }
   return 0;
 }
@@ -174,12 +178,12 @@ int prepare_kernel(int q, int v, int km, int dreg, int dev, int smem_optin) {
 // Largest cluster of split-frame blocks (16, else the portable 8) that the device
 // runs for a field order and message width; 0 when the kernel cannot be prepared.
 // The kernel attributes are set and the device asked once.
-int g_split_max[64][8][2] = {};
+int g_split_max[64][9][2] = {};
 
 int split_max(int q, int mb, int dev, int smem_optin) {
   std::lock_guard<std::mutex> lk(g_attr_mu);
   if (dev < 0 || dev >= 64) return 0;
-  int& mx = g_split_max[dev][nbldpc::ilog2(q) - 1][mb - 1];
+  int& mx = g_split_max[dev][q ? nbldpc::ilog2(q) : 0][mb - 1];
   if (mx == 0) {
     const void* k = split_kernel_for(q, mb);
     mx = k ? split_kernel_prepare(k, nbldpc::kResidentThreads, smem_optin) : 0;
@@ -216,6 +220,10 @@ int reg_scratch(int q, int nthr, int dmax) {
                 : q == 16 ? nbldpc::reg_scratch_bytes<16>(nthr, dmax) : nbldpc::reg_scratch_bytes<32>(nthr, dmax);
 }
 
+// Whether a code takes the register form in the mixed-code kernel: its scratch must leave
+// three blocks on an SM.
+bool mixed_reg(int q, int nthr, int dmax) { return reg_form(q) && reg_scratch(q, nthr, dmax) <= 32768; }
+
 // Plan a launch of kernel (kq, kv, kernel mode km) with fpb frame slots per block for a set of codes.
 // Variants 2 and 3 keep each frame's messages in shared memory: blocks of
 // nbldpc::kResidentThreads threads (1, 2 or 4 frame slots) or of 256 threads with
@@ -243,8 +251,9 @@ int make_plan(int kq, int kv, int km, int fpb, const CodeNeeds* cs, int nc, Plan
   for (int i = 0; i < nc; ++i) {
     const int G = group_lanes(cs[i].q, cs[i].variant & 1);
     if (G > nthr) return NBLDPC_ERR_UNSUPPORTED;
-    const int s = reg ? reg_scratch(cs[i].q, nthr, cs[i].dmax)
-                      : (nthr / G) * group_bytes(cs[i].q, cs[i].dmax, cs[i].mb);
+    const int s = reg || (kq == 0 && mixed_reg(cs[i].q, nthr, cs[i].dmax))
+                      ? reg_scratch(cs[i].q, nthr, cs[i].dmax)
+                      : (nthr / G) * group_bytes(cs[i].q, cs[i].dmax, cs[i].mb, kq == 0 ? cs[i].q >= 128 : (kv & 4) != 0);
     if (s > scratch) scratch = s;
     if (cs[i].blob > pl.blob_cap) pl.blob_cap = cs[i].blob;
     if (cs[i].n > pl.n_cap) pl.n_cap = cs[i].n;
@@ -252,7 +261,7 @@ int make_plan(int kq, int kv, int km, int fpb, const CodeNeeds* cs, int nc, Plan
   }
   pl.blob_cap = (int)round_up((size_t)pl.blob_cap, 16);
   pl.n_cap = (int)round_up((size_t)pl.n_cap, 16);
-  pl.slot_smem = (int)round_up((size_t)(pl.blob_cap + pl.n_cap + 16 + scratch), 16);
+  pl.slot_smem = (int)round_up((size_t)(pl.blob_cap + pl.n_cap + nbldpc::ctl_bytes(kq) + scratch), 16);
   if (resident) {   // the messages follow the slot's scratch
     pl.xs_off = pl.slot_smem;
     pl.slot_smem += (int)round_up(pl.slot_bytes, 16);
@@ -348,11 +357,11 @@ nbldpc::JobDesc job_desc(const nbldpc_code* c, const uint8_t* gamma, int frames,
   j.n = c->n;
   j.m = c->m;
   j.dmax = c->dmax;
-  j.variant = c->variant & 5;          // layout and pruning (a mixed-code kernel keeps messages in the workspace)
   j.work = count ? c->work_counter : nullptr;
   j.vmax = c->vmax;
+  j.perm_at = c->off.perm;
   j.key16 = (255 * (c->vmax + 1) + 1) * c->q <= 65536 ? 1 : 0;
-  j.group_bytes = group_bytes(c->q, c->dmax, c->mb);
+  j.group_bytes = group_bytes(c->q, c->dmax, c->mb, false);
   j.frames = frames;
   j.max_iters = max_iters;
   j.early_stop = early_stop ? 1 : 0;
@@ -391,28 +400,25 @@ int launch_plan(const void* kernel, const Plan& pl, nbldpc::LaunchParams& lp, in
 // Shape of a split launch: ranks per frame, threads per rank, shared memory of a rank.
 struct SplitShape {
   int size = 0, threads = 0, smem = 0;
-  nbldpc::SplitParams p{};
+  nbldpc::SplitLayout lay{};
 };
-
-int split_layout_variant(int q) { return (q >= 16 && q <= 64) ? 1 : 0; }   // kernels.cu: split_kernel_q*
 
 // Lay out a rank's shared memory; size 0 when it does not fit the device.
 SplitShape split_layout(const nbldpc_code* c, int size, int threads) {
   SplitShape s;
-  const int G = group_lanes(c->q, split_layout_variant(c->q));
-  s.p.size = size;
-  s.p.cpc = (c->m + size - 1) / size;
-  s.p.npc = (c->n + size - 1) / size;
-  const long long edges_r = std::min<long long>(c->nnz, (long long)s.p.cpc * c->dmax);
-  const long long edges_n = std::min<long long>(c->nnz, (long long)s.p.npc * c->vmax);
+  const int G = group_lanes(c->q, mixed_layout(c->q));
+  s.lay.cpc = (c->m + size - 1) / size;
+  s.lay.npc = (c->n + size - 1) / size;
+  const long long edges_r = std::min<long long>(c->nnz, (long long)s.lay.cpc * c->dmax);
+  const long long edges_n = std::min<long long>(c->nnz, (long long)s.lay.npc * c->vmax);
   size_t o = c->off.bytes;
   auto take = [&](size_t bytes) { const size_t at = o; o = round_up(o + bytes, 16); return (int)at; };
-  s.p.chat_off = take((size_t)c->n);
-  s.p.flag_off = take(2 * nbldpc::kMaxSplit * sizeof(int));
-  s.p.row_off = take((size_t)edges_n * sizeof(void*));
-  s.p.gam_off = take((size_t)s.p.npc * c->q);
-  s.p.scratch_off = take((size_t)(threads / G) * group_bytes(c->q, c->dmax, c->mb));
-  s.p.x_off = take((size_t)edges_r * c->q * c->mb);
+  s.lay.chat_off = take((size_t)c->n);
+  s.lay.flag_off = take(2 * nbldpc::kMaxSplit * sizeof(int));
+  s.lay.row_off = take((size_t)edges_n * sizeof(void*));
+  s.lay.gam_off = take((size_t)s.lay.npc * c->q);
+  s.lay.scratch_off = take((size_t)(threads / G) * group_bytes(c->q, c->dmax, c->mb, c->mb == 1 && c->q >= 128));
+  s.lay.x_off = take((size_t)edges_r * c->q * c->mb);
   if (o > (size_t)c->smem_optin) return SplitShape{};
   s.size = size;
   s.threads = threads;
@@ -461,7 +467,7 @@ SplitShape split_shape(const nbldpc_code* c, int frames, int early_stop) {
   const long long slots = (long long)c->plan.grid_max * c->plan.fpb;
   if (frames > 2 * slots) return SplitShape{};
   const int sms = c->plan.grid_max / c->plan.per_sm;
-  const int G = group_lanes(c->q, split_layout_variant(c->q));
+  const int G = group_lanes(c->q, mixed_layout(c->q));
   int size = frames <= sms / 8 ? 16 : 8;
   int threads = frames <= 3 * sms / 8 ? 384 : frames <= 3 * sms / 4 ? 256 : 128;
   size = std::min(size, c->split_max);
@@ -479,9 +485,9 @@ SplitShape split_shape(const nbldpc_code* c, int frames, int early_stop) {
   return frames <= most ? s : SplitShape{};
 }
 
-int launch_split(const nbldpc_code* c, SplitShape& s, const nbldpc::JobDesc& job, cudaStream_t st) {
-  s.p.job = job;
-  return split_launch(split_kernel_for(c->q, c->mb), job.frames, s.size, s.threads, s.smem, &s.p, st);
+int launch_split(const nbldpc_code* c, const SplitShape& s, const nbldpc::JobDesc& job, cudaStream_t st) {
+  nbldpc::SplitParams p{job, s.size, s.lay};
+  return split_launch(split_kernel_for(c->q, c->mb), job.frames, s.size, s.threads, s.smem, &p, st);
 }
 
 // split: small batches may go to the split-frame kernel (not while the autotuner times a tuning)
@@ -489,7 +495,7 @@ int launch(const nbldpc_code* c, const uint8_t* gamma, int frames, int max_iters
            int32_t* iters, uint8_t* ok, void* ws, cudaStream_t st, bool count = true, bool split = true) {
   if (frames == 0) return NBLDPC_OK;
   if (split) {
-    SplitShape s = split_shape(c, frames, early_stop);
+    const SplitShape s = split_shape(c, frames, early_stop);
     if (s.size) return launch_split(c, s, job_desc(c, gamma, frames, max_iters, early_stop, sym, iters, ok, 0, count), st);
   }
   nbldpc::LaunchParams lp{};
@@ -541,7 +547,7 @@ int nbldpc_decode_noalloc(const nbldpc_code* c, const uint8_t* gamma_dev, int fr
   }
   st = cuda_status(cudaGetLastError());
   if (st != NBLDPC_OK) return st;
-  SplitShape sp = split_shape(c, frames, early_stop);
+  const SplitShape sp = split_shape(c, frames, early_stop);
   if (sp.size)
     return launch_split(c, sp,
                         job_desc(c, gamma_dev, frames, max_iters, early_stop, out_sym_dev, out_iters_dev, out_ok_dev, 0),
@@ -608,16 +614,16 @@ int nbldpc_code_create(int q, uint32_t prim_poly, int n_cols, int n_rows, const 
   }
   if (dmax > 64 || vmax > 64) return NBLDPC_ERR_UNSUPPORTED;
 
-  // code blob: exp2 | log | row_ptr u16 | edge_col u16 | edge_lh u8 | edge_lhi u8 | vn_ptr u16 | vn_edge u16
+  // code blob: exp2 | log | row_ptr u16 | edge_lh u8 | edge_lhi u8 | edge_col u16 | vn_ptr u16 | vn_edge u16
   nbldpc::CodeBlob off{};
   size_t o = 0;
   auto take = [&](size_t bytes) { const size_t at = o; o = round_up(o + bytes, 16); return (int)at; };
   off.exp2 = take(2 * (size_t)q);
   off.log = take((size_t)q);
   off.row_ptr = take(2 * ((size_t)n_rows + 1));
-  off.edge_col = take(2 * (size_t)nnz);
   off.edge_lh = take((size_t)nnz);
   off.edge_lhi = take((size_t)nnz);
+  off.edge_col = take(2 * (size_t)nnz);
   off.vn_ptr = take(2 * ((size_t)n_cols + 1));
   off.vn_edge = take(2 * (size_t)nnz);
   const int perm_row = q == 8 ? nbldpc::PermRow<8>::bytes : q == 16 ? nbldpc::PermRow<16>::bytes
@@ -832,6 +838,22 @@ int nbldpc_decode(const nbldpc_code* c, const uint8_t* gamma_dev, int frames, in
 }
 
 // ---- mixed-code batches -----------------------------------------------------
+// Frame slots per block that suit a code in the mixed-code kernel: the pinned count, or (register
+// form) enough threads per slot for the checks, or the group form's default.
+static int batch_fpb(const nbldpc_code* c) {
+  if (c->pinned) return c->plan.fpb;
+  if (!reg_form(c->q)) return c->plan.fpb;
+  int fpb = 1;
+  while (fpb < 8 && kThreads / (2 * fpb) >= std::max(32, c->m)) fpb *= 2;
+  return fpb;
+}
+
+// Convolution work of a frame's longest decode (pruned convolutions as a tenth).
+static double frame_work(const nbldpc_job& j) {
+  const nbldpc_code* c = j.code;
+  return (double)j.max_iters * c->nnz * c->q * c->q * (c->q >= 128 ? 0.1 : 1.0);
+}
+
 static int batch_plan(const nbldpc_job* jobs, int n_jobs, Plan* pl, int* total) {
   if (!jobs || n_jobs < 1 || n_jobs > NBLDPC_MAX_BATCH_JOBS) return NBLDPC_ERR_ARG;
   CodeNeeds need[NBLDPC_MAX_BATCH_JOBS];
@@ -843,15 +865,68 @@ static int batch_plan(const nbldpc_job* jobs, int n_jobs, Plan* pl, int* total) 
     const int st = check_device(c);
     if (st != NBLDPC_OK) return st;
     if (kmode(c) != 1) return NBLDPC_ERR_UNSUPPORTED;   // mixed-code launches: 8-bit messages, minimal schedule
-    need[i] = needs_of(c, c->variant & 1, 1);
-    // the all-field kernel runs the group form: its slots are not the register form's
-    const int f = reg_form(c->q) && !c->pinned ? default_fpb(c) : c->plan.fpb;
-    if (f < fpb) fpb = f;
+    need[i] = needs_of(c, mixed_layout(c->q), 1);
+    need[i].blob = c->off.edge_col + c->off.bytes - c->off.perm;   // what the mixed-code kernel stages
+    fpb = std::min(fpb, batch_fpb(c));
     t += jobs[i].frames;
   }
   if (t > 0x7FFFFFFF) return NBLDPC_ERR_ARG;
   *total = (int)t;
+  // few frames: a block each (GF(4) N=48 and GF(8) N=100, 200 frames each: 100 us at two a block, 92 at one)
+  const Plan& pl0 = jobs[0].code->plan;
+  if (t <= 3LL * (pl0.grid_max / pl0.per_sm)) fpb = 1;
   return make_plan(0, -1, 1, fpb, need, n_jobs, pl);
+}
+
+// Shape of a mixed batch whose frames are each decoded on a cluster (size 0: one block per frame
+// slot): the ranks and threads of split_shape, the jobs' layouts one over the other.  Frames count
+// by their work against the longest ones' (an eighth at least): one block per frame ends with the
+// longest frames alone.  Taken up to three such frames per SM with early stop (the serving loop's
+// small groups; 5/8 when q = 16 is the widest field), 3/8 without, and six frames of any kind; not
+// for q <= 8 alone.  Measured on GB300,
+// us per batch against the one-block kernel: 60 / 240 / 450 frames of GF(64) N=576, GF(16) N=1024 and
+// GF(256) N=128 in equal parts 2746 / 3455 / 3878 against 795 / 1444 / 2399; one frame of GF(64)
+// 1243 against 179.
+static int batch_split(const nbldpc_job* jobs, int n_jobs, int total, const Plan& pl, nbldpc::SplitBatchParams* p,
+                       SplitShape* out) {
+  const nbldpc_code* c0 = jobs[0].code;
+  const int sms = pl.grid_max / pl.per_sm;
+  bool stop = true;
+  int q_most = 0;
+  double longest = 0.0, like_longest = 0.0;
+  for (int i = 0; i < n_jobs; ++i)
+    if (jobs[i].frames > 0) {
+      stop = stop && jobs[i].early_stop;
+      q_most = std::max(q_most, jobs[i].code->q);
+      longest = std::max(longest, frame_work(jobs[i]));
+    }
+  if (q_most <= 8 || total > 6 * sms) return 0;
+  for (int i = 0; i < n_jobs; ++i)
+    like_longest += jobs[i].frames * std::max(0.125, longest > 0.0 ? frame_work(jobs[i]) / longest : 1.0);
+  if (like_longest > (!stop ? 3 * sms / 8 : q_most > 16 ? 3 * sms : 5 * sms / 8)) return 0;
+  const int most = split_max(0, 1, c0->device, c0->smem_optin);
+  const int size = std::min(total <= sms / 8 ? 16 : 8, most);
+  if (size < 2) return 0;
+  for (int threads = total <= 3 * sms / 8 ? 384 : total <= 3 * sms / 4 ? 256 : 128; threads >= 64; threads -= 64) {
+    SplitShape all;
+    bool fits = true;
+    for (int i = 0; i < n_jobs && fits; ++i) {
+      const SplitShape s = split_layout(jobs[i].code, size, threads);
+      fits = s.size != 0;
+      p->lay[i] = s.lay;
+      all.smem = std::max(all.smem, s.smem);
+    }
+    if (!fits) continue;
+    all.size = size;
+    all.threads = threads;
+    p->job_off = all.smem;
+    p->sc_off = p->job_off + (int)round_up(sizeof(nbldpc::JobDesc), 16);
+    all.smem = p->sc_off + (int)round_up(sizeof(nbldpc::SplitCtx), 16);
+    if (all.smem > c0->smem_optin) continue;
+    *out = all;
+    return size;
+  }
+  return 0;
 }
 
 int nbldpc_decode_batch_workspace_size(const nbldpc_job* jobs, int n_jobs, size_t* bytes) {
@@ -873,6 +948,13 @@ int nbldpc_decode_batch(const nbldpc_job* jobs, int n_jobs, void* workspace_dev,
   if (!workspace_dev || !aligned(workspace_dev, 16) || workspace_bytes < ws_bytes(pl, total)) return NBLDPC_ERR_ARG;
   nbldpc::LaunchParams lp{};
   int begin = 0;
+  // The jobs with the longest frames first, so that they are not the ones that end the launch.
+  int order[NBLDPC_MAX_BATCH_JOBS];
+  for (int i = 0; i < n_jobs; ++i) order[i] = i;
+  std::stable_sort(order, order + n_jobs, [&](int a, int b) { return frame_work(jobs[a]) > frame_work(jobs[b]); });
+  nbldpc_job sorted[NBLDPC_MAX_BATCH_JOBS];
+  for (int i = 0; i < n_jobs; ++i) sorted[i] = jobs[order[i]];
+  jobs = sorted;
   for (int i = 0; i < n_jobs; ++i) {
     const nbldpc_job& j = jobs[i];
     if (j.frames > 0 && !valid_outputs(j.gamma_dev, j.out_sym_dev, j.out_iters_dev, j.out_ok_dev))
@@ -885,6 +967,22 @@ int nbldpc_decode_batch(const nbldpc_job* jobs, int n_jobs, void* workspace_dev,
   lp.total_items = total;
   st = cuda_status(cudaGetLastError());
   if (st != NBLDPC_OK) return st;
+  if (total > 0) {
+    nbldpc::SplitBatchParams sp{};
+    SplitShape shape;
+    if (batch_split(jobs, n_jobs, total, pl, &sp, &shape)) {
+      memcpy(sp.jobs, lp.jobs, sizeof(sp.jobs));   // (perm_at, reg: the one-block kernel's, set below)
+      sp.njobs = n_jobs;
+      sp.size = shape.size;
+      return split_launch(split_kernel_for(0, 1), total, shape.size, shape.threads, shape.smem, &sp,
+                          reinterpret_cast<cudaStream_t>(cuda_stream));
+    }
+  }
+  for (int i = 0; i < n_jobs; ++i) {
+    const nbldpc_code* c = jobs[i].code;
+    lp.jobs[i].perm_at = c->off.edge_col;          // it stages no edge_col or variable-node view
+    lp.jobs[i].reg = mixed_reg(c->q, pl.threads / pl.fpb, c->dmax) || (c->q == 64 && c->dreg == 4) ? 1 : 0;
+  }
   return launch_plan(kernel_for(0, -1, 1), pl, lp, grid_for(pl, total), workspace_dev,
                      reinterpret_cast<uint8_t*>(workspace_dev) + 256, reinterpret_cast<cudaStream_t>(cuda_stream));
 }

@@ -114,3 +114,35 @@ def test_split_decode_replays_from_a_cuda_graph():
     torch.cuda.synchronize()
     for a, w in zip((sym, its, ok), oracle.decode(code, g.cpu().numpy(), 20, 1, threads=THREADS)):
         assert np.array_equal(a.cpu().numpy(), w)
+
+
+@pytest.mark.parametrize("frames", [(1, 0, 3, 2, 1, 2, 1, 2), (9, 20, 0, 11, 7, 12, 5, 6), (150, 140, 160, 150, 30, 150, 60, 100)])
+@pytest.mark.parametrize("early", [0, 1])
+def test_mixed_batches_of_every_field_order(frames, early):
+    """Ragged codes of every field order in one batch: a few frames (each on a cluster), and more than
+    the one-block kernel holds at once (several frames to a slot, the code description changing
+    under it); every job equals the oracle."""
+    rng = np.random.default_rng(sum(frames))
+    jobs, keep = [], []
+    for k, q in enumerate((2, 4, 8, 16, 32, 64, 128, 256)):
+        n, m, dmax = (24, 9, 6) if q >= 128 else (40, 19, 4) if q == 64 else (61, 31, 6)
+        code = irregular(q, n, m, 5 * q, dmax)
+        f = frames[k]
+        g = rng.integers(0, 48, (f, code.n, q)).astype(np.uint8)
+        if f:
+            g[np.arange(f)[:, None], np.arange(code.n)[None, :], rng.integers(0, q, (f, code.n))] = 0
+        dec, gd = binding.Decoder.from_code(code), torch.as_tensor(g).cuda()
+        out = (torch.empty((f, code.n), dtype=torch.uint8, device="cuda"),
+               torch.empty(f, dtype=torch.int32, device="cuda"), torch.empty(f, dtype=torch.uint8, device="cuda"))
+        keep.append((code, g, dec, gd, out))
+        jobs.append((dec.handle, gd, f, 4 + k % 3, early, *out))
+    ws = torch.empty(binding.nbldpc_decode_batch_workspace_size(jobs), dtype=torch.uint8, device="cuda")
+    before = binding.nbldpc_kernel_launch_count()
+    binding.nbldpc_decode_batch(jobs, ws)
+    torch.cuda.synchronize()
+    assert binding.nbldpc_kernel_launch_count() == before + 1
+    for k, (code, g, dec, gd, out) in enumerate(keep):
+        if g.shape[0]:
+            want = oracle.decode(code, g, 4 + k % 3, early, threads=THREADS)
+            for name, a, w in zip(("symbols", "iterations", "ok"), out, want):
+                assert np.array_equal(a.cpu().numpy(), w), f"q={code.q}: {name}"
