@@ -234,7 +234,8 @@ def _ptr(t) -> int:
 
 def _stream_ptr(stream) -> int:
     if stream is None:
-        return torch.cuda.current_stream().cuda_stream
+        # the raw handle: building a Stream object for it costs twice as much of a call of a few microseconds
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
     if isinstance(stream, torch.cuda.Stream):
         return stream.cuda_stream
     return int(stream)

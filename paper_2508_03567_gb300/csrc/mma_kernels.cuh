@@ -481,18 +481,19 @@ struct JobDesc {
 // Copy the sections of the code description that the min-max kernels read to shared memory:
 // [0, common) bytes, then the permutation selectors.
 __device__ __forceinline__ void stage_blob(unsigned char* sblob, const JobDesc& job, int common_bytes, int tid, int nthr) {
-  const int common = common_bytes / 16, skip = (job.off.perm_src - common_bytes) / 16;
-  const int n = common + (job.off.bytes - job.off.perm) / 16;
-  for (int i = tid; i < n; i += nthr)
-    reinterpret_cast<uint4*>(sblob)[i] = reinterpret_cast<const uint4*>(job.blob)[i < common ? i : i + skip];
+  for (int i = tid; i < common_bytes / 16; i += nthr)
+    reinterpret_cast<uint4*>(sblob)[i] = reinterpret_cast<const uint4*>(job.blob)[i];
+  for (int i = tid; i < (job.off.bytes - job.off.perm) / 16; i += nthr)
+    reinterpret_cast<uint4*>(sblob + common_bytes)[i] = reinterpret_cast<const uint4*>(job.blob + job.off.perm_src)[i];
 }
 
 constexpr int kMaxJobs = 32;
 
-// One launch: up to kMaxJobs jobs whose frames form one work list, served by
-// persistent blocks of `fpb` frame slots each.
-struct LaunchParams {
-  JobDesc jobs[kMaxJobs];
+// One launch: up to N jobs whose frames form one work list, served by
+// persistent blocks of `fpb` frame slots each.  Single-code launches pass the one
+// job alone: a table of 32 is 7 KB of kernel parameters to copy on every launch.
+template <int N> struct LaunchParamsOf {
+  JobDesc jobs[N];
   int njobs, total_items;
   unsigned int* counter;      // next work item
   uint8_t* msg;               // message slots, one per (block, frame slot)
@@ -503,6 +504,7 @@ struct LaunchParams {
   int xs_off;                 // resident launches: shared-memory offset of the slot's messages
   int static_items;           // 1: no more items than frame slots; slot s takes item s (no counter)
 };
+template <int QSEL> using LaunchParams = LaunchParamsOf<QSEL == 0 ? kMaxJobs : 1>;
 
 // Control words of a frame slot, then (mixed-code kernel) a copy of its job.
 __host__ __device__ constexpr int ctl_bytes(int qsel) {
@@ -1663,7 +1665,7 @@ __device__ __forceinline__ void decode_any(const JobDesc& job, const MixedSlot& 
 // degree D (single-field kernels; see decode_frame).
 template <int QSEL, int VSEL, int MB, bool T1 = false, bool XS = false, bool PR = false, int D = 0>
 __global__ void __launch_bounds__(XS ? kResidentThreads : 256, XS ? 2 : PR ? NBLDPC_MINB_PRUNE : MinBlocks<QSEL, VSEL>::v)
-    mma_decode_kernel(const __grid_constant__ LaunchParams p) {
+    mma_decode_kernel(const __grid_constant__ LaunchParams<QSEL> p) {
   static_assert(!XS || (QSEL >= 2 && MB == 1 && !T1), "resident messages: 8-bit, minimal schedule, one field");
   static_assert(!PR || (QSEL >= 2 && MB == 1 && !T1), "pruned convolutions: 8-bit, minimal schedule, one field");
   extern __shared__ __align__(16) unsigned char smem[];

@@ -15,7 +15,7 @@
 #include "mma_kernels.cuh"
 
 static_assert(nbldpc::kMaxJobs == NBLDPC_MAX_BATCH_JOBS, "job table size");
-static_assert(sizeof(nbldpc::LaunchParams) < 32000 && sizeof(nbldpc::SplitBatchParams) < 32000, "kernel parameter space");
+static_assert(sizeof(nbldpc::LaunchParams<0>) < 32000 && sizeof(nbldpc::SplitBatchParams) < 32000, "kernel parameter space");
 
 std::atomic<uint64_t> nbldpc_host::g_launches{0};
 std::mutex nbldpc_host::g_attr_mu;
@@ -371,7 +371,8 @@ nbldpc::JobDesc job_desc(const nbldpc_code* c, const uint8_t* gamma, int frames,
 
 // Queue the counter reset (not needed when every frame has its own slot) and the
 // persistent kernel (grid blocks) on st.
-int launch_plan(const void* kernel, const Plan& pl, nbldpc::LaunchParams& lp, int grid, void* counter, uint8_t* msg,
+template <int N>
+int launch_plan(const void* kernel, const Plan& pl, nbldpc::LaunchParamsOf<N>& lp, int grid, void* counter, uint8_t* msg,
                 cudaStream_t st) {
   if (lp.total_items == 0 || grid < 1) return NBLDPC_OK;
   lp.counter = reinterpret_cast<unsigned int*>(counter);
@@ -498,7 +499,7 @@ int launch(const nbldpc_code* c, const uint8_t* gamma, int frames, int max_iters
     const SplitShape s = split_shape(c, frames, early_stop);
     if (s.size) return launch_split(c, s, job_desc(c, gamma, frames, max_iters, early_stop, sym, iters, ok, 0, count), st);
   }
-  nbldpc::LaunchParams lp{};
+  nbldpc::LaunchParamsOf<1> lp{};
   lp.jobs[0] = job_desc(c, gamma, frames, max_iters, early_stop, sym, iters, ok, 0, count);
   lp.njobs = 1;
   lp.total_items = frames;
@@ -556,7 +557,7 @@ int nbldpc_decode_noalloc(const nbldpc_code* c, const uint8_t* gamma_dev, int fr
   st = noalloc_scratch(&scratch);
   if (st != NBLDPC_OK) return st;
   // the array keeps the previous call's contents: the frame counter is cleared in launch_plan
-  nbldpc::LaunchParams lp{};
+  nbldpc::LaunchParamsOf<1> lp{};
   lp.jobs[0] = job_desc(c, gamma_dev, frames, max_iters, early_stop, out_sym_dev, out_iters_dev, out_ok_dev, 0);
   lp.njobs = 1;
   lp.total_items = frames;
@@ -946,7 +947,7 @@ int nbldpc_decode_batch(const nbldpc_job* jobs, int n_jobs, void* workspace_dev,
   int st = batch_plan(jobs, n_jobs, &pl, &total);
   if (st != NBLDPC_OK) return st;
   if (!workspace_dev || !aligned(workspace_dev, 16) || workspace_bytes < ws_bytes(pl, total)) return NBLDPC_ERR_ARG;
-  nbldpc::LaunchParams lp{};
+  nbldpc::LaunchParams<0> lp{};
   int begin = 0;
   // The jobs with the longest frames first, so that they are not the ones that end the launch.
   int order[NBLDPC_MAX_BATCH_JOBS];
