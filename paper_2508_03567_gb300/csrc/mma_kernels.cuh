@@ -1258,11 +1258,11 @@ __device__ __forceinline__ void decode_frame(const JobDesc& job, int frame, uint
     // a = 16 part + k (k < 16) of edge j = c / CH, part = c % CH, and
     // P_j(h_j a) = alpha_j(a) with h (16 part + k) = h (16 part) ^ h k, both
     // XOR sums of the h x^b = exp2[log h + b] (16-bit messages: 8 symbols a piece)
-    auto scatter_piece = [&](bool first, int e0, int c) {
+    auto scatter_piece = [&](bool first, int e0, int c, unsigned char* base) {
       const int j = c / CH, part = c - j * CH;
       const int lh = edge_lh[e0 + j];
       const int h1 = exp2[lh], h2 = exp2[lh + 1], h4 = exp2[lh + 2];
-      Sym* Pv = vec16(j);
+      Sym* Pv = reinterpret_cast<Sym*>(base + (size_t)j * VB);
       if constexpr (MB == 2) {
         int v[8];
         if (first) load_ints<8>(gam + (size_t)edge_col[e0 + j] * Q + part * 8, v);
@@ -1310,7 +1310,7 @@ __device__ __forceinline__ void decode_frame(const JobDesc& job, int frame, uint
       for (int r = r_first + grp; r < r_last; r += ngroups) {
         const int e0 = row_ptr[r], d = D > 0 ? D : row_ptr[r + 1] - e0;
         if constexpr (kScatter) {
-          for (int c = gl; c < d * CH; c += g::G) scatter_piece(first, e0, c);
+          for (int c = gl; c < d * CH; c += g::G) scatter_piece(first, e0, c, vecs);
         } else {
           // stage incoming alpha rows (alpha^(0) = gamma on the first pass)
           if constexpr (MB == 2) {
@@ -1406,6 +1406,63 @@ __device__ __forceinline__ void decode_frame(const JobDesc& job, int frame, uint
           if (counting && gl == 0) work += (unsigned long long)Q * Q;
         }
         group_sync<g::G>(gmask);
+      }
+    };
+
+    // ---- check-node pass of a rank with at least two warps to a check (pruned, one warp
+    // per convolution): the F chain on one warp and the B chain on the other, then each
+    // every second middle beta, so that a check is 3/2 (d - 2) convolutions long and not
+    // 3 (d - 2) (GF(256) (2,8) N=128, 17 frames: 889 us against 702).  P and F are in
+    // the first warp's scratch, B in the second's.
+    auto cnp_pair = [&](bool first) {
+      if constexpr (PR && SP) {
+        const int r = r_first + (grp >> 1), half = grp & 1;
+        if (r >= r_last) return;
+        auto pair_sync = [&]() { slot_sync(bar_id + 1 + (grp >> 1), 64); };
+        const int e0 = row_ptr[r], d = row_ptr[r + 1] - e0;
+        const int gb = group_scratch_bytes<Q>(job.dmax, 1, true);
+        unsigned char* pf = scratch + (size_t)(grp & ~1) * gb;      // P_j, F_j
+        unsigned char* pb = pf + gb;                                // B_j
+        unsigned char* tmp = vecs + (size_t)(2 * dm - 2) * VB;      // this warp's
+        auto depermute = [&](const Sym* R, int e) {                 // as in cnp: beta(a) = R(h a)
+          const int lh = edge_lh[e], base = da_log0 >= 0 ? (int)exp2[da_log0 + lh] : 0;
+          const int h1 = exp2[lh], h2 = exp2[lh + 1], h4 = exp2[lh + 2];
+          int out[g::BPL];
+#pragma unroll
+          for (int i = 0; i < g::BPL; ++i)
+            out[i] = R[base ^ ((i & 1) ? h1 : 0) ^ ((i & 2) ? h2 : 0) ^ ((i & 4) ? h4 : 0)];
+          store_bytes<g::BPL>(X + (size_t)e * Q + gl * g::BPL, out);
+        };
+        auto at = [&](unsigned char* base, int i) { return reinterpret_cast<Sym*>(base + (size_t)i * VB); };
+        auto convp = [&](const Sym* A, const Sym* B, Sym* C, int kind) {
+          int folded = 0;
+          tpred[kind] = pr_conv<g>(A, B, C, tmp, gl, tpred[kind], counting ? &folded : nullptr);
+          if (counting && gl == 0) work += (unsigned long long)folded * Q;
+          __syncwarp();
+        };
+        for (int c = gl + 32 * half; c < d * CH; c += 64) scatter_piece(first, e0, c, pf);
+        pair_sync();
+        if (half == 0) {
+          const Sym* f = at(pf, 0);
+          for (int j = 1; j <= d - 2; ++j) {
+            convp(f, at(pf, j), at(pf, vF + j), 0);
+            f = at(pf, vF + j);
+          }
+          depermute(f, e0 + d - 1);
+        } else {
+          const Sym* b = at(pf, d - 1);
+          for (int j = d - 2; j >= 1; --j) {
+            convp(b, at(pf, j), at(pb, j), 1);
+            b = at(pb, j);
+          }
+          depermute(b, e0);
+        }
+        pair_sync();
+        for (int j = 1 + half; j <= d - 2; j += 2) {
+          Sym* f = at(pf, j == 1 ? 0 : vF + j - 1);
+          convp(f, j == d - 2 ? at(pf, d - 1) : at(pb, j + 1), f, 2);
+          depermute(f, e0 + j);
+        }
       }
     };
 
@@ -1564,6 +1621,8 @@ __device__ __forceinline__ void decode_frame(const JobDesc& job, int frame, uint
           if (job.dmax <= kRegDeg) cnp_regs4(k == 1); else cnp(k == 1);
         } else if constexpr (reg_form<Q>() && MB == 1 && !T1 && W4) {
           cnp_reg(k == 1);
+        } else if constexpr (PR && SP) {
+          if (2 * (r_last - r_first) <= ngroups) cnp_pair(k == 1); else cnp(k == 1);
         } else {
           cnp((MB == 1 || kScatter) && k == 1);
         }

@@ -474,7 +474,8 @@ SplitShape split_shape(const nbldpc_code* c, int frames, int early_stop) {
   size = std::min(size, c->split_max);
   while (size > 2 && (long long)size * 128 > (long long)c->m * G * 5 / 4) size /= 2;
   const int cpc = (c->m + size - 1) / size;
-  threads = std::min(threads, std::max(128, (int)round_up((size_t)cpc * G, 32)));
+  const int pair = c->mb == 1 && c->q >= 128 && frames <= 3 * sms / 8 ? 2 : 1;   // two warps to a check
+  threads = std::min(threads, std::max(128, (int)round_up((size_t)cpc * G * pair, 32)));
   SplitShape s = split_layout(c, size, threads);
   while (s.size == 0 && threads > 64) s = split_layout(c, size, threads = (threads - 1) / 64 * 64);
   if (s.size == 0) return s;
