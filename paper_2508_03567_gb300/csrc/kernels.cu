@@ -75,10 +75,14 @@ const void* split_kernel_q0() { return reinterpret_cast<const void*>(&mma_split_
 #if NBLDPC_KQ >= 8
 // Address of the kernel that decodes a frame on a cluster of blocks, for mb-byte
 // messages (minimal schedule): the layout and the convolutions of the default variant
-// (GF(8): 16-bit messages only).
-const void* NBLDPC_CAT(split_kernel_q, NBLDPC_KQ)(int mb) {
+// (GF(8): 16-bit messages only); dreg as in kernel_q (GF(64), degree 4).
+const void* NBLDPC_CAT(split_kernel_q, NBLDPC_KQ)(int mb, int dreg) {
+  (void)dreg;
   constexpr int Q = NBLDPC_KQ, V = (Q >= 16 && Q <= 64) ? 1 : 0;
   if (mb == 2) return reinterpret_cast<const void*>(&mma_split_kernel<Q, V, 2, false>);
+#if NBLDPC_KQ == 64
+  if (dreg == 4) return reinterpret_cast<const void*>(&mma_split_kernel<Q, V, 1, false, 4>);
+#endif
 #if NBLDPC_KQ == 8
   return nullptr;
 #else

@@ -1838,13 +1838,14 @@ __device__ __forceinline__ void split_setup(const JobDesc& job, const SplitLayou
   cluster_barrier();           // the row table is complete, and every rank of the cluster runs
 }
 
-template <int Q, int V, int MB, bool PR>
+// D: as in decode_frame.
+template <int Q, int V, int MB, bool PR, int D = 0>
 __global__ void __launch_bounds__(kResidentThreads, 2) mma_split_kernel(const __grid_constant__ SplitParams p) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int rank = blockIdx.x % p.size, frame = blockIdx.x / p.size;
   SplitCtx sc;
   split_setup(p.job, p.lay, frame, rank, p.size, Q, Q * MB, smem, sc);
-  decode_frame<Geo<Q, V>, MB, false, true, PR, false, 0, true>(p.job, frame, smem + p.lay.x_off, smem, smem,
+  decode_frame<Geo<Q, V>, MB, false, true, PR, false, D, true>(p.job, frame, smem + p.lay.x_off, smem, smem,
                                                                smem + p.lay.chat_off, smem + p.lay.scratch_off,
                                                                threadIdx.x, blockDim.x, 1, &sc);
 }

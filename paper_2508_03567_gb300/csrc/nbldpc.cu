@@ -62,12 +62,12 @@ const void* kernel_q64(int v, int mb, int t1, int dreg);
 const void* kernel_q128(int v, int mb, int t1, int dreg);
 const void* kernel_q256(int v, int mb, int t1, int dreg);
 const void* split_kernel_q0();
-const void* split_kernel_q8(int mb);
-const void* split_kernel_q16(int mb);
-const void* split_kernel_q32(int mb);
-const void* split_kernel_q64(int mb);
-const void* split_kernel_q128(int mb);
-const void* split_kernel_q256(int mb);
+const void* split_kernel_q8(int mb, int dreg);
+const void* split_kernel_q16(int mb, int dreg);
+const void* split_kernel_q32(int mb, int dreg);
+const void* split_kernel_q64(int mb, int dreg);
+const void* split_kernel_q128(int mb, int dreg);
+const void* split_kernel_q256(int mb, int dreg);
 }  // namespace nbldpc
 
 namespace {
@@ -103,15 +103,15 @@ int kernel_dreg(int q, int v, int km, int dreg) {
 
 // kernel that decodes a frame on a cluster of blocks (minimal schedule), null where
 // split_shape never takes it; q = 0: mixed codes, 8-bit messages
-const void* split_kernel_for(int q, int mb) {
+const void* split_kernel_for(int q, int mb, int dreg) {
   switch (q) {
     case 0: return nbldpc::split_kernel_q0();
-    case 8: return nbldpc::split_kernel_q8(mb);
-    case 16: return nbldpc::split_kernel_q16(mb);
-    case 32: return nbldpc::split_kernel_q32(mb);
-    case 64: return nbldpc::split_kernel_q64(mb);
-    case 128: return nbldpc::split_kernel_q128(mb);
-    case 256: return nbldpc::split_kernel_q256(mb);
+    case 8: return nbldpc::split_kernel_q8(mb, dreg);
+    case 16: return nbldpc::split_kernel_q16(mb, dreg);
+    case 32: return nbldpc::split_kernel_q32(mb, dreg);
+    case 64: return nbldpc::split_kernel_q64(mb, dreg);
+    case 128: return nbldpc::split_kernel_q128(mb, dreg);
+    case 256: return nbldpc::split_kernel_q256(mb, dreg);
   }
   return nullptr;
 }
@@ -178,14 +178,15 @@ int prepare_kernel(int q, int v, int km, int dreg, int dev, int smem_optin) {
 // Largest cluster of split-frame blocks (16, else the portable 8) that the device
 // runs for a field order and message width; 0 when the kernel cannot be prepared.
 // The kernel attributes are set and the device asked once.
-int g_split_max[64][9][2] = {};
+int g_split_max[64][9][3] = {};
 
-int split_max(int q, int mb, int dev, int smem_optin) {
+int split_max(int q, int mb, int dreg, int dev, int smem_optin) {
   std::lock_guard<std::mutex> lk(g_attr_mu);
   if (dev < 0 || dev >= 64) return 0;
-  int& mx = g_split_max[dev][q ? nbldpc::ilog2(q) : 0][mb - 1];
+  // (the third: 8-bit GF(64) messages and checks of degree 4)
+  int& mx = g_split_max[dev][q ? nbldpc::ilog2(q) : 0][q == 64 && mb == 1 && dreg == 4 ? 2 : mb - 1];
   if (mx == 0) {
-    const void* k = split_kernel_for(q, mb);
+    const void* k = split_kernel_for(q, mb, dreg);
     mx = k ? split_kernel_prepare(k, nbldpc::kResidentThreads, smem_optin) : 0;
     if (mx == 0) mx = -1;
   }
@@ -315,7 +316,7 @@ int configure(nbldpc_code* c, int variant, int fpb) {
   int optin = 0;
   c->split_max = 0;
   if (kmode(c) != 3 && cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device) == cudaSuccess)
-    c->split_max = split_max(c->q, c->mb, c->device, optin);
+    c->split_max = split_max(c->q, c->mb, c->dreg, c->device, optin);
   c->smem_optin = optin;
   return NBLDPC_OK;
 }
@@ -489,7 +490,7 @@ SplitShape split_shape(const nbldpc_code* c, int frames, int early_stop) {
 
 int launch_split(const nbldpc_code* c, const SplitShape& s, const nbldpc::JobDesc& job, cudaStream_t st) {
   nbldpc::SplitParams p{job, s.size, s.lay};
-  return split_launch(split_kernel_for(c->q, c->mb), job.frames, s.size, s.threads, s.smem, &p, st);
+  return split_launch(split_kernel_for(c->q, c->mb, c->dreg), job.frames, s.size, s.threads, s.smem, &p, st);
 }
 
 // split: small batches may go to the split-frame kernel (not while the autotuner times a tuning)
@@ -883,12 +884,12 @@ static int batch_plan(const nbldpc_job* jobs, int n_jobs, Plan* pl, int* total) 
 // Shape of a mixed batch whose frames are each decoded on a cluster (size 0: one block per frame
 // slot): the ranks and threads of split_shape, the jobs' layouts one over the other.  Frames count
 // by their work against the longest ones' (an eighth at least): one block per frame ends with the
-// longest frames alone.  Taken up to three such frames per SM with early stop (the serving loop's
-// small groups; 5/8 when q = 16 is the widest field), 3/8 without, and six frames of any kind; not
-// for q <= 8 alone.  Measured on GB300,
-// us per batch against the one-block kernel: 60 / 240 / 450 frames of GF(64) N=576, GF(16) N=1024 and
-// GF(256) N=128 in equal parts 2746 / 3455 / 3878 against 795 / 1444 / 2399; one frame of GF(64)
-// 1243 against 179.
+// longest frames alone.  Taken with early stop (the serving loop's groups) up to seven such frames per
+// SM, four with GF(256) among the fields and 5/8 when q = 16 is the widest, without up to 3/8, and
+// eight frames of any kind; not for q <= 8 alone.  Measured on GB300, us per batch, the one-block
+// kernel against this: 60 / 240 / 450 frames of GF(64) N=576, GF(16) N=1024 and GF(256) N=128 in
+// equal parts 2746 / 3455 / 3878 against 795 / 1444 / 2399; one frame of GF(64) 1243 against 179; 580
+// of GF(64) 3159 against 2428, of GF(128) N=256 5078 against 3769, of GF(256) N=384 14.6 ms against 15.7.
 static int batch_split(const nbldpc_job* jobs, int n_jobs, int total, const Plan& pl, nbldpc::SplitBatchParams* p,
                        SplitShape* out) {
   const nbldpc_code* c0 = jobs[0].code;
@@ -902,11 +903,12 @@ static int batch_split(const nbldpc_job* jobs, int n_jobs, int total, const Plan
       q_most = std::max(q_most, jobs[i].code->q);
       longest = std::max(longest, frame_work(jobs[i]));
     }
-  if (q_most <= 8 || total > 6 * sms) return 0;
+  if (q_most <= 8 || total > 8 * sms) return 0;
   for (int i = 0; i < n_jobs; ++i)
     like_longest += jobs[i].frames * std::max(0.125, longest > 0.0 ? frame_work(jobs[i]) / longest : 1.0);
-  if (like_longest > (!stop ? 3 * sms / 8 : q_most > 16 ? 3 * sms : 5 * sms / 8)) return 0;
-  const int most = split_max(0, 1, c0->device, c0->smem_optin);
+  const int most_frames = !stop ? 3 * sms / 8 : q_most <= 16 ? 5 * sms / 8 : q_most <= 128 ? 7 * sms : 4 * sms;
+  if (like_longest > most_frames) return 0;
+  const int most = split_max(0, 1, 0, c0->device, c0->smem_optin);
   const int size = std::min(total <= sms / 8 ? 16 : 8, most);
   if (size < 2) return 0;
   for (int threads = total <= 3 * sms / 8 ? 384 : total <= 3 * sms / 4 ? 256 : 128; threads >= 64; threads -= 64) {
@@ -976,7 +978,7 @@ int nbldpc_decode_batch(const nbldpc_job* jobs, int n_jobs, void* workspace_dev,
       memcpy(sp.jobs, lp.jobs, sizeof(sp.jobs));   // (perm_at, reg: the one-block kernel's, set below)
       sp.njobs = n_jobs;
       sp.size = shape.size;
-      return split_launch(split_kernel_for(0, 1), total, shape.size, shape.threads, shape.smem, &sp,
+      return split_launch(split_kernel_for(0, 1, 0), total, shape.size, shape.threads, shape.smem, &sp,
                           reinterpret_cast<cudaStream_t>(cuda_stream));
     }
   }
