@@ -252,9 +252,10 @@ int make_plan(int kq, int kv, int km, int fpb, const CodeNeeds* cs, int nc, Plan
   for (int i = 0; i < nc; ++i) {
     const int G = group_lanes(cs[i].q, cs[i].variant & 1);
     if (G > nthr) return NBLDPC_ERR_UNSUPPORTED;
-    const int s = reg || (kq == 0 && mixed_reg(cs[i].q, nthr, cs[i].dmax))
-                      ? reg_scratch(cs[i].q, nthr, cs[i].dmax)
+    int s = reg ? reg_scratch(cs[i].q, nthr, cs[i].dmax)
                       : (nthr / G) * group_bytes(cs[i].q, cs[i].dmax, cs[i].mb, kq == 0 ? cs[i].q >= 128 : (kv & 4) != 0);
+    if (kq == 0 && mixed_reg(cs[i].q, nthr, cs[i].dmax))    // either form, by the batch's frames
+      s = std::max(s, reg_scratch(cs[i].q, nthr, cs[i].dmax));
     if (s > scratch) scratch = s;
     if (cs[i].blob > pl.blob_cap) pl.blob_cap = cs[i].blob;
     if (cs[i].n > pl.n_cap) pl.n_cap = cs[i].n;
@@ -886,7 +887,8 @@ static int batch_plan(const nbldpc_job* jobs, int n_jobs, Plan* pl, int* total) 
 // by their work against the longest ones' (an eighth at least): one block per frame ends with the
 // longest frames alone.  Taken with early stop (the serving loop's groups) up to seven such frames per
 // SM, four with GF(256) among the fields and 5/8 when q = 16 is the widest, without up to 3/8, and
-// eight frames of any kind; not for q <= 8 alone.  Measured on GB300, us per batch, the one-block
+// eight frames of any kind; not for q <= 8 alone, nor past 3/8 where the longest frames have fewer
+// than 1024 check-node lanes, nor there for q <= 32 at all (and no more 128-thread ranks than lanes).  Measured on GB300, us per batch, the one-block
 // kernel against this: 60 / 240 / 450 frames of GF(64) N=576, GF(16) N=1024 and GF(256) N=128 in
 // equal parts 2746 / 3455 / 3878 against 795 / 1444 / 2399; one frame of GF(64) 1243 against 179; 580
 // of GF(64) 3159 against 2428, of GF(128) N=256 5078 against 3769, of GF(256) N=384 14.6 ms against 15.7.
@@ -895,21 +897,25 @@ static int batch_split(const nbldpc_job* jobs, int n_jobs, int total, const Plan
   const nbldpc_code* c0 = jobs[0].code;
   const int sms = pl.grid_max / pl.per_sm;
   bool stop = true;
-  int q_most = 0;
+  int q_most = 0, lanes = 0;       // widest field, check-node lanes of the longest frames
   double longest = 0.0, like_longest = 0.0;
   for (int i = 0; i < n_jobs; ++i)
     if (jobs[i].frames > 0) {
       stop = stop && jobs[i].early_stop;
       q_most = std::max(q_most, jobs[i].code->q);
-      longest = std::max(longest, frame_work(jobs[i]));
+      if (frame_work(jobs[i]) >= longest) {
+        longest = frame_work(jobs[i]);
+        lanes = jobs[i].code->m * group_lanes(jobs[i].code->q, mixed_layout(jobs[i].code->q));
+      }
     }
   if (q_most <= 8 || total > 8 * sms) return 0;
   for (int i = 0; i < n_jobs; ++i)
     like_longest += jobs[i].frames * std::max(0.125, longest > 0.0 ? frame_work(jobs[i]) / longest : 1.0);
   const int most_frames = !stop ? 3 * sms / 8 : q_most <= 16 ? 5 * sms / 8 : q_most <= 128 ? 7 * sms : 4 * sms;
-  if (like_longest > most_frames) return 0;
+  if (like_longest > most_frames || (lanes < 1024 && (q_most <= 32 || total > 3 * sms / 8))) return 0;
   const int most = split_max(0, 1, 0, c0->device, c0->smem_optin);
-  const int size = std::min(total <= sms / 8 ? 16 : 8, most);
+  int size = std::min(total <= sms / 8 ? 16 : 8, most);
+  while (size > 2 && (long long)size * 128 > (long long)lanes * 5 / 4) size /= 2;
   if (size < 2) return 0;
   for (int threads = total <= 3 * sms / 8 ? 384 : total <= 3 * sms / 4 ? 256 : 128; threads >= 64; threads -= 64) {
     SplitShape all;
@@ -985,7 +991,11 @@ int nbldpc_decode_batch(const nbldpc_job* jobs, int n_jobs, void* workspace_dev,
   for (int i = 0; i < n_jobs; ++i) {
     const nbldpc_code* c = jobs[i].code;
     lp.jobs[i].perm_at = c->off.edge_col;          // it stages no edge_col or variable-node view
-    lp.jobs[i].reg = mixed_reg(c->q, pl.threads / pl.fpb, c->dmax) || (c->q == 64 && c->dreg == 4) ? 1 : 0;
+    // a lane per check takes long with few checks: only when they fill half the slot's lanes or other
+    // frames fill the SM (100 frames of GF(32) N=64 and 200 of GF(4) N=100: 312 us against 109)
+    const int nthr = pl.threads / pl.fpb;
+    const bool fills = 2 * c->m >= nthr || total > pl.grid_max * pl.fpb;
+    lp.jobs[i].reg = (mixed_reg(c->q, nthr, c->dmax) && fills) || (c->q == 64 && c->dreg == 4) ? 1 : 0;
   }
   return launch_plan(kernel_for(0, -1, 1), pl, lp, grid_for(pl, total), workspace_dev,
                      reinterpret_cast<uint8_t*>(workspace_dev) + 256, reinterpret_cast<cudaStream_t>(cuda_stream));
