@@ -256,6 +256,15 @@ int nbldpc_code_autotune(nbldpc_code *code, const uint8_t *gamma_dev, int frames
                          nbldpc_tune_result *results, int max_results, int *n_results);
 
 /*
+ * How a call with these arguments would decode a frame: *blocks is the number of
+ * blocks of the cluster that decodes it, or 0 for the one-block kernels (a
+ * persistent block takes frame after frame).  Host work only; queues nothing.
+ */
+int nbldpc_decode_cluster_blocks(const nbldpc_code *code, int frames, int early_stop, int *blocks);
+int nbldpc_decode_batch_cluster_blocks(const nbldpc_job *jobs, int n_jobs, int *blocks);
+int nbldpc_fftspa_cluster_blocks(const nbldpc_code *code, int frames, int early_stop, int *blocks);
+
+/*
  * ---- Work counter --------------------------------------------------------------
  * With a counter set, every later decode of the code (single-code, batch job,
  * host-buffer and non-allocating decodes; not the autotuner's) adds to

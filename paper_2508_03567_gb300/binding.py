@@ -34,6 +34,7 @@ EXPORTED = ("nbldpc_code_create", "nbldpc_code_destroy", "nbldpc_code_info",
             "nbldpc_code_set_cnp_schedule", "nbldpc_code_get_cnp_schedule", "nbldpc_code_set_work_counter",
             "nbldpc_fftspa_workspace_size", "nbldpc_fftspa_decode",
             "nbldpc_fftspa_decode_host_workspace_size", "nbldpc_fftspa_decode_host",
+            "nbldpc_decode_cluster_blocks", "nbldpc_decode_batch_cluster_blocks", "nbldpc_fftspa_cluster_blocks",
             "nbldpc_server_create", "nbldpc_server_create_custom", "nbldpc_server_submit", "nbldpc_server_poll",
             "nbldpc_server_stats_get", "nbldpc_server_destroy",
             "nbldpc_decode_noalloc", "nbldpc_kernel_launch_count", "nbldpc_probe_minmax",
@@ -118,6 +119,9 @@ def lib() -> ctypes.CDLL:
             ip = ctypes.POINTER(ctypes.c_int)
             L.nbldpc_decode_batch_workspace_size.argtypes = [jp, ctypes.c_int, ctypes.POINTER(sz)]
             L.nbldpc_decode_batch.argtypes = [jp, ctypes.c_int, vp, sz, vp]
+            L.nbldpc_decode_cluster_blocks.argtypes = [vp, ctypes.c_int, ctypes.c_int, ip]
+            L.nbldpc_decode_batch_cluster_blocks.argtypes = [jp, ctypes.c_int, ip]
+            L.nbldpc_fftspa_cluster_blocks.argtypes = [vp, ctypes.c_int, ctypes.c_int, ip]
             L.nbldpc_code_get_tuning.argtypes = [vp, ip, ip]
             L.nbldpc_code_set_tuning.argtypes = [vp, ctypes.c_int, ctypes.c_int]
             L.nbldpc_code_set_message_bits.argtypes = [vp, ctypes.c_int]
@@ -340,6 +344,28 @@ def nbldpc_decode_batch(jobs, workspace, workspace_bytes: int | None = None, str
         workspace_bytes = workspace.numel() * workspace.element_size()
     _check(lib().nbldpc_decode_batch(arr, len(jobs), _ptr(workspace), int(workspace_bytes), _stream_ptr(stream)),
            "nbldpc_decode_batch")
+
+
+def nbldpc_decode_cluster_blocks(handle: int, frames: int, early_stop: int) -> int:
+    """Blocks of the cluster that would decode each frame of such a call (0: the one-block kernels)."""
+    b = ctypes.c_int()
+    _check(lib().nbldpc_decode_cluster_blocks(handle, int(frames), int(early_stop), ctypes.byref(b)),
+           "nbldpc_decode_cluster_blocks")
+    return b.value
+
+
+def nbldpc_decode_batch_cluster_blocks(jobs) -> int:
+    b = ctypes.c_int()
+    _check(lib().nbldpc_decode_batch_cluster_blocks(_jobs_array(jobs), len(jobs), ctypes.byref(b)),
+           "nbldpc_decode_batch_cluster_blocks")
+    return b.value
+
+
+def nbldpc_fftspa_cluster_blocks(handle: int, frames: int, early_stop: int) -> int:
+    b = ctypes.c_int()
+    _check(lib().nbldpc_fftspa_cluster_blocks(handle, int(frames), int(early_stop), ctypes.byref(b)),
+           "nbldpc_fftspa_cluster_blocks")
+    return b.value
 
 
 def nbldpc_code_get_tuning(handle: int):

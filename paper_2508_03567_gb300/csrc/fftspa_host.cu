@@ -257,6 +257,13 @@ int nbldpc_fftspa_workspace_size(const nbldpc_code* c, int frames, size_t* bytes
   return NBLDPC_OK;
 }
 
+int nbldpc_fftspa_cluster_blocks(const nbldpc_code* c, int frames, int early_stop, int* blocks) {
+  if (!c || !blocks || frames < 0) return NBLDPC_ERR_ARG;
+  if (c->fft_status != NBLDPC_OK) return c->fft_status;
+  *blocks = frames ? fft_split_shape(c, frames, early_stop).size : 0;
+  return NBLDPC_OK;
+}
+
 int nbldpc_fftspa_decode(const nbldpc_code* c, const float* prob_dev, int frames, int max_iters, int early_stop,
                          uint8_t* out_sym_dev, int32_t* out_iters_dev, uint8_t* out_ok_dev, float* out_app_dev,
                          void* workspace_dev, size_t workspace_bytes, void* cuda_stream) {

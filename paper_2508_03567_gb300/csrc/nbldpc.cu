@@ -841,6 +841,12 @@ int nbldpc_decode(const nbldpc_code* c, const uint8_t* gamma_dev, int frames, in
                 workspace_dev, reinterpret_cast<cudaStream_t>(cuda_stream));
 }
 
+int nbldpc_decode_cluster_blocks(const nbldpc_code* c, int frames, int early_stop, int* blocks) {
+  if (!c || !blocks || frames < 0) return NBLDPC_ERR_ARG;
+  *blocks = frames ? split_shape(c, frames, early_stop).size : 0;
+  return NBLDPC_OK;
+}
+
 // ---- mixed-code batches -----------------------------------------------------
 // Frame slots per block that suit a code in the mixed-code kernel: the pinned count, or (register
 // form) enough threads per slot for the checks, or the group form's default.
@@ -946,6 +952,18 @@ int nbldpc_decode_batch_workspace_size(const nbldpc_job* jobs, int n_jobs, size_
   const int st = batch_plan(jobs, n_jobs, &pl, &total);
   if (st != NBLDPC_OK) return st;
   *bytes = ws_bytes(pl, total);
+  return NBLDPC_OK;
+}
+
+int nbldpc_decode_batch_cluster_blocks(const nbldpc_job* jobs, int n_jobs, int* blocks) {
+  if (!blocks) return NBLDPC_ERR_ARG;
+  Plan pl{};
+  int total = 0;
+  const int st = batch_plan(jobs, n_jobs, &pl, &total);
+  if (st != NBLDPC_OK) return st;
+  nbldpc::SplitBatchParams sp{};
+  SplitShape shape;
+  *blocks = total > 0 ? batch_split(jobs, n_jobs, total, pl, &sp, &shape) : 0;
   return NBLDPC_OK;
 }
 

@@ -1,0 +1,80 @@
+"""Which kernel a call takes (nbldpc_decode_cluster_blocks and its siblings), and
+parity on the routes that the size rules choose between.  Bar: bit-exact
+against the oracle."""
+import os
+
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2508_03567_gb300 import binding, inputs as I
+from test_gpu_split import irregular
+
+pytestmark = pytest.mark.gpu
+THREADS = os.cpu_count() or 4
+
+
+def sms():
+    return torch.cuda.get_device_properties(0).multi_processor_count
+
+
+def random_gamma(code, frames, seed):
+    """Random reliabilities with a zero per vector: frames that run to their last iteration."""
+    rng = np.random.default_rng(seed)
+    g = rng.integers(0, 48, (frames, code.n, code.q)).astype(np.uint8)
+    if frames:
+        g[np.arange(frames)[:, None], np.arange(code.n)[None, :], rng.integers(0, code.q, (frames, code.n))] = 0
+    return g
+
+
+def batch(specs, iters, early, setup=None):
+    """Jobs of (code, gamma) pairs, each with a handle of its own (setup(k, decoder) tunes it)."""
+    jobs, keep = [], []
+    for k, (code, g) in enumerate(specs):
+        dec, gd, f = binding.Decoder.from_code(code), torch.as_tensor(g).cuda(), g.shape[0]
+        if setup:
+            setup(k, dec)
+        out = (torch.empty((f, code.n), dtype=torch.uint8, device="cuda"),
+               torch.empty(f, dtype=torch.int32, device="cuda"), torch.empty(f, dtype=torch.uint8, device="cuda"))
+        keep.append((dec, gd, out))
+        jobs.append((dec.handle, gd, f, iters, early, *out))
+    return jobs, keep
+
+
+def check_batch(specs, jobs, keep, iters, early):
+    ws = torch.empty(binding.nbldpc_decode_batch_workspace_size(jobs), dtype=torch.uint8, device="cuda")
+    binding.nbldpc_decode_batch(jobs, ws)
+    torch.cuda.synchronize()
+    for (code, g), (_, _, out) in zip(specs, keep):
+        if g.shape[0]:
+            want = oracle.decode(code, g, iters, early, threads=THREADS)
+            for name, a, w in zip(("symbols", "iterations", "ok"), out, want):
+                assert np.array_equal(a.cpu().numpy(), w), f"q={code.q}: {name}"
+
+
+# total frames, as a share of the SMs, of every cluster size and block size that the rule of mixed
+# batches knows for codes with at least 1024 check-node lanes: 16 x 384, 8 x 384, 8 x 256, 8 x 128
+@pytest.mark.parametrize("share,blocks", [(0.08, 16), (0.3, 8), (0.6, 8), (2.0, 8)])
+def test_mixed_batches_on_every_cluster_shape(share, blocks):
+    total = int(share * sms())
+    codes = [I.workload_code("gf64_n576_dv2_dc4"), irregular(256, 61, 27, 261, 7), I.workload_code("gf16_n1024_dv2_dc4"),
+             irregular(4, 61, 31, 20, 10)]
+    counts = [total - 3 * (total // 4), total // 4, total // 4, total // 4]
+    specs = [(c, random_gamma(c, f, 7 * c.q + total)) for c, f in zip(codes, counts)]
+    jobs, keep = batch(specs, 4, 1)
+    assert binding.nbldpc_decode_batch_cluster_blocks(jobs) == blocks
+    check_batch(specs, jobs, keep, 4, 1)
+
+
+def test_small_batches_take_the_cluster_kernels():
+    """The sizes that test_gpu_split.py decodes reach the kernels that it is about."""
+    for q, n, x in ((16, 100, 4), (64, 576, 4), (256, 128, 8)):
+        dec = binding.Decoder.from_code(I.make_regular_code(q, n, 2, x, seed=q + n))
+        for bits in (8, 16):
+            dec.set_message_bits(bits)
+            assert [binding.nbldpc_decode_cluster_blocks(dec.handle, f, 1) > 0 for f in (1, 3, 25)] == [True] * 3
+            assert binding.nbldpc_decode_cluster_blocks(dec.handle, 60000, 1) == 0
+        assert binding.nbldpc_fftspa_cluster_blocks(dec.handle, 60000, 1) == 0
+    dec = binding.Decoder.from_code(I.workload_code("gf64_n576_dv2_dc4"))
+    assert binding.nbldpc_fftspa_cluster_blocks(dec.handle, 1, 1) > 0
