@@ -314,11 +314,11 @@ int configure(nbldpc_code* c, int variant, int fpb) {
   if (st != NBLDPC_OK) return st;
   c->variant = variant;
   c->plan = pl;
+  // (the limit serves the FFT-SPA clusters too, which the min-max settings do not touch)
   int optin = 0;
-  c->split_max = 0;
-  if (kmode(c) != 3 && cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device) == cudaSuccess)
-    c->split_max = split_max(c->q, c->mb, c->dreg, c->device, optin);
+  if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device) != cudaSuccess) optin = 0;
   c->smem_optin = optin;
+  c->split_max = kmode(c) != 3 && optin > 0 ? split_max(c->q, c->mb, c->dreg, c->device, optin) : 0;
   return NBLDPC_OK;
 }
 

@@ -78,3 +78,14 @@ def test_small_batches_take_the_cluster_kernels():
         assert binding.nbldpc_fftspa_cluster_blocks(dec.handle, 60000, 1) == 0
     dec = binding.Decoder.from_code(I.workload_code("gf64_n576_dv2_dc4"))
     assert binding.nbldpc_fftspa_cluster_blocks(dec.handle, 1, 1) > 0
+
+
+def test_fftspa_clusters_do_not_depend_on_the_minmax_schedule():
+    """The Table 1 schedule is a setting of the min-max check-node pass: one FFT-SPA frame decodes on
+    a cluster before and after it."""
+    dec = binding.Decoder.from_code(I.workload_code("gf64_n576_dv2_dc4"))
+    want = binding.nbldpc_fftspa_cluster_blocks(dec.handle, 1, 1)
+    assert want > 0
+    binding.nbldpc_code_set_cnp_schedule(dec.handle, binding.NBLDPC_CNP_TABLE1)
+    assert binding.nbldpc_fftspa_cluster_blocks(dec.handle, 1, 1) == want
+    assert binding.nbldpc_decode_cluster_blocks(dec.handle, 1, 1) == 0      # no Table 1 cluster kernel
