@@ -153,16 +153,18 @@ int nbldpc_decode_host(const nbldpc_code *code, const uint8_t *gamma_host, int f
 
 /*
  * ---- Mixed-code batches -------------------------------------------------
- * One persistent launch decodes the frames of up to NBLDPC_MAX_BATCH_JOBS
+ * One launch decodes the frames of up to NBLDPC_MAX_BATCH_JOBS
  * jobs, each with its own code (any q, N, degrees), reliabilities, iteration
  * limit and outputs.  The frames of all jobs form one work list; a block
  * slot takes the next frame as soon as its previous one has stopped (zero
  * syndrome or max_iters), so codes with different frame counts and frames
- * with different iteration counts share the GPU without idle tails.  Results
- * are identical to nbldpc_decode of each job on its own (frames are
- * independent); only the throughput differs.  The launch is a counter reset
- * plus one kernel on the caller's stream, so it can be captured in a CUDA
- * graph and replayed (same buffers) without host work.  This is the batching
+ * with different iteration counts share the GPU without idle tails.  A batch
+ * of few frames decodes each frame on a cluster of blocks instead (see
+ * Tuning).  Results are identical to nbldpc_decode of each job on its own
+ * (frames are independent); only the throughput differs.  The launch is one
+ * kernel on the caller's stream (and a counter reset when there are more
+ * frames than frame slots), so it can be captured in a CUDA graph and
+ * replayed (same buffers) without host work.  This is the batching
  * form of the paper's multicodeword mapping (Sec. 4: one frame per processing
  * unit, no synchronization between frames), extended to mixed codes.
  */
@@ -183,9 +185,11 @@ typedef struct nbldpc_job {
 int nbldpc_decode_batch_workspace_size(const nbldpc_job *jobs, int n_jobs, size_t *bytes);
 
 /*
- * Queue the batch on `cuda_stream`.  Each code decodes with its own layout
- * variant; the block is split into the smallest frames-per-block value among
- * the jobs' codes.  Errors: NBLDPC_ERR_ARG (n_jobs outside [1,
+ * Queue the batch on `cuda_stream`.  The kernel has one form per field order,
+ * whatever the codes' variants.  A block is split into the smallest
+ * frames-per-block value that suits the jobs' codes; a batch with a code whose
+ * tuning was set by hand (nbldpc_code_set_tuning) keeps these blocks at every
+ * size, with the value set there for that code.  Errors: NBLDPC_ERR_ARG (n_jobs outside [1,
  * NBLDPC_MAX_BATCH_JOBS], bad pointers, short workspace), NBLDPC_ERR_UNSUPPORTED
  * (the combined shared-memory need exceeds the device), NBLDPC_ERR_CUDA.
  */

@@ -864,6 +864,14 @@ static double frame_work(const nbldpc_job& j) {
   return (double)j.max_iters * c->nnz * c->q * c->q * (c->q >= 128 ? 0.1 : 1.0);
 }
 
+// Whether a code that has frames in the batch was tuned by hand: the batch then keeps the one-block
+// kernel and the smallest frames-per-block value among its codes.
+static bool any_pinned(const nbldpc_job* jobs, int n_jobs) {
+  for (int i = 0; i < n_jobs; ++i)
+    if (jobs[i].frames > 0 && jobs[i].code->pinned) return true;
+  return false;
+}
+
 static int batch_plan(const nbldpc_job* jobs, int n_jobs, Plan* pl, int* total) {
   if (!jobs || n_jobs < 1 || n_jobs > NBLDPC_MAX_BATCH_JOBS) return NBLDPC_ERR_ARG;
   CodeNeeds need[NBLDPC_MAX_BATCH_JOBS];
@@ -882,9 +890,10 @@ static int batch_plan(const nbldpc_job* jobs, int n_jobs, Plan* pl, int* total) 
   }
   if (t > 0x7FFFFFFF) return NBLDPC_ERR_ARG;
   *total = (int)t;
-  // few frames: a block each (GF(4) N=48 and GF(8) N=100, 200 frames each: 100 us at two a block, 92 at one)
+  // few frames: a block each (GF(4) N=48 and GF(8) N=100, 200 frames each: 100 us at two a block, 92 at one),
+  // unless a code's frames per block are pinned
   const Plan& pl0 = jobs[0].code->plan;
-  if (t <= 3LL * (pl0.grid_max / pl0.per_sm)) fpb = 1;
+  if (t <= 3LL * (pl0.grid_max / pl0.per_sm) && !any_pinned(jobs, n_jobs)) fpb = 1;
   return make_plan(0, -1, 1, fpb, need, n_jobs, pl);
 }
 
@@ -900,6 +909,7 @@ static int batch_plan(const nbldpc_job* jobs, int n_jobs, Plan* pl, int* total) 
 // of GF(64) 3159 against 2428, of GF(128) N=256 5078 against 3769, of GF(256) N=384 14.6 ms against 15.7.
 static int batch_split(const nbldpc_job* jobs, int n_jobs, int total, const Plan& pl, nbldpc::SplitBatchParams* p,
                        SplitShape* out) {
+  if (any_pinned(jobs, n_jobs)) return 0;
   const nbldpc_code* c0 = jobs[0].code;
   const int sms = pl.grid_max / pl.per_sm;
   bool stop = true;

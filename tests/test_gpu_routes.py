@@ -89,3 +89,23 @@ def test_fftspa_clusters_do_not_depend_on_the_minmax_schedule():
     binding.nbldpc_code_set_cnp_schedule(dec.handle, binding.NBLDPC_CNP_TABLE1)
     assert binding.nbldpc_fftspa_cluster_blocks(dec.handle, 1, 1) == want
     assert binding.nbldpc_decode_cluster_blocks(dec.handle, 1, 1) == 0      # no Table 1 cluster kernel
+
+
+def test_a_pinned_code_keeps_a_mixed_batch_on_the_one_block_kernel():
+    """nbldpc_code_set_tuning holds for batches of every size: no cluster, and the pinned frames per
+    block.  Only a job that has frames counts."""
+    specs = [(I.workload_code("gf64_n576_dv2_dc4"), random_gamma(I.workload_code("gf64_n576_dv2_dc4"), 5, 1)),
+             (I.workload_code("gf16_n1024_dv2_dc4"), random_gamma(I.workload_code("gf16_n1024_dv2_dc4"), 4, 2))]
+    jobs, keep = batch(specs, 4, 1)
+    assert binding.nbldpc_decode_batch_cluster_blocks(jobs) > 0
+    slot = max(-(-c.nnz * c.q // 256) * 256 for c, _ in specs)
+    for fpb in (1, 2):
+        jobs, keep = batch(specs, 4, 1, lambda k, dec: dec.set_tuning(1, fpb))
+        assert binding.nbldpc_decode_batch_cluster_blocks(jobs) == 0
+        # nine frames in blocks of fpb slots
+        assert binding.nbldpc_decode_batch_workspace_size(jobs) == 256 + -(-9 // fpb) * fpb * slot
+        check_batch(specs, jobs, keep, 4, 1)
+    empty = [(specs[0][0], specs[0][1][:0]), specs[0], specs[1]]
+    jobs, keep = batch(empty, 4, 1, lambda k, dec: dec.set_tuning(1, 1) if k == 0 else None)
+    assert binding.nbldpc_decode_batch_cluster_blocks(jobs) > 0
+    check_batch(empty, jobs, keep, 4, 1)
