@@ -240,7 +240,8 @@ int nbldpc_code_get_tuning(const nbldpc_code *code, int *variant, int *frames_pe
 /* Set the tuning by hand (variant 0..7, frames_per_block 1, 2, 4 or 8), for batches of every size;
  * NBLDPC_ERR_UNSUPPORTED if that pair does not fit the device or the code.  Not concurrent with any other call on the same
  * handle (a decode reads the tuning).  Switching a code to 16-bit messages or to the Table 1
- * schedule keeps bit 0 of its variant only. */
+ * schedule then keeps bit 0 of its variant only, also after it is switched back (as after the
+ * autotuner); a code that was never tuned has the default of its current mode. */
 int nbldpc_code_set_tuning(nbldpc_code *code, int variant, int frames_per_block);
 
 /* Device workspace nbldpc_code_autotune needs for `frames` tuning frames. */

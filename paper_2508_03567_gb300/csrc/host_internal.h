@@ -64,6 +64,7 @@ struct nbldpc_code {
   int split_max = 0;                   // largest cluster of the split-frame kernel (0: not for this code's mode)
   int smem_optin = 0;                  // shared memory a block may take
   bool pinned = false;                 // the launch shape was set by nbldpc_code_set_tuning: every batch takes it
+  bool tuned = false;                  // the launch shape was set or measured (else the default of the mode)
   nbldpc_host::Plan plan{};            // single-code launch shape (fpb chosen by default or by the autotuner)
   int fft_status = NBLDPC_ERR_UNSUPPORTED;   // FFT-SPA launch shape below valid when NBLDPC_OK
   int fft_dc = 0, fft_dv = 0;          // FFT-SPA check-node form (dc 0: lane per edge) and column-degree bucket

@@ -344,6 +344,27 @@ int configure_reg(nbldpc_code* c, int variant) {
   return best ? configure(c, variant, best) : NBLDPC_ERR_UNSUPPORTED;
 }
 
+// The launch shape of a handle that nobody tuned, for its message width and schedule.
+// Minimal schedule, 8 bits: the resident-message form (384-thread blocks of 1, 2 or 4 frames)
+// where it fits shared memory, otherwise the same layout with the messages in the workspace.
+int configure_default(nbldpc_code* c) {
+  const int v = default_variant(c->q), fpb = default_fpb(c);
+  if (kmode(c) != 1) return configure(c, v & 1, reg_form(c->q) || v == 0 ? fpb : 1);
+  int st = NBLDPC_ERR_UNSUPPORTED;
+  if (reg_form(c->q)) st = configure_reg(c, v);
+  else if (v >= 2) st = configure(c, v, (v & 2) && fpb > 4 && !warp4_code(c) ? 4 : fpb);
+  return st == NBLDPC_ERR_UNSUPPORTED ? configure(c, v & 1, fpb) : st;
+}
+
+// The launch shape after a change of the message width or the schedule: a tuning that was set or
+// measured keeps the layout (resident messages serve 8-bit codes and the minimal schedule only),
+// any other handle has the default of its new mode, whatever it was before.
+int configure_mode(nbldpc_code* c) {
+  if (!c->tuned) return configure_default(c);
+  const int v = kmode(c) == 1 ? c->variant : c->variant & 1;
+  return configure(c, v, v == c->variant ? c->plan.fpb : reg_form(c->q) && !c->pinned ? default_fpb(c) : 1);
+}
+
 size_t decode_ws_bytes(const nbldpc_code* c, int frames) { return ws_bytes(c->plan, frames); }
 
 nbldpc::JobDesc job_desc(const nbldpc_code* c, const uint8_t* gamma, int frames, int max_iters, int early_stop,
@@ -718,14 +739,7 @@ int nbldpc_code_create(int q, uint32_t prim_poly, int n_cols, int n_rows, const 
   if (e != cudaSuccess) { delete c; return e == cudaErrorMemoryAllocation ? NBLDPC_ERR_NOMEM : NBLDPC_ERR_CUDA; }
   e = cudaMemcpy(c->blob_dev, blob.data(), o, cudaMemcpyHostToDevice);
   int st = cuda_status(e);
-  if (st == NBLDPC_OK) {
-    // the resident-message form (384-thread blocks of 1, 2 or 4 frames) must fit shared
-    // memory; otherwise the same layout with the messages in the workspace
-    const int v = default_variant(q), fpb = default_fpb(c);
-    if (reg_form(q)) st = configure_reg(c, v);
-    else st = v >= 2 ? configure(c, v, (v & 2) && fpb > 4 && !warp4_code(c) ? 4 : fpb) : NBLDPC_ERR_UNSUPPORTED;
-    if (st == NBLDPC_ERR_UNSUPPORTED) st = configure(c, v & 1, fpb);
-  }
+  if (st == NBLDPC_OK) st = configure_default(c);
   if (st == NBLDPC_OK) {
     c->fft_status = fft_configure(c, row_ptr);
     if (c->fft_status == NBLDPC_ERR_CUDA) st = NBLDPC_ERR_CUDA;
@@ -771,7 +785,7 @@ int nbldpc_code_set_tuning(nbldpc_code* c, int variant, int frames_per_block) {
   const int st = check_device(c);
   if (st != NBLDPC_OK) return st;
   const int st2 = configure(c, variant, frames_per_block);
-  if (st2 == NBLDPC_OK) c->pinned = true;
+  if (st2 == NBLDPC_OK) c->pinned = c->tuned = true;
   return st2;
 }
 
@@ -781,9 +795,7 @@ int nbldpc_code_set_message_bits(nbldpc_code* c, int bits) {
   if (check_device(c) != NBLDPC_OK) return check_device(c);
   const int old = c->mb;
   c->mb = bits / 8;
-  // resident messages serve 8-bit codes only: a 16-bit code keeps the layout in the workspace form
-  const int v = c->mb == 1 ? c->variant : c->variant & 1;
-  const int st = configure(c, v, v == c->variant ? c->plan.fpb : reg_form(c->q) && !c->pinned ? default_fpb(c) : 1);
+  const int st = configure_mode(c);
   if (st != NBLDPC_OK) c->mb = old;
   return st;
 }
@@ -800,9 +812,7 @@ int nbldpc_code_set_cnp_schedule(nbldpc_code* c, int schedule) {
   if (check_device(c) != NBLDPC_OK) return check_device(c);
   const int old = c->cnp_schedule;
   c->cnp_schedule = schedule;
-  // the schedule is a separate kernel; resident messages serve the minimal schedule only
-  const int v = schedule == NBLDPC_CNP_MINIMAL ? c->variant : c->variant & 1;
-  const int st = configure(c, v, v == c->variant ? c->plan.fpb : reg_form(c->q) && !c->pinned ? default_fpb(c) : 1);
+  const int st = configure_mode(c);
   if (st != NBLDPC_OK) c->cnp_schedule = old;
   return st;
 }
@@ -1102,6 +1112,7 @@ int nbldpc_code_autotune(nbldpc_code* c, const uint8_t* gamma_dev, int frames, i
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   const int st2 = configure(c, st == NBLDPC_OK ? best_v : v_old, st == NBLDPC_OK ? best_f : f_old);
+  if (st == NBLDPC_OK && st2 == NBLDPC_OK) c->tuned = true;
   if (n_results) *n_results = count;
   return st != NBLDPC_OK ? st : st2;
 }

@@ -109,3 +109,32 @@ def test_a_pinned_code_keeps_a_mixed_batch_on_the_one_block_kernel():
     jobs, keep = batch(empty, 4, 1, lambda k, dec: dec.set_tuning(1, 1) if k == 0 else None)
     assert binding.nbldpc_decode_batch_cluster_blocks(jobs) > 0
     check_batch(empty, jobs, keep, 4, 1)
+
+
+@pytest.mark.parametrize("q,n", [(4, 48), (8, 512), (16, 1024), (32, 600), (64, 576), (128, 96), (256, 96)])
+def test_a_handle_that_was_never_tuned_forgets_its_past_modes(q, n):
+    """To 16-bit messages, or to the Table 1 schedule, and back: the launch shape of a new handle.
+    A tuning that was set keeps its layout bit only, as before."""
+    code = I.make_regular_code(q, n, 2, 4, seed=q + n)
+    dec = binding.Decoder.from_code(code)
+
+    def shape():
+        return (dec.tuning(), binding.nbldpc_decode_workspace_size(dec.handle, 5000),
+                [binding.nbldpc_decode_cluster_blocks(dec.handle, f, e) for f in (1, 60, 300) for e in (0, 1)])
+    new = shape()
+    dec.set_message_bits(16)
+    assert dec.tuning()[0] == new[0][0] & 1
+    dec.set_message_bits(8)
+    assert shape() == new
+    binding.nbldpc_code_set_cnp_schedule(dec.handle, binding.NBLDPC_CNP_TABLE1)
+    assert dec.tuning()[0] == new[0][0] & 1
+    binding.nbldpc_code_set_cnp_schedule(dec.handle, binding.NBLDPC_CNP_MINIMAL)
+    assert shape() == new
+    g = random_gamma(code, 40, q)
+    got = [t.cpu().numpy() for t in dec.decode(torch.as_tensor(g).cuda(), 4, 0)]
+    for a, w in zip(got, oracle.decode(code, g, 4, 0, threads=THREADS)):
+        assert np.array_equal(a, w)
+    dec.set_tuning(*new[0])
+    dec.set_message_bits(16)
+    dec.set_message_bits(8)
+    assert dec.tuning()[0] == new[0][0] & 1
