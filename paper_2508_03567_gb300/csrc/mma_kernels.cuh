@@ -1006,16 +1006,15 @@ template <class T> __device__ __forceinline__ T* at_rank(T* p, int r) {
 // description, chat[n] the decisions, scratch the per-group buffers; X is the
 // slot's message area ([nnz][q] bytes); cold: where edge_col and the variable-node view
 // of the description are (sblob, or the blob in global memory).
-// REG4: q = 4 codes take the register form of the check-node pass (single-field
-// kernels; the all-field kernel keeps the group form).  PR: the check-node
-// convolutions are pruned (pr_conv; 32-lane groups, 8-bit messages, minimal
-// schedule).  W4: a GF(4) frame slot of one warp may take the one-warp form
+// q = 4 codes of check degree <= kRegDeg take the register form of the check-node pass
+// (8-bit messages, minimal schedule).  PR: the check-node convolutions are pruned
+// (pr_conv; 32-lane groups, 8-bit messages, minimal schedule).  W4: a GF(4) frame slot of one warp may take the one-warp form
 // (decode_frame_warp4; resident-message kernels, which have the registers for it).
 // D > 0: every check of the code has degree D (a compile-time loop bound and
 // vector layout; 0: the degrees are read per check).  SP: the threads are those of
 // one rank of a cluster that decodes the frame together (sc; X then holds the
 // message rows of the rank's own edges).
-template <class g, int MB, bool T1, bool REG4 = true, bool PR = false, bool W4 = false, int D = 0, bool SP = false>
+template <class g, int MB, bool T1, bool PR = false, bool W4 = false, int D = 0, bool SP = false>
 __device__ __forceinline__ void decode_frame(const JobDesc& job, int frame, uint8_t* Xown, const unsigned char* sblob,
                                              const unsigned char* cold, uint8_t* chat, unsigned char* scratch,
                                              int stid, int nthr, int bar_id, const SplitCtx* sc = nullptr) {
@@ -1025,7 +1024,7 @@ __device__ __forceinline__ void decode_frame(const JobDesc& job, int frame, uint
   constexpr bool kScatter = scatter_perm<Q>();
   static_assert(MB == 1 || MB == 2, "message bytes");
   static_assert(!PR || (g::G == 32 && MB == 1 && !T1), "pruned convolutions: 32-lane groups, 8-bit, minimal");
-  if constexpr (Q == 4 && MB == 1 && !T1 && REG4 && W4) {
+  if constexpr (Q == 4 && MB == 1 && !T1 && W4) {
     // one warp per frame: a slot of 32 threads
     if (nthr == 32 && decode_frame_warp4<D == 4 ? 4 : 0>(job, frame, Xown, sblob, cold, stid)) return;
   }
@@ -1617,7 +1616,7 @@ __device__ __forceinline__ void decode_frame(const JobDesc& job, int frame, uint
         pass_sync();
       }
       for (int k = 1; k <= job.max_iters; ++k) {
-        if constexpr (Q == 4 && MB == 1 && !T1 && REG4) {
+        if constexpr (Q == 4 && MB == 1 && !T1) {
           if (job.dmax <= kRegDeg) cnp_regs4(k == 1); else cnp(k == 1);
         } else if constexpr (reg_form<Q>() && MB == 1 && !T1 && W4) {
           cnp_reg(k == 1);
@@ -1686,7 +1685,7 @@ __device__ __noinline__ void decode_mixed(MixedSlot m, int frame, int stid, int 
   extern __shared__ __align__(16) unsigned char smem[];
   const JobDesc& job = *reinterpret_cast<const JobDesc*>(smem + m.job);
   uint8_t* X = SP ? smem + m.x : m.X;
-  decode_frame<Geo<Q, mixed_layout<Q>()>, 1, false, true, (Q >= 128), REG, D, SP>(
+  decode_frame<Geo<Q, mixed_layout<Q>()>, 1, false, (Q >= 128), REG, D, SP>(
       job, frame, X, smem + m.blob, SP ? smem + m.blob : job.blob, smem + m.chat, smem + m.scratch, stid, nthr, bar_id,
       reinterpret_cast<const SplitCtx*>(smem + m.sc));
 }
@@ -1718,7 +1717,7 @@ __device__ __forceinline__ void decode_any(const JobDesc& job, const MixedSlot& 
 // MB: message bytes per symbol (1: 8-bit messages; 2: 16-bit, single-field kernels only).
 // T1: the Table 1 check-node schedule (3 d_c - 4 convolutions; single-field kernels only).
 // XS: the frames' messages stay in shared memory (8-bit messages, single-field
-// kernels; kResidentThreads threads, 1, 2 or 4 frame slots per block).
+// kernels; at most kResidentThreads threads, see make_plan).
 // PR: pruned check-node convolutions (single-field kernels whose layout has
 // 32-lane groups; 8-bit messages, minimal schedule).  D > 0: every check has
 // degree D (single-field kernels; see decode_frame).
@@ -1766,8 +1765,7 @@ __global__ void __launch_bounds__(XS ? kResidentThreads : 256, XS ? 2 : PR ? NBL
       slot_sync(bar_id, nthr);
     }
     if constexpr (QSEL != 0)
-      decode_frame<Geo<QSEL, VSEL>, MB, T1, true, PR, XS, D>(job, frame, X, sblob, sblob, chat, scratch, stid, nthr,
-                                                                   bar_id);
+      decode_frame<Geo<QSEL, VSEL>, MB, T1, PR, XS, D>(job, frame, X, sblob, sblob, chat, scratch, stid, nthr, bar_id);
     else
       decode_any<false>(*sjob,
                         MixedSlot{(int)(reinterpret_cast<unsigned char*>(sjob) - smem), (int)(sblob - smem),
@@ -1845,7 +1843,7 @@ __global__ void __launch_bounds__(kResidentThreads, 2) mma_split_kernel(const __
   const int rank = blockIdx.x % p.size, frame = blockIdx.x / p.size;
   SplitCtx sc;
   split_setup(p.job, p.lay, frame, rank, p.size, Q, Q * MB, smem, sc);
-  decode_frame<Geo<Q, V>, MB, false, true, PR, false, D, true>(p.job, frame, smem + p.lay.x_off, smem, smem,
+  decode_frame<Geo<Q, V>, MB, false, PR, false, D, true>(p.job, frame, smem + p.lay.x_off, smem, smem,
                                                                smem + p.lay.chat_off, smem + p.lay.scratch_off,
                                                                threadIdx.x, blockDim.x, 1, &sc);
 }

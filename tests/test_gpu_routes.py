@@ -138,3 +138,32 @@ def test_a_handle_that_was_never_tuned_forgets_its_past_modes(q, n):
     dec.set_message_bits(16)
     dec.set_message_bits(8)
     assert dec.tuning()[0] == new[0][0] & 1
+
+
+def test_gf4_checks_above_degree_8_in_mixed_batches():
+    """The mixed-code kernels' group form of q = 4 (their register form ends at check degree 8): beside a
+    GF(64) code on clusters, and on the one-block kernel."""
+    small = irregular(4, 61, 31, 20, 10)
+    assert np.diff(small.row_ptr).max() > 8
+    for early, counts, cluster in ((1, (9, 20), True), (0, (600, 30), False), (0, (90, 0), False)):
+        specs = [(small, random_gamma(small, counts[0], 5)),
+                 (I.workload_code("gf64_n576_dv2_dc4"), random_gamma(I.workload_code("gf64_n576_dv2_dc4"), counts[1], 6))]
+        jobs, keep = batch(specs, 4, early)
+        assert (binding.nbldpc_decode_batch_cluster_blocks(jobs) > 0) == cluster
+        check_batch(specs, jobs, keep, 4, early)
+
+
+@pytest.mark.parametrize("early,frames", [(1, 8), (0, 130)])
+def test_the_variant_of_a_code_does_not_change_a_mixed_batch(early, frames):
+    """Mixed-code kernels have one form per field order: any variant, on clusters (no code tuned by hand)
+    and on the one-block kernel, gives the oracle's outputs."""
+    codes = [irregular(256, 61, 27, 261, 7), irregular(128, 61, 27, 133, 7), irregular(64, 61, 31, 69, 5),
+             irregular(16, 61, 31, 21, 6)]
+    specs = [(c, random_gamma(c, frames, 11 * c.q)) for c in codes]
+    for variants in (None, (0, 0, 0, 0), (4, 4, 4, 1), (5, 1, 2, 2)):
+        def tune(k, dec):
+            if variants:
+                dec.set_tuning(variants[k], 1)
+        jobs, keep = batch(specs, 3, early, tune)
+        assert (binding.nbldpc_decode_batch_cluster_blocks(jobs) > 0) == (variants is None and early == 1)
+        check_batch(specs, jobs, keep, 3, early)
