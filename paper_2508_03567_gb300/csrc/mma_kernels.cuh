@@ -449,10 +449,11 @@ __device__ __forceinline__ int pr_conv(const uint8_t* A, const uint8_t* B, uint8
 // ---------------------------------------------------------------- parameters
 struct CodeBlob {           // offsets (bytes) into the code blob
   int exp2, log, row_ptr, edge_lh, edge_lhi, edge_col, vn_ptr, vn_edge;   // (in this order)
-  // q = 8, 16, 32: byte selectors of every multiplication (PermRow), staged at `perm`
-  // behind the sections above, from perm_src behind the FFT-SPA section
+  // q = 8, 16, 32: byte selectors of every multiplication (PermRow), bytes - perm of them;
+  // staged at `perm` behind the sections above where the register form runs, from perm_src
+  // behind the FFT-SPA section
   int perm, perm_src;
-  int bytes;                  // staged by the min-max kernels
+  int bytes;                  // the sections above and the selectors
   // FFT-SPA section, from `perm` on (the min-max kernels do not stage it): check of each
   // edge, first check of each warp task, transposed-multiplication basis
   int edge_row, task_c0, at_log, fft_bytes;
@@ -479,12 +480,14 @@ struct JobDesc {
 };
 
 // Copy the sections of the code description that the min-max kernels read to shared memory:
-// [0, common) bytes, then the permutation selectors.
+// [0, common) bytes, then (PERM: the register form, its only reader) the permutation selectors.
+template <bool PERM>
 __device__ __forceinline__ void stage_blob(unsigned char* sblob, const JobDesc& job, int common_bytes, int tid, int nthr) {
   for (int i = tid; i < common_bytes / 16; i += nthr)
     reinterpret_cast<uint4*>(sblob)[i] = reinterpret_cast<const uint4*>(job.blob)[i];
-  for (int i = tid; i < (job.off.bytes - job.off.perm) / 16; i += nthr)
-    reinterpret_cast<uint4*>(sblob + common_bytes)[i] = reinterpret_cast<const uint4*>(job.blob + job.off.perm_src)[i];
+  if constexpr (PERM)
+    for (int i = tid; i < (job.off.bytes - job.off.perm) / 16; i += nthr)
+      reinterpret_cast<uint4*>(sblob + common_bytes)[i] = reinterpret_cast<const uint4*>(job.blob + job.off.perm_src)[i];
 }
 
 constexpr int kMaxJobs = 32;
@@ -1756,7 +1759,7 @@ __global__ void __launch_bounds__(XS ? kResidentThreads : 256, XS ? 2 : PR ? NBL
     const JobDesc& job = (QSEL == 0) ? p.jobs[j] : p.jobs[0];
     const int frame = item - job.item_begin;
     if (j != staged) {      // stage the code description (GF tables, H, variable-node view)
-      stage_blob(sblob, job, job.perm_at, stid, nthr);
+      stage_blob<QSEL == 0 || (XS && reg_form<QSEL>())>(sblob, job, job.perm_at, stid, nthr);
       if constexpr (QSEL == 0) {
         for (int i = stid; i < (int)(sizeof(JobDesc) / 4); i += nthr)
           reinterpret_cast<uint32_t*>(sjob)[i] = reinterpret_cast<const uint32_t*>(&job)[i];
@@ -1800,7 +1803,7 @@ struct SplitBatchParams {     // mixed codes; the jobs' frames form one list
 __device__ __forceinline__ void split_setup(const JobDesc& job, const SplitLayout& p, int frame, int rank, int size,
                                             int q, int rs, unsigned char* smem, SplitCtx& sc) {
   const int tid = threadIdx.x, nthr = blockDim.x;
-  stage_blob(smem, job, job.off.perm, tid, nthr);
+  stage_blob<false>(smem, job, job.off.perm, tid, nthr);
   sc.rank = rank;
   sc.size = size;
   sc.r0 = min(rank * p.cpc, job.m);

@@ -194,15 +194,15 @@ int split_max(int q, int mb, int dreg, int dev, int smem_optin) {
 }
 
 struct CodeNeeds {       // what one code asks of a frame slot
-  int q, variant, mb, dmax, blob, n;
+  int q, variant, mb, dmax, blob, perm, n;   // blob: staged sections; perm: the register form's selectors
   size_t msg;
   int dreg;              // regular check degree (0: the rows differ)
   int m;
 };
 
 CodeNeeds needs_of(const nbldpc_code* c, int variant, int mb) {
-  return CodeNeeds{c->q, variant, mb, c->dmax, c->off.bytes, c->n, round_up((size_t)c->nnz * c->q * mb, 256),
-                   c->dreg, c->m};
+  return CodeNeeds{c->q, variant, mb, c->dmax, c->off.perm, c->off.bytes - c->off.perm, c->n,
+                   round_up((size_t)c->nnz * c->q * mb, 256), c->dreg, c->m};
 }
 
 // Field orders whose resident-message kernels take the register form of the check-node
@@ -257,7 +257,8 @@ int make_plan(int kq, int kv, int km, int fpb, const CodeNeeds* cs, int nc, Plan
     if (kq == 0 && mixed_reg(cs[i].q, nthr, cs[i].dmax))    // either form, by the batch's frames
       s = std::max(s, reg_scratch(cs[i].q, nthr, cs[i].dmax));
     if (s > scratch) scratch = s;
-    if (cs[i].blob > pl.blob_cap) pl.blob_cap = cs[i].blob;
+    const int blob = cs[i].blob + (reg || kq == 0 ? cs[i].perm : 0);
+    if (blob > pl.blob_cap) pl.blob_cap = blob;
     if (cs[i].n > pl.n_cap) pl.n_cap = cs[i].n;
     if (cs[i].msg > pl.slot_bytes) pl.slot_bytes = cs[i].msg;
   }
@@ -435,7 +436,7 @@ SplitShape split_layout(const nbldpc_code* c, int size, int threads) {
   s.lay.npc = (c->n + size - 1) / size;
   const long long edges_r = std::min<long long>(c->nnz, (long long)s.lay.cpc * c->dmax);
   const long long edges_n = std::min<long long>(c->nnz, (long long)s.lay.npc * c->vmax);
-  size_t o = c->off.bytes;
+  size_t o = c->off.perm;
   auto take = [&](size_t bytes) { const size_t at = o; o = round_up(o + bytes, 16); return (int)at; };
   s.lay.chat_off = take((size_t)c->n);
   s.lay.flag_off = take(2 * nbldpc::kMaxSplit * sizeof(int));
@@ -894,7 +895,7 @@ static int batch_plan(const nbldpc_job* jobs, int n_jobs, Plan* pl, int* total) 
     if (st != NBLDPC_OK) return st;
     if (kmode(c) != 1) return NBLDPC_ERR_UNSUPPORTED;   // mixed-code launches: 8-bit messages, minimal schedule
     need[i] = needs_of(c, mixed_layout(c->q), 1);
-    need[i].blob = c->off.edge_col + c->off.bytes - c->off.perm;   // what the mixed-code kernel stages
+    need[i].blob = c->off.edge_col;   // the mixed-code kernel stages no edge_col or variable-node view
     fpb = std::min(fpb, batch_fpb(c));
     t += jobs[i].frames;
   }

@@ -167,3 +167,23 @@ def test_the_variant_of_a_code_does_not_change_a_mixed_batch(early, frames):
         jobs, keep = batch(specs, 3, early, tune)
         assert (binding.nbldpc_decode_batch_cluster_blocks(jobs) > 0) == (variants is None and early == 1)
         check_batch(specs, jobs, keep, 3, early)
+
+
+@pytest.mark.parametrize("q,n", [(32, 13936), (16, 13940)])
+def test_the_largest_codes_leave_no_room_for_unused_tables(q, n):
+    """Regular (2,4) codes within 100 bytes of the block's shared memory in the group form (15 n bytes of
+    description, n of decisions, the groups' scratch): it stages no table of the register form.  The
+    same code with 16-bit messages and under the Table 1 schedule, against the oracle."""
+    code = I.make_regular_code(q, n, 2, 4, seed=q, encoder=False)
+    dec = binding.Decoder.from_code(code)
+    g = random_gamma(code, 3, q)
+    gd = torch.as_tensor(g).cuda()
+    for a, w in zip(dec.decode(gd, 4, 1), oracle.decode(code, g, 4, 1, threads=THREADS)):
+        assert np.array_equal(a.cpu().numpy(), w)
+    binding.nbldpc_code_set_cnp_schedule(dec.handle, binding.NBLDPC_CNP_TABLE1)
+    for a, w in zip(dec.decode(gd, 4, 0), oracle.decode(code, g, 4, 0, threads=THREADS)):
+        assert np.array_equal(a.cpu().numpy(), w)
+    binding.nbldpc_code_set_cnp_schedule(dec.handle, binding.NBLDPC_CNP_MINIMAL)
+    dec.set_message_bits(16)
+    for a, w in zip(dec.decode(gd, 4, 0), oracle.decode(code, g, 4, 0, threads=THREADS, cap=65535)):
+        assert np.array_equal(a.cpu().numpy(), w)
