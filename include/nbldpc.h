@@ -207,8 +207,7 @@ int nbldpc_decode_batch(const nbldpc_job *jobs, int n_jobs, void *workspace_dev,
  * blocks of 384 threads with 1, 2 or 4 frames or of 256 threads with 8, and
  * the messages must fit beside the block's other shared data; otherwise
  * NBLDPC_ERR_UNSUPPORTED; GF(8), GF(16) and GF(32) decode a check per thread
- * there, with as many threads per frame as its checks need, 384 per block at
- * most).  With one warp per frame (8 frames per block, or
+ * there, with no more threads per frame than its checks need).  With one warp per frame (8 frames per block, or
  * any single-code launch whose frame slots are 32 threads) a GF(4) code of at
  * most 32 checks of degree <= 4 and columns of degree <= 2 is decoded by that
  * warp alone, with no block-wide barrier.

@@ -470,8 +470,9 @@ struct JobDesc {
   uint8_t* out_ok;            // [frames]
   int q, n, m, dmax, vmax;    // field order, columns, rows, largest row and column degree
   int perm_at;                // where the permutation selectors are staged, behind the other staged sections
-  int reg;                    // mixed-code kernel: register form of the check-node pass (q = 8, 16, 32), or
-                              // every check of degree 4 (q = 64)
+  int reg;                    // q = 8, 16, 32: lanes that take a check each in the register form of the
+                              // check-node pass (mixed-code kernel: 0, the group form); q = 64 in the
+                              // mixed-code kernel: not 0 when every check has degree 4
   int key16;                  // (255 * (max column degree + 1) + 1) * q <= 65536: 16-bit argmin keys
   int group_bytes;            // per-group shared scratch for this code
   int frames, max_iters, early_stop;
@@ -790,7 +791,7 @@ template <int NB> __device__ __forceinline__ void pack_row(const uint32_t (&v)[2
   for (int i = 0; i < NB; ++i) r[i] = __byte_perm(v[2 * i], v[2 * i + 1], 0x6420);
 }
 
-// shared scratch of a frame slot of nthr lanes: F_1..F_{d-3} of each lane's check, as bytes
+// shared scratch of nthr lanes: F_1..F_{d-3} of each lane's check, as bytes
 template <int Q> __host__ __device__ constexpr int reg_scratch_bytes(int nthr, int dmax) {
   return dmax > 3 ? nthr * (dmax - 3) * Q : 0;
 }
@@ -1557,8 +1558,10 @@ __device__ __forceinline__ void decode_frame(const JobDesc& job, int frame, uint
           pack_row<NB>(R, r);
           store_packed(e, r);
         };
-        uint8_t* fs = scratch + (size_t)stid * Q;                // F_j of this lane: fs + (j - 1) * nthr * Q
-        for (int r = r_first + stid; r < r_last; r += nthr) {
+        const int lanes = job.reg;
+        if (stid >= lanes) return;
+        uint8_t* fs = scratch + (size_t)stid * Q;                // F_j of this lane: fs + (j - 1) * lanes * Q
+        for (int r = r_first + stid; r < r_last; r += lanes) {
           const int e0 = row_ptr[r], d = D > 0 ? D : row_ptr[r + 1] - e0;
           if (counting && d > 2) work += (unsigned long long)Q * Q * 3 * (d - 2);
           uint32_t a[W], b[W], c[W];
@@ -1571,7 +1574,7 @@ __device__ __forceinline__ void decode_frame(const JobDesc& job, int frame, uint
             if (j <= d - 3) {
               uint32_t f[NB];
               pack_row<NB>(c, f);
-              store_row<Q>(fs + (size_t)(j - 1) * nthr * Q, f);
+              store_row<Q>(fs + (size_t)(j - 1) * lanes * Q, f);
             }
 #pragma unroll
             for (int w = 0; w < W; ++w) a[w] = c[w];
@@ -1585,7 +1588,7 @@ __device__ __forceinline__ void decode_frame(const JobDesc& job, int frame, uint
               load_p(e0, a);
             } else {
               uint32_t f[NB];
-              load_row<Q>(fs + (size_t)(j - 2) * nthr * Q, f);
+              load_row<Q>(fs + (size_t)(j - 2) * lanes * Q, f);
               unpack_row<NB>(f, a);
             }
             uint32_t be[NB];

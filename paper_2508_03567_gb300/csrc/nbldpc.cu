@@ -209,10 +209,10 @@ CodeNeeds needs_of(const nbldpc_code* c, int variant, int mb) {
 // pass (one lane per check).
 bool reg_form(int q) { return q == 8 || q == 16 || q == 32; }
 
-// Threads of a frame slot of those kernels: the checks in as few rounds as 384 threads
+// Threads of a frame slot of those kernels: the checks in as few rounds as `most` threads
 // allow, and no more threads than these rounds need.
-int reg_threads(int m) {
-  const int rounds = (m + nbldpc::kResidentThreads - 1) / nbldpc::kResidentThreads;
+int reg_threads(int m, int most = nbldpc::kResidentThreads) {
+  const int rounds = (m + most - 1) / most;
   return (int)round_up((size_t)(m + rounds - 1) / rounds, 32);
 }
 
@@ -228,8 +228,8 @@ bool mixed_reg(int q, int nthr, int dmax) { return reg_form(q) && reg_scratch(q,
 // Plan a launch of kernel (kq, kv, kernel mode km) with fpb frame slots per block for a set of codes.
 // Variants 2 and 3 keep each frame's messages in shared memory: blocks of
 // nbldpc::kResidentThreads threads (1, 2 or 4 frame slots) or of 256 threads with
-// 8 one-warp slots (q = 8, 16, 32: at most nbldpc::kResidentThreads threads, as many
-// a slot as its checks need), no message slots in the workspace.
+// 8 one-warp slots (q = 8, 16, 32: no more threads a slot than its checks need, and as
+// many of them with a check as their scratch leaves room for), no message slots in the workspace.
 int make_plan(int kq, int kv, int km, int fpb, const CodeNeeds* cs, int nc, Plan* out) {
   int dev = 0, sms = 0, optin = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
@@ -238,16 +238,15 @@ int make_plan(int kq, int kv, int km, int fpb, const CodeNeeds* cs, int nc, Plan
     return NBLDPC_ERR_CUDA;
   const bool resident = kv >= 0 && (kv & 2);
   const bool reg = resident && reg_form(kq);
-  const int threads = reg ? fpb * reg_threads(cs[0].m)
-                          : resident ? (fpb == 8 ? kThreads : nbldpc::kResidentThreads) : kThreads;
-  if (fpb < 1 || threads % fpb) return NBLDPC_ERR_ARG;
-  if (reg && threads > nbldpc::kResidentThreads) return NBLDPC_ERR_UNSUPPORTED;
+  const int most = resident && fpb != 8 ? nbldpc::kResidentThreads : kThreads;
+  if (fpb < 1 || most % fpb) return NBLDPC_ERR_ARG;
   if (resident && km != 1) return NBLDPC_ERR_UNSUPPORTED;
-  const int nthr = threads / fpb;
+  int nthr = most / fpb;
   if (nthr < 32 || nthr % 32) return NBLDPC_ERR_UNSUPPORTED;
+  if (reg) nthr = std::min(nthr, reg_threads(cs[0].m, nthr));
   Plan pl{};
   pl.fpb = fpb;
-  pl.threads = threads;
+  pl.threads = fpb * nthr;
   int scratch = 0;
   for (int i = 0; i < nc; ++i) {
     const int G = group_lanes(cs[i].q, cs[i].variant & 1);
@@ -264,7 +263,18 @@ int make_plan(int kq, int kv, int km, int fpb, const CodeNeeds* cs, int nc, Plan
   }
   pl.blob_cap = (int)round_up((size_t)pl.blob_cap, 16);
   pl.n_cap = (int)round_up((size_t)pl.n_cap, 16);
-  pl.slot_smem = (int)round_up((size_t)(pl.blob_cap + pl.n_cap + nbldpc::ctl_bytes(kq) + scratch), 16);
+  const int fixed = pl.blob_cap + pl.n_cap + nbldpc::ctl_bytes(kq);
+  if (reg) {
+    pl.lanes = nthr;
+    const int row = reg_scratch(kq, 1, cs[0].dmax);   // a lane's scratch
+    const int room = optin / fpb / 16 * 16 - (int)round_up((size_t)fixed, 16) - (int)round_up(pl.slot_bytes, 16);
+    if (scratch > room) {
+      pl.lanes = room < row ? 0 : std::min(nthr, room / 16 * 16 / row);
+      if (pl.lanes < 1) return NBLDPC_ERR_UNSUPPORTED;
+      scratch = pl.lanes * row;
+    }
+  }
+  pl.slot_smem = (int)round_up((size_t)(fixed + scratch), 16);
   if (resident) {   // the messages follow the slot's scratch
     pl.xs_off = pl.slot_smem;
     pl.slot_smem += (int)round_up(pl.slot_bytes, 16);
@@ -337,7 +347,7 @@ int configure_reg(nbldpc_code* c, int variant) {
     Plan pl{};
     const int st = make_plan(c->q, variant, kmode(c), fpb, &need, 1, &pl);
     if (st == NBLDPC_ERR_CUDA) return st;
-    if (st == NBLDPC_OK && pl.per_sm * pl.threads >= most) {
+    if (st == NBLDPC_OK && pl.lanes == nthr && pl.per_sm * pl.threads >= most) {
       most = pl.per_sm * pl.threads;
       best = fpb;
     }
@@ -526,6 +536,7 @@ int launch(const nbldpc_code* c, const uint8_t* gamma, int frames, int max_iters
   }
   nbldpc::LaunchParamsOf<1> lp{};
   lp.jobs[0] = job_desc(c, gamma, frames, max_iters, early_stop, sym, iters, ok, 0, count);
+  lp.jobs[0].reg = c->plan.lanes;
   lp.njobs = 1;
   lp.total_items = frames;
   return launch_plan(kernel_for(c->q, c->variant, kmode(c), c->dreg), c->plan, lp, grid_for(c->plan, frames), ws,
@@ -584,6 +595,7 @@ int nbldpc_decode_noalloc(const nbldpc_code* c, const uint8_t* gamma_dev, int fr
   // the array keeps the previous call's contents: the frame counter is cleared in launch_plan
   nbldpc::LaunchParamsOf<1> lp{};
   lp.jobs[0] = job_desc(c, gamma_dev, frames, max_iters, early_stop, out_sym_dev, out_iters_dev, out_ok_dev, 0);
+  lp.jobs[0].reg = pl.lanes;
   lp.njobs = 1;
   lp.total_items = frames;
   return launch_plan(kernel_for(c->q, c->variant, kmode(c), c->dreg), pl, lp, grid, scratch,
@@ -1034,7 +1046,7 @@ int nbldpc_decode_batch(const nbldpc_job* jobs, int n_jobs, void* workspace_dev,
     // frames fill the SM (100 frames of GF(32) N=64 and 200 of GF(4) N=100: 312 us against 109)
     const int nthr = pl.threads / pl.fpb;
     const bool fills = 2 * c->m >= nthr || total > pl.grid_max * pl.fpb;
-    lp.jobs[i].reg = (mixed_reg(c->q, nthr, c->dmax) && fills) || (c->q == 64 && c->dreg == 4) ? 1 : 0;
+    lp.jobs[i].reg = (mixed_reg(c->q, nthr, c->dmax) && fills) || (c->q == 64 && c->dreg == 4) ? nthr : 0;
   }
   return launch_plan(kernel_for(0, -1, 1), pl, lp, grid_for(pl, total), workspace_dev,
                      reinterpret_cast<uint8_t*>(workspace_dev) + 256, reinterpret_cast<cudaStream_t>(cuda_stream));

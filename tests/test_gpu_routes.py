@@ -187,3 +187,33 @@ def test_the_largest_codes_leave_no_room_for_unused_tables(q, n):
     dec.set_message_bits(16)
     for a, w in zip(dec.decode(gd, 4, 0), oracle.decode(code, g, 4, 0, threads=THREADS, cap=65535)):
         assert np.array_equal(a.cpu().numpy(), w)
+
+
+def one_heavy_check(q, n, m, seed):
+    """Checks of degree 3, and one of degree 60."""
+    rng = np.random.default_rng(seed)
+    h = np.zeros((m, n), np.int64)
+    for r in range(m):
+        d = 60 if r == m // 2 else 3
+        h[r, (3 * r + np.arange(d)) % n] = rng.integers(1, q, d)
+    return I.code_from_dense(h, q, I.PRIMITIVE_POLY[q])
+
+
+@pytest.mark.parametrize("q,n,tunings", [(16, 1024, ((2, 1), (3, 2), (3, 4))), (32, 600, ((3, 1), (2, 2))),
+                                         (8, 512, ((2, 1), (3, 2), (2, 4), (2, 8))),
+                                         (16, 64, ((3, 4), (2, 8))), (32, 64, ((3, 2), (2, 4)))])
+def test_resident_tunings_of_the_register_form(q, n, tunings):
+    """Variants 2 and 3 at every frames-per-block whose messages fit, also where a frame has more checks
+    than its share of the block's threads (n >= 512), or its checks want more scratch than is left (n =
+    64: lanes without a check at 4 and 8 frames): taken, and equal to the oracle."""
+    code = one_heavy_check(q, n, 40, q) if n == 64 else I.make_regular_code(q, n, 2, 4, seed=q + n)
+    dec = binding.Decoder.from_code(code)
+    g = random_gamma(code, 21, q + n)
+    gd = torch.as_tensor(g).cuda()
+    for v, fpb in tunings:
+        dec.set_tuning(v, fpb)
+        assert dec.tuning() == (v, fpb)
+        for iters, early in ((4, 1), (2, 0)):
+            want = oracle.decode(code, g, iters, early, threads=THREADS)
+            for a, w in zip(dec.decode(gd, iters, early), want):
+                assert np.array_equal(a.cpu().numpy(), w), f"variant {v}, {fpb} frames per block"
