@@ -25,6 +25,7 @@ struct Plan {
   int grid_max = 0;     // resident blocks on the device
   int blob_cap = 0, n_cap = 0;
   size_t slot_bytes = 0;  // message slot per frame slot in the workspace (0: messages in shared memory)
+  bool mixed_reg = false; // mixed-code launches: room for the register form of the check-node pass
   int lanes = 0;          // register form: lanes of a frame slot that take a check each
   int xs_off = 0;         // shared-memory offset of the messages (resident launches)
 };

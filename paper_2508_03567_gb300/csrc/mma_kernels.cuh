@@ -481,12 +481,12 @@ struct JobDesc {
 };
 
 // Copy the sections of the code description that the min-max kernels read to shared memory:
-// [0, common) bytes, then (PERM: the register form, its only reader) the permutation selectors.
-template <bool PERM>
-__device__ __forceinline__ void stage_blob(unsigned char* sblob, const JobDesc& job, int common_bytes, int tid, int nthr) {
+// [0, common) bytes, then (perm: the register form, their only reader) the permutation selectors.
+__device__ __forceinline__ void stage_blob(unsigned char* sblob, const JobDesc& job, int common_bytes, bool perm, int tid,
+                                           int nthr) {
   for (int i = tid; i < common_bytes / 16; i += nthr)
     reinterpret_cast<uint4*>(sblob)[i] = reinterpret_cast<const uint4*>(job.blob)[i];
-  if constexpr (PERM)
+  if (perm)
     for (int i = tid; i < (job.off.bytes - job.off.perm) / 16; i += nthr)
       reinterpret_cast<uint4*>(sblob + common_bytes)[i] = reinterpret_cast<const uint4*>(job.blob + job.off.perm_src)[i];
 }
@@ -1762,7 +1762,7 @@ __global__ void __launch_bounds__(XS ? kResidentThreads : 256, XS ? 2 : PR ? NBL
     const JobDesc& job = (QSEL == 0) ? p.jobs[j] : p.jobs[0];
     const int frame = item - job.item_begin;
     if (j != staged) {      // stage the code description (GF tables, H, variable-node view)
-      stage_blob<QSEL == 0 || (XS && reg_form<QSEL>())>(sblob, job, job.perm_at, stid, nthr);
+      stage_blob(sblob, job, job.perm_at, QSEL == 0 ? job.reg != 0 : XS && reg_form<QSEL>(), stid, nthr);
       if constexpr (QSEL == 0) {
         for (int i = stid; i < (int)(sizeof(JobDesc) / 4); i += nthr)
           reinterpret_cast<uint32_t*>(sjob)[i] = reinterpret_cast<const uint32_t*>(&job)[i];
@@ -1806,7 +1806,7 @@ struct SplitBatchParams {     // mixed codes; the jobs' frames form one list
 __device__ __forceinline__ void split_setup(const JobDesc& job, const SplitLayout& p, int frame, int rank, int size,
                                             int q, int rs, unsigned char* smem, SplitCtx& sc) {
   const int tid = threadIdx.x, nthr = blockDim.x;
-  stage_blob<false>(smem, job, job.off.perm, tid, nthr);
+  stage_blob(smem, job, job.off.perm, false, tid, nthr);
   sc.rank = rank;
   sc.size = size;
   sc.r0 = min(rank * p.cpc, job.m);

@@ -230,7 +230,9 @@ bool mixed_reg(int q, int nthr, int dmax) { return reg_form(q) && reg_scratch(q,
 // nbldpc::kResidentThreads threads (1, 2 or 4 frame slots) or of 256 threads with
 // 8 one-warp slots (q = 8, 16, 32: no more threads a slot than its checks need, and as
 // many of them with a check as their scratch leaves room for), no message slots in the workspace.
-int make_plan(int kq, int kv, int km, int fpb, const CodeNeeds* cs, int nc, Plan* out) {
+// mixed: the mixed-code kernel's (kq = 0) register form has its scratch and selectors beside the group
+// form's, so that a launch may take either; without them where both do not fit.
+int make_plan(int kq, int kv, int km, int fpb, const CodeNeeds* cs, int nc, Plan* out, bool mixed = true) {
   int dev = 0, sms = 0, optin = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
@@ -253,10 +255,10 @@ int make_plan(int kq, int kv, int km, int fpb, const CodeNeeds* cs, int nc, Plan
     if (G > nthr) return NBLDPC_ERR_UNSUPPORTED;
     int s = reg ? reg_scratch(cs[i].q, nthr, cs[i].dmax)
                       : (nthr / G) * group_bytes(cs[i].q, cs[i].dmax, cs[i].mb, kq == 0 ? cs[i].q >= 128 : (kv & 4) != 0);
-    if (kq == 0 && mixed_reg(cs[i].q, nthr, cs[i].dmax))    // either form, by the batch's frames
-      s = std::max(s, reg_scratch(cs[i].q, nthr, cs[i].dmax));
+    const bool either = kq == 0 && mixed && mixed_reg(cs[i].q, nthr, cs[i].dmax);
+    if (either) s = std::max(s, reg_scratch(cs[i].q, nthr, cs[i].dmax));
     if (s > scratch) scratch = s;
-    const int blob = cs[i].blob + (reg || kq == 0 ? cs[i].perm : 0);
+    const int blob = cs[i].blob + (reg || either ? cs[i].perm : 0);
     if (blob > pl.blob_cap) pl.blob_cap = blob;
     if (cs[i].n > pl.n_cap) pl.n_cap = cs[i].n;
     if (cs[i].msg > pl.slot_bytes) pl.slot_bytes = cs[i].msg;
@@ -264,6 +266,9 @@ int make_plan(int kq, int kv, int km, int fpb, const CodeNeeds* cs, int nc, Plan
   pl.blob_cap = (int)round_up((size_t)pl.blob_cap, 16);
   pl.n_cap = (int)round_up((size_t)pl.n_cap, 16);
   const int fixed = pl.blob_cap + pl.n_cap + nbldpc::ctl_bytes(kq);
+  if (kq == 0 && mixed && fpb * (int)round_up((size_t)(fixed + scratch), 16) > optin)
+    return make_plan(kq, kv, km, fpb, cs, nc, out, false);
+  pl.mixed_reg = kq == 0 && mixed;
   if (reg) {
     pl.lanes = nthr;
     const int row = reg_scratch(kq, 1, cs[0].dmax);   // a lane's scratch
@@ -1046,7 +1051,7 @@ int nbldpc_decode_batch(const nbldpc_job* jobs, int n_jobs, void* workspace_dev,
     // frames fill the SM (100 frames of GF(32) N=64 and 200 of GF(4) N=100: 312 us against 109)
     const int nthr = pl.threads / pl.fpb;
     const bool fills = 2 * c->m >= nthr || total > pl.grid_max * pl.fpb;
-    lp.jobs[i].reg = (mixed_reg(c->q, nthr, c->dmax) && fills) || (c->q == 64 && c->dreg == 4) ? nthr : 0;
+    lp.jobs[i].reg = (pl.mixed_reg && mixed_reg(c->q, nthr, c->dmax) && fills) || (c->q == 64 && c->dreg == 4) ? nthr : 0;
   }
   return launch_plan(kernel_for(0, -1, 1), pl, lp, grid_for(pl, total), workspace_dev,
                      reinterpret_cast<uint8_t*>(workspace_dev) + 256, reinterpret_cast<cudaStream_t>(cuda_stream));

@@ -189,12 +189,12 @@ def test_the_largest_codes_leave_no_room_for_unused_tables(q, n):
         assert np.array_equal(a.cpu().numpy(), w)
 
 
-def one_heavy_check(q, n, m, seed):
-    """Checks of degree 3, and one of degree 60."""
+def one_heavy_check(q, n, m, seed, heavy=60):
+    """Checks of degree 3, and one of degree `heavy`."""
     rng = np.random.default_rng(seed)
     h = np.zeros((m, n), np.int64)
     for r in range(m):
-        d = 60 if r == m // 2 else 3
+        d = heavy if r == m // 2 else 3
         h[r, (3 * r + np.arange(d)) % n] = rng.integers(1, q, d)
     return I.code_from_dense(h, q, I.PRIMITIVE_POLY[q])
 
@@ -217,3 +217,16 @@ def test_resident_tunings_of_the_register_form(q, n, tunings):
             want = oracle.decode(code, g, iters, early, threads=THREADS)
             for a, w in zip(dec.decode(gd, iters, early), want):
                 assert np.array_equal(a.cpu().numpy(), w), f"variant {v}, {fpb} frames per block"
+
+
+def test_mixed_batch_of_a_code_whose_register_scratch_does_not_fit():
+    """32 checks, one of degree 34, eight frames to a block: the register form's scratch (31 KB a frame)
+    does not fit eight times, the group form's does, and the batch takes it."""
+    code = one_heavy_check(32, 34, 32, 7, heavy=34)
+    assert code.m == 32 and np.diff(code.row_ptr).max() == 34
+    frames = 4 * sms()
+    specs = [(code, random_gamma(code, frames, 8))]
+    for early in (0, 1):
+        jobs, keep = batch(specs, 3, early)
+        check_batch(specs, jobs, keep, 3, early)
+    assert binding.nbldpc_decode_batch_workspace_size(jobs) % (8 * (-(-code.nnz * 32 // 256) * 256)) == 256
