@@ -55,7 +55,7 @@ const void* fft_kernel_for(int q, int dc, int dv, int form, int* threads = nullp
 #endif
 
 // device, log2(q) - 1, check-node form, column-degree bucket: the kernels' attributes are
-// set; the largest cluster of the split-frame kernel (-1: none)
+// set; the largest cluster of the split-frame kernel (0: not asked, -1: none)
 bool g_fft_attr_done[64][8][3][3][2] = {};
 int g_fft_split_max[64][8][3][3] = {};
 
@@ -115,9 +115,10 @@ int nbldpc_host::fft_configure(nbldpc_code* c, const int32_t* row_ptr) {
       if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, optin) != cudaSuccess)
         return NBLDPC_ERR_CUDA;
       if (split == 0) split = split_kernel_prepare(fft_kernel_for(c->q, dc, dv, 2), threads, optin);
+      if (split == 0) split = -1;
       done = true;
     }
-    c->fft_split_max = split;
+    c->fft_split_max = split < 0 ? 0 : split;
     c->fft_split_threads = threads;
   }
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pl.per_sm, k, pl.threads, pl.smem) != cudaSuccess)

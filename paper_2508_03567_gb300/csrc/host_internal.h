@@ -95,28 +95,38 @@ inline int check_device(const nbldpc_code* c) {
 int fft_configure(nbldpc_code* c, const int32_t* row_ptr);
 
 // ---- frames split over the blocks of a cluster ------------------------------
-// Set a split-frame kernel's attributes; the largest cluster that the device runs
-// for it (16, else the portable 8), or 0 when it cannot be prepared.
+// Largest cluster, of 16 (only if `wide`: beyond the portable size), 8, 4 and 2 blocks, that
+// `runs` says the device can run, or 0: frames then keep one block each.
+template <class Runs> int largest_cluster(bool wide, Runs runs) {
+  for (int size = wide ? nbldpc::kMaxSplit : 8; size >= 2; size /= 2)
+    if (runs(size)) return size;
+  return 0;
+}
+
+// Set a split-frame kernel's attributes; the largest cluster of blocks of this shape that the
+// device runs for it, or 0 when there is none or the kernel cannot be prepared.
 inline int split_kernel_prepare(const void* kernel, int threads, int smem_optin) {
   if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_optin) != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }
-  cudaLaunchConfig_t cfg{};
-  cudaLaunchAttribute at{};
-  at.id = cudaLaunchAttributeClusterDimension;
-  at.val.clusterDim.x = nbldpc::kMaxSplit;
-  at.val.clusterDim.y = at.val.clusterDim.z = 1;
-  cfg.gridDim = dim3(nbldpc::kMaxSplit);
-  cfg.blockDim = dim3((unsigned)threads);
-  cfg.dynamicSmemBytes = (size_t)smem_optin;
-  cfg.attrs = &at;
-  cfg.numAttrs = 1;
-  int n = 0;
-  const bool wide = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
-                    cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) == cudaSuccess && n >= 1;
+  const bool wide = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+  const int most = largest_cluster(wide, [&](int size) {
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = (unsigned)size;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.gridDim = dim3((unsigned)size);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = (size_t)smem_optin;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    int n = 0;
+    return cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) == cudaSuccess && n >= 1;
+  });
   cudaGetLastError();          // a refused query is not a later call's error
-  return wide ? nbldpc::kMaxSplit : 8;
+  return most;
 }
 
 // Queue one cluster of `size` blocks per frame.

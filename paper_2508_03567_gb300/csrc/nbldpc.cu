@@ -175,9 +175,9 @@ int prepare_kernel(int q, int v, int km, int dreg, int dev, int smem_optin) {
   return NBLDPC_OK;
 }
 
-// Largest cluster of split-frame blocks (16, else the portable 8) that the device
-// runs for a field order and message width; 0 when the kernel cannot be prepared.
-// The kernel attributes are set and the device asked once.
+// Largest cluster of split-frame blocks (16, 8, 4 or 2) that the device runs for a field
+// order and message width; 0 when there is none.  The kernel attributes are set and the
+// device asked once (-1: asked, none).
 int g_split_max[64][9][3] = {};
 
 int split_max(int q, int mb, int dreg, int dev, int smem_optin) {
