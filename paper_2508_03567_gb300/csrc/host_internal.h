@@ -27,6 +27,7 @@ struct Plan {
   size_t slot_bytes = 0;  // message slot per frame slot in the workspace (0: messages in shared memory)
   bool mixed_reg = false; // mixed-code launches: room for the register form of the check-node pass
   int lanes = 0;          // register form: lanes of a frame slot that take a check each
+  int dreg = 0;           // check degree that selects the kernel (see kernel_for)
   int xs_off = 0;         // shared-memory offset of the messages (resident launches)
 };
 

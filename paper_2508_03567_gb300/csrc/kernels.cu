@@ -28,7 +28,8 @@ template <int Q> const void* pruned_kernel(int layout) {
 // groups only, not with bit 1), mb-byte messages and the check-node schedule t1
 // (1: Table 1's 3 d_c - 4 convolutions, 8-bit messages only) of this unit's
 // field order; dreg: the code's check degree when all are equal (GF(4) and
-// GF(64) have resident-message kernels for degree 4), else 0; null when there is none.
+// GF(64) have resident-message kernels for degree 4), else 0, or -1 for the register form
+// with fewer lanes than threads; null when there is none.
 const void* NBLDPC_CAT(kernel_q, NBLDPC_KQ)(int v, int mb, int t1, int dreg) {
   (void)dreg;
 #if NBLDPC_KQ == 0
@@ -49,10 +50,12 @@ const void* NBLDPC_CAT(kernel_q, NBLDPC_KQ)(int v, int mb, int t1, int dreg) {
 #endif
 #if NBLDPC_KQ == 8 || NBLDPC_KQ == 16 || NBLDPC_KQ == 32
     // (one lane per check: the layouts of the group form do not differ here)
-    return reinterpret_cast<const void*>(&mma_decode_kernel<NBLDPC_KQ, 0, 1, false, true>);
-#endif
+    return dreg < 0 ? reinterpret_cast<const void*>(&mma_decode_kernel<NBLDPC_KQ, 0, 1, false, true, false, -1>)
+                    : reinterpret_cast<const void*>(&mma_decode_kernel<NBLDPC_KQ, 0, 1, false, true>);
+#else
     return (v & 1) ? reinterpret_cast<const void*>(&mma_decode_kernel<NBLDPC_KQ, 1, 1, false, true>)
                    : reinterpret_cast<const void*>(&mma_decode_kernel<NBLDPC_KQ, 0, 1, false, true>);
+#endif
   }
   if (t1) {
     if (mb != 1) return nullptr;

@@ -471,8 +471,9 @@ struct JobDesc {
   int q, n, m, dmax, vmax;    // field order, columns, rows, largest row and column degree
   int perm_at;                // where the permutation selectors are staged, behind the other staged sections
   int reg;                    // q = 8, 16, 32: lanes that take a check each in the register form of the
-                              // check-node pass (mixed-code kernel: 0, the group form); q = 64 in the
-                              // mixed-code kernel: not 0 when every check has degree 4
+                              // check-node pass (the slot's threads, or D = -1 fewer; mixed-code kernel:
+                              // 0, the group form); q = 64 in the mixed-code kernel: not 0 when every
+                              // check has degree 4
   int key16;                  // (255 * (max column degree + 1) + 1) * q <= 65536: 16-bit argmin keys
   int group_bytes;            // per-group shared scratch for this code
   int frames, max_iters, early_stop;
@@ -1015,7 +1016,8 @@ template <class T> __device__ __forceinline__ T* at_rank(T* p, int r) {
 // (pr_conv; 32-lane groups, 8-bit messages, minimal schedule).  W4: a GF(4) frame slot of one warp may take the one-warp form
 // (decode_frame_warp4; resident-message kernels, which have the registers for it).
 // D > 0: every check of the code has degree D (a compile-time loop bound and
-// vector layout; 0: the degrees are read per check).  SP: the threads are those of
+// vector layout; 0: the degrees are read per check; -1: so they are, and not every
+// lane of the slot has room for a check in the register form).  SP: the threads are those of
 // one rank of a cluster that decodes the frame together (sc; X then holds the
 // message rows of the rank's own edges).
 template <class g, int MB, bool T1, bool PR = false, bool W4 = false, int D = 0, bool SP = false>
@@ -1558,8 +1560,10 @@ __device__ __forceinline__ void decode_frame(const JobDesc& job, int frame, uint
           pack_row<NB>(R, r);
           store_packed(e, r);
         };
-        const int lanes = job.reg;
-        if (stid >= lanes) return;
+        // (a stride from the job costs up to 10 % where the pass is short: GF(16) N=64, 9,000 frames
+        // 330 us against 300, so launches with all lanes have a kernel without it)
+        const int lanes = D < 0 ? job.reg : nthr;
+        if (D < 0 && stid >= lanes) return;
         uint8_t* fs = scratch + (size_t)stid * Q;                // F_j of this lane: fs + (j - 1) * lanes * Q
         for (int r = r_first + stid; r < r_last; r += lanes) {
           const int e0 = row_ptr[r], d = D > 0 ? D : row_ptr[r + 1] - e0;

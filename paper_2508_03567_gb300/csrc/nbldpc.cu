@@ -78,8 +78,9 @@ int kmode(const nbldpc_code* c) { return c->mb == 2 ? 2 : (c->cnp_schedule == NB
 
 // kernel compiled for one field order, variant (bit 0: layout; bit 1: messages
 // resident in shared memory; bit 2: pruned convolutions), kernel mode and the
-// code's regular check degree (dreg: 0 when the rows differ; a field order may
-// have a kernel for it), or for every field order (q = 0, mode 1)
+// code's regular check degree (dreg: 0 when the rows differ, -1 for a register form
+// with fewer lanes than threads; a field order may have a kernel for it), or for every
+// field order (q = 0, mode 1)
 const void* kernel_for(int q, int v, int km, int dreg = 0) {
   const int mb = km == 2 ? 2 : 1, t1 = km == 3 ? 1 : 0;
   switch (q) {
@@ -150,14 +151,15 @@ int group_bytes(int q, int dmax, int mb, bool pr) {
 
 // Every kernel may use up to the opt-in shared memory of the device (set once
 // per device and kernel; occupancy still follows the bytes of each launch).
-bool g_attr_done[64][85] = {};
+bool g_attr_done[64][88] = {};
 
 // per field order: 3 kernel modes x 2 layouts, the 2 resident-message kernels,
 // then the 2 pruned-convolution kernels; after them the 2 GF(64) and the 2 GF(4)
-// resident kernels of check degree 4
+// resident kernels of check degree 4 and the GF(8), GF(16), GF(32) ones of few lanes
 int kernel_slot(int q, int v, int km, int dreg) {
   if (q == 0) return 0;
   if (kernel_dreg(q, v, km, dreg)) return (q == 64 ? 81 : 83) + (v & 1);
+  if (dreg < 0) return 85 + nbldpc::ilog2(q) - 3;
   return 1 + 10 * (nbldpc::ilog2(q) - 1) + ((v & 4) ? 8 + (v & 1) : (v & 2) ? 6 + (v & 1) : 2 * (km - 1) + (v & 1));
 }
 
@@ -287,7 +289,7 @@ int make_plan(int kq, int kv, int km, int fpb, const CodeNeeds* cs, int nc, Plan
   }
   pl.smem = fpb * pl.slot_smem;
   if (pl.smem > optin) return NBLDPC_ERR_UNSUPPORTED;
-  const int dreg = (kq != 0 && nc == 1) ? cs[0].dreg : 0;
+  const int dreg = pl.dreg = reg ? (pl.lanes < nthr ? -1 : 0) : (kq != 0 && nc == 1) ? cs[0].dreg : 0;
   int st = prepare_kernel(kq, kv, km, dreg, dev, optin);
   if (st != NBLDPC_OK) return st;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pl.per_sm, kernel_for(kq, kv, km, dreg), pl.threads, pl.smem) !=
@@ -546,7 +548,7 @@ int launch(const nbldpc_code* c, const uint8_t* gamma, int frames, int max_iters
   lp.jobs[0].reg = c->plan.lanes;
   lp.njobs = 1;
   lp.total_items = frames;
-  return launch_plan(kernel_for(c->q, c->variant, kmode(c), c->dreg), c->plan, lp, grid_for(c->plan, frames), ws,
+  return launch_plan(kernel_for(c->q, c->variant, kmode(c), c->plan.dreg), c->plan, lp, grid_for(c->plan, frames), ws,
                      reinterpret_cast<uint8_t*>(ws) + 256, st);
 }
 
@@ -605,7 +607,7 @@ int nbldpc_decode_noalloc(const nbldpc_code* c, const uint8_t* gamma_dev, int fr
   lp.jobs[0].reg = pl.lanes;
   lp.njobs = 1;
   lp.total_items = frames;
-  return launch_plan(kernel_for(c->q, c->variant, kmode(c), c->dreg), pl, lp, grid, scratch,
+  return launch_plan(kernel_for(c->q, c->variant, kmode(c), pl.dreg), pl, lp, grid, scratch,
                      reinterpret_cast<uint8_t*>(scratch) + 256,
                      reinterpret_cast<cudaStream_t>(cuda_stream));
 }
