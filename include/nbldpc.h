@@ -211,7 +211,7 @@ int nbldpc_decode_batch(const nbldpc_job *jobs, int n_jobs, void *workspace_dev,
  * any single-code launch whose frame slots are 32 threads) a GF(4) code of at
  * most 32 checks of degree <= 4 and columns of degree <= 2 is decoded by that
  * warp alone, with no block-wide barrier.
- * The workspace of such a code is 256 bytes.  Bit 2 (variants 4 and 5) prunes
+ * The workspace of a code tuned to variant 2 or 3 is 256 bytes.  Bit 2 (variants 4 and 5) prunes
  * the check-node convolutions: C(x) = min_y max(A(y), B(x ^ y)) equals the
  * minimum over the y with A(y) <= T for any T >= max_x C(x) (any other y gives
  * a maximum above C(x)), and likewise with A and B exchanged, so each
@@ -221,7 +221,9 @@ int nbldpc_decode_batch(const nbldpc_job *jobs, int n_jobs, void *workspace_dev,
  * 8-bit messages and the minimal schedule, and excludes bit 1 (otherwise
  * NBLDPC_ERR_UNSUPPORTED).  Mixed-code batches have one kernel form per field
  * order whatever the variant (GF(128) and GF(256) pruned).  nbldpc_code_create picks a default variant
- * per field order and a frames-per-block value from the code size;
+ * per field order and a frames-per-block value from the code size (GF(8) to GF(32) take fewer
+ * frames per block, and short GF(16) and GF(32) codes variant 1, when a call has too few frames
+ * for that; nbldpc_decode_workspace_size counts the slots);
  * nbldpc_code_autotune measures every valid pair on the caller's frames and
  * keeps the fastest.  A batch of too few frames to fill the GPU this way (how
  * few depends on the code, the message width and early_stop; minimal schedule)

@@ -69,6 +69,8 @@ struct nbldpc_code {
   bool pinned = false;                 // the launch shape was set by nbldpc_code_set_tuning: every batch takes it
   bool tuned = false;                  // the launch shape was set or measured (else the default of the mode)
   nbldpc_host::Plan plan{};            // single-code launch shape (fpb chosen by default or by the autotuner)
+  bool has_group = false;              // untuned register-form handles: the group form's launch shape, for the
+  nbldpc_host::Plan group{};           // calls with too few frames for a lane per check (variant & 1)
   int fft_status = NBLDPC_ERR_UNSUPPORTED;   // FFT-SPA launch shape below valid when NBLDPC_OK
   int fft_dc = 0, fft_dv = 0;          // FFT-SPA check-node form (dc 0: lane per edge) and column-degree bucket
   int fft_split_max = 0, fft_split_threads = 0;   // largest cluster and block of the FFT-SPA split-frame kernel

@@ -332,6 +332,7 @@ int configure(nbldpc_code* c, int variant, int fpb) {
   if (st != NBLDPC_OK) return st;
   c->variant = variant;
   c->plan = pl;
+  c->has_group = false;
   // (the limit serves the FFT-SPA clusters too, which the min-max settings do not touch)
   int optin = 0;
   if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device) != cudaSuccess) optin = 0;
@@ -362,6 +363,32 @@ int configure_reg(nbldpc_code* c, int variant) {
   return best ? configure(c, variant, best) : NBLDPC_ERR_UNSUPPORTED;
 }
 
+// Frames up to which an untuned GF(16) or GF(32) handle decodes in the group form.  A lane per
+// check takes long with few checks, and a chip that is not full does not make up for it; the
+// group form spreads a check over 8 (q = 16) or 16 lanes.  The limits are frames per SM, from
+// sweeps of 20 to 16,000 frames over codes of 32 to 512 checks on GB300 (us per decode of up to
+// 30 iterations with early stop, group form against register form with the frames per block
+// of choose_plan):
+//  - GF(16): N=64, 100 / 1,300 / 4,000 frames 75 / 140 / 253 against 126 / 158 / 255; N=96 (3,6),
+//    152 / 1,300 / 2,700 frames 185 / 340 / 535 against 197 / 436 / 560; N=128 (64 checks), 300
+//    frames 160 against 128.
+//  - GF(32): N=64, 600 / 4,000 / 16,000 frames 199 / 541 / 1,689 against 449 / 781 / 1,743; N=128,
+//    1,300 / 8,000 frames 522 / 1,766 against 649 / 1,652; N=256 (128 checks), 600 frames 725
+//    against 610.
+//  - Fixed iterations fill the chip sooner: N=64, 100 / 600 frames 29 / 52 against 47 / 48 at
+//    GF(16), 50 / 111 against 152 / 156 at GF(32); GF(32) N=160, 450 / 600 frames 197 / 250
+//    against 236 / 235; 32 checks of degree 4 and 8, 1,900 frames 320 and 743 against 300 and 936.
+int group_frames(const nbldpc_code* c, int early_stop) {
+  int per_sm = 0;
+  if (c->q == 16 && c->m <= 50) per_sm = early_stop ? 16 : c->m <= 32 ? 3 : 1;
+  if (c->q == 32) {
+    if (c->m <= 32) per_sm = early_stop ? 1 << 16 : c->n <= 2 * c->m ? 12 : 18;
+    else if (c->m <= 100) per_sm = early_stop ? 36 : 3;
+    else if (c->m < 192) per_sm = early_stop ? 0 : 1;
+  }
+  return per_sm * (c->plan.grid_max / c->plan.per_sm);
+}
+
 // The launch shape of a handle that nobody tuned, for its message width and schedule.
 // Minimal schedule, 8 bits: the resident-message form (384-thread blocks of 1, 2 or 4 frames)
 // where it fits shared memory, otherwise the same layout with the messages in the workspace.
@@ -369,8 +396,15 @@ int configure_default(nbldpc_code* c) {
   const int v = default_variant(c->q), fpb = default_fpb(c);
   if (kmode(c) != 1) return configure(c, v & 1, reg_form(c->q) || v == 0 ? fpb : 1);
   int st = NBLDPC_ERR_UNSUPPORTED;
-  if (reg_form(c->q)) st = configure_reg(c, v);
-  else if (v >= 2) st = configure(c, v, (v & 2) && fpb > 4 && !warp4_code(c) ? 4 : fpb);
+  if (reg_form(c->q)) {
+    st = configure_reg(c, v);
+    if (st == NBLDPC_OK && group_frames(c, 0) + group_frames(c, 1) > 0) {
+      const CodeNeeds need = needs_of(c, v & 1, c->mb);
+      const int st2 = make_plan(c->q, v & 1, 1, fpb, &need, 1, &c->group);
+      if (st2 == NBLDPC_ERR_CUDA) return st2;
+      c->has_group = st2 == NBLDPC_OK;
+    }
+  } else if (v >= 2) st = configure(c, v, (v & 2) && fpb > 4 && !warp4_code(c) ? 4 : fpb);
   return st == NBLDPC_ERR_UNSUPPORTED ? configure(c, v & 1, fpb) : st;
 }
 
@@ -383,7 +417,35 @@ int configure_mode(nbldpc_code* c) {
   return configure(c, v, v == c->variant ? c->plan.fpb : reg_form(c->q) && !c->pinned ? default_fpb(c) : 1);
 }
 
-size_t decode_ws_bytes(const nbldpc_code* c, int frames) { return ws_bytes(c->plan, frames); }
+// The one-block launch shape of a call: a tuning that was set or measured as it is.  An untuned
+// handle's frames share blocks only as long as that leaves three blocks to two SMs (GF(16)
+// N=100, 300 frames 127 us in blocks of one frame, 159 in blocks of four; 10 fixed iterations of
+// 900 frames of N=64 86 us in blocks of one, 60 in blocks of four).
+Plan choose_plan(const nbldpc_code* c, int frames, int early_stop, int* variant) {
+  *variant = c->variant;
+  if (c->has_group && frames <= group_frames(c, early_stop)) {
+    *variant = c->variant & 1;
+    return c->group;
+  }
+  Plan pl = c->plan;
+  if (c->tuned || pl.lanes == 0) return pl;
+  const int sms = pl.grid_max / pl.per_sm;
+  while (pl.fpb > 1 && 2 * frames < 3 * pl.fpb * sms) {
+    pl.fpb /= 2;
+    pl.threads /= 2;
+    pl.smem /= 2;
+    pl.grid_max *= 2;
+  }
+  return pl;
+}
+
+// Enough for `frames` frames and any smaller number, with and without early stop.
+size_t decode_ws_bytes(const nbldpc_code* c, int frames) {
+  size_t most = ws_bytes(c->plan, frames);
+  if (c->has_group)
+    most = std::max(most, ws_bytes(c->group, std::min(frames, std::max(group_frames(c, 0), group_frames(c, 1)))));
+  return most;
+}
 
 nbldpc::JobDesc job_desc(const nbldpc_code* c, const uint8_t* gamma, int frames, int max_iters, int early_stop,
                          uint8_t* sym, int32_t* iters, uint8_t* ok, int item_begin, bool count = true) {
@@ -493,6 +555,9 @@ int split_resident(const nbldpc_code* c, const SplitShape& s) {
 //  - No more 128-thread ranks than the frame has check-node lanes for.
 //  - q <= 8 stays (GF(8) N=512, one frame 83 against 109: the passes are shorter
 //    than the cluster's barriers), but for the 16-bit messages of q = 8.
+//  - GF(16) codes of one 256-thread block per frame keep it (N=64: 75 us against 99 to 110); the
+//    few ranks of short GF(32) codes have a thread per lane up to one frame per SM (N=96 (3,6),
+//    152 frames: 318 us with 128 threads, 245 with 256).
 //  - The register form (q = 16, 32) is fast enough alone from 5/8 frame per SM on at
 //    q = 16 (200 frames of N=1024 351 against 346, of N=444 251 against 284), from
 //    three on at q = 32 (700 frames 1960 against 1985); 3/8 and 5/8 without early stop
@@ -515,7 +580,9 @@ SplitShape split_shape(const nbldpc_code* c, int frames, int early_stop) {
   int size = frames <= sms / 8 ? 16 : 8;
   int threads = frames <= 3 * sms / 8 ? 384 : frames <= 3 * sms / 4 ? 256 : 128;
   size = std::min(size, c->split_max);
+  if (c->has_group && c->q == 16 && c->m * G <= 256) return SplitShape{};
   while (size > 2 && (long long)size * 128 > (long long)c->m * G * 5 / 4) size /= 2;
+  if (c->has_group && size < 8 && threads == 128 && frames <= sms) threads = 256;
   const int cpc = (c->m + size - 1) / size;
   const int pair = c->mb == 1 && c->q >= 128 && frames <= 3 * sms / 8 ? 2 : 1;   // two warps to a check
   threads = std::min(threads, std::max(128, (int)round_up((size_t)cpc * G * pair, 32)));
@@ -535,20 +602,23 @@ int launch_split(const nbldpc_code* c, const SplitShape& s, const nbldpc::JobDes
   return split_launch(split_kernel_for(c->q, c->mb, c->dreg), job.frames, s.size, s.threads, s.smem, &p, st);
 }
 
-// split: small batches may go to the split-frame kernel (not while the autotuner times a tuning)
+// choose: the kernel follows the number of frames (not while the autotuner times a tuning)
 int launch(const nbldpc_code* c, const uint8_t* gamma, int frames, int max_iters, int early_stop, uint8_t* sym,
-           int32_t* iters, uint8_t* ok, void* ws, cudaStream_t st, bool count = true, bool split = true) {
+           int32_t* iters, uint8_t* ok, void* ws, cudaStream_t st, bool count = true, bool choose = true) {
   if (frames == 0) return NBLDPC_OK;
-  if (split) {
+  int variant = c->variant;
+  Plan pl = c->plan;
+  if (choose) {
     const SplitShape s = split_shape(c, frames, early_stop);
     if (s.size) return launch_split(c, s, job_desc(c, gamma, frames, max_iters, early_stop, sym, iters, ok, 0, count), st);
+    pl = choose_plan(c, frames, early_stop, &variant);
   }
   nbldpc::LaunchParamsOf<1> lp{};
   lp.jobs[0] = job_desc(c, gamma, frames, max_iters, early_stop, sym, iters, ok, 0, count);
-  lp.jobs[0].reg = c->plan.lanes;
+  lp.jobs[0].reg = pl.lanes;
   lp.njobs = 1;
   lp.total_items = frames;
-  return launch_plan(kernel_for(c->q, c->variant, kmode(c), c->plan.dreg), c->plan, lp, grid_for(c->plan, frames), ws,
+  return launch_plan(kernel_for(c->q, variant, kmode(c), pl.dreg), pl, lp, grid_for(pl, frames), ws,
                      reinterpret_cast<uint8_t*>(ws) + 256, st);
 }
 
@@ -583,7 +653,8 @@ int nbldpc_decode_noalloc(const nbldpc_code* c, const uint8_t* gamma_dev, int fr
   if (!valid_outputs(gamma_dev, out_sym_dev, out_iters_dev, out_ok_dev)) return NBLDPC_ERR_ARG;
   int st = check_device(c);
   if (st != NBLDPC_OK) return st;
-  const Plan& pl = c->plan;
+  int variant = 0;
+  const Plan pl = choose_plan(c, frames, early_stop, &variant);
   const size_t per_block = (size_t)pl.fpb * pl.slot_bytes;   // 0 when the messages stay in shared memory
   if (256 + per_block > (size_t)NBLDPC_NOALLOC_SCRATCH_BYTES) return NBLDPC_ERR_UNSUPPORTED;
   int grid = grid_for(pl, frames);
@@ -607,7 +678,7 @@ int nbldpc_decode_noalloc(const nbldpc_code* c, const uint8_t* gamma_dev, int fr
   lp.jobs[0].reg = pl.lanes;
   lp.njobs = 1;
   lp.total_items = frames;
-  return launch_plan(kernel_for(c->q, c->variant, kmode(c), pl.dreg), pl, lp, grid, scratch,
+  return launch_plan(kernel_for(c->q, variant, kmode(c), pl.dreg), pl, lp, grid, scratch,
                      reinterpret_cast<uint8_t*>(scratch) + 256,
                      reinterpret_cast<cudaStream_t>(cuda_stream));
 }
@@ -1133,7 +1204,8 @@ int nbldpc_code_autotune(nbldpc_code* c, const uint8_t* gamma_dev, int frames, i
     }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
-  const int st2 = configure(c, st == NBLDPC_OK ? best_v : v_old, st == NBLDPC_OK ? best_f : f_old);
+  const int st2 = st == NBLDPC_OK ? configure(c, best_v, best_f)
+                                  : c->tuned ? configure(c, v_old, f_old) : configure_default(c);
   if (st == NBLDPC_OK && st2 == NBLDPC_OK) c->tuned = true;
   if (n_results) *n_results = count;
   return st != NBLDPC_OK ? st : st2;

@@ -230,3 +230,44 @@ def test_mixed_batch_of_a_code_whose_register_scratch_does_not_fit():
         jobs, keep = batch(specs, 3, early)
         check_batch(specs, jobs, keep, 3, early)
     assert binding.nbldpc_decode_batch_workspace_size(jobs) % (8 * (-(-code.nnz * 32 // 256) * 256)) == 256
+
+
+@pytest.mark.parametrize("q,n,dv,dc", [(8, 64, 2, 4), (16, 64, 2, 4), (16, 100, 2, 4), (16, 128, 2, 8), (32, 64, 2, 4),
+                                       (32, 96, 3, 6), (32, 160, 2, 4), (32, 128, 2, 4)])
+def test_short_codes_at_every_number_of_frames(q, n, dv, dc):
+    """The form and the frames per block of an untuned handle follow the frames of a call: on each side of
+    the limits (cluster limits, frames per SM, the whole chip), through
+    nbldpc_decode and nbldpc_decode_noalloc, the oracle's outputs; a workspace of the largest call
+    serves every smaller one."""
+    code = I.make_regular_code(q, n, dv, dc, seed=q + n)
+    dec = binding.Decoder.from_code(code)
+    frames = [1, sms() // 3, sms(), sms() + 1, 3 * sms(), 3 * sms() + 1, 8 * sms(), 16 * sms(), 16 * sms() + 1, 37 * sms()]
+    need = [binding.nbldpc_decode_workspace_size(dec.handle, f) for f in frames]
+    assert need == sorted(need)
+    g = random_gamma(code, frames[-1], q + n)
+    gd = torch.as_tensor(g).cuda()
+    want = {es: oracle.decode(code, g, 3, es, threads=THREADS) for es in (0, 1)}
+    for f in reversed(frames):
+        for es in (0, 1):
+            got = dec.decode(gd[:f], 3, es)                 # (the workspace of the largest call)
+            for a, w in zip(got, want[es]):
+                assert np.array_equal(a.cpu().numpy(), w[:f]), f"{f} frames, early {es}"
+            out = [torch.empty_like(t) for t in got]
+            binding.nbldpc_decode_noalloc(dec.handle, gd, f, 3, es, *out)
+            for a, b in zip(out, got):
+                assert torch.equal(a, b), f"noalloc: {f} frames, early {es}"
+
+
+def test_short_codes_take_the_group_form_until_the_chip_is_full():
+    """Message slots in the workspace: the group form of GF(16) N=64 and GF(32) N=64.  A GF(16) N=1024
+    code, and a tuning that was set, keep the register form, which has none."""
+    for q in (16, 32):
+        code = I.make_regular_code(q, 64, 2, 4, seed=q + 64)
+        dec = binding.Decoder.from_code(code)
+        slot = -(-code.nnz * q // 256) * 256
+        assert dec.tuning()[0] == 3
+        assert binding.nbldpc_decode_workspace_size(dec.handle, 2 * sms()) == 256 + 2 * sms() * slot
+        dec.set_tuning(*dec.tuning())
+        assert binding.nbldpc_decode_workspace_size(dec.handle, 2 * sms()) == 256
+    dec = binding.Decoder.from_code(I.workload_code("gf16_n1024_dv2_dc4"))
+    assert binding.nbldpc_decode_workspace_size(dec.handle, 5000) == 256
