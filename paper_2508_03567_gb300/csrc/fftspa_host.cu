@@ -178,7 +178,11 @@ FftSplitShape fft_split_layout(const nbldpc_code* c, int size, int threads) {
 //    a half frames per SM; from 1024 on, 3/8 (GF(256) (2,8) N=128, 48 / 96 frames:
 //    519 / 519 against 366 / 550); from 400 on, and in the lane-per-edge form, 1/8
 //    (GF(4) N=1024, 1 / 96 frames: 132 / 130 against 95 / 161), none below (GF(16)
-//    N=100, one frame: 72 against 80).
+//    N=100, one frame: 72 against 80).  A lane of the lane-per-edge form has q products
+//    and sums a pass: from 1024 lanes on at q <= 4 (GF(4) N=48, N=200, N=500, one frame:
+//    39, 44 and 69 against 60, 62 and 66; GF(2) N=200 (3,6) 51 against 72), from 512 on at
+//    GF(8) and GF(16) ((2,12) N=120, 320 lanes: 75 and 98 against 93 and 103; GF(16) N=240, 640
+//    lanes: 165 against 107), any number for wider fields (GF(32) (2,12) N=120: 188 against 126).
 //  - Equal iterations for every frame have no tail to shorten: up to 3/8 frame
 //    per SM (96 frames of GF(64) N=576: 164 against 229), and for q <= 32 between
 //    one frame per SM and four thirds, which the one-block kernel takes in two
@@ -187,19 +191,22 @@ FftSplitShape fft_split_shape(const nbldpc_code* c, int frames, int early_stop) 
   if (c->fft_split_max == 0) return FftSplitShape{};
   const bool lane_form = c->fft_dc == 0;
   const int sms = c->fft_plan.grid_max / c->fft_plan.per_sm;
-  const int lanes = lane_form ? 512 : c->m * (c->q == 256 ? 32 : c->q / 4);
-  if (lanes < 400) return FftSplitShape{};
-  const int few = lanes < 1024 ? sms / 8 : 3 * sms / 8;
-  const bool more = lanes >= 2000 && (early_stop ? frames <= 3 * sms / 2
+  const int lanes = lane_form ? 32 * c->ntasks : c->m * (c->q == 256 ? 32 : c->q / 4);
+  if (lanes < (!lane_form ? 400 : c->q <= 4 ? 1024 : c->q <= 16 ? 512 : 0)) return FftSplitShape{};
+  const int few = lane_form || lanes < 1024 ? sms / 8 : 3 * sms / 8;
+  const bool more = !lane_form && lanes >= 2000 && (early_stop ? frames <= 3 * sms / 2
                                                  : c->q <= 32 && frames > sms && frames <= 4 * sms / 3);
   if (frames > few && !more) return FftSplitShape{};
   int size = frames <= sms / 8 ? 16 : frames <= 3 * sms / 4 ? 8 : 4;
   int threads = c->q == 64 || c->q == 128 ? c->fft_split_threads / 2 : 256;
-  if (lanes < 1024) {
+  if (lane_form || lanes < 1024) {
     size = 8;
     threads = lane_form ? 256 : 128;
   }
+  if (lane_form)
+    while (size > c->ntasks) size /= 2;
   size = std::min(size, c->fft_split_max);
+  if (size < 2) return FftSplitShape{};
   FftSplitShape s = fft_split_layout(c, size, threads);
   while (s.size == 0 && threads > 64) s = fft_split_layout(c, size, threads = (threads - 1) / 64 * 64);
   return s;

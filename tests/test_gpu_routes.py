@@ -271,3 +271,23 @@ def test_short_codes_take_the_group_form_until_the_chip_is_full():
         assert binding.nbldpc_decode_workspace_size(dec.handle, 2 * sms()) == 256
     dec = binding.Decoder.from_code(I.workload_code("gf16_n1024_dv2_dc4"))
     assert binding.nbldpc_decode_workspace_size(dec.handle, 5000) == 256
+
+
+def test_fftspa_clusters_of_the_lane_per_edge_form_follow_the_tasks():
+    """A warp task holds up to 32 edges: short GF(2) and GF(4) codes, whose few tasks leave most ranks
+    without work, keep one block per frame, and no cluster has more blocks than the code has tasks."""
+    for q, n, dv, dc, clusters in ((2, 64, 2, 4, False), (2, 200, 3, 6, False), (4, 48, 2, 4, False),
+                                   (4, 200, 2, 4, False), (4, 1024, 2, 4, True), (2, 1536, 2, 4, True),
+                                   (8, 120, 2, 12, False), (16, 240, 2, 12, True), (64, 192, 2, 12, True)):
+        dec = binding.Decoder.from_code(I.make_regular_code(q, n, dv, dc, seed=q + n))
+        assert (binding.nbldpc_fftspa_cluster_blocks(dec.handle, 1, 1) > 0) == clusters, (q, n, dc)
+    code = irregular(32, 40, 6, 55, 20)            # six checks, one above degree 8: few tasks
+    assert np.diff(code.row_ptr).max() > 8
+    dec = binding.Decoder.from_code(code)
+    assert 2 <= binding.nbldpc_fftspa_cluster_blocks(dec.handle, 1, 1) <= 6
+    p = np.random.default_rng(16).dirichlet(np.full(32, 0.05), (300, code.n)).astype(np.float32) + np.float32(1e-6)
+    pd = torch.as_tensor(p).cuda()
+    ref = dec.fftspa_decode(pd, 4, 0, want_app=True)
+    got = dec.fftspa_decode(pd[:5].contiguous(), 4, 0, want_app=True)
+    for a, b in zip(got, ref):
+        assert torch.equal(a, b[:5])
