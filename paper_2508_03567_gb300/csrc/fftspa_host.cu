@@ -183,8 +183,12 @@ FftSplitShape fft_split_layout(const nbldpc_code* c, int size, int threads) {
 //    39, 44 and 69 against 60, 62 and 66; GF(2) N=200 (3,6) 51 against 72), from 512 on at
 //    GF(8) and GF(16) ((2,12) N=120, 320 lanes: 75 and 98 against 93 and 103; GF(16) N=240, 640
 //    lanes: 165 against 107), any number for wider fields (GF(32) (2,12) N=120: 188 against 126).
-//  - Equal iterations for every frame have no tail to shorten: up to 3/8 frame
-//    per SM (96 frames of GF(64) N=576: 164 against 229), and for q <= 32 between
+//  - Equal iterations for every frame have no tail to shorten, so a second wave of
+//    clusters costs its whole time: 16 ranks up to a tenth of a frame per SM, 8 up to a
+//    quarter, 4 up to 3/8 (one block, these, and 16 / 8 / 8 ranks, 5 iterations: GF(128)
+//    N=128, 19 / 42 / 57 frames 69, 47, 71 / 70, 66, 87 / 70, 70, 91; GF(64) N=256 70, 47,
+//    71 / 71, 63, 87 / 71, 66, 91; GF(256) (2,8) N=128 133, 77, 116 / 133, 105, 145 / 135,
+//    115, 155; below 2000 lanes at q = 128 none past a quarter: N=96 55, 60, 78) (96 frames of GF(64) N=576: 164 against 229), and for q <= 32 between
 //    one frame per SM and four thirds, which the one-block kernel takes in two
 //    waves (200 frames of GF(32) N=600, 5 iterations: 292 against 279).
 FftSplitShape fft_split_shape(const nbldpc_code* c, int frames, int early_stop) {
@@ -199,6 +203,11 @@ FftSplitShape fft_split_shape(const nbldpc_code* c, int frames, int early_stop) 
   if (frames > few && !more) return FftSplitShape{};
   int size = frames <= sms / 8 ? 16 : frames <= 3 * sms / 4 ? 8 : 4;
   int threads = c->q == 64 || c->q == 128 ? c->fft_split_threads / 2 : 256;
+  if (!early_stop && frames <= 3 * sms / 8) {
+    size = frames <= sms / 10 ? 16 : frames <= sms / 4 ? 8 : 4;
+    if (size == 4) threads = 256;
+    if (size == 4 && c->q == 128 && lanes < 2000) return FftSplitShape{};
+  }
   if (lane_form || lanes < 1024) {
     size = 8;
     threads = lane_form ? 256 : 128;

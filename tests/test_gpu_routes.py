@@ -291,3 +291,21 @@ def test_fftspa_clusters_of_the_lane_per_edge_form_follow_the_tasks():
     got = dec.fftspa_decode(pd[:5].contiguous(), 4, 0, want_app=True)
     for a, b in zip(got, ref):
         assert torch.equal(a, b[:5])
+
+
+@pytest.mark.parametrize("q,n,want", [(64, 256, (16, 8, 8, 4, 0)), (128, 128, (16, 8, 8, 4, 0)), (128, 96, (16, 8, 8, 0, 0)),
+                                      (256, 128, (16, 8, 8, 4, 0))])
+def test_fftspa_clusters_of_fixed_iterations_take_one_wave(q, n, want):
+    """Without early stop the frames' clusters run side by side or not at all: the more frames, the fewer
+    blocks; outputs as inside a large batch."""
+    code = I.make_regular_code(q, n, 2, 4, seed=q + n)
+    dec = binding.Decoder.from_code(code)
+    counts = [1, sms() // 8, sms() // 5, sms() // 3, sms() // 2]
+    assert tuple(binding.nbldpc_fftspa_cluster_blocks(dec.handle, f, 0) for f in counts) == want
+    p = np.random.default_rng(q).dirichlet(np.full(q, 0.05), (2 * sms(), code.n)).astype(np.float32) + np.float32(1e-6)
+    pd = torch.as_tensor(p).cuda()
+    ref = dec.fftspa_decode(pd, 3, 0, want_app=True)
+    for f in counts:
+        got = dec.fftspa_decode(pd[:f].contiguous(), 3, 0, want_app=True)
+        for a, b in zip(got, ref):
+            assert torch.equal(a, b[:f])
