@@ -236,10 +236,16 @@ def _ptr(t) -> int:
     return int(t)
 
 
+# the raw handle of a device's current stream: building a Stream object for it costs twice as much of a
+# call of a few microseconds (a private name: without it the object is built)
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream_ptr(stream) -> int:
     if stream is None:
-        # the raw handle: building a Stream object for it costs twice as much of a call of a few microseconds
-        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+        if _raw_stream is not None:
+            return _raw_stream(torch.cuda.current_device())
+        return torch.cuda.current_stream().cuda_stream
     if isinstance(stream, torch.cuda.Stream):
         return stream.cuda_stream
     return int(stream)
