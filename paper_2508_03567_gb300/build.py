@@ -40,6 +40,7 @@ def _units():
     # (the mixed-code kernels call a function per field order: the launch bounds' 80 registers bind those too)
     units = [(os.path.join(CSRC, "kernels.cu"), f"kernels_q{q}.o",
               [f"-DNBLDPC_KQ={q}"] + (["-maxrregcount=80"] if q == 0 else [])) for q in KERNEL_UNITS]
+    units.insert(0, (os.path.join(CSRC, "kernels.cu"), "kernels_q0_wide.o", ["-DNBLDPC_KQ=0", "-DNBLDPC_MIXED_WIDE"]))
     units += [(os.path.join(CSRC, "fftspa.cu"), f"fftspa_q{q}.o", [f"-DNBLDPC_FQ={q}"]) for q in FFT_UNITS]
     units.append((os.path.join(CSRC, "nbldpc.cu"), "nbldpc.o", []))
     units.append((os.path.join(CSRC, "fftspa_host.cu"), "fftspa_host.o", []))

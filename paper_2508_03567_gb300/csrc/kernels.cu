@@ -1,7 +1,8 @@
 // One translation unit per kernel family, so the field orders compile in
 // parallel: built with -DNBLDPC_KQ=q for the two layout variants of field
-// order q (single-code launches), or -DNBLDPC_KQ=0 for the kernel that
-// serves every field order (mixed-code launches).
+// order q (single-code launches), or -DNBLDPC_KQ=0 for the kernels that
+// serve every field order (mixed-code launches; with -DNBLDPC_MIXED_WIDE the one
+// for batches that do not fill the chip).
 #include "mma_kernels.cuh"
 
 #ifndef NBLDPC_KQ
@@ -23,6 +24,10 @@ template <int Q> const void* pruned_kernel(int layout) {
   return nullptr;
 }
 
+#ifdef NBLDPC_MIXED_WIDE
+// Address of the mixed-code kernel for batches that do not fill the chip (two blocks an SM).
+const void* kernel_q0_wide() { return reinterpret_cast<const void*>(&mma_decode_kernel<0, -2, 1>); }
+#else
 // Address of the decode kernel for variant v (bit 0: layout; bit 1: messages
 // resident in shared memory; bit 2: pruned convolutions, layouts of 32-lane
 // groups only, not with bit 1), mb-byte messages and the check-node schedule t1
@@ -93,5 +98,6 @@ const void* NBLDPC_CAT(split_kernel_q, NBLDPC_KQ)(int mb, int dreg) {
 #endif
 }
 #endif
+#endif  // NBLDPC_MIXED_WIDE
 
 }  // namespace nbldpc

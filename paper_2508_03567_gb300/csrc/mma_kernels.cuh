@@ -1655,7 +1655,7 @@ __device__ __forceinline__ void decode_frame(const JobDesc& job, int frame, uint
 // Persistent blocks of fpb frame slots; every slot takes work items (a frame
 // of one job) from a global counter until the list is exhausted.  QSEL = q,
 // VSEL = variant compiles the path of one field order and layout (single-code
-// launches); QSEL = 0, VSEL = -1 compiles every field order (mixed-code launches).
+// launches); QSEL = 0, VSEL = -1 or -2 compiles every field order (mixed-code launches).
 // Resident 256-thread blocks per SM the register allocation must allow: the
 // q >= 128 paths need more than 85 registers per thread without spilling.
 #ifndef NBLDPC_MINB_64
@@ -1670,9 +1670,11 @@ __device__ __forceinline__ void decode_frame(const JobDesc& job, int frame, uint
 #ifndef NBLDPC_MINB_PRUNE
 #define NBLDPC_MINB_PRUNE 3
 #endif
-// The mixed-code kernel (QSEL = 0) has no dense q >= 128 path and fits 80 registers too.
+// The mixed-code kernel (QSEL = 0) has no dense q >= 128 path and comes in two forms: VSEL = -1
+// for batches that fill the chip, three blocks at 80 registers with a function per field order,
+// VSEL = -2 for the others, two blocks with every path in line.
 template <int QSEL, int VSEL> struct MinBlocks {
-  static constexpr int v = QSEL == 0 ? 3 : QSEL >= 128 ? NBLDPC_MINB_WIDE
+  static constexpr int v = QSEL == 0 ? (VSEL == -2 ? 2 : 3) : QSEL >= 128 ? NBLDPC_MINB_WIDE
                          : (QSEL == 64 ? (VSEL == 1 ? 3 : NBLDPC_MINB_64) : 4);
 };
 
@@ -1687,11 +1689,9 @@ struct MixedSlot {
   uint8_t* X;
 };
 
-// A function of its own: in line, the persistent kernel's frame loop kept a dozen registers
-// across every path, and the paths spilled at 80.  It takes offsets, so that its accesses are
-// shared-memory ones.
-template <int Q, bool REG, bool SP, int D = 0>
-__device__ __noinline__ void decode_mixed(MixedSlot m, int frame, int stid, int nthr, int bar_id) {
+// It takes offsets, so that its accesses are shared-memory ones.
+template <int Q, bool REG, bool SP, int D>
+__device__ __forceinline__ void decode_mixed_inline(const MixedSlot& m, int frame, int stid, int nthr, int bar_id) {
   extern __shared__ __align__(16) unsigned char smem[];
   const JobDesc& job = *reinterpret_cast<const JobDesc*>(smem + m.job);
   uint8_t* X = SP ? smem + m.x : m.X;
@@ -1700,27 +1700,43 @@ __device__ __noinline__ void decode_mixed(MixedSlot m, int frame, int stid, int 
       reinterpret_cast<const SplitCtx*>(smem + m.sc));
 }
 
-template <bool SP>
+// As a function: at 80 registers, in line, the persistent kernel's frame loop kept a dozen registers
+// across every path and the paths spilled.  A call costs 5 to 30 % of a frame's time, also without a
+// spill: us per iteration of 20 frames, as a function and in line at 128 registers: GF(8) N=100 3.0
+// and 2.4, GF(32) N=64 4.6 and 3.9, GF(64) N=576 69 and 65, GF(128) N=256 171 and 127, GF(256) (2,8)
+// N=128 132 and 107.
+template <int Q, bool REG, bool SP, int D>
+__device__ __noinline__ void decode_mixed_call(MixedSlot m, int frame, int stid, int nthr, int bar_id) {
+  decode_mixed_inline<Q, REG, SP, D>(m, frame, stid, nthr, bar_id);
+}
+
+template <bool CALL, int Q, bool REG, bool SP, int D = 0>
+__device__ __forceinline__ void decode_mixed(const MixedSlot& m, int frame, int stid, int nthr, int bar_id) {
+  if constexpr (CALL) decode_mixed_call<Q, REG, SP, D>(m, frame, stid, nthr, bar_id);
+  else decode_mixed_inline<Q, REG, SP, D>(m, frame, stid, nthr, bar_id);
+}
+
+template <bool SP, bool CALL>
 __device__ __forceinline__ void decode_any(const JobDesc& job, const MixedSlot& m, int frame, int stid, int nthr,
                                            int bar_id) {
   if constexpr (!SP) {
     if (job.reg) {
-      if (job.q == 64) decode_mixed<64, false, SP, 4>(m, frame, stid, nthr, bar_id);
-      else if (job.q == 8) decode_mixed<8, true, SP>(m, frame, stid, nthr, bar_id);
-      else if (job.q == 16) decode_mixed<16, true, SP>(m, frame, stid, nthr, bar_id);
-      else decode_mixed<32, true, SP>(m, frame, stid, nthr, bar_id);
+      if (job.q == 64) decode_mixed<CALL, 64, false, SP, 4>(m, frame, stid, nthr, bar_id);
+      else if (job.q == 8) decode_mixed<CALL, 8, true, SP>(m, frame, stid, nthr, bar_id);
+      else if (job.q == 16) decode_mixed<CALL, 16, true, SP>(m, frame, stid, nthr, bar_id);
+      else decode_mixed<CALL, 32, true, SP>(m, frame, stid, nthr, bar_id);
       return;
     }
   }
   switch (job.q) {
-    case 2: decode_mixed<2, false, SP>(m, frame, stid, nthr, bar_id); break;
-    case 4: decode_mixed<4, !SP, SP>(m, frame, stid, nthr, bar_id); break;
-    case 8: decode_mixed<8, false, SP>(m, frame, stid, nthr, bar_id); break;
-    case 16: decode_mixed<16, false, SP>(m, frame, stid, nthr, bar_id); break;
-    case 32: decode_mixed<32, false, SP>(m, frame, stid, nthr, bar_id); break;
-    case 64: decode_mixed<64, false, SP>(m, frame, stid, nthr, bar_id); break;
-    case 128: decode_mixed<128, false, SP>(m, frame, stid, nthr, bar_id); break;
-    default: decode_mixed<256, false, SP>(m, frame, stid, nthr, bar_id); break;
+    case 2: decode_mixed<CALL, 2, false, SP>(m, frame, stid, nthr, bar_id); break;
+    case 4: decode_mixed<CALL, 4, !SP, SP>(m, frame, stid, nthr, bar_id); break;
+    case 8: decode_mixed<CALL, 8, false, SP>(m, frame, stid, nthr, bar_id); break;
+    case 16: decode_mixed<CALL, 16, false, SP>(m, frame, stid, nthr, bar_id); break;
+    case 32: decode_mixed<CALL, 32, false, SP>(m, frame, stid, nthr, bar_id); break;
+    case 64: decode_mixed<CALL, 64, false, SP>(m, frame, stid, nthr, bar_id); break;
+    case 128: decode_mixed<CALL, 128, false, SP>(m, frame, stid, nthr, bar_id); break;
+    default: decode_mixed<CALL, 256, false, SP>(m, frame, stid, nthr, bar_id); break;
   }
 }
 
@@ -1777,7 +1793,7 @@ __global__ void __launch_bounds__(XS ? kResidentThreads : 256, XS ? 2 : PR ? NBL
     if constexpr (QSEL != 0)
       decode_frame<Geo<QSEL, VSEL>, MB, T1, PR, XS, D>(job, frame, X, sblob, sblob, chat, scratch, stid, nthr, bar_id);
     else
-      decode_any<false>(*sjob,
+      decode_any<false, VSEL == -1>(*sjob,
                         MixedSlot{(int)(reinterpret_cast<unsigned char*>(sjob) - smem), (int)(sblob - smem),
                                   (int)(chat - smem), (int)(scratch - smem), 0, 0, X},
                         frame, stid, nthr, bar_id);
@@ -1875,7 +1891,7 @@ __global__ void __launch_bounds__(kResidentThreads, 2) mma_split_batch_kernel(co
   split_setup(job, lay, frame, rank, p.size, job.q, job.q, smem, sc);
   if (threadIdx.x == 0) *reinterpret_cast<SplitCtx*>(smem + p.sc_off) = sc;
   __syncthreads();
-  decode_any<true>(*sjob, MixedSlot{p.job_off, 0, lay.chat_off, lay.scratch_off, lay.x_off, p.sc_off, nullptr}, frame,
+  decode_any<true, true>(*sjob, MixedSlot{p.job_off, 0, lay.chat_off, lay.scratch_off, lay.x_off, p.sc_off, nullptr}, frame,
                    threadIdx.x, blockDim.x, 1);
 }
 

@@ -53,6 +53,7 @@ bool build_field(int q, uint32_t poly, std::vector<uint8_t>& exp2, std::vector<u
 
 namespace nbldpc {   // defined in kernels.cu, one translation unit per field order
 const void* kernel_q0(int v, int mb, int t1, int dreg);
+const void* kernel_q0_wide();
 const void* kernel_q2(int v, int mb, int t1, int dreg);
 const void* kernel_q4(int v, int mb, int t1, int dreg);
 const void* kernel_q8(int v, int mb, int t1, int dreg);
@@ -80,11 +81,11 @@ int kmode(const nbldpc_code* c) { return c->mb == 2 ? 2 : (c->cnp_schedule == NB
 // resident in shared memory; bit 2: pruned convolutions), kernel mode and the
 // code's regular check degree (dreg: 0 when the rows differ, -1 for a register form
 // with fewer lanes than threads; a field order may have a kernel for it), or for every
-// field order (q = 0, mode 1)
+// field order (q = 0, mode 1; v = -1 at three blocks an SM, -2 at two)
 const void* kernel_for(int q, int v, int km, int dreg = 0) {
   const int mb = km == 2 ? 2 : 1, t1 = km == 3 ? 1 : 0;
   switch (q) {
-    case 0: return nbldpc::kernel_q0(-1, mb, t1, 0);
+    case 0: return v == -2 ? nbldpc::kernel_q0_wide() : nbldpc::kernel_q0(-1, mb, t1, 0);
     case 2: return nbldpc::kernel_q2(v, mb, t1, dreg);
     case 4: return nbldpc::kernel_q4(v, mb, t1, dreg);
     case 8: return nbldpc::kernel_q8(v, mb, t1, dreg);
@@ -151,13 +152,13 @@ int group_bytes(int q, int dmax, int mb, bool pr) {
 
 // Every kernel may use up to the opt-in shared memory of the device (set once
 // per device and kernel; occupancy still follows the bytes of each launch).
-bool g_attr_done[64][88] = {};
+bool g_attr_done[64][89] = {};
 
 // per field order: 3 kernel modes x 2 layouts, the 2 resident-message kernels,
 // then the 2 pruned-convolution kernels; after them the 2 GF(64) and the 2 GF(4)
 // resident kernels of check degree 4 and the GF(8), GF(16), GF(32) ones of few lanes
 int kernel_slot(int q, int v, int km, int dreg) {
-  if (q == 0) return 0;
+  if (q == 0) return v == -2 ? 88 : 0;
   if (kernel_dreg(q, v, km, dreg)) return (q == 64 ? 81 : 83) + (v & 1);
   if (dreg < 0) return 85 + nbldpc::ilog2(q) - 3;
   return 1 + 10 * (nbldpc::ilog2(q) - 1) + ((v & 4) ? 8 + (v & 1) : (v & 2) ? 6 + (v & 1) : 2 * (km - 1) + (v & 1));
@@ -995,9 +996,11 @@ static int batch_plan(const nbldpc_job* jobs, int n_jobs, Plan* pl, int* total) 
   *total = (int)t;
   // few frames: a block each (GF(4) N=48 and GF(8) N=100, 200 frames each: 100 us at two a block, 92 at one),
   // unless a code's frames per block are pinned
-  const Plan& pl0 = jobs[0].code->plan;
+  const nbldpc_code* c0 = jobs[0].code;
+  const Plan& pl0 = c0->plan;
   if (t <= 3LL * (pl0.grid_max / pl0.per_sm) && !any_pinned(jobs, n_jobs)) fpb = 1;
-  return make_plan(0, -1, 1, fpb, need, n_jobs, pl);
+  const int st = prepare_kernel(0, -2, 1, 0, c0->device, c0->smem_optin);
+  return st != NBLDPC_OK ? st : make_plan(0, -1, 1, fpb, need, n_jobs, pl);
 }
 
 // Shape of a mixed batch whose frames are each decoded on a cluster (size 0: one block per frame
@@ -1056,6 +1059,37 @@ static int batch_split(const nbldpc_job* jobs, int n_jobs, int total, const Plan
     return size;
   }
   return 0;
+}
+
+// Whether a mixed batch takes the two-block kernel with its paths in line.  It decodes a frame 5 to 30 %
+// sooner (see decode_mixed_call), the three-block kernel has more of them side by side; three to a
+// block of rounds (frame slots of three blocks an SM), measured on GB300, us per batch, two against
+// three blocks:
+//  - With early stop the last frames decide until the chip has been full six times over: GF(64) N=576,
+//    1,100 / 1,400 / 6,000 frames 4,406 / 5,520 / 19,957 against 4,537 / 5,686 / 19,672; GF(64) N=88,
+//    N=522 and N=232, 2,123 in all 2,340 against 2,791; GF(256) N=384, 2,000 39.4 against 39.2 ms; 532
+//    of GF(16) N=716, GF(64) N=126 and others 1,333 against 1,541.
+//  - Fields up to GF(8) gain little from it: where their rounds are not fewer than four thirds of the
+//    other kernel's, the third block wins (GF(8) (3,6) N=580, 361 frames 220 against 164; GF(2) N=534,
+//    1,290 697 against 612; 20 of GF(16) N=64 and 30 of GF(8) N=100 64 against 78).
+//  - Fixed iterations: up to two and a half frames per SM (GF(64) N=576, 300 frames 939 against 979; 399
+//    of four GF(64) codes 649 against 730; GF(256) N=177, 416 2,982 against 2,588), and for GF(128) and
+//    GF(256) where rounds allow (GF(256) N=384, 600 frames 6,973 against 8,427).
+static bool batch_wide(const nbldpc_job* jobs, int n_jobs, int total, const Plan& pl) {
+  bool stop = true;
+  double small = 0.0, middle = 0.0, large = 0.0;     // work of the fields up to GF(8), up to GF(64), above
+  for (int i = 0; i < n_jobs; ++i) {
+    if (jobs[i].frames == 0) continue;
+    stop = stop && jobs[i].early_stop;
+    const int q = jobs[i].code->q;
+    (q <= 8 ? small : q <= 64 ? middle : large) += jobs[i].frames * frame_work(jobs[i]);
+  }
+  const long long want = (total + pl.fpb - 1) / pl.fpb, sms = pl.grid_max / pl.per_sm;
+  const long long two = (want + 2 * sms - 1) / (2 * sms), three = (want + pl.grid_max - 1) / pl.grid_max;
+  const bool fewer = three <= 3 && 3 * two < 4 * three;
+  if (small > middle + large) return fewer;
+  if (stop) return three <= 6;
+  return 2 * want <= 5 * sms || (large > middle + small && fewer);
 }
 
 int nbldpc_decode_batch_workspace_size(const nbldpc_job* jobs, int n_jobs, size_t* bytes) {
@@ -1128,7 +1162,9 @@ int nbldpc_decode_batch(const nbldpc_job* jobs, int n_jobs, void* workspace_dev,
     const bool fills = 2 * c->m >= nthr || total > pl.grid_max * pl.fpb;
     lp.jobs[i].reg = (pl.mixed_reg && mixed_reg(c->q, nthr, c->dmax) && fills) || (c->q == 64 && c->dreg == 4) ? nthr : 0;
   }
-  return launch_plan(kernel_for(0, -1, 1), pl, lp, grid_for(pl, total), workspace_dev,
+  const bool wide = batch_wide(jobs, n_jobs, total, pl);
+  const int grid = std::min(grid_for(pl, total), wide ? 2 * (pl.grid_max / pl.per_sm) : pl.grid_max);
+  return launch_plan(kernel_for(0, wide ? -2 : -1, 1), pl, lp, grid, workspace_dev,
                      reinterpret_cast<uint8_t*>(workspace_dev) + 256, reinterpret_cast<cudaStream_t>(cuda_stream));
 }
 

@@ -309,3 +309,21 @@ def test_fftspa_clusters_of_fixed_iterations_take_one_wave(q, n, want):
         got = dec.fftspa_decode(pd[:f].contiguous(), 3, 0, want_app=True)
         for a, b in zip(got, ref):
             assert torch.equal(a, b[:f])
+
+
+@pytest.mark.parametrize("early,per_sm", [(1, 1), (1, 5), (1, 30), (0, 2), (0, 3), (0, 9)])
+@pytest.mark.parametrize("family", ["all", "small", "wide"])
+def test_mixed_batches_on_both_one_block_kernels(family, early, per_sm):
+    """Frames per SM on each side of the limits between the two-block kernel (paths in line) and the
+    three-block one (a function per field order), for the mixes that have limits of their own; ragged
+    codes below the sizes that take clusters, several frames to a slot at the largest."""
+    fields = {"all": (2, 4, 8, 16, 32, 64, 128, 256), "small": (2, 4, 8), "wide": (128, 256)}[family]
+    frames = per_sm * sms() // len(fields) + 1
+    specs = []
+    for q in fields:
+        n, m, dmax = (24, 9, 6) if q >= 128 else (40, 19, 4) if q == 64 else (61, 31, 6)
+        code = irregular(q, n, m, 5 * q, dmax)
+        specs.append((code, random_gamma(code, frames, q + per_sm)))
+    jobs, keep = batch(specs, 3, early, lambda k, dec: dec.set_tuning(0, 1 + (per_sm > 9)) if k == 0 else None)
+    assert binding.nbldpc_decode_batch_cluster_blocks(jobs) == 0
+    check_batch(specs, jobs, keep, 3, early)
