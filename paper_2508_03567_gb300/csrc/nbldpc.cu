@@ -952,14 +952,29 @@ int nbldpc_decode_cluster_blocks(const nbldpc_code* c, int frames, int early_sto
 }
 
 // ---- mixed-code batches -----------------------------------------------------
-// Frame slots per block that suit a code in the mixed-code kernel: the pinned count, or (register
-// form) enough threads per slot for the checks, or the group form's default.
-static int batch_fpb(const nbldpc_code* c) {
-  if (c->pinned) return c->plan.fpb;
-  if (!reg_form(c->q)) return c->plan.fpb;
+// Frame slots per block with enough threads each for a check a thread.
+static int reg_fpb(const nbldpc_code* c) {
   int fpb = 1;
   while (fpb < 8 && kThreads / (2 * fpb) >= std::max(32, c->m)) fpb *= 2;
   return fpb;
+}
+
+// Whether a job may take the register form in the mixed-code kernels: GF(32) codes of up to 100 checks
+// for more frames than an untuned handle decodes in the group form, and with a check for four fifths
+// of the lanes (1,000 frames of GF(32) N=64 and 2,000 of GF(4) N=100: 416 us against 265; 2,106 of
+// (2,8) N=280, 70 checks on 128 lanes, fixed iterations 2,011 against 1,608).
+static bool batch_reg(const nbldpc_job& j) {
+  const nbldpc_code* c = j.code;
+  if (!reg_form(c->q)) return false;
+  return c->q != 32 || c->m > 100 ||
+         (j.frames > group_frames(c, j.early_stop) && 5 * c->m > 4 * (kThreads / reg_fpb(c)));
+}
+
+// Frame slots per block that suit a job in the mixed-code kernels: the pinned count, or (register
+// form) enough threads per slot for the checks, or the group form's default.
+static int batch_fpb(const nbldpc_job& j) {
+  if (j.code->pinned || !reg_form(j.code->q)) return j.code->plan.fpb;
+  return batch_reg(j) ? reg_fpb(j.code) : default_fpb(j.code);
 }
 
 // Convolution work of a frame's longest decode (pruned convolutions as a tenth).
@@ -989,7 +1004,7 @@ static int batch_plan(const nbldpc_job* jobs, int n_jobs, Plan* pl, int* total) 
     if (kmode(c) != 1) return NBLDPC_ERR_UNSUPPORTED;   // mixed-code launches: 8-bit messages, minimal schedule
     need[i] = needs_of(c, mixed_layout(c->q), 1);
     need[i].blob = c->off.edge_col;   // the mixed-code kernel stages no edge_col or variable-node view
-    fpb = std::min(fpb, batch_fpb(c));
+    fpb = std::min(fpb, batch_fpb(jobs[i]));
     t += jobs[i].frames;
   }
   if (t > 0x7FFFFFFF) return NBLDPC_ERR_ARG;
@@ -1160,7 +1175,8 @@ int nbldpc_decode_batch(const nbldpc_job* jobs, int n_jobs, void* workspace_dev,
     // frames fill the SM (100 frames of GF(32) N=64 and 200 of GF(4) N=100: 312 us against 109)
     const int nthr = pl.threads / pl.fpb;
     const bool fills = 2 * c->m >= nthr || total > pl.grid_max * pl.fpb;
-    lp.jobs[i].reg = (pl.mixed_reg && mixed_reg(c->q, nthr, c->dmax) && fills) || (c->q == 64 && c->dreg == 4) ? nthr : 0;
+    const bool reg = pl.mixed_reg && mixed_reg(c->q, nthr, c->dmax) && fills && batch_reg(jobs[i]);
+    lp.jobs[i].reg = reg || (c->q == 64 && c->dreg == 4) ? nthr : 0;
   }
   const bool wide = batch_wide(jobs, n_jobs, total, pl);
   const int grid = std::min(grid_for(pl, total), wide ? 2 * (pl.grid_max / pl.per_sm) : pl.grid_max);

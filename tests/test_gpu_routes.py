@@ -224,11 +224,10 @@ def test_mixed_batch_of_a_code_whose_register_scratch_does_not_fit():
     does not fit eight times, the group form's does, and the batch takes it."""
     code = one_heavy_check(32, 34, 32, 7, heavy=34)
     assert code.m == 32 and np.diff(code.row_ptr).max() == 34
-    frames = 4 * sms()
+    frames = 13 * sms()                             # more than the group form is taken for anyway
     specs = [(code, random_gamma(code, frames, 8))]
-    for early in (0, 1):
-        jobs, keep = batch(specs, 3, early)
-        check_batch(specs, jobs, keep, 3, early)
+    jobs, keep = batch(specs, 3, 0)
+    check_batch(specs, jobs, keep, 3, 0)
     assert binding.nbldpc_decode_batch_workspace_size(jobs) % (8 * (-(-code.nnz * 32 // 256) * 256)) == 256
 
 
@@ -327,3 +326,14 @@ def test_mixed_batches_on_both_one_block_kernels(family, early, per_sm):
     jobs, keep = batch(specs, 3, early, lambda k, dec: dec.set_tuning(0, 1 + (per_sm > 9)) if k == 0 else None)
     assert binding.nbldpc_decode_batch_cluster_blocks(jobs) == 0
     check_batch(specs, jobs, keep, 3, early)
+
+
+@pytest.mark.parametrize("early", [0, 1])
+@pytest.mark.parametrize("n,dc,per_sm", [(64, 4, 2), (64, 4, 13), (128, 4, 2), (128, 4, 4), (280, 8, 4)])
+def test_mixed_batches_of_short_gf32_codes(n, dc, per_sm, early):
+    """Group form and register form of GF(32) in a mixed batch (32, 64 and 70 checks), on each side of the
+    limits in frames, beside a GF(4) code that shares the frame slots: the oracle's outputs."""
+    codes = [I.make_regular_code(32, n, 2, dc, seed=32 + n), irregular(4, 61, 31, 20, 6)]
+    specs = [(c, random_gamma(c, per_sm * sms() + 1, n + dc)) for c in codes]
+    jobs, keep = batch(specs, 2, early)
+    check_batch(specs, jobs, keep, 2, early)
