@@ -337,3 +337,18 @@ def test_mixed_batches_of_short_gf32_codes(n, dc, per_sm, early):
     specs = [(c, random_gamma(c, per_sm * sms() + 1, n + dc)) for c in codes]
     jobs, keep = batch(specs, 2, early)
     check_batch(specs, jobs, keep, 2, early)
+
+
+def test_mixed_batches_leave_the_clusters_where_frames_fill_the_chip():
+    """Frames per SM up to which a batch of one code decodes on clusters, by field, check-node lanes and check
+    degree."""
+    for q, n, dv, dc, per_sm in ((16, 1024, 2, 4, 0.625), (32, 600, 3, 6, 2), (32, 128, 2, 4, 0.75), (64, 576, 2, 4, 4),
+                                 (64, 160, 2, 4, 1.5), (128, 256, 2, 4, 3), (256, 192, 2, 4, 3), (256, 192, 2, 6, 2.5),
+                                 (256, 280, 2, 8, 1.5)):
+        code = I.make_regular_code(q, n, dv, dc, seed=q + n, encoder=False)
+        dec = binding.Decoder.from_code(code)
+        for frames, cluster in ((int(per_sm * sms()), True), (int(per_sm * sms()) + 1, False)):
+            job = (dec.handle, None, frames, 10, 1, None, None, None)
+            assert (binding.nbldpc_decode_batch_cluster_blocks([job]) > 0) == cluster, (q, n, dc, frames)
+            job = (dec.handle, None, frames, 10, 0, None, None, None)
+            assert (binding.nbldpc_decode_batch_cluster_blocks([job]) > 0) == (frames <= 3 * sms() // 8)
