@@ -1020,15 +1020,16 @@ static int batch_plan(const nbldpc_job* jobs, int n_jobs, Plan* pl, int* total) 
 
 // Shape of a mixed batch whose frames are each decoded on a cluster (size 0: one block per frame
 // slot): the ranks and threads of split_shape, the jobs' layouts one over the other.  Frames count
-// by their work against the longest ones' (an eighth at least): one block per frame ends with the
-// longest frames alone.  Taken with early stop (the serving loop's groups) up to a number of such
-// frames per SM that follows the widest field: q = 16 5/8; q = 32 two, below 1400 check-node lanes 3/4;
+// by their work against the longest ones' (an eighth at least; whole for q <= 8, which a cluster does not
+// shorten: 565 frames of GF(8) and GF(4) codes and 5 of GF(32) N=728 647 us on clusters, 358 on one block
+// each; 53 of GF(8) and 57 of GF(16) 195 and 132): one block per frame ends with the longest frames
+// alone.  Taken with early stop (the serving loop's groups) up to a number of such frames per SM that follows the widest field: q = 16 5/8; q = 32 two, below 1400 check-node lanes 3/4;
 // q = 64 four and q = 128 three, below 1400 lanes one and a half; q = 256 three, two and a half above
 // check degree 4 and one and a half from 8 on; without early stop 3/8; and eight frames of any kind.  Not
 // for q <= 8 alone, nor past 3/8 where the longest frames have fewer than 1024 lanes, nor there for
 // q <= 32 at all (and no more 128-thread ranks than lanes).  Measured on GB300, us per batch, the faster
-// one-block kernel against this: 60 / 240 / 450 frames of GF(64) N=576, GF(16) N=1024 and GF(256) N=128 in equal parts 2746 /
-// 3455 / 3878 against 795 / 1444 / 2399; one frame of GF(64) 1243 against 179; 580 of GF(64) 2854
+// one-block kernel against this: 60 / 240 / 450 frames of GF(64) N=576, GF(16) N=1024 and GF(256) N=128
+// in equal parts 2746 / 3455 / 3878 against 795 / 1444 / 2399; one frame of GF(64) 1243 against 179; 580 of GF(64) 2854
 // against 2558; beyond the limits 823 of GF(32) N=716 1100 against 1421, 947 of GF(128) N=138 1582
 // against 2020, 263 of GF(256) (2,8) N=280 3132 against 4940, 213 of two GF(32) codes of 1184 lanes
 // 300 against 372.
@@ -1052,7 +1053,8 @@ static int batch_split(const nbldpc_job* jobs, int n_jobs, int total, const Plan
     }
   if (q_most <= 8 || total > 8 * sms) return 0;
   for (int i = 0; i < n_jobs; ++i)
-    like_longest += jobs[i].frames * std::max(0.125, longest > 0.0 ? frame_work(jobs[i]) / longest : 1.0);
+    like_longest += jobs[i].frames *
+                    (jobs[i].code->q <= 8 ? 1.0 : std::max(0.125, longest > 0.0 ? frame_work(jobs[i]) / longest : 1.0));
   const int most_frames = !stop          ? 3 * sms / 8
                           : q_most <= 16  ? 5 * sms / 8
                           : q_most <= 32  ? (lanes < 1400 ? 3 * sms / 4 : 2 * sms)

@@ -352,3 +352,16 @@ def test_mixed_batches_leave_the_clusters_where_frames_fill_the_chip():
             assert (binding.nbldpc_decode_batch_cluster_blocks([job]) > 0) == cluster, (q, n, dc, frames)
             job = (dec.handle, None, frames, 10, 0, None, None, None)
             assert (binding.nbldpc_decode_batch_cluster_blocks([job]) > 0) == (frames <= 3 * sms() // 8)
+
+
+def test_frames_of_small_fields_do_not_take_clusters_for_the_sake_of_a_few():
+    """A few GF(32) or GF(16) frames among many of GF(8): one block per frame; the same few alone, and a few of
+    both, on clusters."""
+    codes = [I.workload_code("gf16_n1024_dv2_dc4"), irregular(8, 70, 33, 41, 6)]
+    decs = [binding.Decoder.from_code(c) for c in codes]
+    for counts, cluster in (((5, 0), True), ((5, 30), True), ((sms() // 3, sms() // 3), False), ((5, 2 * sms()), False)):
+        jobs = [(d.handle, None, f, 4, 1, None, None, None) for d, f in zip(decs, counts)]
+        assert (binding.nbldpc_decode_batch_cluster_blocks(jobs) > 0) == cluster, counts
+    specs = [(c, random_gamma(c, f, f)) for c, f in zip(codes, (5, 2 * sms()))]
+    jobs, keep = batch(specs, 4, 1)
+    check_batch(specs, jobs, keep, 4, 1)
