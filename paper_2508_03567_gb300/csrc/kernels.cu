@@ -34,7 +34,8 @@ const void* kernel_q0_wide() { return reinterpret_cast<const void*>(&mma_decode_
 // (1: Table 1's 3 d_c - 4 convolutions, 8-bit messages only) of this unit's
 // field order; dreg: the code's check degree when all are equal (GF(4) and
 // GF(64) have resident-message kernels for degree 4), else 0, or -1 for the register form
-// with fewer lanes than threads; null when there is none.
+// with fewer lanes than threads, -1 or -4 for GF(4) codes that a warp decodes alone; null
+// when there is none.
 const void* NBLDPC_CAT(kernel_q, NBLDPC_KQ)(int v, int mb, int t1, int dreg) {
   (void)dreg;
 #if NBLDPC_KQ == 0
@@ -47,6 +48,11 @@ const void* NBLDPC_CAT(kernel_q, NBLDPC_KQ)(int v, int mb, int t1, int dreg) {
   }
   if (v >= 2) {
     if (mb != 1 || t1) return nullptr;
+#if NBLDPC_KQ == 4
+    if (dreg < 0)    // the one-warp form alone
+      return dreg == -4 ? reinterpret_cast<const void*>(&mma_decode_kernel<4, 0, 1, false, true, false, -4>)
+                        : reinterpret_cast<const void*>(&mma_decode_kernel<4, 0, 1, false, true, false, -1>);
+#endif
 #if NBLDPC_KQ == 64 || NBLDPC_KQ == 4
     // every check of degree 4 (the regular (2,4) codes): a compile-time check degree
     if (dreg == 4)

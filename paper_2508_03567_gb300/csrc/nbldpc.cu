@@ -80,7 +80,7 @@ int kmode(const nbldpc_code* c) { return c->mb == 2 ? 2 : (c->cnp_schedule == NB
 // kernel compiled for one field order, variant (bit 0: layout; bit 1: messages
 // resident in shared memory; bit 2: pruned convolutions), kernel mode and the
 // code's regular check degree (dreg: 0 when the rows differ, -1 for a register form
-// with fewer lanes than threads; a field order may have a kernel for it), or for every
+// with fewer lanes than threads, -1 or -4 for a GF(4) code in the one-warp form; a field order may have a kernel for it), or for every
 // field order (q = 0, mode 1; v = -1 at three blocks an SM, -2 at two)
 const void* kernel_for(int q, int v, int km, int dreg = 0) {
   const int mb = km == 2 ? 2 : 1, t1 = km == 3 ? 1 : 0;
@@ -152,7 +152,7 @@ int group_bytes(int q, int dmax, int mb, bool pr) {
 
 // Every kernel may use up to the opt-in shared memory of the device (set once
 // per device and kernel; occupancy still follows the bytes of each launch).
-bool g_attr_done[64][89] = {};
+bool g_attr_done[64][91] = {};
 
 // per field order: 3 kernel modes x 2 layouts, the 2 resident-message kernels,
 // then the 2 pruned-convolution kernels; after them the 2 GF(64) and the 2 GF(4)
@@ -160,7 +160,7 @@ bool g_attr_done[64][89] = {};
 int kernel_slot(int q, int v, int km, int dreg) {
   if (q == 0) return v == -2 ? 88 : 0;
   if (kernel_dreg(q, v, km, dreg)) return (q == 64 ? 81 : 83) + (v & 1);
-  if (dreg < 0) return 85 + nbldpc::ilog2(q) - 3;
+  if (dreg < 0) return q == 4 ? (dreg == -4 ? 90 : 89) : 85 + nbldpc::ilog2(q) - 3;
   return 1 + 10 * (nbldpc::ilog2(q) - 1) + ((v & 4) ? 8 + (v & 1) : (v & 2) ? 6 + (v & 1) : 2 * (km - 1) + (v & 1));
 }
 
@@ -201,11 +201,17 @@ struct CodeNeeds {       // what one code asks of a frame slot
   size_t msg;
   int dreg;              // regular check degree (0: the rows differ)
   int m;
+  bool warp4;            // a GF(4) code that one warp decodes alone
 };
+
+// GF(4) codes a single warp decodes alone (one-warp frame slots: at most 32
+// checks of degree <= 4, columns of degree <= 2): GF(4) N=48 (2,4) 17-18 us per
+// 1,000-frame decode at 8 frames per block against 24.5 at 4.
+bool warp4_code(const nbldpc_code* c) { return c->q == 4 && c->m <= 32 && c->dmax <= 4 && c->vmax <= 2; }
 
 CodeNeeds needs_of(const nbldpc_code* c, int variant, int mb) {
   return CodeNeeds{c->q, variant, mb, c->dmax, c->off.perm, c->off.bytes - c->off.perm, c->n,
-                   round_up((size_t)c->nnz * c->q * mb, 256), c->dreg, c->m};
+                   round_up((size_t)c->nnz * c->q * mb, 256), c->dreg, c->m, warp4_code(c)};
 }
 
 // Field orders whose resident-message kernels take the register form of the check-node
@@ -290,7 +296,9 @@ int make_plan(int kq, int kv, int km, int fpb, const CodeNeeds* cs, int nc, Plan
   }
   pl.smem = fpb * pl.slot_smem;
   if (pl.smem > optin) return NBLDPC_ERR_UNSUPPORTED;
-  const int dreg = pl.dreg = reg ? (pl.lanes < nthr ? -1 : 0) : (kq != 0 && nc == 1) ? cs[0].dreg : 0;
+  const bool w4 = kq == 4 && resident && nthr == 32 && cs[0].warp4;
+  const int dreg = pl.dreg = reg ? (pl.lanes < nthr ? -1 : 0)
+                             : w4 ? (cs[0].dreg == 4 ? -4 : -1) : (kq != 0 && nc == 1) ? cs[0].dreg : 0;
   int st = prepare_kernel(kq, kv, km, dreg, dev, optin);
   if (st != NBLDPC_OK) return st;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pl.per_sm, kernel_for(kq, kv, km, dreg), pl.threads, pl.smem) !=
@@ -309,11 +317,6 @@ int make_plan(int kq, int kv, int km, int fpb, const CodeNeeds* cs, int nc, Plan
 // 2.8x the dense kernel; GF(128) (2,4) N=256: 35.6 against 41.1 ms); otherwise
 // layout 0).
 int default_variant(int q) { return q >= 128 ? 4 : (q >= 16 && q <= 64) ? 3 : q >= 4 ? 2 : 0; }
-
-// GF(4) codes a single warp decodes alone (one-warp frame slots: at most 32
-// checks of degree <= 4, columns of degree <= 2): GF(4) N=48 (2,4) 17-18 us per
-// 1,000-frame decode at 8 frames per block against 24.5 at 4.
-bool warp4_code(const nbldpc_code* c) { return c->q == 4 && c->m <= 32 && c->dmax <= 4 && c->vmax <= 2; }
 
 // Frame slots per block when nothing better is known: enough threads per slot
 // for the checks and variable nodes of one frame, at least one warp.

@@ -365,3 +365,23 @@ def test_frames_of_small_fields_do_not_take_clusters_for_the_sake_of_a_few():
     specs = [(c, random_gamma(c, f, f)) for c, f in zip(codes, (5, 2 * sms()))]
     jobs, keep = batch(specs, 4, 1)
     check_batch(specs, jobs, keep, 4, 1)
+
+
+def test_gf4_codes_at_eight_frames_per_block():
+    """One warp per frame: regular and ragged codes that the one-warp kernels serve (up to 32 checks of degree
+    <= 4, columns of degree <= 2), and the nearest codes that they do not (33 checks, degree 5, a column of
+    degree 3): the oracle's outputs at few and many frames."""
+    ragged = [irregular(4, 61, 32, 9, 4), irregular(4, 61, 33, 9, 4), irregular(4, 61, 30, 10, 5)]
+    assert [(c.m, int(np.diff(c.row_ptr).max())) for c in ragged] == [(32, 4), (33, 4), (30, 5)]
+    codes = [I.workload_code("gf4_n48_dv2_dc4"), *ragged, I.make_regular_code(4, 60, 3, 6, seed=64)]
+    assert [int(np.bincount(c.col_idx).max()) for c in codes] == [2, 2, 2, 2, 3]
+    for code in codes:
+        dec = binding.Decoder.from_code(code)
+        g = random_gamma(code, 9 * sms(), code.n + code.m)
+        gd = torch.as_tensor(g).cuda()
+        for v in (2, 3):
+            dec.set_tuning(v, 8)
+            for frames, iters, early in ((1, 5, 1), (13, 2, 0), (9 * sms(), 3, 1), (9 * sms(), 0, 0)):
+                want = oracle.decode(code, g[:frames], iters, early, threads=THREADS)
+                for a, w in zip(dec.decode(gd[:frames].contiguous(), iters, early), want):
+                    assert np.array_equal(a.cpu().numpy(), w), (code.m, v, frames)
