@@ -511,6 +511,9 @@ struct SplitShape {
   nbldpc::SplitLayout lay{};
 };
 
+// What a rank of a mixed batch keeps behind its sections (its job and SplitCtx).
+constexpr size_t kSplitTail = (sizeof(nbldpc::JobDesc) + 15) / 16 * 16 + (sizeof(nbldpc::SplitCtx) + 15) / 16 * 16;
+
 // Lay out a rank's shared memory; size 0 when it does not fit the device.
 SplitShape split_layout(const nbldpc_code* c, int size, int threads) {
   SplitShape s;
@@ -519,16 +522,24 @@ SplitShape split_layout(const nbldpc_code* c, int size, int threads) {
   s.lay.npc = (c->n + size - 1) / size;
   const long long edges_r = std::min<long long>(c->nnz, (long long)s.lay.cpc * c->dmax);
   const long long edges_n = std::min<long long>(c->nnz, (long long)s.lay.npc * c->vmax);
-  // every section on a 128-byte line, all banks: where the scratch of two groups of a warp starts in
-  // the middle of one, their vectors meet in the banks (GF(32) (3,6) N=600, 25 frames: 345 us, 335 on lines)
-  size_t o = round_up((size_t)c->off.perm, 128);
-  auto take = [&](size_t bytes) { const size_t at = o; o = round_up(o + bytes, 128); return (int)at; };
-  s.lay.chat_off = take((size_t)c->n);
-  s.lay.flag_off = take(2 * nbldpc::kMaxSplit * sizeof(int));
-  s.lay.row_off = take((size_t)edges_n * sizeof(void*));
-  s.lay.gam_off = take((size_t)s.lay.npc * c->q);
-  s.lay.scratch_off = take((size_t)(threads / G) * group_bytes(c->q, c->dmax, c->mb, c->mb == 1 && c->q >= 128));
-  s.lay.x_off = take((size_t)edges_r * c->q * c->mb);
+  // Every section on a 128-byte line, all banks, unless the padding costs a resident block: where the
+  // scratch of two groups of a warp starts in the middle of a line, their vectors meet in the banks (GF(32)
+  // (3,6) N=600, 25 frames: 345 us, 335 on lines; but 225 frames of GF(256) (2,8) N=156 and 9 of N=280 in
+  // one batch 5,040 us with three blocks an SM, 3,767 with four).
+  auto lay_out = [&](size_t line) {
+    size_t o = round_up((size_t)c->off.perm, line);
+    auto take = [&](size_t bytes) { const size_t at = o; o = round_up(o + bytes, line); return (int)at; };
+    s.lay.chat_off = take((size_t)c->n);
+    s.lay.flag_off = take(2 * nbldpc::kMaxSplit * sizeof(int));
+    s.lay.row_off = take((size_t)edges_n * sizeof(void*));
+    s.lay.gam_off = take((size_t)s.lay.npc * c->q);
+    s.lay.scratch_off = take((size_t)(threads / G) * group_bytes(c->q, c->dmax, c->mb, c->mb == 1 && c->q >= 128));
+    s.lay.x_off = take((size_t)edges_r * c->q * c->mb);
+    return o;
+  };
+  auto blocks = [&](size_t smem) { return ((size_t)c->smem_optin + 1024) / (smem + kSplitTail + 1024); };
+  const size_t tight = lay_out(16), lines = lay_out(128);
+  const size_t o = lines > (size_t)c->smem_optin || blocks(lines) < blocks(tight) ? lay_out(16) : lines;
   if (o > (size_t)c->smem_optin) return SplitShape{};
   s.size = size;
   s.threads = threads;
