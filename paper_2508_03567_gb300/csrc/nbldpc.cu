@@ -991,6 +991,14 @@ static int batch_fpb(const nbldpc_job& j) {
   return batch_reg(j) ? reg_fpb(j.code) : default_fpb(j.code);
 }
 
+// Time (us) of a frame's longest decode alone on a block: ns per edge and iteration as measured on
+// GB300 (20 frames, two-block kernel: GF(4) N=400 5.0 us an iteration, GF(8) N=512 4.4, GF(16) N=1024
+// 12.7, GF(32) N=600 52, GF(64) N=576 65, GF(128) N=256 127, GF(256) (2,8) N=128 107), and 1.5 us.
+static double frame_us(const nbldpc_job& j) {
+  static const double ns[9] = {0, 6, 5, 6, 10, 30, 56, 250, 420};
+  return j.max_iters * (1.5 + 1e-3 * ns[nbldpc::ilog2(j.code->q)] * j.code->nnz);
+}
+
 // Convolution work of a frame's longest decode (pruned convolutions as a tenth).
 static double frame_work(const nbldpc_job& j) {
   const nbldpc_code* c = j.code;
@@ -1034,19 +1042,20 @@ static int batch_plan(const nbldpc_job* jobs, int n_jobs, Plan* pl, int* total) 
 
 // Shape of a mixed batch whose frames are each decoded on a cluster (size 0: one block per frame
 // slot): the ranks and threads of split_shape, the jobs' layouts one over the other.  Frames count
-// by their work against the longest ones' (an eighth at least; whole for q <= 8, which a cluster does not
-// shorten: 565 frames of GF(8) and GF(4) codes and 5 of GF(32) N=728 647 us on clusters, 358 on one block
-// each; 53 of GF(8) and 57 of GF(16) 195 and 132): one block per frame ends with the longest frames
-// alone.  Taken with early stop (the serving loop's groups) up to a number of such frames per SM that follows the widest field: q = 16 5/8; q = 32 two, below 1400 check-node lanes 3/4;
-// q = 64 four and q = 128 three, below 1400 lanes one and a half; q = 256 three, two and a half above
-// check degree 4 and one and a half from 8 on; without early stop 3/8; and eight frames of any kind.  Not
-// for q <= 8 alone, nor past 3/8 where the longest frames have fewer than 1024 lanes, nor there for
-// q <= 32 at all (and no more 128-thread ranks than lanes).  Measured on GB300, us per batch, the faster
-// one-block kernel against this: 60 / 240 / 450 frames of GF(64) N=576, GF(16) N=1024 and GF(256) N=128
-// in equal parts 2746 / 3455 / 3878 against 795 / 1444 / 2399; one frame of GF(64) 1243 against 179; 580 of GF(64) 2854
-// against 2558; beyond the limits 823 of GF(32) N=716 1100 against 1421, 947 of GF(128) N=138 1582
-// against 2020, 263 of GF(256) (2,8) N=280 3132 against 4940, 213 of two GF(32) codes of 1184 lanes
-// 300 against 372.
+// by their time against the longest ones' (an eighth at least; five times that for q <= 8, which a
+// cluster hardly shortens: 565 frames of GF(8) and GF(4) codes and 5 of GF(32) N=728 647 us on
+// clusters, 358 on one block each; but 406 of GF(4) N=194 with one of GF(256) N=180 and 75 others 499
+// and 1438): one block per frame ends with the longest frames alone.  Taken with early stop (the
+// serving loop's groups) up to a number of such frames per SM that follows the widest field: q = 16
+// 5/8; q = 32 two, below 1200 check-node lanes 3/4; q = 64 four and q = 128 three, below 1200 lanes
+// one and a half; q = 256 three, two and a half above check degree 4 and one and a half from 8 on;
+// without early stop 3/8; and eight frames of any kind.  Not for q <= 8 alone, nor past 3/8 where the
+// longest frames have fewer than 1024 lanes, nor there for q <= 32 at all (and no more 128-thread
+// ranks than lanes).  Measured on GB300, us per batch, the faster one-block kernel against this: 60 /
+// 240 / 450 frames of GF(64) N=576, GF(16) N=1024 and GF(256) N=128 in equal parts 2746 / 3455 / 3878
+// against 795 / 1444 / 2399; one frame of GF(64) 1243 against 179; 580 of GF(64) 2854 against 2558;
+// beyond the limits 823 of GF(32) N=716 1100 against 1421, 947 of GF(128) N=138 1582 against 2020,
+// 263 of GF(256) (2,8) N=280 3132 against 4940, 213 of two GF(32) codes of 1184 lanes 300 against 372.
 static int batch_split(const nbldpc_job* jobs, int n_jobs, int total, const Plan& pl, nbldpc::SplitBatchParams* p,
                        SplitShape* out) {
   if (any_pinned(jobs, n_jobs)) return 0;
@@ -1059,20 +1068,21 @@ static int batch_split(const nbldpc_job* jobs, int n_jobs, int total, const Plan
     if (jobs[i].frames > 0) {
       stop = stop && jobs[i].early_stop;
       q_most = std::max(q_most, jobs[i].code->q);
-      if (frame_work(jobs[i]) >= longest) {
-        longest = frame_work(jobs[i]);
+      if (frame_us(jobs[i]) >= longest) {
+        longest = frame_us(jobs[i]);
         lanes = jobs[i].code->m * group_lanes(jobs[i].code->q, mixed_layout(jobs[i].code->q));
         degree = jobs[i].code->dmax;
       }
     }
   if (q_most <= 8 || total > 8 * sms) return 0;
-  for (int i = 0; i < n_jobs; ++i)
-    like_longest += jobs[i].frames *
-                    (jobs[i].code->q <= 8 ? 1.0 : std::max(0.125, longest > 0.0 ? frame_work(jobs[i]) / longest : 1.0));
+  for (int i = 0; i < n_jobs; ++i) {
+    const double like = longest > 0.0 ? frame_us(jobs[i]) / longest : 1.0;
+    like_longest += jobs[i].frames * std::min(1.0, std::max(0.125, jobs[i].code->q <= 8 ? 5 * like : like));
+  }
   const int most_frames = !stop          ? 3 * sms / 8
                           : q_most <= 16  ? 5 * sms / 8
-                          : q_most <= 32  ? (lanes < 1400 ? 3 * sms / 4 : 2 * sms)
-                          : q_most <= 128 ? (lanes < 1400 ? 3 * sms / 2 : q_most <= 64 ? 4 * sms : 3 * sms)
+                          : q_most <= 32  ? (lanes < 1200 ? 3 * sms / 4 : 2 * sms)
+                          : q_most <= 128 ? (lanes < 1200 ? 3 * sms / 2 : q_most <= 64 ? 4 * sms : 3 * sms)
                           : degree <= 4   ? 3 * sms
                                           : (degree < 8 ? 5 : 3) * sms / 2;
   if (like_longest > most_frames || (lanes < 1024 && (q_most <= 32 || total > 3 * sms / 8))) return 0;
@@ -1110,27 +1120,29 @@ static int batch_split(const nbldpc_job* jobs, int n_jobs, int total, const Plan
 //    1,100 / 1,400 / 6,000 frames 4,406 / 5,520 / 19,957 against 4,537 / 5,686 / 19,672; GF(64) N=88,
 //    N=522 and N=232, 2,123 in all 2,340 against 2,791; GF(256) N=384, 2,000 39.4 against 39.2 ms; 532
 //    of GF(16) N=716, GF(64) N=126 and others 1,333 against 1,541.
-//  - Fields up to GF(8) gain little from it: where their rounds are not fewer than four thirds of the
+//  - Fields up to GF(16) gain little from it: where their rounds are not fewer than four thirds of the
 //    other kernel's, the third block wins (GF(8) (3,6) N=580, 361 frames 220 against 164; GF(2) N=534,
-//    1,290 697 against 612; 20 of GF(16) N=64 and 30 of GF(8) N=100 64 against 78).
+//    1,290 697 against 612; GF(16) N=308, 818 553 against 512, four GF(16) codes, 1,643 1,383 against 1,297;
+//    20 of GF(16) N=64 and 30 of GF(8) N=100 64 against 78), but for GF(16) frames that the three blocks
+//    take at once (436 of N=216 and N=272 266 against 319).
 //  - Fixed iterations: up to two and a half frames per SM (GF(64) N=576, 300 frames 939 against 979; 399
 //    of four GF(64) codes 649 against 730; GF(256) N=177, 416 2,982 against 2,588), and for GF(128) and
 //    GF(256) where rounds allow (GF(256) N=384, 600 frames 6,973 against 8,427).
 static bool batch_wide(const nbldpc_job* jobs, int n_jobs, int total, const Plan& pl) {
   bool stop = true;
-  double small = 0.0, middle = 0.0, large = 0.0;     // work of the fields up to GF(8), up to GF(64), above
+  double small = 0.0, q16 = 0.0, middle = 0.0, large = 0.0;   // work up to GF(8), of GF(16), up to GF(64), above
   for (int i = 0; i < n_jobs; ++i) {
     if (jobs[i].frames == 0) continue;
     stop = stop && jobs[i].early_stop;
     const int q = jobs[i].code->q;
-    (q <= 8 ? small : q <= 64 ? middle : large) += jobs[i].frames * frame_work(jobs[i]);
+    (q <= 8 ? small : q == 16 ? q16 : q <= 64 ? middle : large) += jobs[i].frames * frame_work(jobs[i]);
   }
   const long long want = (total + pl.fpb - 1) / pl.fpb, sms = pl.grid_max / pl.per_sm;
   const long long two = (want + 2 * sms - 1) / (2 * sms), three = (want + pl.grid_max - 1) / pl.grid_max;
   const bool fewer = three <= 3 && 3 * two < 4 * three;
-  if (small > middle + large) return fewer;
+  if (small + q16 > middle + large) return fewer || (q16 > small && stop && three == 1);
   if (stop) return three <= 6;
-  return 2 * want <= 5 * sms || (large > middle + small && fewer);
+  return 2 * want <= 5 * sms || (large > small + q16 + middle && fewer);
 }
 
 int nbldpc_decode_batch_workspace_size(const nbldpc_job* jobs, int n_jobs, size_t* bytes) {

@@ -343,7 +343,7 @@ def test_mixed_batches_leave_the_clusters_where_frames_fill_the_chip():
     """Frames per SM up to which a batch of one code decodes on clusters, by field, check-node lanes and check
     degree."""
     for q, n, dv, dc, per_sm in ((16, 1024, 2, 4, 0.625), (32, 600, 3, 6, 2), (32, 128, 2, 4, 0.75), (64, 576, 2, 4, 4),
-                                 (64, 160, 2, 4, 1.5), (128, 256, 2, 4, 3), (256, 192, 2, 4, 3), (256, 192, 2, 6, 2.5),
+                                 (64, 144, 2, 4, 1.5), (128, 256, 2, 4, 3), (256, 192, 2, 4, 3), (256, 192, 2, 6, 2.5),
                                  (256, 280, 2, 8, 1.5)):
         code = I.make_regular_code(q, n, dv, dc, seed=q + n, encoder=False)
         dec = binding.Decoder.from_code(code)
@@ -354,17 +354,17 @@ def test_mixed_batches_leave_the_clusters_where_frames_fill_the_chip():
             assert (binding.nbldpc_decode_batch_cluster_blocks([job]) > 0) == (frames <= 3 * sms() // 8)
 
 
-def test_frames_of_small_fields_do_not_take_clusters_for_the_sake_of_a_few():
-    """A few GF(32) or GF(16) frames among many of GF(8): one block per frame; the same few alone, and a few of
-    both, on clusters."""
-    codes = [I.workload_code("gf16_n1024_dv2_dc4"), irregular(8, 70, 33, 41, 6)]
-    decs = [binding.Decoder.from_code(c) for c in codes]
-    for counts, cluster in (((5, 0), True), ((5, 30), True), ((sms() // 3, sms() // 3), False), ((5, 2 * sms()), False)):
-        jobs = [(d.handle, None, f, 4, 1, None, None, None) for d, f in zip(decs, counts)]
+def test_frames_of_small_fields_on_clusters_for_the_sake_of_a_few():
+    """Many GF(8) frames as long as half of a GF(16) frame keep one block each with a few of those; many short
+    GF(4) frames follow a few GF(256) frames, which take a hundred times as long, onto clusters."""
+    a = [I.workload_code("gf16_n1024_dv2_dc4"), I.make_regular_code(8, 512, 2, 4, seed=520)]
+    b = [I.workload_code("gf256_n128_dv2_dc8"), irregular(4, 61, 31, 20, 6)]
+    for codes, counts, cluster in ((a, (5, 0), True), (a, (5, 30), True), (a, (sms() // 3, sms() // 3), False),
+                                   (a, (5, 2 * sms()), False), (b, (3, sms()), True)):
+        specs = [(c, random_gamma(c, f, f + c.q)) for c, f in zip(codes, counts)]
+        jobs, keep = batch(specs, 3, 1)
         assert (binding.nbldpc_decode_batch_cluster_blocks(jobs) > 0) == cluster, counts
-    specs = [(c, random_gamma(c, f, f)) for c, f in zip(codes, (5, 2 * sms()))]
-    jobs, keep = batch(specs, 4, 1)
-    check_batch(specs, jobs, keep, 4, 1)
+        check_batch(specs, jobs, keep, 3, 1)
 
 
 def test_gf4_codes_at_eight_frames_per_block():
