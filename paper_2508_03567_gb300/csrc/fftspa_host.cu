@@ -171,14 +171,14 @@ FftSplitShape fft_split_layout(const nbldpc_code* c, int size, int threads) {
 // throughput it is slower (GF(64) N=576, 4096 frames: 5.5 ms against 8.2 ms at
 // best), so it serves batches that leave SMs idle.  Measured on GB300, us per
 // decode of up to 20 iterations with early stop, one block against this rule:
-// GF(64) N=576, 1 / 48 / 200 frames 299 / 356 / 628 against 88 / 245 / 586; GF(16)
-// N=1024, 1 / 96 / 200 frames 299 / 304 / 400 against 116 / 235 / 357; GF(256) N=384,
-// 1 / 96 / 200 frames 1872 / 1881 / 2421 against 276 / 1054 / 2096.
+// GF(64) N=576, 1 / 48 / 200 frames 284 / 336 / 579 against 72 / 175 / 501; GF(16)
+// N=1024, 1 / 96 / 200 frames 283 / 285 / 343 against 97 / 182 / 293; GF(256) N=384,
+// 1 / 96 / 200 frames 1851 / 1851 / 2190 against 257 / 832 / 1668.
 //  - The fewer check-node lanes a frame has, the fewer frames: from 2000 on, one and
-//    a half frames per SM; from 1024 on, 3/8 (GF(256) (2,8) N=128, 48 / 96 frames:
-//    519 / 519 against 366 / 550); from 400 on, and in the lane-per-edge form, 1/8
-//    (GF(4) N=1024, 1 / 96 frames: 132 / 130 against 95 / 161), none below (GF(16)
-//    N=100, one frame: 72 against 80).  A lane of the lane-per-edge form has q products
+//    a half frames per SM; from 1024 on, 3/8 (GF(256) (2,8) N=128, 48 frames:
+//    499 against 301; 96 frames 519 against 550); from 400 on, and in the lane-per-edge form, 1/8
+//    (GF(4) N=1024, one frame: 113 against 75; 96 frames 130 against 161), none below
+//    (GF(16) N=100, one frame: 72 against 80).  A lane of the lane-per-edge form has q products
 //    and sums a pass: from 1024 lanes on at q <= 4 (GF(4) N=48, N=200, N=500, one frame:
 //    39, 44 and 69 against 60, 62 and 66; GF(2) N=200 (3,6) 51 against 72), from 512 on at
 //    GF(8) and GF(16) ((2,12) N=120, 320 lanes: 75 and 98 against 93 and 103; GF(16) N=240, 640
@@ -188,9 +188,10 @@ FftSplitShape fft_split_layout(const nbldpc_code* c, int size, int threads) {
 //    quarter, 4 up to 3/8 (one block, these, and 16 / 8 / 8 ranks, 5 iterations: GF(128)
 //    N=128, 19 / 42 / 57 frames 69, 47, 71 / 70, 66, 87 / 70, 70, 91; GF(64) N=256 70, 47,
 //    71 / 71, 63, 87 / 71, 66, 91; GF(256) (2,8) N=128 133, 77, 116 / 133, 105, 145 / 135,
-//    115, 155; below 2000 lanes at q = 128 none past a quarter: N=96 55, 60, 78) (96 frames of GF(64) N=576: 164 against 229), and for q <= 32 between
-//    one frame per SM and four thirds, which the one-block kernel takes in two
-//    waves (200 frames of GF(32) N=600, 5 iterations: 292 against 279).
+//    115, 155; below 2000 lanes at q = 128 none past a quarter: N=96 55, 60, 78), none above
+//    (96 frames of GF(64) N=576: 164 against 229), and for q <= 32 between one frame per SM
+//    and four thirds, which the one-block kernel takes in two waves (200 frames of GF(32)
+//    N=600, 5 iterations: 276 against 260).
 FftSplitShape fft_split_shape(const nbldpc_code* c, int frames, int early_stop) {
   if (c->fft_split_max == 0) return FftSplitShape{};
   const bool lane_form = c->fft_dc == 0;

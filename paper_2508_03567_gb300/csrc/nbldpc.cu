@@ -314,7 +314,7 @@ int make_plan(int kq, int kv, int km, int fpb, const CodeNeeds* cs, int nc, Plan
 // benchmark codes on GB300 (GF(8) to GF(64): layout 1 from GF(16) on, with the
 // messages in shared memory; GF(4): layout 0 with the messages in shared
 // memory; GF(128), GF(256): pruned convolutions, layout 0 (GF(256) (2,6) N=384:
-// 2.8x the dense kernel; GF(128) (2,4) N=256: 35.6 against 41.1 ms); otherwise
+// 3.2x the dense kernel; GF(128) (2,4) N=256: 35.6 against 41.1 ms); otherwise
 // layout 0).
 int default_variant(int q) { return q >= 128 ? 4 : (q >= 16 && q <= 64) ? 3 : q >= 4 ? 2 : 0; }
 
@@ -557,14 +557,14 @@ int split_resident(const nbldpc_code* c, const SplitShape& s) {
 //
 // One block per frame leaves SMs idle below their number, and with early stop
 // it leaves them idle at the end of a batch, when the last frames run all their
-// iterations (a GF(64) N=576 frame: 58 us an iteration on one SM, 9.5 us on
+// iterations (a GF(64) N=576 frame: 56 us an iteration on one SM, 6.4 us on
 // 16).  Measured on GB300, us per decode of up to 20 or 30 iterations, one
-// block per frame against this rule: GF(64) N=576, 1 / 96 / 200 / 1000 frames
-// 1103 / 1158 / 1937 / 3721 against 180 / 481 / 846 / 3299; GF(256) (2,6) N=384,
-// 1 / 96 / 200 frames 7328 / 7818 / 9626 against 689 / 3498 / 8051; GF(256) (2,8)
-// N=128, 17 frames 3939 against 1217; GF(32) N=600, 1 / 96 / 450 frames (register
-// form) 836 / 841 / 1576 against 171 / 439 / 1353; GF(16) N=1024, 1 / 48 frames
-// 235 / 236 against 116 / 182.
+// block per frame against this rule: GF(64) N=576, 1 / 96 / 200 frames
+// 1085 / 1142 / 1915 against 158 / 494 / 794; GF(256) (2,6) N=384 6080 / 6609 /
+// 8330 against 502 / 2206 / 4519; GF(256) (2,8) N=128, 17 frames 2135 against
+// 464; GF(32) N=600 (register form), 1 / 96 / 450 frames 814 / 814 / 1612
+// against 151 / 436 / 1357; GF(16) N=1024, 1 / 48 frames 213 / 215 against
+// 97 / 175.
 //  - More ranks and threads for fewer frames, so that the SMs are filled and the
 //    frame's chain of passes is as short as they allow.
 //  - No more 128-thread ranks than the frame has check-node lanes for.
@@ -583,9 +583,9 @@ int split_resident(const nbldpc_code* c, const SplitShape& s) {
 //    (GF(256): 400 frames of N=384 12.9 ms against 15.6); a third when
 //    every frame runs the same iterations (no tail: 1000 frames 7.1 ms against 7.7).
 //  - 16-bit messages: as many frames as the one-block kernels hold, half at q = 8
-//    (GF(64) N=576, 1 / 96 / 450 frames 1583 / 1655 / 3662 against 187 / 574 / 1910;
-//    GF(256) N=384, 200 frames 26.3 against 11.8 ms; GF(8) N=512, 200 / 450 frames
-//    243 / 271 against 184 / 324).
+//    (GF(64) N=576, 1 / 96 / 450 frames 1548 / 1629 / 3643 against 165 / 564 / 1890;
+//    GF(256) N=384, 200 frames 26.3 against 12.1 ms; GF(8) N=512, 200 frames
+//    217 against 167).
 SplitShape split_shape(const nbldpc_code* c, int frames, int early_stop) {
   if (c->split_max == 0 || c->pinned) return SplitShape{};
   const long long slots = (long long)c->plan.grid_max * c->plan.fpb;
